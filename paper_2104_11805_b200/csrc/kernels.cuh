@@ -50,8 +50,8 @@ struct Sliced {
     float*     val;
     const int* order;
     int idx16;
-    const int* out;         // forward kernels: tile row that unit u's output goes to (NULL: row u), for layers whose rows are
-                            // stored group by group while their neurons carry the numbers the next layer's grouping gave them
+    const int* out;         // tile row that stored row u stands for (NULL: row u): ragged layers, whose rows are stored by length,
+                            // and layers stored group by group (neurons numbered by the next layer's grouping)
 };
 
 __device__ __forceinline__ float4 ld_f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -497,6 +497,7 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
     int row, base, nch;
     SDNN_UNIT_SHAPE(m, unit, nunits, row, base, nch)
     float b = (row < n) ? bias[row] : 0.0f;
+    int to = (m.out && row < n) ? m.out[row] : row;       // tile row this row writes
     if (unit < nunits && lane == 0) prefetch_unit(m, unit, RPW, n, UPS);
     IdxChunk<I16> c[CPS];
 #pragma unroll
@@ -514,6 +515,7 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         int nrow, nbase, nnch;
         SDNN_UNIT_SHAPE(m, nunit, nunits, nrow, nbase, nnch)
         const float nb = (nrow < n) ? bias[nrow] : 0.0f;
+        const int nto = (m.out && nrow < n) ? m.out[nrow] : nrow;
         if (nunit < nunits && lane == 0) prefetch_unit(m, nunit, RPW, n, UPS);
 
         Lane<V> acc;
@@ -537,10 +539,10 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         if (nch == 0 && nnch > 0) load_idx<CPS, I16>(c, m, nbase);      // empty slice: nothing prefetched across the boundary yet
         if (row < n) {
             lane_activate(acc, act, clamp);
-            lane_store(tile_row(xout + boff, m.out ? m.out[row] : row, pitch), acc);      // regrouped layer: the neuron's tile row
+            lane_store(tile_row(xout + boff, to, pitch), acc);
             if (live_flags) live |= lane_nonzero_bits(acc);
         }
-        unit = nunit; row = nrow; base = nbase; nch = nnch; b = nb;
+        unit = nunit; row = nrow; base = nbase; nch = nnch; b = nb; to = nto;
     }
     if (live_flags) {
 #pragma unroll
@@ -1138,6 +1140,7 @@ forward_ep_kernel(Sliced m, const float* __restrict__ bias, const float* __restr
     IdxChunk<I16> c[EP_IT];
     SDNN_EP_LOAD_IDX(c, 0, EP_IT)
     const float b = (e.item < n) ? bias[e.item] : 0.0f;
+    const int to = (m.out && e.item < n) ? m.out[e.item] : e.item;
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
     Lane<4> acc;
@@ -1164,7 +1167,7 @@ forward_ep_kernel(Sliced m, const float* __restrict__ bias, const float* __restr
     if (e.h == 0 && e.item < n) {
         acc.a.x += b; acc.a.y += b; acc.a.z += b; acc.a.w += b;
         lane_activate(acc, act, clamp);
-        lane_store(xout + (size_t)(m.out ? m.out[e.item] : e.item) * 4, acc);
+        lane_store(xout + (size_t)to * 4, acc);
     }
     if (pdl == 1) grid_launch_dependents();
 }
@@ -1236,13 +1239,14 @@ backward_row_ep_kernel(Sliced m, float* __restrict__ bias, const float* __restri
     IdxChunk<I16> c[EP_IT];
     SDNN_EP_LOAD_IDX(c, 0, EP_IT)
     const int len = (e.item < n) ? m.len[e.item] : 0;
+    const int lab = (m.out && e.item < n) ? m.out[e.item] : e.item;
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
     const float inv_b = sp->inv_b;
     const float step = sp->eta * inv_b;
     Lane<4> d;
     lane_fill(d, 0.0f);
-    if (e.item < n) lane_load(d, dk + (size_t)(m.out ? m.out[e.item] : e.item) * 4);
+    if (e.item < n) lane_load(d, dk + (size_t)lab * 4);
     if (update_bias && e.h == 0 && e.item < n) bias[e.item] -= step * lane_sum(d);
     for (int t0 = 0; t0 < e.nch; t0 += 2 * EP_IT) {
         float4 w[EP_IT];
