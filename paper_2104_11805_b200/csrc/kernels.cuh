@@ -898,6 +898,7 @@ struct BackwardArgs {
     int act;                  // activation (ACT_*)
     int update_bias, skip_dead, pdl;
     int cols_only;            // MIRROR: leave the row units to a separate launch (which may run beside the next layer's column units)
+    int alternate;            // column units: see backward_col_units
     const float* warm;        // tile the NEXT backward launch will gather from (x^{k-2}), or NULL: asked into L2 now,
     unsigned warm_bytes;      // because it was written a whole forward pass ago and has left the cache
 };
@@ -906,7 +907,7 @@ struct BackwardArgs {
 template <int G, int V, int CPS, bool I16>
 __device__ __forceinline__ void backward_col_units(const Sliced m, const float* __restrict__ xprev, const float* __restrict__ dk,
                                                    float* __restrict__ dprev, int n, float clamp, int act, float step, float inv_b,
-                                                   int first, int stride, int pdl) {
+                                                   int first, int stride, int pdl, int alternate) {
     constexpr int RPW = 32 / G;
     constexpr int UPS = (RPW >= SLICE) ? 1 : SLICE / RPW;
     constexpr unsigned pitch = 4u * V * G;
@@ -918,7 +919,10 @@ __device__ __forceinline__ void backward_col_units(const Sliced m, const float* 
     float* val = m.val;
     const float* dg = dk + boff;
 
-    int u = first, item, base, nch;
+    // The columns come by descending length.  alternate: a warp that takes several units takes them from alternating ends of
+    // its rounds, so that every warp gets long and short columns (two units each, no row units beside them: 18.3 -> 17.3 us per
+    // layer at 65536 neurons and 16 inputs, 13.4 -> 12.8 at 16384 and 64; row units fill the tail as well and gain nothing by it)
+    int u = first, item, base, nch, round = 0;
     SDNN_UNIT_SHAPE(m, u, nunits, item, base, nch)
     if (u < nunits && lane == 0) prefetch_unit(m, u, RPW, n, UPS);
     int len = 0, j = 0;
@@ -935,7 +939,8 @@ __device__ __forceinline__ void backward_col_units(const Sliced m, const float* 
     if (pdl == 2) grid_launch_dependents();
 
     while (u < nunits) {
-        const int nu = u + stride;
+        ++round;
+        const int nu = round * stride + ((alternate & round & 1) ? stride - 1 - first : first);
         int nitem, nbase, nnch, nlen = 0, nj = 0;
         SDNN_UNIT_SHAPE(m, nu, nunits, nitem, nbase, nnch)
         if (nitem < n) { nlen = m.len[nitem]; nj = m.order[nitem]; }
@@ -1088,7 +1093,7 @@ backward_kernel(const BackwardArgs a) {
     // step parameters: written once per step, long before any backward launch
     const float inv_b = a.sp->inv_b;
     const float step = a.sp->eta * inv_b;
-    if (MIRROR) backward_col_units<G, V, CPS, I16>(a.cols, a.xprev, a.dk, a.dprev, a.n, a.clamp, a.act, step, inv_b, first, stride, a.pdl);
+    if (MIRROR) backward_col_units<G, V, CPS, I16>(a.cols, a.xprev, a.dk, a.dprev, a.n, a.clamp, a.act, step, inv_b, first, stride, a.pdl, a.alternate);
     else {
         if (a.pdl) grid_dependency_wait();
         if (a.pdl == 2) grid_launch_dependents();
@@ -1280,11 +1285,137 @@ backward_row_ep_kernel(Sliced m, float* __restrict__ bias, const float* __restri
 #undef SDNN_EP_LOAD_IDX
 
 // ---------------------------------------------------------------------------------------------
+// Update of the row-major copy from the transposed one.  The column units have just computed the layer's new values, so the
+// row-major copy only needs them moved: no second gather of x^{k-1} per entry, no second gradient, no old values.  Both copies
+// are cut into blocks of `block` consecutive elements, and the move is two passes through shared memory with a buffer T between
+// them, ordered by (block of the transposed copy, block of the row-major copy):
+//   split_values : a CTA reads one block of the transposed copy and writes its part of T (both contiguous)
+//   merge_values : a CTA collects its row-major block from the `nb` runs of T that belong to it (about 32 entries each: the
+//                  block size is chosen for that) and writes it
+// pos_a[t] / pos_b[t]: place of T's element t within its block of the transposed / row-major copy.  Nothing is scattered in
+// global memory: fetching each value by its 4-byte address instead costs a request per entry (about one per clock and SM,
+// 7 us for 2 M entries, and slower than the row units it would replace).  CTAs of 128 threads and at most 32 registers a
+// thread take the place of one one-warp CTA of the column units, beside which they run.
+struct Move {
+    const int* start;             // [nb * (nb + 1)] first element of run (block of the transposed copy, block of the row-major copy) in T
+    const int2* runs;             // [nb * nb] the same by row-major block: (first element, length)
+    const unsigned short* pos_a;
+    const unsigned short* pos_b;
+    int nb, block;
+};
+constexpr int MOVE_THREADS = 256;
+__global__ void __launch_bounds__(MOVE_THREADS, 4)
+split_values_kernel(Move m, const float* __restrict__ cval, int c_elems, float* __restrict__ T) {
+    extern __shared__ __align__(16) float move_smem[];
+    constexpr int AHEAD = 4;
+    const int cb = blockIdx.x, lo = cb * m.block, cnt = min(m.block, c_elems - lo);      // both multiples of 4
+    for (int q = threadIdx.x * 4; q < cnt; q += MOVE_THREADS * 4) cp_async16(move_smem + q, cval + lo + q);
+    cp_async_commit();
+    const int t0 = m.start[cb * (m.nb + 1)], t1 = m.start[cb * (m.nb + 1) + m.nb];      // t0 a multiple of 4; T is padded to one
+    ushort4 p[AHEAD];
+    bool waited = false;
+    for (int t = t0 + threadIdx.x * 4; __syncthreads_or(t < t1 || !waited); t += AHEAD * MOVE_THREADS * 4) {
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+            if (t + i * MOVE_THREADS * 4 < t1) p[i] = __ldcs(reinterpret_cast<const ushort4*>(m.pos_a + t + i * MOVE_THREADS * 4));
+        if (!waited) { cp_async_wait<0>(); __syncthreads(); waited = true; }
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+            if (t + i * MOVE_THREADS * 4 < t1)
+                st_f4(T + t + i * MOVE_THREADS * 4, make_float4(move_smem[p[i].x], move_smem[p[i].y], move_smem[p[i].z], move_smem[p[i].w]));
+    }
+}
+__global__ void __launch_bounds__(MOVE_THREADS, 4)
+merge_values_kernel(Move m, const float* __restrict__ T, float* __restrict__ rval, int r_elems) {
+    extern __shared__ __align__(16) float move_smem[];
+    constexpr int TEAMS = MOVE_THREADS / 16, RUNS = 4, DEEP = 3;                        // 16 threads share a run; 12 elements in flight per thread
+    int2* runs = reinterpret_cast<int2*>(move_smem + m.block);
+    const int rb = blockIdx.x, lo = rb * m.block, cnt = min(m.block, r_elems - lo);
+    const int sub = threadIdx.x & 15, team = threadIdx.x >> 4;
+    for (int q = threadIdx.x; q < m.nb; q += MOVE_THREADS) runs[q] = m.runs[(size_t)rb * m.nb + q];
+    for (int q = threadIdx.x * 4; q < cnt; q += MOVE_THREADS * 4) st_f4(move_smem + q, make_float4(0.f, 0.f, 0.f, 0.f));      // padding
+    __syncthreads();
+    for (int cb = team; cb < m.nb; cb += TEAMS * RUNS) {
+        int2 r[RUNS];
+        float v[RUNS * DEEP];
+        unsigned short at[RUNS * DEEP];
+#pragma unroll
+        for (int u = 0; u < RUNS; ++u) {
+            r[u] = cb + u * TEAMS < m.nb ? runs[cb + u * TEAMS] : make_int2(0, 0);
+#pragma unroll
+            for (int d = 0; d < DEEP; ++d)
+                if (sub + 16 * d < r[u].y) {
+                    v[u * DEEP + d] = T[r[u].x + sub + 16 * d];
+                    at[u * DEEP + d] = __ldcs(m.pos_b + r[u].x + sub + 16 * d);
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < RUNS; ++u) {
+#pragma unroll
+            for (int d = 0; d < DEEP; ++d)
+                if (sub + 16 * d < r[u].y) move_smem[at[u * DEEP + d]] = v[u * DEEP + d];
+            for (int q = sub + 16 * DEEP; q < r[u].y; q += 16) move_smem[m.pos_b[r[u].x + q]] = T[r[u].x + q];
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x * 4; q < cnt; q += MOVE_THREADS * 4) __stcs(reinterpret_cast<float4*>(rval + lo + q), ld_f4(move_smem + q));
+}
+// Set-up of a Move, from `from` (place in the transposed copy of each element of the row-major copy, -1: padding): run
+// lengths, run starts (each block of the transposed copy begins at a multiple of 4 in T), places.
+__global__ void move_count_kernel(const int* __restrict__ from, int r_elems, int block, int nb, int* __restrict__ count) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < r_elems; e += gridDim.x * blockDim.x)
+        if (from[e] >= 0) atomicAdd(count + (from[e] / block) * nb + e / block, 1);
+}
+__global__ void __launch_bounds__(1024) move_starts_kernel(int* __restrict__ count, int nb, int* __restrict__ start, int2* __restrict__ runs) {
+    __shared__ int first[1025];
+    const int cb = threadIdx.x;                                                         // nb <= 1024
+    int total = 0;
+    if (cb < nb) for (int rb = 0; rb < nb; ++rb) total += count[cb * nb + rb];
+    if (cb < nb) first[cb + 1] = (total + 3) / 4 * 4;
+    __syncthreads();
+    if (cb == 0) { first[0] = 0; for (int q = 1; q <= nb; ++q) first[q] += first[q - 1]; }
+    __syncthreads();
+    if (cb >= nb) return;
+    int at = first[cb];
+    for (int rb = 0; rb < nb; ++rb) {
+        const int c = count[cb * nb + rb];
+        start[cb * (nb + 1) + rb] = at; runs[(size_t)rb * nb + cb] = make_int2(at, c);
+        count[cb * nb + rb] = at;                                                       // from here on: cursor of the run
+        at += c;
+    }
+    start[cb * (nb + 1) + nb] = at;
+}
+__global__ void move_places_kernel(const int* __restrict__ from, int r_elems, int block, int nb, int* __restrict__ cursor,
+                                   unsigned short* __restrict__ pos_a, unsigned short* __restrict__ pos_b) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < r_elems; e += gridDim.x * blockDim.x) {
+        const int p = from[e];
+        if (p < 0) continue;
+        const int t = atomicAdd(cursor + (p / block) * nb + e / block, 1);
+        pos_a[t] = (unsigned short)(p % block); pos_b[t] = (unsigned short)(e % block);
+    }
+}
+
+// b^k -= step * sum over the batch of delta^k (biases trained: read as one more column of W^k whose input is the constant 1).
+// A thread per stored row; the padding columns of delta are zero.
+__global__ void __launch_bounds__(256)
+update_bias_kernel(float* __restrict__ bias, const float* __restrict__ dk, const int* __restrict__ out, int n, int ld,
+                   const StepParams* __restrict__ sp) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= n) return;
+    const float* d = dk + (size_t)(out ? out[row] : row) * ld;
+    float s = 0.0f;
+    for (int b = 0; b < ld; b += 4) { const float4 v = ld_f4(d + b); s += (v.x + v.y) + (v.z + v.w); }
+    bias[row] -= sp->eta * sp->inv_b * s;
+}
+
+// ---------------------------------------------------------------------------------------------
 // Fills the transposed copy's values from the row-major copy: entry (column j, row i) of the transposed
 // copy is looked up by binary search in row i (ascending columns).  One warp per transposed unit.
 // With `mismatch` non-NULL nothing is written; entries whose bits differ from the row-major copy are counted.
-// row_of (or NULL): stored row of the row-major copy that holds neuron i, for layers whose rows were regrouped.
-__global__ void mirror_values_kernel(Sliced rows, Sliced cols, int n, unsigned long long* mismatch, const int* __restrict__ row_of) {
+// row_of (or NULL): stored row of the row-major copy that holds neuron i, for layers whose rows are not in neuron order.
+// from (or NULL): also notes where each entry of the row-major copy has its twin in the transposed one (see Move).
+__global__ void mirror_values_kernel(Sliced rows, Sliced cols, int n, unsigned long long* mismatch, const int* __restrict__ row_of,
+                                     int* __restrict__ from) {
     const int cc = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (cc >= n) return;
     const int len = cols.len[cc];
@@ -1303,6 +1434,7 @@ __global__ void mirror_values_kernel(Sliced rows, Sliced cols, int n, unsigned l
         }
         if (at < 0) { if (mismatch) atomicAdd(mismatch, 1ull << 32); continue; }     // pattern error: high word
         const float w = rows.val[rb + (at >> 2) * CHUNK_ROW + (at & 3)];
+        if (from) from[rb + (at >> 2) * CHUNK_ROW + (at & 3)] = pos;
         if (mismatch) {
             if (__float_as_uint(w) != __float_as_uint(cols.val[pos])) atomicAdd(mismatch, 1ull);
         } else {

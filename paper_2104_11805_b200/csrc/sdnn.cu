@@ -61,6 +61,7 @@ struct LayerMem {
     bool r_chunks_mult4 = false;           // every slice of the row-major copy has a multiple of 4 chunks
     int* r_idx = nullptr; float* r_val = nullptr; float* r_grad = nullptr;
     int* c_idx = nullptr; float* c_val = nullptr;
+    Move move{};                           // how r_val is filled from c_val after an update (nb = 0: row units compute theirs)
     std::vector<int> r_slice_off;          // host copy of the row-major slice offsets
     RowShape shape;
     // set-up reordering (SDNN_FLAG_REORDER): how the stored rows and entries map back to the caller's CSR arrays
@@ -116,10 +117,12 @@ struct sdnn {
     float* d_dl = nullptr;              // delta^L tile (atomics realisation)
     float* d_delta_all = nullptr;       // split backward: [L][N][ld], every delta^k of the step
     bool split = false;                 // transposed realisation with the row units as launches of their own on side streams
-    static constexpr int MAX_SIDE = 2;
-    cudaStream_t side_streams[MAX_SIDE] = {nullptr, nullptr};   // the row-unit launches alternate between these
-    cudaEvent_t ev_side_join[MAX_SIDE] = {nullptr, nullptr};
+    static constexpr int MAX_SIDE = 4, ROW_SIDE = 2;
+    cudaStream_t side_streams[MAX_SIDE] = {};           // row-unit launches alternate between the first two, moves between all
+    cudaEvent_t ev_side_join[MAX_SIDE] = {};
     int n_side = 0;
+    float* d_move[MAX_SIDE] = {};       // T of split_values_kernel / merge_values_kernel
+    size_t move_elems[MAX_SIDE] = {};
     cudaStream_t launch_stream = nullptr;     // where launch_k currently enqueues (NULL = stream)
     std::vector<cudaEvent_t> ev_delta;  // [L] delta^k (0-based layer) complete
     cudaEvent_t ev_fork = nullptr;
@@ -172,6 +175,7 @@ struct sdnn {
     int64_t stage_idx_cap = 0;
 
     std::map<std::tuple<const void*, int, int>, std::pair<int, int>> plans;   // (kernel, units, chunks) -> (grid.x, block)
+    std::map<const void*, bool> carved;                                       // kernels given the shared-memory split of the move kernels
     std::map<std::pair<const void*, int>, int> occupancy;                     // (kernel, block) -> resident CTAs per SM
 
     int64_t launches = 0;
@@ -441,6 +445,16 @@ Sliced cols_of(sdnn* h, int layer) {
     return m;
 }
 
+// Gives a kernel that runs beside the move kernels their split of an SM's memory between L1 and shared memory: an SM changes
+// the split only when it is empty, so that kernels with different ones take turns instead of running side by side (65536
+// neurons, 64 inputs: backward 60 us per layer without this, 52 with it; the gathers do not miss the L1).
+constexpr int MOVE_SMEM_KB = 100;
+void carve(sdnn* h, const void* kernel) {
+    if (h->carved[kernel]) return;
+    h->carved[kernel] = true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, MOVE_SMEM_KB * 100 / 228) != cudaSuccess) cudaGetLastError();
+}
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_k(sdnn* h, void (*kernel)(KArgs...), dim3 grid, dim3 block, bool pdl, Args... args) {
     cudaLaunchConfig_t lc = {};
@@ -593,6 +607,15 @@ void launch_forward_window(sdnn* h, int layer, const float* xin, float* xout, in
     count_launch(h);
 }
 
+// Whether the row-major copy of a layer gets its new values moved from the transposed one (see Move in kernels.cuh) instead of
+// computing them in row units.  A row unit's gather costs by its bytes from 128-byte rows on, a move the same at any
+// width, and two short launches must be worth their own round trips.  Backward us per layer, row units / move: 4096 neurons, 32
+// inputs 5.0 / 5.5, 128 inputs 9.2 / 8.4; 16384 neurons, 16 inputs 8.5 / 9.8, 32 inputs 9.1 / 8.6, 64 inputs 16.8 / 13.8, 128
+// inputs 33.5 / 25.3; 65536 neurons, 16 inputs 23.2 / 23.5, 32 inputs 32.3 / 29.1, 64 inputs 66.1 / 52.0.
+constexpr int MOVE_WIDTH = 32;
+constexpr int64_t MOVE_WORK = 8 << 20;      // stored elements x padded batch
+bool moves(const LayerMem& lm, int ld) { return ld >= MOVE_WIDTH && lm.r_elems * ld >= MOVE_WORK; }
+
 // delta tile of layer `layer` (0-based; the paper's delta^{layer+1}) in the transposed realisation
 float* delta_tile(sdnn* h, int layer, size_t tile) {
     if (h->d_dbg_delta) return h->d_dbg_delta + (size_t)layer * tile;
@@ -637,6 +660,7 @@ void launch_backward_gvc(sdnn* h, int layer, int ld, int part) {
         } else {                                                                               \
             auto plan = plan_grid(h, (const void*)backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>, units, 1, os_);  \
             if (a.pdl && (plan.first <= h->sms || MIR)) a.pdl = PDL_EARLY;                     \
+            if (part != 0 && h->lay[layer].move.nb > 0) carve(h, (const void*)backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>); \
             launch_k(h, backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>, dim3(plan.first), dim3(plan.second), a.pdl != 0, a); \
         }                                                                                      \
     } while (0)
@@ -646,6 +670,7 @@ void launch_backward_gvc(sdnn* h, int layer, int ld, int part) {
             a.cols = cols_of(h, layer);
             a.dprev = delta_tile(h, layer - 1, tile);
             a.cols_only = part == 1 ? 1 : 0;
+            a.alternate = a.cols_only && h->lay[layer].move.nb > 0 && moves(h->lay[layer], ld) ? 1 : 0;
             SDNN_BWD(false, false, true);
         } else if (part != 1) {
             if (part == 2) { a.pdl = 0; a.warm = nullptr; }
@@ -712,6 +737,23 @@ void launch_backward_i(sdnn* h, int layer, int ld, int part) {
     count_launch(h);
 }
 
+// Row-major copy of a layer whose transposed copy the column units have just updated (see Move), on side stream `side`.
+void launch_move(sdnn* h, int layer, int ld, int side) {
+    const LayerMem& lm = h->lay[layer];
+    const Move& m = lm.move;
+    const size_t smem = (size_t)m.block * sizeof(float);
+    carve(h, (const void*)split_values_kernel);
+    carve(h, (const void*)merge_values_kernel);
+    split_values_kernel<<<m.nb, MOVE_THREADS, smem, h->launch_stream>>>(m, (const float*)lm.c_val, (int)lm.c_elems, h->d_move[side]);
+    merge_values_kernel<<<m.nb, MOVE_THREADS, smem + (size_t)m.nb * sizeof(int2), h->launch_stream>>>(m, (const float*)h->d_move[side], lm.r_val, (int)lm.r_elems);
+    count_launch(h, 2);
+    if (h->cfg.update_bias) {
+        update_bias_kernel<<<(h->N + 255) / 256, 256, 0, h->launch_stream>>>(h->d_bias + (size_t)layer * h->N, (const float*)delta_tile(h, layer, (size_t)h->N * ld),
+                                                                           (const int*)lm.r_out, h->N, ld, (const StepParams*)h->d_sp);
+        count_launch(h);
+    }
+}
+
 void launch_backward(sdnn* h, int layer, int ld, int part = 0) {
     if (h->idx16) launch_backward_i<true>(h, layer, ld, part);
     else launch_backward_i<false>(h, layer, ld, part);
@@ -737,22 +779,27 @@ void launch_transpose_in(sdnn* h, const float* src, float* dst, int cnt, int col
 // backward chain of one train step over tiles of padded width ld
 void enqueue_backward_chain(sdnn* h, int ld) {
     if (h->split) {
-        // column units chain on the main stream; the row units of layer k only need delta^k and x^{k-1}, so they run on
-        // the side streams beside the column units of the layers below
+        // Column units chain on the main stream.  The update of the row-major copy runs on the side streams beside the column
+        // units of the layers below: moved over from the transposed copy once the layer's own column units are done, or (first
+        // layer, which has no transposed copy, and handles that keep the gradient) computed by row units, which need only
+        // delta^k and x^{k-1}.
         cudaEventRecord(h->ev_fork, h->stream);
         for (int q = 0; q < h->n_side; ++q) cudaStreamWaitEvent(h->side_streams[q], h->ev_fork, 0);
         cudaEventRecord(h->ev_delta[h->L - 1], h->stream);
         for (int k = h->L - 1; k >= 0; --k) {
             NvtxRange pass("backward layer", k + 1);
-            cudaStream_t side = h->side_streams[k % h->n_side];
-            cudaStreamWaitEvent(side, h->ev_delta[k], 0);
-            h->launch_stream = side;
-            launch_backward(h, k, ld, 2);
-            h->launch_stream = nullptr;
+            const bool move = h->lay[k].move.nb > 0 && moves(h->lay[k], ld);
+            const int q = k % (move ? h->n_side : sdnn::ROW_SIDE);
             if (k > 0) {
                 launch_backward(h, k, ld, 1);
                 cudaEventRecord(h->ev_delta[k - 1], h->stream);
             }
+            cudaStream_t side = h->side_streams[q];
+            cudaStreamWaitEvent(side, h->ev_delta[move ? k - 1 : k], 0);
+            h->launch_stream = side;
+            if (move) launch_move(h, k, ld, q);
+            else launch_backward(h, k, ld, 2);
+            h->launch_stream = nullptr;
         }
         for (int q = 0; q < h->n_side; ++q) {
             cudaEventRecord(h->ev_side_join[q], h->side_streams[q]);
@@ -1109,10 +1156,12 @@ int convert_values(sdnn* h, int layer) {
     return SDNN_OK;
 }
 
-int refresh_mirror(sdnn* h, int layer, unsigned long long* mismatch_dev) {
+// `from`: also notes the place of every row-major entry's twin (see mirror_values_kernel)
+int refresh_mirror(sdnn* h, int layer, unsigned long long* mismatch_dev, int* from = nullptr) {
     const int wpb = 8;
     mirror_values_kernel<<<(h->N + wpb - 1) / wpb, wpb * 32, 0, h->stream>>>(rows_of(h, layer), cols_of(h, layer), h->N, mismatch_dev,
-                                                                             (const int*)h->lay[layer].r_row_of);
+                                                                             (const int*)h->lay[layer].r_row_of,
+                                                                             from);
     CU(h, cudaGetLastError());
     return SDNN_OK;
 }
@@ -1135,6 +1184,44 @@ int upload_indices(sdnn* h, int* dst, const std::vector<int>& src) {      // syn
     for (int64_t q = 0; q < (int64_t)src.size(); ++q) narrow[(size_t)q] = (unsigned short)src[(size_t)q];
     CU(h, cudaMemcpyAsync(dst, narrow.data(), narrow.size() * sizeof(unsigned short), cudaMemcpyHostToDevice, h->stream));
     CU(h, cudaStreamSynchronize(h->stream));
+    return SDNN_OK;
+}
+
+// Fills the transposed copy's values and, where the row-major copy is to be updated from them (see Move), lays down the
+// maps for that.  Blocks of 2^k elements (256 .. 8192: at most 32 KB of shared memory) so that a run has about 32 entries.
+// Not with the gradient kept for inspection, which the row units record; and not beyond 1024 blocks (8 M stored elements a
+// layer), where runs would get long tables: there the row units compute the update themselves.
+int build_move(sdnn* h, int layer) {
+    LayerMem& lm = h->lay[layer];
+    const int64_t most = std::max(lm.r_elems, lm.c_elems);
+    int block = 256;
+    while (block < 8192 && (int64_t)block * block < 24 * most) block *= 2;
+    const int nb = (int)((most + block - 1) / block);
+    if (!h->split || lm.r_grad || !moves(lm, h->ld_max) || nb < 1 || nb > 1024) return refresh_mirror(h, layer, nullptr);
+    int rc;
+    int *from = nullptr, *start = nullptr;
+    int2* runs = nullptr;
+    unsigned short* pos[2] = {nullptr, nullptr};
+    const size_t t_elems = (size_t)h->nnz[layer] + 4 * (size_t)nb;
+    if ((rc = dev_alloc(h, &start, (size_t)nb * (nb + 1), false)) || (rc = dev_alloc(h, &runs, (size_t)nb * nb, false)) ||
+        (rc = dev_alloc(h, &pos[0], t_elems, true)) || (rc = dev_alloc(h, &pos[1], t_elems, true))) return rc;
+    for (int q = 0; q < h->n_side; ++q)
+        if (t_elems > h->move_elems[q]) {      // one T per side stream, grown to the largest layer
+            if ((rc = dev_alloc(h, &h->d_move[q], t_elems, false))) return rc;
+            h->move_elems[q] = t_elems;
+        }
+    CU(h, cudaMallocAsync((void**)&from, (size_t)(lm.r_elems + (int64_t)nb * nb) * sizeof(int), h->stream));
+    int* count = from + lm.r_elems;
+    CU(h, cudaMemsetAsync(from, 0xff, (size_t)lm.r_elems * sizeof(int), h->stream));
+    CU(h, cudaMemsetAsync(count, 0, (size_t)nb * nb * sizeof(int), h->stream));
+    if ((rc = refresh_mirror(h, layer, nullptr, from))) return rc;
+    const int grid = (int)std::min<int64_t>((lm.r_elems + 255) / 256, 8 * (int64_t)h->sms);
+    move_count_kernel<<<grid, 256, 0, h->stream>>>(from, (int)lm.r_elems, block, nb, count);
+    move_starts_kernel<<<1, 1024, 0, h->stream>>>(count, nb, start, runs);
+    move_places_kernel<<<grid, 256, 0, h->stream>>>(from, (int)lm.r_elems, block, nb, count, pos[0], pos[1]);
+    CU(h, cudaFreeAsync(from, h->stream));
+    CU(h, cudaGetLastError());
+    lm.move = Move{start, runs, pos[0], pos[1], nb, block};
     return SDNN_OK;
 }
 
@@ -1258,7 +1345,7 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
         CU(h, cudaMemcpyAsync(h->d_c_len + (size_t)layer * N, c_len.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         CU(h, cudaMemcpyAsync(h->d_c_order + (size_t)layer * N, order.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         if (lm.c_elems && (rc = upload_indices(h, lm.c_idx, c_idx))) return rc;
-        if ((rc = refresh_mirror(h, layer, nullptr))) return rc;
+        if ((rc = build_move(h, layer))) return rc;      // fills the transposed copy's values too
     }
     CU(h, cudaStreamSynchronize(h->stream));   // the host vectors above go out of scope; the caller may reuse its arrays
     {
@@ -1615,7 +1702,9 @@ int sdnn_create_deferred(sdnn_t** out, int32_t n_layers, int32_t n_neurons, cons
         h->split = h->mirror && !(cfg->flags & SDNN_FLAG_BWD_ONE_LAUNCH);
         if (h->split) {
             if (!(cfg->flags & SDNN_FLAG_KEEP_DEBUG) && (rc = dev_alloc(h, &h->d_delta_all, L * tile, true))) return bail(rc);
-            h->n_side = 2;      // row-unit launches of neighbouring layers do not depend on each other: two streams let them overlap
+            // row-unit launches of neighbouring layers do not depend on each other: two streams let them overlap; a move is
+            // two short launches in a row, mostly round trips beside a saturated load path: four streams
+            h->n_side = h->ld_max >= MOVE_WIDTH ? sdnn::MAX_SIDE : sdnn::ROW_SIDE;
             for (int q = 0; q < h->n_side; ++q) {
                 if ((e = cudaStreamCreateWithFlags(&h->side_streams[q], cudaStreamNonBlocking)) != cudaSuccess) return bail(cuda_fail(h, e, "cudaStreamCreate"));
                 if ((e = cudaEventCreateWithFlags(&h->ev_side_join[q], cudaEventDisableTiming)) != cudaSuccess) return bail(cuda_fail(h, e, "cudaEventCreate"));

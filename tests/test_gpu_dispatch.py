@@ -3,7 +3,8 @@ smallest and largest nets of a rule's range, each against the float64 oracle."""
 import numpy as np
 import pytest
 
-from parity_util import ragged_net
+from oracle import OracleNet
+from parity_util import check_close, ragged_net
 from test_gpu_parity import BWD_MODES, infer_parity, sdnn, torch_cuda, train_parity  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -23,3 +24,36 @@ def test_ragged_rows_stored_by_length(torch_cuda, n, B):  # noqa: F811
     train_parity(torch_cuda, arrays, [(vectors(rng, B, n), vectors(rng, B, n)) for _ in range(2)], eta=0.02, update_bias=True,
                  activation="sigmoid", expect_live=True)
     infer_parity(torch_cuda, arrays, vectors(rng, 3 * B, n), 2 * B, expect_nonempty=True)
+
+
+@pytest.mark.parametrize("n,k,B", [(4097, 48, 100), (1500, 300, 33), (8200, 32, 33)])
+def test_row_major_copy_moved_from_the_transposed_one(torch_cuda, n, k, B):  # noqa: F811
+    """Layers large enough to have their row-major copy filled from the transposed one after an update (blocks of 2048 to 4096
+    elements, the last one partial, ragged rows and columns), two steps of one handle at the full batch and one at a batch
+    narrow enough for row units, against the oracle; both copies hold the same bits."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n)
+    rps, cols, vals, biases = [], [], [], []
+    for _ in range(2):
+        length = rng.integers(0, 2 * k, size=n)
+        rp = np.zeros(n + 1, dtype=np.int32)
+        rp[1:] = np.cumsum(length)
+        cols.append(np.concatenate([np.sort(rng.choice(n, size=m, replace=False)) for m in length]).astype(np.int32))
+        rps.append(rp)
+        vals.append((rng.standard_normal(rp[-1]) * 0.1).astype(np.float32))
+        biases.append((rng.standard_normal(n) * 0.1).astype(np.float32))
+    h = pkg.Sdnn.create(rps, cols, vals, biases, max_batch=B, train=True, update_bias=True, activation=pkg.ACT_SIGMOID)
+    ora = OracleNet(rps, cols, vals, biases, update_bias=True, activation="sigmoid")
+    for b in (B, B, 5):
+        ora.quantize_state()
+        for l in range(2):
+            h.set_weights(l, ora.w[l], ora.bias[l])
+        x0, y = vectors(rng, b, n), vectors(rng, b, n)
+        h.train_step(torch.from_numpy(x0).cuda(), torch.from_numpy(y).cuda(), b, 0.5)
+        ora.train_step(x0, y, 0.5, keep=())
+        for l in range(2):
+            w, bias = h.get_weights(l)
+            check_close(w, ora.w[l], f"W^{l + 1} at B = {b}")
+            check_close(bias, ora.bias[l], f"b^{l + 1} at B = {b}")
+            assert h.mirror_mismatches(l) == 0
+    h.destroy()
