@@ -4,6 +4,7 @@
 // arithmetic step runs in the kernels of kernels.cuh.
 #include "../../include/sdnn.h"
 #include "kernels.cuh"
+#include "vector.cuh"
 #include "reorder.h"
 
 #include <nvtx3/nvToolsExt.h>
@@ -14,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <tuple>
@@ -156,6 +158,9 @@ struct sdnn {
     int* d_in_label = nullptr;          // [N] tile row of input neuron i (NULL: identity)
     std::vector<std::vector<int>> labels;   // [L + 1] host: tile row of neuron i at boundary k (x^k, delta^k); empty = identity
     int windowed_layers = 0;
+    VectorLayer* d_vector = nullptr;    // [L] table of vector_infer_kernel (NULL: the net is not for it)
+    int vector_kpad = 0;                // entries per row of every slice of every layer (the same everywhere, or no table)
+    int* vector_status = nullptr;       // pinned: raised by a whole-network kernel whose wait for its neighbours ran out
     bool compaction = false;            // SDNN_FLAG_SKIP_DEAD asked for; effective while no bias is positive
     std::vector<char> bias_nonpositive; // per layer
     bool live_valid = false;
@@ -1006,6 +1011,113 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     return SDNN_OK;
 }
 
+// ---------------------------------------------------------------------------------------------
+// Whole networks in one launch for one to four inputs (vector.cuh): nets whose rows all have the same padded length, up to 4096
+// neurons x (padded) inputs.  120 layers of 1024 neurons, one launch per layer / one launch: 1 input 255 / 121 us, 4 inputs 252 /
+// 176; 60 layers of 2048: 1 input 143 / 98, 4 inputs 142 / 159; of 4096: 1 input 149 / 156, 2 inputs 149 / 195.  And it leaves 132
+// SMs to other handles: three of them asked in turn answer an input in 47 us each instead of 240 (1024 x 120).
+constexpr int VECTOR_WORK = 4096, VECTOR_DEPTH = 2048;
+
+// Status words that kernels raise and the host reads without waiting: one page of pinned memory for all handles (pinning one
+// takes longer than loading a small net), given back when the last of them goes.
+struct StatusPage {
+    static constexpr int WORDS = 1024;
+    std::mutex mutex;
+    int* words = nullptr;
+    std::vector<char> taken;
+    int users = 0;
+    int* get() {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (!words) {
+            if (cudaHostAlloc((void**)&words, WORDS * sizeof(int), cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); words = nullptr; return nullptr; }
+            taken.assign(WORDS, 0);
+        }
+        for (int q = 0; q < WORDS; ++q)
+            if (!taken[q]) { taken[q] = 1; ++users; words[q] = 0; return words + q; }
+        return nullptr;
+    }
+    void put(int* p) {
+        std::lock_guard<std::mutex> lock(mutex);
+        taken[p - words] = 0;
+        if (--users == 0) { cudaFreeHost(words); words = nullptr; }
+    }
+};
+StatusPage& status_page() { static StatusPage page; return page; }
+
+// table of layer pointers (called by sdnn_finalize)
+int build_vector(sdnn* h) {
+    if (h->reorder || h->compaction || !h->idx16 || h->N > VECTOR_WORK || h->L > VECTOR_DEPTH) return SDNN_OK;
+    int rc;
+    std::vector<VectorLayer> table(h->L);
+    for (int k = 0; k < h->L; ++k) {
+        const LayerMem& lm = h->lay[k];
+        const int kpad = lm.r_slice_off[1] / SLICE;
+        if (lm.r_out || kpad == 0 || (k > 0 && kpad != h->vector_kpad)) return SDNN_OK;
+        for (int sl = 0; sl < h->NS; ++sl) if (lm.r_slice_off[sl + 1] - lm.r_slice_off[sl] != kpad * SLICE) return SDNN_OK;
+        table[k] = VectorLayer{reinterpret_cast<const unsigned short*>(lm.r_idx), lm.r_val};
+        h->vector_kpad = kpad;
+    }
+    if (!(h->vector_status = status_page().get())) return SDNN_OK;      // no word left: the launches per layer do it
+    if ((rc = dev_alloc(h, &h->d_vector, (size_t)h->L, false))) return rc;
+    CU(h, cudaMemcpyAsync(h->d_vector, table.data(), table.size() * sizeof(VectorLayer), cudaMemcpyHostToDevice, h->stream));
+    CU(h, cudaStreamSynchronize(h->stream));
+    return SDNN_OK;
+}
+
+int vector_check(sdnn* h) {
+    if (!h->vector_status || !*h->vector_status) return SDNN_OK;
+    *h->vector_status = 0;
+    return fail(h, SDNN_ERR_CUDA, "a whole-network launch gave up waiting for its neighbours: the results of that call are not valid");
+}
+
+// shared memory of vector_infer_kernel<v> without its ring of entries, and a stage of the ring
+size_t vector_smem(const sdnn* h, int v, size_t* stage) {
+    const size_t blocks = (h->N + VECTOR_CTAS * VECTOR_BLOCK - 1) / (VECTOR_CTAS * VECTOR_BLOCK);
+    *stage = blocks * VECTOR_BLOCK * (size_t)h->vector_kpad * 6;
+    return 2 * (((size_t)h->N * v * 4 + 15) & ~(size_t)15) + 2 * blocks * VECTOR_BLOCK * v * 4 + (size_t)h->L * sizeof(VectorLayer) + 128;
+}
+constexpr size_t VECTOR_SMEM = 226 * 1024;
+// stages of the ring that fit; below three a layer's entries would be waited for
+int vector_stages(const sdnn* h, int v) {
+    size_t stage = 0;
+    const size_t base = vector_smem(h, v, &stage);
+    return base >= VECTOR_SMEM ? 0 : (int)std::min<size_t>(VECTOR_STAGES, (VECTOR_SMEM - base) / stage);
+}
+
+template <int V>
+int launch_vector(sdnn* h, VectorArgs a) {
+    size_t stage = 0;
+    const size_t base = vector_smem(h, V, &stage), smem = base + vector_stages(h, V) * stage;
+    a.stages = vector_stages(h, V);
+    const void* kernel = (const void*)vector_infer_kernel<V>;
+    if (!h->carved[kernel]) {
+        CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VECTOR_SMEM));
+        CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        h->carved[kernel] = true;
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(VECTOR_CTAS); lc.blockDim = dim3(VECTOR_THREADS); lc.dynamicSmemBytes = smem; lc.stream = h->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = VECTOR_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    lc.attrs = at; lc.numAttrs = 1;
+    CU(h, cudaLaunchKernelEx(&lc, vector_infer_kernel<V>, a));
+    count_launch(h);
+    return SDNN_OK;
+}
+
+bool takes_vector(const sdnn* h, int cnt) {
+    const int v = cnt <= 2 ? cnt : 4;
+    return h->d_vector && (int64_t)h->N * v <= VECTOR_WORK && vector_stages(h, v) >= 3;
+}
+
+// All layers for one to four inputs: x0 [cnt][N] -> y and nonzero counts (either may be NULL).
+int infer_vector(sdnn* h, const float* x0, int cnt, float* y, int* nz_count) {
+    NvtxRange call("sdnn whole-network inference");
+    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, h->vector_kpad, 0, x0, cnt, y, nz_count, h->vector_status, h->cfg.clamp, h->cfg.activation};
+    return cnt == 1 ? launch_vector<1>(h, a) : cnt == 2 ? launch_vector<2>(h, a) : launch_vector<4>(h, a);
+}
+
 // Inputs per inference tile.  The gathers of a layer read the whole activation tile at random, so the two
 // ping-pong tiles should sit in L2: unless every layer's pattern is local (each block of rows reads few tile rows,
 // which the cache then holds whatever the tile's size), the tile is narrowed to the widest power of two >= 128
@@ -1631,6 +1743,7 @@ void sdnn_destroy(sdnn_t* h) {
         if (h->ev_pin[q]) cudaEventDestroy(h->ev_pin[q]);
         if (h->pin[q]) cudaFreeHost(h->pin[q]);
     }
+    if (h->vector_status) status_page().put(h->vector_status);
     for (void* p : h->allocs) cudaFree(p);
     if (h->own_stream) cudaStreamDestroy(h->stream);
     delete h;
@@ -1768,6 +1881,10 @@ int sdnn_finalize(sdnn_t* h) {
         int rc = build_reordered(h);
         if (rc) return rc;
     }
+    {
+        int rc = build_vector(h);
+        if (rc) return rc;
+    }
     CU(h, cudaStreamSynchronize(h->stream));
     h->finalized = true;
     return SDNN_OK;
@@ -1834,6 +1951,8 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
     int rc = check_infer_args(h, x0, n_inputs, nz_index_out, nz_index_capacity);
     if (rc) return rc;
     CU(h, cudaSetDevice(h->device));
+    if ((rc = vector_check(h))) return rc;
+    if (n_inputs >= 1 && n_inputs <= 4 && takes_vector(h, (int)n_inputs) && !nz_index_out && !nz_total_out) return infer_vector(h, x0, (int)n_inputs, y_out, nz_count_out);
     const bool want_sets = nz_count_out || nz_index_out || nz_total_out;
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     const int T = infer_tile_width(h);

@@ -57,3 +57,31 @@ def test_row_major_copy_moved_from_the_transposed_one(torch_cuda, n, k, B):  # n
             check_close(bias, ora.bias[l], f"b^{l + 1} at B = {b}")
             assert h.mirror_mismatches(l) == 0
     h.destroy()
+
+
+@pytest.mark.parametrize("n,k,layers", [(9, 3, 2), (64, 5, 3), (1000, 32, 4), (1024, 33, 9), (1025, 32, 5), (2047, 8, 12), (4096, 16, 3)])
+@pytest.mark.parametrize("cnt", [1, 2, 3])
+@pytest.mark.parametrize("act", ["clamped_relu", "sigmoid"])
+def test_whole_network_launch(torch_cuda, n, k, layers, cnt, act):  # noqa: F811
+    """One to four inputs through a net whose rows all have the same length: a block of 64 rows per CTA and one or more, the
+    last one partial or empty, fewer rows than CTAs, rows of more than 32 entries, more layers than the ring of entries has
+    stages; twice, so that the second call meets what the first one left."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + k)
+    rp = [np.arange(n + 1, dtype=np.int32) * k] * layers
+    cols = [np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for _ in range(n)]).astype(np.int32) for _ in range(layers)]
+    vals = [(rng.standard_normal(n * k) * (2.0 / k) ** 0.5).astype(np.float32) for _ in range(layers)]
+    bias = [(rng.standard_normal(n) * 0.1).astype(np.float32) for _ in range(layers)]
+    h = pkg.Sdnn.create(rp, cols, vals, bias, max_batch=64, activation=pkg.ACT_SIGMOID if act == "sigmoid" else pkg.ACT_CLAMPED_RELU)
+    ora = OracleNet(rp, cols, vals, bias, activation=act)
+    for _ in range(2):
+        x0 = vectors(rng, cnt, n)
+        y = torch.full((cnt, n), -1.0, device="cuda")
+        c = torch.full((cnt,), -1, dtype=torch.int32, device="cuda")
+        before = h.kernel_launches()
+        h.infer_batch(torch.from_numpy(x0).cuda(), cnt, y, c)
+        torch.cuda.synchronize()
+        assert (h.kernel_launches() - before == 1) == (n * (cnt if cnt <= 2 else 4) <= 4096)
+        check_close(y.cpu().numpy(), ora.infer(x0), "x^L")
+        assert np.array_equal(c.cpu().numpy(), np.count_nonzero(y.cpu().numpy(), axis=1))
+    h.destroy()
