@@ -42,6 +42,8 @@ struct RowShape {
 // Buffers of one inference tile in flight.  Tiles are independent of one another (so are the inputs), and a
 // handle may work on two at a time, each on its own stream, so that the ramp and tail of one tile's launches are
 // filled by the other's.
+struct TileGraph { int cols = 0, pdl = 0; bool track = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0, used = 0; };
+
 struct InferLane {
     cudaStream_t stream = nullptr;         // lane 0: the handle's stream
     float* tile[2] = {nullptr, nullptr};   // ping-pong activation tiles
@@ -52,6 +54,7 @@ struct InferLane {
     int* live_hist = nullptr;              // [L] live inputs after each layer of this lane's most recent tile
     float* stage_out = nullptr;            // host entry point: staged x^L and counts of this lane's tile
     int* stage_cnt = nullptr;
+    TileGraph graphs[4];                   // captured layer chains of this lane's tiles, by width
     cudaEvent_t ev_scan = nullptr;         // this lane's last scan of the running id total is done
     cudaEvent_t ev_done = nullptr;         // everything this lane was given in the current call is done
     bool ready = false;
@@ -149,6 +152,7 @@ struct sdnn {
     InferLane* cur = nullptr;           // lane the launch helpers currently work for
     cudaEvent_t last_scan_ev = nullptr, ev_lane_start = nullptr;
     int live_lane = 0;
+    int64_t infer_calls = 0;
     long long* d_running = nullptr;
     int l2_bytes = 0;
     std::vector<char> local_pattern;    // per layer: blocks of 1024 rows touch few distinct columns (see infer_tile_width)
@@ -944,6 +948,44 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     return SDNN_OK;
 }
 
+// The launches of a tile's layers, as a graph from a handle's second call on: one launch of the host's instead of one per
+// layer, which take 2.2 us each and which a layer of a narrow net does not outlast (1024 neurons x 120 layers, 256 inputs, three
+// handles in turn: 300 us a call of launches).  The first call launches directly, so that a net that is asked once does not pay for
+// the graph.  A lane keeps four, for as many tile widths.
+template <typename Layers>
+int enqueue_layers(sdnn* h, InferLane& ln, int cols, bool track, const Layers& layers) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (h->infer_calls < 2 || h->L < 4 || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
+        capturing != cudaStreamCaptureStatusNone) {
+        layers();
+        return SDNN_OK;
+    }
+    TileGraph* g = &ln.graphs[0];
+    for (TileGraph& q : ln.graphs) {
+        if (q.exec && q.cols == cols && q.track == track && q.pdl == h->fwd_pdl) { g = &q; break; }
+        if (g->exec && (!q.exec || q.used < g->used)) g = &q;      // the one not used for longest
+    }
+    if (!g->exec || g->cols != cols || g->track != track || g->pdl != h->fwd_pdl) {
+        if (g->exec) { cudaGraphExecDestroy(g->exec); g->exec = nullptr; }
+        cudaGraph_t graph = nullptr;
+        const int64_t before = h->launches;
+        CU(h, cudaStreamBeginCapture(ln.stream, cudaStreamCaptureModeThreadLocal));
+        layers();
+        cudaError_t e = cudaStreamEndCapture(ln.stream, &graph);
+        g->launches = h->launches - before;
+        h->launches = before;
+        if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
+        e = cudaGraphInstantiate(&g->exec, graph, 0);
+        cudaGraphDestroy(graph);
+        if (e != cudaSuccess) { g->exec = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
+        g->cols = cols; g->track = track; g->pdl = h->fwd_pdl;
+    }
+    g->used = h->infer_calls;
+    CU(h, cudaGraphLaunch(g->exec, ln.stream));
+    h->launches += g->launches;
+    return SDNN_OK;
+}
+
 // One tile of inference on device buffers, on lane `ln`: x0 [cnt][N] -> outputs for these cnt inputs.
 int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, int* cnt_out, int* idx_out, long long capacity,
                bool want_sets) {
@@ -954,35 +996,43 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     h->cur = &ln;
     h->launch_stream = st;
     launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
-    int cur = 0;
     bool track = h->compaction && h->cfg.activation == SDNN_ACT_CLAMPED_RELU;      // sigmoid(b) is never 0: nothing ever dies
     for (int l = 0; l < h->L && track; ++l) track = h->bias_nonpositive[l] != 0;     // the zero vector must be a fixed point
+    auto layers = [&]() {
+        int cur = 0;
+        if (track) {
+            const Geometry q = geometry(cols);
+            const int chunk = q.g * q.v;
+            const int rows_grid = std::min((h->N + 7) / 8, h->sms * 8);
+            for (int k = 0; k < h->L; ++k) {
+                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, true);
+                cur ^= 1;
+                live_kernel<<<1, 1024, 0, st>>>(ln.cs, ln.live_hist + k, chunk);
+                compact_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], h->N, ld, chunk);
+                count_launch(h, 2);
+            }
+            expand_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], ln.tile[cur ^ 1], h->N, cols, ld);
+            count_launch(h);
+        } else {
+            for (int k = 0; k < h->L; ++k) {
+                NvtxRange pass("forward layer", k + 1);
+                if (h->lay[k].windowed) launch_forward_window(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
+                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
+                cur ^= 1;
+            }
+        }
+    };
     if (track) {
-        const Geometry q = geometry(cols);
-        const int chunk = q.g * q.v;
-        const int rows_grid = std::min((h->N + 7) / 8, h->sms * 8);
         cols_init_kernel<<<(ld + 255) / 256, 256, 0, st>>>(ln.cs, cnt, ld);
         count_launch(h);
-        for (int k = 0; k < h->L; ++k) {
-            launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, true);
-            cur ^= 1;
-            live_kernel<<<1, 1024, 0, st>>>(ln.cs, ln.live_hist + k, chunk);
-            compact_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], h->N, ld, chunk);
-            count_launch(h, 2);
-        }
-        expand_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], ln.tile[cur ^ 1], h->N, cols, ld);
-        count_launch(h);
-        cur ^= 1;
         h->live_valid = true;
         h->live_lane = (int)(&ln - h->lane);
-    } else {
-        for (int k = 0; k < h->L; ++k) {
-            NvtxRange pass("forward layer", k + 1);
-            if (h->lay[k].windowed) launch_forward_window(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
-            else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
-            cur ^= 1;
-        }
     }
+    {
+        const int rc = enqueue_layers(h, ln, cols, track, layers);
+        if (rc) return rc;
+    }
+    const int cur = (h->L + (track ? 1 : 0)) & 1;
     h->launch_stream = nullptr;
     h->cur = &h->lane[0];
     const float* xl = ln.tile[cur];
@@ -1147,6 +1197,7 @@ int infer_lanes(const sdnn* h, int /*T*/) {
 // handle's stream ends up behind everything lane 1 did
 int lanes_begin(sdnn* h, int lanes) {
     h->last_scan_ev = nullptr;
+    ++h->infer_calls;
     // with two tiles in flight, CTAs of a tile's next layer that only wait would hold SM slots the other tile can use
     // (config 4 and uniform N = 65536: 1.4 % slower when released early)
     h->fwd_pdl = lanes > 1 ? PDL_AT_END : PDL_EARLY;
@@ -1729,6 +1780,7 @@ void sdnn_destroy(sdnn_t* h) {
     for (InferLane& ln : h->lane) {
         if (ln.ev_scan) cudaEventDestroy(ln.ev_scan);
         if (ln.ev_done) cudaEventDestroy(ln.ev_done);
+        for (TileGraph& g : ln.graphs) if (g.exec) cudaGraphExecDestroy(g.exec);
         if (ln.stream && ln.stream != h->stream) { cudaStreamSynchronize(ln.stream); cudaStreamDestroy(ln.stream); }
     }
     if (h->ev_lane_start) cudaEventDestroy(h->ev_lane_start);
