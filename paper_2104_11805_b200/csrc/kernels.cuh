@@ -347,55 +347,78 @@ __global__ void set_step_params_kernel(StepParams* p, float eta, int batch, doub
 // belong to the caller and cannot be re-laid out (sdnn_infer_noalloc).
 // The arrays are the caller's and were never validated on the host: a column index outside [0, n) is not followed
 // (its entry contributes nothing) and is counted in *bad_columns, which the host can read afterwards.
-template <int G>
+// G lanes share a row, V inputs each.  Rows start anywhere, so the lanes of a row fetch the entries of a step (each lane OWN of
+// them side by side, one step ahead; as vectors where the row starts at a multiple of four), check their columns once and hand them
+// round by shuffles: STEP gathers of every row are in flight whatever the row's alignment (rows of 8 .. 56 entries, 4096
+// neurons, 100 inputs: 14.7 -> 8.5 us per layer, where rows off a multiple of four had taken their entries one at a time).
+template <int G, int V, int STEP>
 __global__ void __launch_bounds__(256)
 forward_csr_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ val,
                    const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
                    int n, int ld, float clamp, unsigned long long* __restrict__ bad_columns) {
-    constexpr int RPW = 32 / G;
+    constexpr int RPW = 32 / G, OWN = (STEP + G - 1) / G;      // entries of a step that a lane fetches (G > STEP: only the first STEP lanes do)
     const int lane = threadIdx.x & 31;
-    const int sub = lane % G, grp = lane / G;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int row = warp * RPW + grp;
-    if (row >= n) return;
-    const int boff = blockIdx.y * (4 * G) + sub * 4;
+    const int sub = lane % G, lead = lane - sub;
+    const int row = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RPW + lane / G;
+    int p = 0, e = 0;
+    float b = 0.0f;
+    if (row < n) { p = row_ptr[row]; e = row_ptr[row + 1]; b = bias[row]; }
+    const int boff = blockIdx.y * (V * G) + sub * V;
     const float* xg = xin + boff;
-
-    const int s = row_ptr[row], e = row_ptr[row + 1];
-    const float b = bias[row];
-    float4 acc = make_float4(b, b, b, b);
-    int p = s;
+    const unsigned pitch = (unsigned)ld * 4u;
     unsigned bad = 0;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-#define SDNN_FMA4(W, X) acc.x = fmaf(W, X.x, acc.x); acc.y = fmaf(W, X.y, acc.y); acc.z = fmaf(W, X.z, acc.z); acc.w = fmaf(W, X.w, acc.w);
-#define SDNN_X(C) ((unsigned)(C) < (unsigned)n ? gather_f4(xg + (size_t)(C) * ld) : (++bad, zero))
-    if (((s | e) & 3) == 0) {
-        for (; p + 8 <= e; p += 8) {
-            const int4 c0 = *reinterpret_cast<const int4*>(col + p), c1 = *reinterpret_cast<const int4*>(col + p + 4);
-            const float4 w0 = ld_f4(val + p), w1 = ld_f4(val + p + 4);
-            const float4 x0 = SDNN_X(c0.x), x1 = SDNN_X(c0.y), x2 = SDNN_X(c0.z), x3 = SDNN_X(c0.w);
-            const float4 x4 = SDNN_X(c1.x), x5 = SDNN_X(c1.y), x6 = SDNN_X(c1.z), x7 = SDNN_X(c1.w);
-            SDNN_FMA4(w0.x, x0) SDNN_FMA4(w0.y, x1) SDNN_FMA4(w0.z, x2) SDNN_FMA4(w0.w, x3)
-            SDNN_FMA4(w1.x, x4) SDNN_FMA4(w1.y, x5) SDNN_FMA4(w1.z, x6) SDNN_FMA4(w1.w, x7)
+    int c[OWN];
+    float w[OWN];
+    const bool aligned = (p & 3) == 0;
+    auto fetch = [&](int at) {
+        const int first = at + sub * OWN;
+        if (OWN >= 4 && aligned && first + OWN <= e) {
+#pragma unroll
+            for (int i = 0; i + 3 < OWN; i += 4) {
+                const int4 cv = __ldg(reinterpret_cast<const int4*>(col + first + i));
+                const float4 wv = __ldg(reinterpret_cast<const float4*>(val + first + i));
+                c[i] = cv.x; c[i + 1] = cv.y; c[i + 2] = cv.z; c[i + 3] = cv.w;
+                w[i] = wv.x; w[i + 1] = wv.y; w[i + 2] = wv.z; w[i + 3] = wv.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < OWN; ++i) {
+                const bool on = first + i < e && sub * OWN < STEP;
+                c[i] = on ? __ldg(col + first + i) : 0;
+                w[i] = on ? __ldg(val + first + i) : 0.0f;
+            }
         }
-        for (; p < e; p += 4) {
-            const int4 c0 = *reinterpret_cast<const int4*>(col + p);
-            const float4 w0 = ld_f4(val + p);
-            const float4 x0 = SDNN_X(c0.x), x1 = SDNN_X(c0.y), x2 = SDNN_X(c0.z), x3 = SDNN_X(c0.w);
-            SDNN_FMA4(w0.x, x0) SDNN_FMA4(w0.y, x1) SDNN_FMA4(w0.z, x2) SDNN_FMA4(w0.w, x3)
+#pragma unroll
+        for (int i = 0; i < OWN; ++i)
+            if ((unsigned)c[i] >= (unsigned)n) { ++bad; c[i] = 0; w[i] = 0.0f; }      // not followed, counted once
+    };
+    fetch(p);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    Lane<V> acc;
+    lane_fill(acc, b);
+    // the rows of a warp take as many steps as its longest: the shuffles want all lanes
+    int steps = (e - p + STEP - 1) / STEP;
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) steps = max(steps, __shfl_xor_sync(0xffffffffu, steps, o));
+    for (int t = 0; t < steps; ++t, p += STEP) {
+        Lane<V> x[STEP];
+        float ww[STEP];
+#pragma unroll
+        for (int j = 0; j < STEP; ++j) {
+            const int cc = __shfl_sync(0xffffffffu, c[j % OWN], lead + j / OWN);
+            ww[j] = __shfl_sync(0xffffffffu, w[j % OWN], lead + j / OWN);
+            if (p + j < e) lane_gather(x[j], tile_row(xg, cc, pitch)); else lane_fill(x[j], 0.0f);
         }
-    } else {
-        for (; p < e; ++p) {
-            const float w = val[p];
-            const float4 x = SDNN_X(col[p]);
-            SDNN_FMA4(w, x)
-        }
+        fetch(p + STEP);
+#pragma unroll
+        for (int j = 0; j < STEP; ++j) if (p + j < e) lane_fma(ww[j], x[j], acc);
     }
-#undef SDNN_X
-    if (bad && sub == 0) atomicAdd(bad_columns, (unsigned long long)bad);      // the lanes of a row see the same columns
-    acc.x = clampf(acc.x, clamp); acc.y = clampf(acc.y, clamp);
-    acc.z = clampf(acc.z, clamp); acc.w = clampf(acc.w, clamp);
-    st_f4(xout + (size_t)row * ld + boff, acc);
+    if (bad) atomicAdd(bad_columns, (unsigned long long)bad);
+    if (row < n) {
+        lane_activate(acc, ACT_CLAMPED_RELU, clamp);
+        lane_store(tile_row(xout + boff, row, pitch), acc);
+    }
 }
 
 // ---------------------------------------------------------------------------------------------

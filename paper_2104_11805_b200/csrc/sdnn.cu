@@ -2839,7 +2839,7 @@ namespace {
 static __device__ __align__(256) float g_noalloc_scratch[2 * SDNN_NOALLOC_MAX_TILE_FLOATS];
 static __device__ unsigned long long g_noalloc_bad_columns;      // out-of-range column indices met so far (never followed)
 
-// tile geometry of this entry point (plain CSR kernel: 4 batch entries per lane, chunks of 128 columns)
+// tile geometry of this entry point (plain CSR kernel: 8 batch entries per lane, chunks of 128 columns)
 int noalloc_padded_width(int b) {
     if (b <= 4) return 4;
     if (b <= 128) { int w = 4; while (w < b) w <<= 1; return w; }
@@ -2874,12 +2874,18 @@ int noalloc_scratch(float** out, unsigned long long** bad_out) {
     return SDNN_OK;
 }
 
-template <int G>
+// a layer may start its prologue (its rows' places, first entries) under the tail of the one before
+template <int G, int V, int STEP = 8>
 void noalloc_forward_g(cudaStream_t st, const int* rp, const int* col, const float* val, const float* bias,
                        const float* xin, float* xout, int n, int ld, int chunks, float clamp, unsigned long long* bad) {
-    const int rows_per_block = 8 * (32 / G);
-    dim3 grid((n + rows_per_block - 1) / rows_per_block, chunks);
-    forward_csr_kernel<G><<<grid, 256, 0, st>>>(rp, col, val, bias, xin, xout, n, ld, clamp, bad);
+    const int warps = (n + 32 / G - 1) / (32 / G), wpb = warps * chunks < 4096 ? 2 : 4;      // small CTAs: more SMs, finer tails
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((warps + wpb - 1) / wpb, chunks); lc.blockDim = dim3(32 * wpb); lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at; lc.numAttrs = 1;
+    cudaLaunchKernelEx(&lc, forward_csr_kernel<G, V, STEP>, rp, col, val, bias, xin, xout, n, ld, clamp, bad);
 }
 
 }  // namespace
@@ -2912,7 +2918,7 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
     if (rc) return rc;
     float* tile[2] = {scratch, scratch + SDNN_NOALLOC_MAX_TILE_FLOATS};
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    const struct { int g, chunks; } q = {ld <= 128 ? ld / 4 : 32, ld <= 128 ? 1 : ld / 128};
+    const int chunks = ld <= 128 ? 1 : ld / 128;
     {
         dim3 grid((n_neurons + 31) / 32, (ld + 31) / 32), block(32, 8);
         transpose_in_kernel<<<grid, block, 0, st>>>(x0, tile[0], n_neurons, n_inputs, ld, ld, nullptr);
@@ -2923,14 +2929,17 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
         const int* col = col_idx + layer_offset[l];
         const float* val = values + layer_offset[l];
         const float* b = bias + (size_t)l * n_neurons;
-        switch (q.g) {
-            case 1: noalloc_forward_g<1>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, q.chunks, clamp, bad); break;
-            case 2: noalloc_forward_g<2>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, q.chunks, clamp, bad); break;
-            case 4: noalloc_forward_g<4>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, q.chunks, clamp, bad); break;
-            case 8: noalloc_forward_g<8>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, q.chunks, clamp, bad); break;
-            case 16: noalloc_forward_g<16>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, q.chunks, clamp, bad); break;
-            default: noalloc_forward_g<32>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, q.chunks, clamp, bad); break;
+#define SDNN_NOALLOC(...) noalloc_forward_g<__VA_ARGS__>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, chunks, clamp, bad)
+        // up to 32 inputs a row has few lanes, so that 16 of its entries in flight per step still fit the registers
+        switch (ld / chunks) {
+            case 4: SDNN_NOALLOC(1, 4, 16); break;
+            case 8: SDNN_NOALLOC(1, 8); break;
+            case 16: SDNN_NOALLOC(4, 4, 16); break;
+            case 32: SDNN_NOALLOC(8, 4, 16); break;
+            case 64: SDNN_NOALLOC(8, 8); break;
+            default: SDNN_NOALLOC(16, 8); break;
         }
+#undef SDNN_NOALLOC
         cur ^= 1;
     }
     {
