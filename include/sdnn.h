@@ -65,7 +65,7 @@ typedef enum {
 #define SDNN_FLAG_KEEP_DEBUG  0x04u /* train handles: also store delta^k and the gradient G^k of the last step     */
 #define SDNN_FLAG_SKIP_DEAD   0x08u /* allow data-dependent skipping; default is dense mode: every layer streams   */
                                     /* its weights and processes every input.  Inference: inputs whose activation  */
-                                    /* vector has become all zero are dropped from the tile (whole chunks of 256   */
+                                    /* vector has become all zero are dropped from the tile (whole chunks of 64    */
                                     /* columns at a time); only done while no layer has a positive bias, because   */
                                     /* only then does an all-zero vector stay all zero.  Training: a unit of rows  */
                                     /* whose delta is zero for every input skips its entries (not for B <= 4,      */

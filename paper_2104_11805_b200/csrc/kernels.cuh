@@ -498,7 +498,9 @@ __device__ __forceinline__ void prefetch_unit(const Sliced& m, int u, int rpw, i
 // While it works on a unit a warp asks for the entries of its next unit to be brought into L2.
 // CG: the gathers go past L1 (64-byte rows of a layer without padding entries).
 // SPAN: a CTA takes a run of `span` consecutive units instead of walking the units in a grid-wide stride.
-template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false>
+// TRACK (dropping dead inputs): one grid for all chunks, whose warps walk the units of the chunks that still hold live inputs
+// (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.
+template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false, bool TRACK = false>
 __global__ void __launch_bounds__(256, CPS > 2 ? 1 : 2)
 forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
                int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span) {
@@ -510,12 +512,14 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
     const int all_units = (n + RPW - 1) / RPW;
     const int nunits = SPAN ? min(all_units, ((int)blockIdx.x + 1) * span) : all_units;
     const int stride = SPAN ? wpb : gridDim.x * wpb;
-    const int boff = blockIdx.y * (V * G) + sub * V;
-    const float* xg = xin + boff;
+    int boff = (TRACK ? 0 : blockIdx.y * (V * G)) + sub * V;
     const unsigned pitch = (unsigned)ld * 4u;
     const float* __restrict__ val = m.val;
 
     int unit = (SPAN ? blockIdx.x * span : blockIdx.x * wpb) + (threadIdx.x >> 5);
+    int chunks_left = 0x7fffffff;      // TRACK: chunks from the current one on
+#define SDNN_WRAP(U, BOFF, LEFT) if (TRACK && (U) >= nunits) { const int q_ = (U) / nunits; (U) -= q_ * nunits; BOFF += q_ * (V * G); LEFT -= q_; }
+    SDNN_WRAP(unit, boff, chunks_left)
     // prologue that does not depend on the previous layer: shape of the first row, its entries on their way to L2
     int row, base, nch;
     SDNN_UNIT_SHAPE(m, unit, nunits, row, base, nch)
@@ -528,13 +532,13 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
     if (nch > 0) load_idx<CPS, I16>(c, m, base);
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
-    // compaction mode: only the first *ncols_dev columns of the tile still hold live inputs
-    if (ncols_dev && blockIdx.y * (V * G) >= *ncols_dev) return;
+    if (TRACK) chunks_left += (*ncols_dev + V * G - 1) / (V * G) - 0x7fffffff;
     unsigned live = 0u;       // bit e: column boff + e of some row this lane produced is nonzero
 
-    while (unit < nunits) {
+    while (unit < nunits && (!TRACK || chunks_left > 0)) {
         // shape of this group's row in the warp's next unit (used when this unit's last step prefetches across the boundary)
-        const int nunit = unit + stride;
+        int nunit = unit + stride, nboff = boff, nleft = chunks_left;
+        SDNN_WRAP(nunit, nboff, nleft)
         int nrow, nbase, nnch;
         SDNN_UNIT_SHAPE(m, nunit, nunits, nrow, nbase, nnch)
         const float nb = (nrow < n) ? bias[nrow] : 0.0f;
@@ -544,6 +548,7 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         Lane<V> acc;
         lane_fill(acc, b);
         const float* vp = val + base;
+        const float* xg = xin + boff;
         for (int t = 0; t < nch; t += CPS) {
             float4 w[CPS];
             Lane<V> x[4 * CPS];
@@ -563,15 +568,18 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         if (row < n) {
             lane_activate(acc, act, clamp);
             lane_store(tile_row(xout + boff, to, pitch), acc);
-            if (live_flags) live |= lane_nonzero_bits(acc);
+            if (TRACK) live |= lane_nonzero_bits(acc);
+        }
+        if (TRACK && live && (nboff != boff || nleft <= 0)) {      // this warp's last unit of the chunk
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+                if ((live >> e) & 1u) live_flags[boff + e] = 1;      // many lanes may store the same 1
+            live = 0u;
         }
         unit = nunit; row = nrow; base = nbase; nch = nnch; b = nb; to = nto;
+        if (TRACK) { boff = nboff; chunks_left = nleft; }
     }
-    if (live_flags) {
-#pragma unroll
-        for (int e = 0; e < V; ++e)
-            if ((live >> e) & 1u) live_flags[boff + e] = 1;      // many lanes may store the same 1
-    }
+#undef SDNN_WRAP
     if (pdl == 1) grid_launch_dependents();
 }
 
@@ -1491,9 +1499,10 @@ sliced_csr_kernel(Sliced m, float* __restrict__ csr, const int* __restrict__ sta
 // activation vector has become all zero stays all zero when no bias is positive).  The tile keeps its live
 // inputs in its first *ncols columns; colmap[c] = position in the caller's tile of the input in column c.
 //   cols_init : ncols = cnt, colmap = identity, flags cleared
-//   live      : after a forward layer has marked the columns that still hold a nonzero: count them, record
-//               the count for this layer, and - if that frees at least one whole chunk of columns - renumber
-//               (perm[new] = old column, colmap follows, ncols = count, *do_compact = 1).  Single block.
+//   live      : after a forward layer has marked the columns that still hold a nonzero: count them and - if that frees at least
+//               one whole chunk of columns - renumber (perm[new] = old column, colmap follows, ncols = count, *do_compact = 1).
+//               Single block; only after some of the layers, since renumbering costs two launches in the chain of layers
+//   count     : live columns after every layer, from the marks, once per tile
 //   compact   : moves the columns of every row to their new places, in place (a warp reads the part of a row it
 //               is about to overwrite before it writes), and clears the rest of the last live chunk
 //   expand    : final tile back to the caller's column positions, dead inputs all zero
@@ -1503,24 +1512,24 @@ struct ColState {
     int* do_compact;
     int* colmap;       // [ld]
     int* perm;         // [ld]
-    int* flags;        // [ld]
+    int* flags;        // [L][ld]: marks of each layer
 };
 
 __global__ void cols_init_kernel(ColState s, int cnt, int ld) {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ld; c += gridDim.x * blockDim.x) {
-        s.colmap[c] = c; s.perm[c] = c; s.flags[c] = 0;
+        s.colmap[c] = c; s.perm[c] = c;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) { *s.ncols = cnt; *s.old_ncols = cnt; *s.do_compact = 0; }
 }
 
-__global__ void __launch_bounds__(1024) live_kernel(ColState s, int* __restrict__ live_after_layer, int chunk) {
+__global__ void __launch_bounds__(1024) live_kernel(ColState s, const int* __restrict__ flags, int chunk) {
     __shared__ int warp_tot[32];
     __shared__ int carry, total;
     const int n = *s.ncols;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // pass 1: how many columns are still live
     int cnt = 0;
-    for (int b = threadIdx.x; b < n; b += 1024) cnt += (s.flags[b] != 0);
+    for (int b = threadIdx.x; b < n; b += 1024) cnt += (flags[b] != 0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
     if (lane == 0) warp_tot[wid] = cnt;
@@ -1529,7 +1538,6 @@ __global__ void __launch_bounds__(1024) live_kernel(ColState s, int* __restrict_
         int t = 0;
         for (int q = 0; q < 32; ++q) t += warp_tot[q];
         total = t; carry = 0;
-        *live_after_layer = t;
     }
     __syncthreads();
     const int live = total;
@@ -1538,7 +1546,7 @@ __global__ void __launch_bounds__(1024) live_kernel(ColState s, int* __restrict_
         // pass 2: stable renumbering, 1024 columns at a time (new position <= old position)
         for (int base = 0; base < n; base += 1024) {
             const int b = base + threadIdx.x;
-            const int f = (b < n && s.flags[b] != 0) ? 1 : 0;
+            const int f = (b < n && flags[b] != 0) ? 1 : 0;
             const int cm = (b < n) ? s.colmap[b] : 0;
             int incl = f;
 #pragma unroll
@@ -1557,11 +1565,22 @@ __global__ void __launch_bounds__(1024) live_kernel(ColState s, int* __restrict_
             __syncthreads();
         }
     }
-    for (int b = threadIdx.x; b < n; b += 1024) s.flags[b] = 0;
     if (threadIdx.x == 0) {
         *s.do_compact = renumber ? 1 : 0;
         if (renumber) { *s.old_ncols = n; *s.ncols = live; }
     }
+}
+
+// a block per layer; columns that a layer did not process are not marked
+__global__ void __launch_bounds__(256) live_count_kernel(const int* __restrict__ flags, int* __restrict__ live_after_layer, int ld) {
+    __shared__ int part[8];
+    int cnt = 0;
+    for (int b = threadIdx.x; b < ld; b += 256) cnt += (flags[(size_t)blockIdx.x * ld + b] != 0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) live_after_layer[blockIdx.x] = part[0] + part[1] + part[2] + part[3] + part[4] + part[5] + part[6] + part[7];
 }
 
 __global__ void __launch_bounds__(256) compact_kernel(ColState s, float* __restrict__ tile, int n, int ld, int chunk) {

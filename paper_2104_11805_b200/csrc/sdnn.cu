@@ -495,7 +495,7 @@ cudaError_t launch_k(sdnn* h, void (*kernel)(KArgs...), dim3 grid, dim3 block, b
 }
 
 template <bool I16, int G, int V, int CPS = 2>
-void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld, int chunks, bool track) {
+void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld, int chunks) {
     constexpr int RPW = 32 / G;
     const int units = (h->N + RPW - 1) / RPW;
     const float* bias = h->d_bias + (size_t)layer * h->N;
@@ -517,7 +517,7 @@ void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld
 #define SDNN_FWD(CG_, SPAN_)                                                                                                   \
     launch_k(h, forward_kernel<G, V, CPS, I16, CG_, SPAN_>, dim3(plan.first, chunks), dim3(plan.second), h->pdl, rows_of(h, layer), \
              bias, xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,                              \
-             track ? (const int*)h->cur->cs.ncols : (const int*)nullptr, track ? h->cur->cs.flags : (int*)nullptr, span)
+             (const int*)nullptr, (int*)nullptr, span)
     // the grid-stride instantiation is the one the wide inference tiles take: it carries nothing of the other walk
     if (cg) { if (span > 0) SDNN_FWD((G == 2 && V == 8 && CPS == 2), true); else SDNN_FWD((G == 2 && V == 8 && CPS == 2), false); }
     else if (span > 0) SDNN_FWD(false, true);
@@ -525,7 +525,30 @@ void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld
 #undef SDNN_FWD
 }
 
-// track: compaction mode (process only the live columns, mark the columns that stay live)
+// A layer while dead inputs are being dropped: chunks of 64 inputs at most, which is the width that columns are dropped by (as fast per
+// input as 256 on dense tiles of 4096 neurons; of 1024 inputs a third of which survive, 6 of 16 such chunks are left, not 2 of 4
+// of 256), only the live ones, and each column that stays live marked.
+constexpr int TRACK_CHUNK = 64;
+template <bool I16, int G, int V>
+void launch_forward_tracked(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
+    const int units = (h->N + 32 / G - 1) / (32 / G), chunks = cols / (V * G);
+    auto plan = plan_grid(h, (const void*)forward_kernel<G, V, 2, I16, false, false, true>, units * chunks, 1);
+    launch_k(h, forward_kernel<G, V, 2, I16, false, false, true>, dim3(plan.first), dim3(plan.second), h->pdl, rows_of(h, layer),
+             (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,
+             (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0);
+    count_launch(h);
+}
+template <bool I16>
+void launch_forward_tracked_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
+    switch (std::min(cols, TRACK_CHUNK)) {
+        case 4: launch_forward_tracked<I16, 1, 4>(h, layer, xin, xout, ld, cols); break;
+        case 8: launch_forward_tracked<I16, 1, 8>(h, layer, xin, xout, ld, cols); break;
+        case 16: launch_forward_tracked<I16, 2, 8>(h, layer, xin, xout, ld, cols); break;
+        case 32: launch_forward_tracked<I16, 4, 8>(h, layer, xin, xout, ld, cols); break;
+        default: launch_forward_tracked<I16, 8, 8>(h, layer, xin, xout, ld, cols); break;
+    }
+}
+
 // Tiles of padded width 4 take the kernels that give a lane a row's chunk instead of a row (see kernels.cuh), unless
 // the handle asked for one of the other backward realisations: those keep the common kernels at every width.
 bool entry_parallel(const sdnn* h, int ld) {
@@ -533,25 +556,25 @@ bool entry_parallel(const sdnn* h, int ld) {
 }
 
 template <bool I16>
-void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, bool track) {
+void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
     const Geometry q = geometry(cols);
-    if (q.v == 4 && !track && entry_parallel(h, ld)) {
+    if (q.v == 4 && entry_parallel(h, ld)) {
         const int wf = h->NS <= h->sms ? 1 : 4;      // few slices: one per CTA, so that they spread over as many SMs
         launch_k(h, forward_ep_kernel<I16>, dim3((h->NS + wf - 1) / wf), dim3(32 * wf), h->pdl, rows_of(h, layer),
                  (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0);
-    } else if (q.v == 4) launch_forward_gv<I16, 1, 4>(h, layer, xin, xout, ld, q.chunks, track);
+    } else if (q.v == 4) launch_forward_gv<I16, 1, 4>(h, layer, xin, xout, ld, q.chunks);
     else switch (q.g) {
-        case 1: launch_forward_gv<I16, 1, 8>(h, layer, xin, xout, ld, q.chunks, track); break;
-        case 2: launch_forward_gv<I16, 2, 8>(h, layer, xin, xout, ld, q.chunks, track); break;
-        case 4: launch_forward_gv<I16, 4, 8>(h, layer, xin, xout, ld, q.chunks, track); break;
-        case 8: launch_forward_gv<I16, 8, 8>(h, layer, xin, xout, ld, q.chunks, track); break;
-        case 16: launch_forward_gv<I16, 16, 8>(h, layer, xin, xout, ld, q.chunks, track); break;
+        case 1: launch_forward_gv<I16, 1, 8>(h, layer, xin, xout, ld, q.chunks); break;
+        case 2: launch_forward_gv<I16, 2, 8>(h, layer, xin, xout, ld, q.chunks); break;
+        case 4: launch_forward_gv<I16, 4, 8>(h, layer, xin, xout, ld, q.chunks); break;
+        case 8: launch_forward_gv<I16, 8, 8>(h, layer, xin, xout, ld, q.chunks); break;
+        case 16: launch_forward_gv<I16, 16, 8>(h, layer, xin, xout, ld, q.chunks); break;
         default:
             // a launch of at most one warp-row per resident slot is bound by its chain of round trips: four chunks (16
             // entries) of a row in flight per step instead of two, where every slice has whole steps of that size
-            if (!track && h->lay[layer].r_chunks_mult4 && (int64_t)h->N * q.chunks <= (int64_t)h->sms * 8)
-                launch_forward_gv<I16, 32, 8, 4>(h, layer, xin, xout, ld, q.chunks, track);
-            else launch_forward_gv<I16, 32, 8>(h, layer, xin, xout, ld, q.chunks, track);
+            if (h->lay[layer].r_chunks_mult4 && (int64_t)h->N * q.chunks <= (int64_t)h->sms * 8)
+                launch_forward_gv<I16, 32, 8, 4>(h, layer, xin, xout, ld, q.chunks);
+            else launch_forward_gv<I16, 32, 8>(h, layer, xin, xout, ld, q.chunks);
             break;
     }
     count_launch(h);
@@ -559,8 +582,11 @@ void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld,
 
 // the kernels are instantiated for both index widths of the sliced copies
 void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, bool track = false) {
-    if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, track);
-    else launch_forward_i<false>(h, layer, xin, xout, ld, cols, track);
+    if (track) {
+        if (h->idx16) launch_forward_tracked_i<true>(h, layer, xin, xout, ld, cols);
+        else launch_forward_tracked_i<false>(h, layer, xin, xout, ld, cols);
+    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols);
+    else launch_forward_i<false>(h, layer, xin, xout, ld, cols);
 }
 
 // Windowed layers (rows grouped by shared columns at set-up): the group's window of the input tile is staged in shared
@@ -958,9 +984,9 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     if ((rc = dev_alloc(h, &ln.offs, (size_t)h->ld_max, false))) return rc;
     if (h->compaction) {
         int* blk = nullptr;
-        if ((rc = dev_alloc(h, &blk, 3 * (size_t)h->ld_max + 4, true))) return rc;
+        if ((rc = dev_alloc(h, &blk, (2 + (size_t)h->L) * (size_t)h->ld_max + 4, true))) return rc;
         ln.cs.colmap = blk; ln.cs.perm = blk + h->ld_max; ln.cs.flags = blk + 2 * (size_t)h->ld_max;
-        ln.cs.ncols = blk + 3 * (size_t)h->ld_max; ln.cs.old_ncols = ln.cs.ncols + 1; ln.cs.do_compact = ln.cs.ncols + 2;
+        ln.cs.ncols = blk + (2 + (size_t)h->L) * (size_t)h->ld_max; ln.cs.old_ncols = ln.cs.ncols + 1; ln.cs.do_compact = ln.cs.ncols + 2;
         if ((rc = dev_alloc(h, &ln.live_hist, (size_t)h->L, true))) return rc;
     }
     ln.ready = true;
@@ -1020,18 +1046,24 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     auto layers = [&]() {
         int cur = 0;
         if (track) {
-            const Geometry q = geometry(cols);
-            const int chunk = q.g * q.v;
+            const int chunk = std::min(cols, TRACK_CHUNK);
             const int rows_grid = std::min((h->N + 7) / 8, h->sms * 8);
+            cudaMemsetAsync(ln.cs.flags, 0, (size_t)h->L * ld * sizeof(int), st);
             for (int k = 0; k < h->L; ++k) {
                 launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, true);
                 cur ^= 1;
-                live_kernel<<<1, 1024, 0, st>>>(ln.cs, ln.live_hist + k, chunk);
-                compact_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], h->N, ld, chunk);
-                count_launch(h, 2);
+                // dropping what has died: after each of the first layers, where most do, then at growing distances (after 1, 2, 3, 4,
+                // 6, 8, 12, 16, 24, ... layers)
+                const int q = k + 1, high = q < 4 ? 1 : 1 << (31 - __builtin_clz(q));
+                if (k + 1 < h->L && (q < 4 || q == high || q == high + high / 2)) {
+                    live_kernel<<<1, 1024, 0, st>>>(ln.cs, ln.cs.flags + (size_t)k * ld, chunk);
+                    compact_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], h->N, ld, chunk);
+                    count_launch(h, 2);
+                }
             }
+            live_count_kernel<<<h->L, 256, 0, st>>>(ln.cs.flags, ln.live_hist, ld);
             expand_kernel<<<rows_grid, 256, 0, st>>>(ln.cs, ln.tile[cur], ln.tile[cur ^ 1], h->N, cols, ld);
-            count_launch(h);
+            count_launch(h, 2);
         } else {
             for (int k = 0; k < h->L; ++k) {
                 NvtxRange pass("forward layer", k + 1);
