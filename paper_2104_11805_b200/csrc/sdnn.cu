@@ -48,6 +48,7 @@ struct InferLane {
     cudaStream_t stream = nullptr;         // lane 0: the handle's stream
     float* tile[2] = {nullptr, nullptr};   // ping-pong activation tiles
     int* seg_cnt = nullptr;
+    unsigned* nz_bits = nullptr;           // nonzero bits of the final tile, 32 rows a word
     int* tile_cnt = nullptr;
     long long* offs = nullptr;
     ColState cs{};                         // live-column bookkeeping (SDNN_FLAG_SKIP_DEAD)
@@ -825,7 +826,7 @@ void launch_output_gradient(sdnn* h, int ld) {
 }
 
 void launch_transpose_in(sdnn* h, const float* src, float* dst, int cnt, int cols, int ld, const int* row_map = nullptr) {
-    dim3 grid((h->N + 31) / 32, (cols + 31) / 32), block(32, 8);
+    dim3 grid((h->N + TRANSPOSE_ROWS - 1) / TRANSPOSE_ROWS, (cols + 31) / 32), block(256);
     transpose_in_kernel<<<grid, block, 0, h->launch_stream ? h->launch_stream : h->stream>>>(src, dst, h->N, cnt, cols, ld, row_map);
     count_launch(h);
 }
@@ -980,6 +981,7 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     if ((rc = dev_alloc(h, &ln.tile[0], tile, false))) return rc;
     if ((rc = dev_alloc(h, &ln.tile[1], tile, false))) return rc;
     if ((rc = dev_alloc(h, &ln.seg_cnt, nseg * (size_t)h->ld_max, false))) return rc;
+    if ((rc = dev_alloc(h, &ln.nz_bits, ((size_t)h->N + 31) / 32 * (size_t)h->ld_max, false))) return rc;
     if ((rc = dev_alloc(h, &ln.tile_cnt, (size_t)h->ld_max, false))) return rc;
     if ((rc = dev_alloc(h, &ln.offs, (size_t)h->ld_max, false))) return rc;
     if (h->compaction) {
@@ -996,11 +998,14 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
 // The launches of a tile's layers, as a graph from a handle's second call on: one launch of the host's instead of one per
 // layer, which take 2.2 us each and which a layer of a narrow net does not outlast (1024 neurons x 120 layers, 256 inputs, three
 // handles in turn: 300 us a call of launches).  The first call launches directly, so that a net that is asked once does not pay for
-// the graph.  A lane keeps four, for as many tile widths.
+// the graph.  A lane keeps four, for as many tile widths.  Layers that outlast their launch calls several times over are
+// launched directly (4096 neurons, tiles of 1024: 27 us a layer, 1 % slower as graphs on two streams), unless dead inputs are
+// being dropped: nobody knows what is left of those.
+constexpr int64_t GRAPH_WORK = 32 << 20;      // stored elements x inputs per layer: about 7 us
 template <typename Layers>
 int enqueue_layers(sdnn* h, InferLane& ln, int cols, bool track, const Layers& layers) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (h->infer_calls < 2 || h->L < 4 || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
+    if (h->infer_calls < 2 || h->L < 4 || (!track && h->lay[0].r_elems * cols > GRAPH_WORK) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
         capturing != cudaStreamCaptureStatusNone) {
         layers();
         return SDNN_OK;
@@ -1088,14 +1093,14 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     h->cur = &h->lane[0];
     const float* xl = ln.tile[cur];
     if (y_out) {
-        dim3 grid((h->N + 31) / 32, (cnt + 31) / 32), block(32, 8);
+        dim3 grid((h->N + TRANSPOSE_ROWS - 1) / TRANSPOSE_ROWS, (cnt + 31) / 32), block(256);
         transpose_out_kernel<<<grid, block, 0, st>>>(xl, y_out, h->N, cnt, ld);
         count_launch(h);
     }
     if (want_sets) {
         const int nseg = (h->N + NZ_SEG - 1) / NZ_SEG;
-        dim3 grid(nseg, (cnt + 127) / 128);
-        nz_count_kernel<<<grid, 128, 0, st>>>(xl, ln.seg_cnt, h->N, cnt, ld);
+        dim3 grid(nseg, (cnt + 31) / 32);
+        nz_count_kernel<<<grid, 256, 0, st>>>(xl, ln.nz_bits, ln.seg_cnt, h->N, cnt, ld);
         nz_scan_segments_kernel<<<(cnt + 127) / 128, 128, 0, st>>>(ln.seg_cnt, ln.tile_cnt, nseg, cnt, ld);
         // the running total of ids is carried from tile to tile: the scans of successive tiles run in order
         if (h->last_scan_ev && h->last_scan_ev != ln.ev_scan) CU(h, cudaStreamWaitEvent(st, h->last_scan_ev, 0));
@@ -1104,7 +1109,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
         h->last_scan_ev = ln.ev_scan;
         count_launch(h, 3);
         if (idx_out) {
-            nz_fill_kernel<<<grid, 128, 0, st>>>(xl, ln.seg_cnt, ln.offs, idx_out, capacity, h->N, cnt, ld);
+            nz_fill_kernel<<<grid, 256, 0, st>>>(ln.nz_bits, ln.seg_cnt, ln.offs, idx_out, capacity, h->N, cnt, ld);
             count_launch(h);
         }
     }
@@ -2971,7 +2976,7 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int chunks = ld <= 128 ? 1 : ld / 128;
     {
-        dim3 grid((n_neurons + 31) / 32, (ld + 31) / 32), block(32, 8);
+        dim3 grid((n_neurons + TRANSPOSE_ROWS - 1) / TRANSPOSE_ROWS, (ld + 31) / 32), block(256);
         transpose_in_kernel<<<grid, block, 0, st>>>(x0, tile[0], n_neurons, n_inputs, ld, ld, nullptr);
     }
     int cur = 0;
@@ -2994,7 +2999,7 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
         cur ^= 1;
     }
     {
-        dim3 grid((n_neurons + 31) / 32, (n_inputs + 31) / 32), block(32, 8);
+        dim3 grid((n_neurons + TRANSPOSE_ROWS - 1) / TRANSPOSE_ROWS, (n_inputs + 31) / 32), block(256);
         transpose_out_kernel<<<grid, block, 0, st>>>(tile[cur], y_out, n_neurons, n_inputs, ld);
     }
     cudaError_t e = cudaGetLastError();
