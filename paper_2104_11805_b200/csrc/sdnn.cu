@@ -42,7 +42,7 @@ struct RowShape {
 // Buffers of one inference tile in flight.  Tiles are independent of one another (so are the inputs), and a
 // handle may work on two at a time, each on its own stream, so that the ramp and tail of one tile's launches are
 // filled by the other's.
-struct TileGraph { int cols = 0, pdl = 0; bool track = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0, used = 0; };
+struct TileGraph { int cw = 0, cols = 0, pdl = 0; bool track = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0, used = 0; };
 
 struct InferLane {
     cudaStream_t stream = nullptr;         // lane 0: the handle's stream
@@ -267,12 +267,30 @@ int padded_width(int b) {
     return (b + 255) / 256 * 256;
 }
 
-// lanes per row group (g), batch entries per lane (v), (g*v)-wide chunks per tile row
-struct Geometry { int g; int v; int chunks; };
-Geometry geometry(int cols) {
-    if (cols <= 4) return {1, 4, 1};
-    if (cols <= 256) return {cols / 8, 8, 1};
-    return {32, 8, cols / 256};
+// lanes per row group (g) and batch entries per lane (v) for a chunk of cw inputs (a power of two up to 256)
+struct Geometry { int g; int v; };
+Geometry geometry(int cw) {
+    if (cw <= 4) return {1, 4};
+    return {cw / 8, 8};
+}
+
+// How the columns of an inference tile of `cnt` inputs are padded and cut: chunks of cw inputs, cols of them in all.  One chunk up
+// to 256 inputs and chunks of 256 beyond, unless chunks of 128 or 64 save more padding than the 5 or 10 % they may cost, in
+// layers that are bound by their gathers: 4096 neurons, 300 inputs are 320 columns, not 512 (960 -> 681 us for 60 layers),
+// 16384 neurons, 150 inputs 192, not 256 (631 -> 434 us for 20).  Smaller layers are bound by their chain of round trips, which
+// padding does not lengthen and more chunks do (1024 neurons, 300 inputs: 517 -> 555 us for 120).
+constexpr int64_t SHAPE_WORK = 32 << 20;      // stored elements x inputs per layer
+struct TileShape { int cw, cols; };
+TileShape tile_shape(int cnt, int64_t elems) {
+    TileShape best{std::min(padded_width(cnt), 256), padded_width(cnt)};
+    if (cnt <= 64 || elems * cnt < SHAPE_WORK) return best;
+    double least = best.cols;
+    for (int cw = 128; cw >= 64; cw /= 2) {
+        const int cols = (cnt + cw - 1) / cw * cw;
+        const double work = cols * (cw == 64 ? 1.10 : 1.05);
+        if (work < least) { least = work; best = {cw, cols}; }
+    }
+    return best;
 }
 
 int validate_cfg(const sdnn_config* cfg) {
@@ -557,37 +575,38 @@ bool entry_parallel(const sdnn* h, int ld) {
 }
 
 template <bool I16>
-void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
-    const Geometry q = geometry(cols);
+void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw) {
+    const Geometry q = geometry(cw);
+    const int chunks = cols / cw;
     if (q.v == 4 && entry_parallel(h, ld)) {
         const int wf = h->NS <= h->sms ? 1 : 4;      // few slices: one per CTA, so that they spread over as many SMs
         launch_k(h, forward_ep_kernel<I16>, dim3((h->NS + wf - 1) / wf), dim3(32 * wf), h->pdl, rows_of(h, layer),
                  (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0);
-    } else if (q.v == 4) launch_forward_gv<I16, 1, 4>(h, layer, xin, xout, ld, q.chunks);
+    } else if (q.v == 4) launch_forward_gv<I16, 1, 4>(h, layer, xin, xout, ld, chunks);
     else switch (q.g) {
-        case 1: launch_forward_gv<I16, 1, 8>(h, layer, xin, xout, ld, q.chunks); break;
-        case 2: launch_forward_gv<I16, 2, 8>(h, layer, xin, xout, ld, q.chunks); break;
-        case 4: launch_forward_gv<I16, 4, 8>(h, layer, xin, xout, ld, q.chunks); break;
-        case 8: launch_forward_gv<I16, 8, 8>(h, layer, xin, xout, ld, q.chunks); break;
-        case 16: launch_forward_gv<I16, 16, 8>(h, layer, xin, xout, ld, q.chunks); break;
+        case 1: launch_forward_gv<I16, 1, 8>(h, layer, xin, xout, ld, chunks); break;
+        case 2: launch_forward_gv<I16, 2, 8>(h, layer, xin, xout, ld, chunks); break;
+        case 4: launch_forward_gv<I16, 4, 8>(h, layer, xin, xout, ld, chunks); break;
+        case 8: launch_forward_gv<I16, 8, 8>(h, layer, xin, xout, ld, chunks); break;
+        case 16: launch_forward_gv<I16, 16, 8>(h, layer, xin, xout, ld, chunks); break;
         default:
             // a launch of at most one warp-row per resident slot is bound by its chain of round trips: four chunks (16
             // entries) of a row in flight per step instead of two, where every slice has whole steps of that size
-            if (h->lay[layer].r_chunks_mult4 && (int64_t)h->N * q.chunks <= (int64_t)h->sms * 8)
-                launch_forward_gv<I16, 32, 8, 4>(h, layer, xin, xout, ld, q.chunks);
-            else launch_forward_gv<I16, 32, 8>(h, layer, xin, xout, ld, q.chunks);
+            if (h->lay[layer].r_chunks_mult4 && (int64_t)h->N * chunks <= (int64_t)h->sms * 8)
+                launch_forward_gv<I16, 32, 8, 4>(h, layer, xin, xout, ld, chunks);
+            else launch_forward_gv<I16, 32, 8>(h, layer, xin, xout, ld, chunks);
             break;
     }
     count_launch(h);
 }
 
 // the kernels are instantiated for both index widths of the sliced copies
-void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, bool track = false) {
+void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, bool track = false) {
     if (track) {
         if (h->idx16) launch_forward_tracked_i<true>(h, layer, xin, xout, ld, cols);
         else launch_forward_tracked_i<false>(h, layer, xin, xout, ld, cols);
-    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols);
-    else launch_forward_i<false>(h, layer, xin, xout, ld, cols);
+    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, cw);
+    else launch_forward_i<false>(h, layer, xin, xout, ld, cols, cw);
 }
 
 // Windowed layers (rows grouped by shared columns at set-up): the group's window of the input tile is staged in shared
@@ -879,7 +898,7 @@ void enqueue_step_body(sdnn* h, int ld, unsigned flags, bool averaged) {
         NvtxRange chain("sdnn forward chain");
         for (int k = 0; k < h->L; ++k) {
             NvtxRange pass("forward layer", k + 1);
-            launch_forward(h, k, h->d_acts + (size_t)k * tile, h->d_acts + (size_t)(k + 1) * tile, ld, ld);
+            launch_forward(h, k, h->d_acts + (size_t)k * tile, h->d_acts + (size_t)(k + 1) * tile, ld, ld, ld);
         }
     }
     cudaEventRecordWithFlags(h->ev[1], h->stream, flags);
@@ -1003,7 +1022,7 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
 // being dropped: nobody knows what is left of those.
 constexpr int64_t GRAPH_WORK = 32 << 20;      // stored elements x inputs per layer: about 7 us
 template <typename Layers>
-int enqueue_layers(sdnn* h, InferLane& ln, int cols, bool track, const Layers& layers) {
+int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, bool track, const Layers& layers) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (h->infer_calls < 2 || h->L < 4 || (!track && h->lay[0].r_elems * cols > GRAPH_WORK) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
         capturing != cudaStreamCaptureStatusNone) {
@@ -1012,10 +1031,10 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cols, bool track, const Layers& l
     }
     TileGraph* g = &ln.graphs[0];
     for (TileGraph& q : ln.graphs) {
-        if (q.exec && q.cols == cols && q.track == track && q.pdl == h->fwd_pdl) { g = &q; break; }
+        if (q.exec && q.cw == cw && q.cols == cols && q.track == track && q.pdl == h->fwd_pdl) { g = &q; break; }
         if (g->exec && (!q.exec || q.used < g->used)) g = &q;      // the one not used for longest
     }
-    if (!g->exec || g->cols != cols || g->track != track || g->pdl != h->fwd_pdl) {
+    if (!g->exec || g->cw != cw || g->cols != cols || g->track != track || g->pdl != h->fwd_pdl) {
         if (g->exec) { cudaGraphExecDestroy(g->exec); g->exec = nullptr; }
         cudaGraph_t graph = nullptr;
         const int64_t before = h->launches;
@@ -1028,7 +1047,7 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cols, bool track, const Layers& l
         e = cudaGraphInstantiate(&g->exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) { g->exec = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
-        g->cols = cols; g->track = track; g->pdl = h->fwd_pdl;
+        g->cw = cw; g->cols = cols; g->track = track; g->pdl = h->fwd_pdl;
     }
     g->used = h->infer_calls;
     CU(h, cudaGraphLaunch(g->exec, ln.stream));
@@ -1041,13 +1060,15 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
                bool want_sets) {
     NvtxRange call("sdnn inference tile");
     const int ld = h->ld_max;
-    const int cols = padded_width(cnt);
     cudaStream_t st = ln.stream;
     h->cur = &ln;
     h->launch_stream = st;
-    launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     bool track = h->compaction && h->cfg.activation == SDNN_ACT_CLAMPED_RELU;      // sigmoid(b) is never 0: nothing ever dies
     for (int l = 0; l < h->L && track; ++l) track = h->bias_nonpositive[l] != 0;     // the zero vector must be a fixed point
+    // dropping dead inputs works on chunks of 64 whatever the padding
+    const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->lay[0].r_elems);
+    const int cw = shape.cw, cols = shape.cols;
+    launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     auto layers = [&]() {
         int cur = 0;
         if (track) {
@@ -1055,7 +1076,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
             const int rows_grid = std::min((h->N + 7) / 8, h->sms * 8);
             cudaMemsetAsync(ln.cs.flags, 0, (size_t)h->L * ld * sizeof(int), st);
             for (int k = 0; k < h->L; ++k) {
-                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, true);
+                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, true);
                 cur ^= 1;
                 // dropping what has died: after each of the first layers, where most do, then at growing distances (after 1, 2, 3, 4,
                 // 6, 8, 12, 16, 24, ... layers)
@@ -1073,7 +1094,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
             for (int k = 0; k < h->L; ++k) {
                 NvtxRange pass("forward layer", k + 1);
                 if (h->lay[k].windowed) launch_forward_window(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
-                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
+                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw);
                 cur ^= 1;
             }
         }
@@ -1085,7 +1106,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
         h->live_lane = (int)(&ln - h->lane);
     }
     {
-        const int rc = enqueue_layers(h, ln, cols, track, layers);
+        const int rc = enqueue_layers(h, ln, cw, cols, track, layers);
         if (rc) return rc;
     }
     const int cur = (h->L + (track ? 1 : 0)) & 1;

@@ -85,3 +85,15 @@ def test_whole_network_launch(torch_cuda, n, k, layers, cnt, act):  # noqa: F811
         check_close(y.cpu().numpy(), ora.infer(x0), "x^L")
         assert np.array_equal(c.cpu().numpy(), np.count_nonzero(y.cpu().numpy(), axis=1))
     h.destroy()
+
+
+@pytest.mark.parametrize("cnt", [65, 129, 150, 300, 449, 513])
+def test_tile_widths_between_powers_of_two(torch_cuda, cnt):  # noqa: F811
+    """Layers large enough for tiles cut into chunks of 64 or 128 inputs: widths just above a chunk, a few chunks, and one that
+    keeps chunks of 256; outputs, counts and id lists."""
+    rng = np.random.default_rng(cnt)
+    n, k = 8200, 64
+    cols = [np.concatenate([np.sort(rng.integers(0, n - k + 1, size=k)) + np.arange(k) for _ in range(n)]).astype(np.int32) for _ in range(2)]
+    vals = [(rng.standard_normal(n * k) * (2.0 / k) ** 0.5).astype(np.float32) for _ in range(2)]
+    arrays = ([np.arange(n + 1, dtype=np.int32) * k] * 2, cols, vals, [np.zeros(n, dtype=np.float32)] * 2)
+    infer_parity(torch_cuda, arrays, vectors(rng, cnt, n), 600, expect_nonempty=True)
