@@ -97,3 +97,11 @@ def test_tile_widths_between_powers_of_two(torch_cuda, cnt):  # noqa: F811
     vals = [(rng.standard_normal(n * k) * (2.0 / k) ** 0.5).astype(np.float32) for _ in range(2)]
     arrays = ([np.arange(n + 1, dtype=np.int32) * k] * 2, cols, vals, [np.zeros(n, dtype=np.float32)] * 2)
     infer_parity(torch_cuda, arrays, vectors(rng, cnt, n), 600, expect_nonempty=True)
+
+
+@pytest.mark.parametrize("cnt", [255, 256, 300, 500])
+def test_host_batches_cut_in_two(torch_cuda, cnt):  # noqa: F811
+    """Host batches of one tile around the size from which they are halved: outputs, counts and ids in the order of the inputs."""
+    rng = np.random.default_rng(cnt)
+    arrays = ragged_net(rng, n=2111, layers=3, kmax=40, scale=0.3)
+    infer_parity(torch_cuda, arrays, vectors(rng, cnt, 2111), 512, host=True, expect_nonempty=True)
