@@ -176,7 +176,9 @@ struct sdnn {
     float* d_stage_a2 = nullptr;        // second input stage of sdnn_infer_batch_host: tile t+1 is copied while tile t computes
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_consumed[2] = {nullptr, nullptr};
+    float* d_stage_b2 = nullptr;        // output stage of the second tile in flight
     int* d_stage_cnt = nullptr;
+    int* d_stage_cnt2 = nullptr;
     float* d_stage_w = nullptr;         // one layer's values in the caller's order (sdnn_get/set_weights)
     static constexpr int PINS = 4;      // pinned pieces that results for pageable memory travel through
     char* pin[PINS] = {nullptr, nullptr, nullptr, nullptr};
@@ -997,8 +999,8 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     else ln.stream = h->stream;
     CU(h, cudaEventCreateWithFlags(&ln.ev_scan, cudaEventDisableTiming));
     CU(h, cudaEventCreateWithFlags(&ln.ev_done, cudaEventDisableTiming));
-    if ((rc = dev_alloc(h, &ln.tile[0], tile, false))) return rc;
-    if ((rc = dev_alloc(h, &ln.tile[1], tile, false))) return rc;
+    if ((rc = dev_alloc(h, &ln.tile[0], 2 * tile, false))) return rc;
+    ln.tile[1] = ln.tile[0] + tile;
     if ((rc = dev_alloc(h, &ln.seg_cnt, nseg * (size_t)h->ld_max, false))) return rc;
     if ((rc = dev_alloc(h, &ln.nz_bits, ((size_t)h->N + 31) / 32 * (size_t)h->ld_max, false))) return rc;
     if ((rc = dev_alloc(h, &ln.tile_cnt, (size_t)h->ld_max, false))) return rc;
@@ -2133,25 +2135,28 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     // two input stages and a copy stream: the copy of tile t+1 runs under the layers of tile t
     const int T = host_tile_width(h, n_inputs);
+    const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // the two halves share the stages of one tile
     if (!h->copy_stream) {
         CU(h, cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
         for (int q = 0; q < 2; ++q) {
             CU(h, cudaEventCreateWithFlags(&h->ev_copied[q], cudaEventDisableTiming));
             CU(h, cudaEventCreateWithFlags(&h->ev_consumed[q], cudaEventDisableTiming));
         }
-        if ((rc = dev_alloc(h, &h->d_stage_a2, (size_t)h->cfg.max_batch * h->N, false))) return rc;
     }
-    float* stage[2] = {h->d_stage_a, h->d_stage_a2};
+    if (!halved && !h->d_stage_a2 && (rc = dev_alloc(h, &h->d_stage_a2, (size_t)h->cfg.max_batch * h->N, false))) return rc;
+    float* stage[2] = {h->d_stage_a, halved ? h->d_stage_a + (size_t)T * h->N : h->d_stage_a2};
     CU(h, cudaEventRecord(h->ev_consumed[0], h->stream));       // the stages may still be read by earlier work on the stream
     CU(h, cudaEventRecord(h->ev_consumed[1], h->stream));
     const int lanes = n_inputs > T ? infer_lanes(h, T) : 1;
     if ((rc = lanes_begin(h, lanes))) return rc;
+    if (lanes == 2 && !halved && !h->d_stage_b2) {
+        if ((rc = dev_alloc(h, &h->d_stage_b2, (size_t)h->cfg.max_batch * h->N, false))) return rc;
+        if ((rc = dev_alloc(h, &h->d_stage_cnt2, (size_t)h->cfg.max_batch, false))) return rc;
+    }
     h->lane[0].stage_out = h->d_stage_b;
     h->lane[0].stage_cnt = h->d_stage_cnt;
-    if (lanes == 2 && !h->lane[1].stage_out) {
-        if ((rc = dev_alloc(h, &h->lane[1].stage_out, (size_t)h->cfg.max_batch * h->N, false))) return rc;
-        if ((rc = dev_alloc(h, &h->lane[1].stage_cnt, (size_t)h->cfg.max_batch, false))) return rc;
-    }
+    h->lane[1].stage_out = halved ? h->d_stage_b + (size_t)T * h->N : h->d_stage_b2;
+    h->lane[1].stage_cnt = halved ? h->d_stage_cnt + T : h->d_stage_cnt2;
     int64_t tile_no = 0;
     for (int64_t t0 = 0; t0 < n_inputs; t0 += T, ++tile_no) {
         const int cnt = (int)((n_inputs - t0 < T) ? (n_inputs - t0) : T);
