@@ -30,7 +30,7 @@
 
 namespace sdnn_kernels {
 
-struct StepParams {     // written by set_step_params before each train step; read by the graph's kernels
+struct StepParams {     // written by start_step_kernel at the start of each train step; read by the graph's kernels
     float eta;          // learning rate
     float inv_b;        // 1 / B
     int   batch;        // B (valid inputs; the tile is zero-padded to ld)
@@ -309,8 +309,8 @@ __device__ __forceinline__ void chunk_update(float* vp, float* gp, const float4&
 // With 4-byte accesses and 32 x 32 tiles 65536 x 1024 floats took 213 us in and 178 us out; HBM needs 83.
 // row_map (or NULL): tile row of input neuron i, for nets whose input neurons were renumbered at set-up.
 constexpr int TRANSPOSE_ROWS = 128, TRANSPOSE_PITCH = 33;
-__global__ void __launch_bounds__(256)
-transpose_in_kernel(const float* __restrict__ src, float* __restrict__ dst, int n, int cnt, int cols, int ld, const int* __restrict__ row_map) {
+__device__ __forceinline__ void transpose_in(const float* __restrict__ src, float* __restrict__ dst, int n, int cnt, int cols, int ld,
+                                             const int* __restrict__ row_map) {
     __shared__ float t[TRANSPOSE_ROWS * TRANSPOSE_PITCH];      // [neuron][input]
     const int i0 = blockIdx.x * TRANSPOSE_ROWS, b0 = blockIdx.y * 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = i0 + lane * 4;
@@ -346,6 +346,11 @@ transpose_in_kernel(const float* __restrict__ src, float* __restrict__ dst, int 
             st_f4(dst + (size_t)(row_map ? row_map[i0 + r] : i0 + r) * ld + b0 + quad * 4, make_float4(s[0], s[1], s[2], s[3]));
         }
     }
+}
+
+__global__ void __launch_bounds__(256)
+transpose_in_kernel(const float* __restrict__ src, float* __restrict__ dst, int n, int cnt, int cols, int ld, const int* __restrict__ row_map) {
+    transpose_in(src, dst, n, cnt, cols, ld, row_map);
 }
 
 // tile [n][ld] -> y [cnt][n]; the same blocks
@@ -386,9 +391,19 @@ transpose_out_kernel(const float* __restrict__ src, float* __restrict__ dst, int
     }
 }
 
-__global__ void set_step_params_kernel(StepParams* p, float eta, int batch, double* loss) {
-    p->eta = eta; p->inv_b = 1.0f / (float)batch; p->batch = batch; p->pad = 0;
-    *loss = 0.0;
+// Start of a train step in one launch: the input tile (blockIdx.z = 0), the target tile (1), and the step's parameters.  sp_batch
+// (or NULL): the averaged form, whose backward chain runs on a single vector (sp) while its means are over the batch (sp_batch).
+__global__ void __launch_bounds__(256)
+start_step_kernel(const float* __restrict__ x0, float* __restrict__ x_tile, const float* __restrict__ target, float* __restrict__ y_tile, int n, int batch,
+                  int ld, const int* __restrict__ row_map, StepParams* sp, StepParams* sp_batch, float eta, double* loss) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
+        const int b = sp_batch ? 1 : batch;
+        sp->eta = eta; sp->inv_b = 1.0f / (float)b; sp->batch = b; sp->pad = 0;
+        if (sp_batch) { sp_batch->eta = eta; sp_batch->inv_b = 1.0f / (float)batch; sp_batch->batch = batch; sp_batch->pad = 0; }
+        *loss = 0.0;
+    }
+    if (blockIdx.z == 0) transpose_in(x0, x_tile, n, batch, ld, ld, row_map);
+    else transpose_in(target, y_tile, n, batch, ld, ld, nullptr);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -936,15 +936,11 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
             if ((rc = dev_alloc(h, &h->d_mean, (size_t)(h->L + 1) * h->N * 4, true))) return rc;
             if ((rc = dev_alloc(h, &h->d_sp_batch, 1, true))) return rc;
         }
-        set_step_params_kernel<<<1, 1, 0, h->stream>>>(h->d_sp_batch, eta, B, h->d_loss);
-        set_step_params_kernel<<<1, 1, 0, h->stream>>>(h->d_sp, eta, 1, h->d_loss);
-        count_launch(h, 2);
-    } else {
-        set_step_params_kernel<<<1, 1, 0, h->stream>>>(h->d_sp, eta, B, h->d_loss);
-        count_launch(h);
     }
-    launch_transpose_in(h, x0, h->d_acts, B, ld, ld, h->d_in_label);
-    launch_transpose_in(h, target, h->d_yt, B, ld, ld);
+    const dim3 start_grid((h->N + TRANSPOSE_ROWS - 1) / TRANSPOSE_ROWS, (ld + 31) / 32, 2);
+    start_step_kernel<<<start_grid, 256, 0, h->stream>>>(x0, h->d_acts, target, h->d_yt, h->N, B, ld, (const int*)h->d_in_label, h->d_sp,
+                                                         averaged ? h->d_sp_batch : (StepParams*)nullptr, eta, h->d_loss);
+    count_launch(h);
     if (h->cfg.flags & SDNN_FLAG_NO_GRAPH) {
         enqueue_step_body(h, ld, cudaEventRecordDefault, averaged);
     } else {
@@ -1357,6 +1353,12 @@ void sliced_to_csr(const sdnn* h, const LayerMem& lm, const std::vector<float>& 
 // engine fills some while the host cores empty the others, so that the page faults of a fresh array are taken by several
 // cores and under the transfer (sdnn_get_weights of 2 M entries, 8 MB: 3.7 -> 0.7 ms; of 0.5 M entries: 0.7 -> 0.13 ms).
 constexpr size_t PIN_BYTES = 1 << 20;
+int ensure_pin(sdnn* h, int q) {
+    if (h->pin[q]) return SDNN_OK;
+    CU(h, cudaMallocHost((void**)&h->pin[q], PIN_BYTES));
+    CU(h, cudaEventCreateWithFlags(&h->ev_pin[q], cudaEventDisableTiming));
+    return SDNN_OK;
+}
 int copy_to_caller(sdnn* h, void* dst, const void* src, size_t bytes) {
     cudaPointerAttributes at{};
     const bool pageable = cudaPointerGetAttributes(&at, dst) != cudaSuccess || at.type == cudaMemoryTypeUnregistered;
@@ -1369,10 +1371,7 @@ int copy_to_caller(sdnn* h, void* dst, const void* src, size_t bytes) {
     const int64_t pieces = (int64_t)((bytes + PIN_BYTES - 1) / PIN_BYTES);
     auto issue = [&](int64_t p) -> int {
         const int q = (int)(p % sdnn::PINS);
-        if (!h->pin[q]) {
-            CU(h, cudaMallocHost((void**)&h->pin[q], PIN_BYTES));
-            CU(h, cudaEventCreateWithFlags(&h->ev_pin[q], cudaEventDisableTiming));
-        }
+        if (const int rc_pin = ensure_pin(h, q)) return rc_pin;
         const size_t lo = (size_t)p * PIN_BYTES;
         CU(h, cudaMemcpyAsync(h->pin[q], static_cast<const char*>(src) + lo, std::min(PIN_BYTES, bytes - lo), cudaMemcpyDeviceToHost, h->stream));
         CU(h, cudaEventRecord(h->ev_pin[q], h->stream));
@@ -1402,9 +1401,9 @@ int ensure_stage_w(sdnn* h) {
 
 // values of a layer whose stored entries are the caller's, row by row: device staging buffer <-> sliced copy
 template <bool TO_CSR>
-int convert_values(sdnn* h, int layer) {
+int convert_values(sdnn* h, int layer, float* csr) {
     const LayerMem& lm = h->lay[layer];
-    sliced_csr_kernel<TO_CSR><<<(h->N + 15) / 16, 512, 0, h->stream>>>(rows_of(h, layer), h->d_stage_w, (const int*)lm.r_start, lm.shape.uniform_k, h->N);
+    sliced_csr_kernel<TO_CSR><<<(h->N + 15) / 16, 512, 0, h->stream>>>(rows_of(h, layer), csr, (const int*)lm.r_start, lm.shape.uniform_k, h->N);
     count_launch(h);
     CU(h, cudaGetLastError());
     return SDNN_OK;
@@ -2197,7 +2196,12 @@ int sdnn_get_weights(sdnn_t* h, int32_t layer, float* values_out, float* bias_ou
     const int64_t nnz = h->nnz[layer];
     if (values_out && nnz && lm.entry_src.empty()) {
         int rc;
-        if ((rc = ensure_stage_w(h)) || (rc = convert_values<true>(h, layer)) || (rc = copy_to_caller(h, values_out, h->d_stage_w, (size_t)nnz * sizeof(float)))) return rc;
+        const size_t bytes = (size_t)nnz * sizeof(float);
+        if (bytes <= PIN_BYTES / 4) {      // a small layer: the kernel writes to pinned memory itself, one launch and one wait
+            if ((rc = ensure_pin(h, 0)) || (rc = convert_values<true>(h, layer, reinterpret_cast<float*>(h->pin[0])))) return rc;
+            CU(h, cudaStreamSynchronize(h->stream));
+            memcpy(values_out, h->pin[0], bytes);
+        } else if ((rc = ensure_stage_w(h)) || (rc = convert_values<true>(h, layer, h->d_stage_w)) || (rc = copy_to_caller(h, values_out, h->d_stage_w, bytes))) return rc;
     } else if (values_out && nnz) {      // entries in another order than the caller's (SDNN_FLAG_REORDER)
         CU(h, cudaStreamSynchronize(h->stream));
         std::vector<float> stored((size_t)nnz);
@@ -2250,7 +2254,7 @@ int sdnn_set_weights(sdnn_t* h, int32_t layer, const float* values, const float*
             int rc;
             if ((rc = ensure_stage_w(h))) return rc;
             CU(h, cudaMemcpyAsync(h->d_stage_w, values, (size_t)nnz * sizeof(float), cudaMemcpyHostToDevice, h->stream));
-            if ((rc = convert_values<false>(h, layer))) return rc;
+            if ((rc = convert_values<false>(h, layer, h->d_stage_w))) return rc;
             CU(h, cudaStreamSynchronize(h->stream));
         } else if (lm.windowed) {
             tmp.assign((size_t)lm.w_elems, 0.0f);
