@@ -144,7 +144,7 @@ struct sdnn {
     StepParams* d_sp_batch = nullptr;   // the real batch, while d_sp describes the single backpropagated vector
     const float* bwd_acts = nullptr;    // activations the backward launches read (NULL: d_acts)
     cudaGraphExec_t graph = nullptr, graph_avg = nullptr;
-    int graph_ld = 0, graph_avg_ld = 0;
+    int graph_ld = 0, graph_avg_ld = 0, graph_v = 0, graph_avg_v = 0;
     int64_t graph_launches = 0, graph_avg_launches = 0;   // kernel nodes of the captured steps
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};   // before forward chain, between, after backward chain
 
@@ -889,16 +889,136 @@ void enqueue_backward_chain(sdnn* h, int ld) {
     }
 }
 
-// forward + backward chain of one train step on the internal buffers; `flags` selects how the three
+// ---------------------------------------------------------------------------------------------
+// Whole networks in one launch for one to four inputs (vector.cuh): nets whose rows all have the same padded length, up to 4096
+// neurons x (padded) inputs.  120 layers of 1024 neurons, one launch per layer / one launch: 1 input 255 / 121 us, 4 inputs 252 /
+// 176; 60 layers of 2048: 1 input 143 / 98, 4 inputs 142 / 159; of 4096: 1 input 149 / 156, 2 inputs 149 / 195.  And it leaves 132
+// SMs to other handles: three of them asked in turn answer an input in 47 us each instead of 240 (1024 x 120).
+constexpr int VECTOR_WORK = 4096, VECTOR_DEPTH = 2048;
+
+// Status words that kernels raise and the host reads without waiting: one page of pinned memory for all handles (pinning one
+// takes longer than loading a small net), given back when the last of them goes.
+struct StatusPage {
+    static constexpr int WORDS = 1024;
+    std::mutex mutex;
+    int* words = nullptr;
+    std::vector<char> taken;
+    int users = 0;
+    int* get() {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (!words) {
+            if (cudaHostAlloc((void**)&words, WORDS * sizeof(int), cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); words = nullptr; return nullptr; }
+            taken.assign(WORDS, 0);
+        }
+        for (int q = 0; q < WORDS; ++q)
+            if (!taken[q]) { taken[q] = 1; ++users; words[q] = 0; return words + q; }
+        return nullptr;
+    }
+    void put(int* p) {
+        std::lock_guard<std::mutex> lock(mutex);
+        taken[p - words] = 0;
+        if (--users == 0) { cudaFreeHost(words); words = nullptr; }
+    }
+};
+StatusPage& status_page() { static StatusPage page; return page; }
+
+// table of layer pointers (called by sdnn_finalize)
+int build_vector(sdnn* h) {
+    if (h->reorder || h->compaction || !h->idx16 || h->N > VECTOR_WORK || h->L > VECTOR_DEPTH) return SDNN_OK;
+    int rc;
+    std::vector<VectorLayer> table(h->L);
+    for (int k = 0; k < h->L; ++k) {
+        const LayerMem& lm = h->lay[k];
+        const int kpad = lm.r_slice_off[1] / SLICE;
+        if (lm.r_out || kpad == 0 || (k > 0 && kpad != h->vector_kpad)) return SDNN_OK;
+        for (int sl = 0; sl < h->NS; ++sl) if (lm.r_slice_off[sl + 1] - lm.r_slice_off[sl] != kpad * SLICE) return SDNN_OK;
+        table[k] = VectorLayer{reinterpret_cast<const unsigned short*>(lm.r_idx), lm.r_val};
+        h->vector_kpad = kpad;
+    }
+    if (!(h->vector_status = status_page().get())) return SDNN_OK;      // no word left: the launches per layer do it
+    if ((rc = dev_alloc(h, &h->d_vector, (size_t)h->L, false))) return rc;
+    CU(h, cudaMemcpyAsync(h->d_vector, table.data(), table.size() * sizeof(VectorLayer), cudaMemcpyHostToDevice, h->stream));
+    CU(h, cudaStreamSynchronize(h->stream));
+    return SDNN_OK;
+}
+
+int vector_check(sdnn* h) {
+    if (!h->vector_status || !*h->vector_status) return SDNN_OK;
+    *h->vector_status = 0;
+    return fail(h, SDNN_ERR_CUDA, "a whole-network launch gave up waiting for its neighbours: the results of that call are not valid");
+}
+
+// shared memory of vector_infer_kernel<v> without its ring of entries, and a stage of the ring
+size_t vector_smem(const sdnn* h, int v, size_t* stage) {
+    const size_t blocks = (h->N + VECTOR_CTAS * VECTOR_BLOCK - 1) / (VECTOR_CTAS * VECTOR_BLOCK);
+    *stage = blocks * VECTOR_BLOCK * (size_t)h->vector_kpad * 6;
+    return 2 * (((size_t)h->N * v * 4 + 15) & ~(size_t)15) + 2 * blocks * VECTOR_BLOCK * v * 4 + (size_t)h->L * sizeof(VectorLayer) + 128;
+}
+constexpr size_t VECTOR_SMEM = 226 * 1024;
+// stages of the ring that fit; below three a layer's entries would be waited for
+int vector_stages(const sdnn* h, int v) {
+    size_t stage = 0;
+    const size_t base = vector_smem(h, v, &stage);
+    return base >= VECTOR_SMEM ? 0 : (int)std::min<size_t>(VECTOR_STAGES, (VECTOR_SMEM - base) / stage);
+}
+
+template <int V>
+int launch_vector(sdnn* h, VectorArgs a) {
+    size_t stage = 0;
+    const size_t base = vector_smem(h, V, &stage), smem = base + vector_stages(h, V) * stage;
+    a.stages = vector_stages(h, V);
+    const void* kernel = (const void*)vector_infer_kernel<V>;
+    if (!h->carved[kernel]) {
+        CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VECTOR_SMEM));
+        CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        h->carved[kernel] = true;
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(VECTOR_CTAS); lc.blockDim = dim3(VECTOR_THREADS); lc.dynamicSmemBytes = smem; lc.stream = h->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = VECTOR_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    lc.attrs = at; lc.numAttrs = 1;
+    CU(h, cudaLaunchKernelEx(&lc, vector_infer_kernel<V>, a));
+    count_launch(h);
+    return SDNN_OK;
+}
+
+bool takes_vector(const sdnn* h, int cnt) {
+    const int v = cnt <= 2 ? cnt : 4;
+    return h->d_vector && (int64_t)h->N * v <= VECTOR_WORK && vector_stages(h, v) >= 3;
+}
+
+// Forward chain of a train step by the same kernel, where its latency counts alone: 48 layers of 1024 neurons, one input
+// 80 -> 57 us, two 80 -> 63; four, and one through 2048 neurons, the same either way.
+constexpr int VECTOR_TRAIN_WORK = 2048;
+int train_vector_width(const sdnn* h, int B) {
+    const int v = B <= 2 ? B : 4;
+    return B <= 4 && h->split && h->N < VECTOR_TRAIN_WORK && h->N * v <= VECTOR_TRAIN_WORK && takes_vector(h, B) ? v : 0;
+}
+int forward_vector(sdnn* h, int v) {
+    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, h->vector_kpad, 0, nullptr, v, nullptr, nullptr, h->d_acts, h->vector_status, h->cfg.clamp, h->cfg.activation};
+    return v == 1 ? launch_vector<1>(h, a) : v == 2 ? launch_vector<2>(h, a) : launch_vector<4>(h, a);
+}
+
+// All layers for one to four inputs: x0 [cnt][N] -> y and nonzero counts (either may be NULL).
+int infer_vector(sdnn* h, const float* x0, int cnt, float* y, int* nz_count) {
+    NvtxRange call("sdnn whole-network inference");
+    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, h->vector_kpad, 0, x0, cnt, y, nz_count, nullptr, h->vector_status, h->cfg.clamp, h->cfg.activation};
+    return cnt == 1 ? launch_vector<1>(h, a) : cnt == 2 ? launch_vector<2>(h, a) : launch_vector<4>(h, a);
+}
+
+// forward + backward chain of one train step on the internal buffers; v: see train_vector_width; `flags` selects how the three
 // timing events are recorded (as external event-record nodes while capturing a graph).
 // averaged: the forward chain runs on the whole batch, then the batch means of x^0..x^L and the averaged delta^L are
 // formed and the backward chain runs on those single vectors (tiles of padded width 4).
-void enqueue_step_body(sdnn* h, int ld, unsigned flags, bool averaged) {
+void enqueue_step_body(sdnn* h, int ld, int v, unsigned flags, bool averaged) {
     const size_t tile = (size_t)h->N * ld;
     cudaEventRecordWithFlags(h->ev[0], h->stream, flags);
     {
         NvtxRange chain("sdnn forward chain");
-        for (int k = 0; k < h->L; ++k) {
+        if (v) forward_vector(h, v);
+        else for (int k = 0; k < h->L; ++k) {
             NvtxRange pass("forward layer", k + 1);
             launch_forward(h, k, h->d_acts + (size_t)k * tile, h->d_acts + (size_t)(k + 1) * tile, ld, ld, ld);
         }
@@ -928,7 +1048,8 @@ void enqueue_step_body(sdnn* h, int ld, unsigned flags, bool averaged) {
 
 int train_step_device(sdnn* h, const float* x0, const float* target, int B, float eta, float* loss_out, bool averaged = false) {
     NvtxRange call(averaged ? "sdnn_train_step_averaged" : "sdnn_train_step");
-    const int ld = padded_width(B);
+    const int ld = padded_width(B), v = train_vector_width(h, B);      // v: the forward chain as one launch for v inputs (0: a launch per layer)
+    if (const int rc = vector_check(h)) return rc;
     h->fwd_pdl = PDL_EARLY;
     if (averaged) {
         if (!h->d_mean) {
@@ -942,17 +1063,18 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
                                                          averaged ? h->d_sp_batch : (StepParams*)nullptr, eta, h->d_loss);
     count_launch(h);
     if (h->cfg.flags & SDNN_FLAG_NO_GRAPH) {
-        enqueue_step_body(h, ld, cudaEventRecordDefault, averaged);
+        enqueue_step_body(h, ld, v, cudaEventRecordDefault, averaged);
     } else {
         cudaGraphExec_t& graph = averaged ? h->graph_avg : h->graph;
         int& graph_ld = averaged ? h->graph_avg_ld : h->graph_ld;
+        int& graph_v = averaged ? h->graph_avg_v : h->graph_v;
         int64_t& graph_launches = averaged ? h->graph_avg_launches : h->graph_launches;
-        if (!graph || graph_ld != ld) {
+        if (!graph || graph_ld != ld || graph_v != v) {
             if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
             cudaGraph_t g = nullptr;
             const int64_t before = h->launches;
             CU(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-            enqueue_step_body(h, ld, cudaEventRecordExternal, averaged);
+            enqueue_step_body(h, ld, v, cudaEventRecordExternal, averaged);
             cudaError_t e = cudaStreamEndCapture(h->stream, &g);
             graph_launches = h->launches - before;
             h->launches = before;
@@ -960,7 +1082,7 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
             e = cudaGraphInstantiate(&graph, g, 0);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) { graph = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
-            graph_ld = ld;
+            graph_ld = ld; graph_v = v;
         }
         CU(h, cudaGraphLaunch(graph, h->stream));
         count_launch(h, (int)graph_launches);
@@ -973,6 +1095,7 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
         CU(h, cudaMemcpyAsync(&j, h->d_loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         CU(h, cudaStreamSynchronize(h->stream));
         *loss_out = (float)j;
+        return vector_check(h);
     }
     return SDNN_OK;
 }
@@ -1136,113 +1259,6 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     }
     CU(h, cudaGetLastError());
     return SDNN_OK;
-}
-
-// ---------------------------------------------------------------------------------------------
-// Whole networks in one launch for one to four inputs (vector.cuh): nets whose rows all have the same padded length, up to 4096
-// neurons x (padded) inputs.  120 layers of 1024 neurons, one launch per layer / one launch: 1 input 255 / 121 us, 4 inputs 252 /
-// 176; 60 layers of 2048: 1 input 143 / 98, 4 inputs 142 / 159; of 4096: 1 input 149 / 156, 2 inputs 149 / 195.  And it leaves 132
-// SMs to other handles: three of them asked in turn answer an input in 47 us each instead of 240 (1024 x 120).
-constexpr int VECTOR_WORK = 4096, VECTOR_DEPTH = 2048;
-
-// Status words that kernels raise and the host reads without waiting: one page of pinned memory for all handles (pinning one
-// takes longer than loading a small net), given back when the last of them goes.
-struct StatusPage {
-    static constexpr int WORDS = 1024;
-    std::mutex mutex;
-    int* words = nullptr;
-    std::vector<char> taken;
-    int users = 0;
-    int* get() {
-        std::lock_guard<std::mutex> lock(mutex);
-        if (!words) {
-            if (cudaHostAlloc((void**)&words, WORDS * sizeof(int), cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); words = nullptr; return nullptr; }
-            taken.assign(WORDS, 0);
-        }
-        for (int q = 0; q < WORDS; ++q)
-            if (!taken[q]) { taken[q] = 1; ++users; words[q] = 0; return words + q; }
-        return nullptr;
-    }
-    void put(int* p) {
-        std::lock_guard<std::mutex> lock(mutex);
-        taken[p - words] = 0;
-        if (--users == 0) { cudaFreeHost(words); words = nullptr; }
-    }
-};
-StatusPage& status_page() { static StatusPage page; return page; }
-
-// table of layer pointers (called by sdnn_finalize)
-int build_vector(sdnn* h) {
-    if (h->reorder || h->compaction || !h->idx16 || h->N > VECTOR_WORK || h->L > VECTOR_DEPTH) return SDNN_OK;
-    int rc;
-    std::vector<VectorLayer> table(h->L);
-    for (int k = 0; k < h->L; ++k) {
-        const LayerMem& lm = h->lay[k];
-        const int kpad = lm.r_slice_off[1] / SLICE;
-        if (lm.r_out || kpad == 0 || (k > 0 && kpad != h->vector_kpad)) return SDNN_OK;
-        for (int sl = 0; sl < h->NS; ++sl) if (lm.r_slice_off[sl + 1] - lm.r_slice_off[sl] != kpad * SLICE) return SDNN_OK;
-        table[k] = VectorLayer{reinterpret_cast<const unsigned short*>(lm.r_idx), lm.r_val};
-        h->vector_kpad = kpad;
-    }
-    if (!(h->vector_status = status_page().get())) return SDNN_OK;      // no word left: the launches per layer do it
-    if ((rc = dev_alloc(h, &h->d_vector, (size_t)h->L, false))) return rc;
-    CU(h, cudaMemcpyAsync(h->d_vector, table.data(), table.size() * sizeof(VectorLayer), cudaMemcpyHostToDevice, h->stream));
-    CU(h, cudaStreamSynchronize(h->stream));
-    return SDNN_OK;
-}
-
-int vector_check(sdnn* h) {
-    if (!h->vector_status || !*h->vector_status) return SDNN_OK;
-    *h->vector_status = 0;
-    return fail(h, SDNN_ERR_CUDA, "a whole-network launch gave up waiting for its neighbours: the results of that call are not valid");
-}
-
-// shared memory of vector_infer_kernel<v> without its ring of entries, and a stage of the ring
-size_t vector_smem(const sdnn* h, int v, size_t* stage) {
-    const size_t blocks = (h->N + VECTOR_CTAS * VECTOR_BLOCK - 1) / (VECTOR_CTAS * VECTOR_BLOCK);
-    *stage = blocks * VECTOR_BLOCK * (size_t)h->vector_kpad * 6;
-    return 2 * (((size_t)h->N * v * 4 + 15) & ~(size_t)15) + 2 * blocks * VECTOR_BLOCK * v * 4 + (size_t)h->L * sizeof(VectorLayer) + 128;
-}
-constexpr size_t VECTOR_SMEM = 226 * 1024;
-// stages of the ring that fit; below three a layer's entries would be waited for
-int vector_stages(const sdnn* h, int v) {
-    size_t stage = 0;
-    const size_t base = vector_smem(h, v, &stage);
-    return base >= VECTOR_SMEM ? 0 : (int)std::min<size_t>(VECTOR_STAGES, (VECTOR_SMEM - base) / stage);
-}
-
-template <int V>
-int launch_vector(sdnn* h, VectorArgs a) {
-    size_t stage = 0;
-    const size_t base = vector_smem(h, V, &stage), smem = base + vector_stages(h, V) * stage;
-    a.stages = vector_stages(h, V);
-    const void* kernel = (const void*)vector_infer_kernel<V>;
-    if (!h->carved[kernel]) {
-        CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VECTOR_SMEM));
-        CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        h->carved[kernel] = true;
-    }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(VECTOR_CTAS); lc.blockDim = dim3(VECTOR_THREADS); lc.dynamicSmemBytes = smem; lc.stream = h->stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = VECTOR_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    lc.attrs = at; lc.numAttrs = 1;
-    CU(h, cudaLaunchKernelEx(&lc, vector_infer_kernel<V>, a));
-    count_launch(h);
-    return SDNN_OK;
-}
-
-bool takes_vector(const sdnn* h, int cnt) {
-    const int v = cnt <= 2 ? cnt : 4;
-    return h->d_vector && (int64_t)h->N * v <= VECTOR_WORK && vector_stages(h, v) >= 3;
-}
-
-// All layers for one to four inputs: x0 [cnt][N] -> y and nonzero counts (either may be NULL).
-int infer_vector(sdnn* h, const float* x0, int cnt, float* y, int* nz_count) {
-    NvtxRange call("sdnn whole-network inference");
-    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, h->vector_kpad, 0, x0, cnt, y, nz_count, h->vector_status, h->cfg.clamp, h->cfg.activation};
-    return cnt == 1 ? launch_vector<1>(h, a) : cnt == 2 ? launch_vector<2>(h, a) : launch_vector<4>(h, a);
 }
 
 // Inputs per inference tile.  The gathers of a layer read the whole activation tile at random, so the two

@@ -37,6 +37,7 @@ struct VectorArgs {
     int cnt;
     float* y;                       // [cnt][n] or NULL
     int* nz_count;                  // [cnt] or NULL
+    float* acts;                    // training: tiles [depth + 1][n][4] of x^0 (read instead of x) and x^1 .. (written); else NULL
     int* status;
     float clamp;
     int act;
@@ -110,7 +111,8 @@ vector_infer_kernel(const VectorArgs a) {
     // the input vectors, in every CTA
     for (int i = threadIdx.x; i < n; i += VECTOR_THREADS)
 #pragma unroll
-        for (int b = 0; b < V; ++b) reinterpret_cast<float*>(vector_smem)[i * V + b] = b < a.cnt ? a.x[(size_t)b * n + i] : 0.0f;
+        for (int b = 0; b < V; ++b)
+            reinterpret_cast<float*>(vector_smem)[i * V + b] = a.acts ? a.acts[i * 4 + b] : b < a.cnt ? a.x[(size_t)b * n + i] : 0.0f;
     // receivers: warp w sends to CTAs w and w + 8
     const unsigned my_x = x0 + rank * (VECTOR_BLOCK * PITCH);
     const unsigned to_x[2] = {cluster_addr(my_x, warp), cluster_addr(my_x, warp + VECTOR_WARPS)};
@@ -191,6 +193,12 @@ vector_infer_kernel(const VectorArgs a) {
 #pragma unroll
                 for (int b = 0; b < V; ++b) acc0.a[b] = a.act == ACT_SIGMOID ? activate(acc0.a[b] + bb, ACT_SIGMOID, a.clamp) : clampf(acc0.a[b] + bb, a.clamp);
                 vec_st(send + (unsigned)(d * VECTOR_BLOCK + warp * 8 + lane) * PITCH, acc0);
+                if (a.acts && row0 + d * STRIDE < n) {
+                    float4 v = make_float4(acc0.a[0], 0.f, 0.f, 0.f);
+                    if (V > 1) v.y = acc0.a[V > 1 ? 1 : 0];
+                    if (V > 2) { v.z = acc0.a[V > 2 ? 2 : 0]; v.w = acc0.a[V > 2 ? 3 : 0]; }
+                    st_f4(a.acts + ((size_t)(k + 1) * n + row0 + d * STRIDE) * 4, v);
+                }
             }
         }
         __syncthreads();

@@ -105,3 +105,29 @@ def test_host_batches_cut_in_two(torch_cuda, cnt):  # noqa: F811
     rng = np.random.default_rng(cnt)
     arrays = ragged_net(rng, n=2111, layers=3, kmax=40, scale=0.3)
     infer_parity(torch_cuda, arrays, vectors(rng, cnt, 2111), 512, host=True, expect_nonempty=True)
+
+
+@pytest.mark.parametrize("n,k,B", [(33, 7, 4), (1000, 32, 1), (1024, 32, 2), (1030, 40, 1), (2047, 16, 1)])
+def test_train_with_the_forward_chain_in_one_launch(torch_cuda, n, k, B):  # noqa: F811
+    """Narrow nets with rows of one length, up to four inputs: everything a step leaves behind against the oracle, ending with a
+    smaller batch of the same padded width, which takes another variant of the launch."""
+    rng = np.random.default_rng(n + B)
+    cols = [np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for _ in range(n)]).astype(np.int32) for _ in range(3)]
+    vals = [rng.uniform(-1, 1, size=n * k).astype(np.float32) for _ in range(3)]
+    arrays = ([np.arange(n + 1, dtype=np.int32) * k] * 3, cols, vals, [(rng.standard_normal(n) * 0.1).astype(np.float32)] * 3)
+    batches = [(vectors(rng, B, n), vectors(rng, B, n)) for _ in range(2)]
+    train_parity(torch_cuda, arrays, batches, eta=0.02, update_bias=True, activation="sigmoid", expect_live=True)
+    torch, pkg = torch_cuda, sdnn()
+    h = pkg.Sdnn.create(*arrays, max_batch=4, train=True, activation=pkg.ACT_SIGMOID)
+    ora = OracleNet(*arrays, activation="sigmoid")
+    for b in (B, 1, 3):
+        ora.quantize_state()
+        for l in range(3):
+            h.set_weights(l, ora.w[l], ora.bias[l])
+        x0, y = vectors(rng, b, n), vectors(rng, b, n)
+        loss = h.train_step(torch.from_numpy(x0).cuda(), torch.from_numpy(y).cuda(), b, 0.1, want_loss=True)
+        want = ora.train_step(x0, y, 0.1, keep=())["loss"]
+        assert abs(loss - want) <= 1e-4 * want
+        for l in range(3):
+            check_close(h.get_weights(l, want_bias=False), ora.w[l], f"W^{l + 1} at B = {b}")
+    h.destroy()
