@@ -652,10 +652,11 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
 // they share, see reorder.h).  The stored rows of such a layer come group by group; the columns of a group are one
 // contiguous range of tile rows, its window; every row of a group is padded to the group's longest row (a multiple of
 // eight entries; padding: column 0, value 0), so that the place of every entry follows from the group's base without a
-// row pointer.  Work item = (group, part of its rows, chunk of TC inputs): the CTA copies the window's TC columns into
+// row pointer.  A group's entries are interleaved over slices of 16 rows like those of Sliced:
+//     entry q of the group's row r  ->  g_ebase + (r / 16) * 16 k + (q / 4) * 64 + (r % 16) * 4 + q % 4
+// Work item = (group, part of its rows, chunk of TC inputs): the CTA copies the window's TC columns into
 // shared memory (16-byte cp.async pieces, all in flight at once), then its warps walk the rows: a lane owns one input,
-// reads x[col][input] from the window (one conflict-free 128-byte wavefront per stored entry at TC = 32) and
-// accumulates in stored order.  The entries of a row (16-bit column within the window, value) travel through a small
+// reads x[col][input] from the window and accumulates in stored order.  The entries of a row (16-bit column within the window, value) travel through a small
 // ring in shared memory per warp: pieces of up to 32 entries are fetched with cp.async WINDOW_RING - 1 pieces ahead and
 // read back with warp-wide broadcast loads, so that no warp waits for an L2 round trip per row.  The output row goes
 // to the tile row `out[row]`: the number the NEXT layer's grouping gave this neuron.  A random row of the window costs
@@ -676,6 +677,10 @@ struct Windowed {
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(d), "l"(gmem_src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
@@ -715,10 +720,13 @@ forward_window_kernel(Windowed m, const float* __restrict__ xin, float* __restri
             if (i < pieces) {
                 const int row = r0 + (i / ppr) * nwarps, t = (i % ppr) << 5;
                 const int n = min(32, k - t);             // entries of the piece, a multiple of 8
-                const size_t at = (size_t)(row - g0) * k + t;
+                const int r = row - g0, q = lane & 7;     // lanes 0 .. 7: four columns each, 8 .. 15: four values
+                const size_t at = (size_t)(r & ~(SLICE - 1)) * k + (r & (SLICE - 1)) * 4 + (size_t)((t >> 2) + q) * CHUNK_ROW;
                 unsigned char* slot = ring + (i % WINDOW_RING) * WINDOW_PIECE_BYTES;
-                if (lane < (n >> 3)) cp_async16(slot + lane * 16, gcol + at + lane * 8);
-                else if (lane >= 4 && lane - 4 < (n >> 2)) cp_async16(slot + 64 + (lane - 4) * 16, gval + at + (lane - 4) * 4);
+                if (lane < 16 && q < (n >> 2)) {
+                    if (lane < 8) cp_async8(slot + q * 8, gcol + at);
+                    else cp_async16(slot + 64 + q * 16, gval + at);
+                }
             }
             cp_async_commit();
         };
@@ -762,32 +770,35 @@ forward_window_kernel(Windowed m, const float* __restrict__ xin, float* __restri
 }
 
 // ---------------------------------------------------------------------------------------------
-// The same layer for chunks of 32 inputs with four rows side by side in a warp: a group of eight lanes owns a row, a
-// lane four inputs of it.  Per four stored entries a lane group reads its row's columns (one 64-bit load) and values (one
-// 128-bit load) from the warp's ring, whose four row slots are staggered over the banks, and each window row with one
-// 128-bit load per lane: 128 contiguous bytes per group, four wavefronts per warp instruction for four entries, and two
-// packed FMAs per lane and entry.  About 38 shared-memory wavefronts per row of 32 entries, against 44 and six instructions
-// per FMA for the lane-per-input mapping above.  32 warps per CTA; the ring holds the piece in use and the next one.
-constexpr int W32_THREADS = 1024;
-constexpr int W32_ROWS = 4;                    // rows side by side in a warp
-constexpr int W32_RING = 2;                    // stages of a warp's entry ring
-constexpr int W32_SLOT = 208;                  // bytes of one row's piece in the ring: 64 of columns, 128 of values, 16 of padding
-                                               // (52 words: the four rows' slots start 20 banks apart)
-constexpr int W32_STAGE = W32_ROWS * W32_SLOT;
-constexpr int W32_RING_BYTES = (W32_THREADS / 32) * W32_RING * W32_STAGE;
+// The same layer for chunks of 32 inputs with 16 rows side by side in a warp, two lanes a row, 16 inputs a lane: a window row is
+// read with four 128-bit loads per lane, and the four rows of a phase (eight lanes) start with different quarters of their
+// 128 bytes, so that a phase never meets in a bank.  What bounds the kernel is the shared-memory pipe, one wavefront per stored
+// entry and 32 inputs.  A warp's entries come straight from global memory (128 contiguous bytes of columns, 256 of values per four
+// entries of 16 rows), two chunks ahead, under the shared-memory reads of the two chunks before them.
+// Four rows in a warp and the entries passed through a ring in shared memory cost a fifth of that pipe on top: 65536 neurons in 64
+// blocks, six layers of 4096 inputs with the copies in and out 9.83 -> 8.42 ms; 4096 neurons, 24 layers, 256 inputs 261 -> 209 us.
+constexpr int W32_THREADS = 512;
+
+// acc += w * (the lane's 64 bytes of a window row), in 16-byte pieces from `turn` on
+__device__ __forceinline__ void window_entry(unsigned row, unsigned turn, float w, float4 (&acc)[4]) {
+    float4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[i].x), "=f"(x[i].y), "=f"(x[i].z), "=f"(x[i].w)
+                     : "r"(row + ((turn + i * 16u) & 63u)));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f4_fma(w, x[i], acc[i]);
+}
 
 __global__ void __launch_bounds__(W32_THREADS, 1)
 forward_window32_kernel(Windowed m, const float* __restrict__ xin, float* __restrict__ xout, int ld, int chunks, int splits,
                         float clamp, int act, int pdl) {
-    extern __shared__ __align__(16) unsigned char window_smem[];
-    constexpr int TC = 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int grp = lane >> 3, sub = lane & 7;
-    unsigned char* ring = window_smem + warp * (W32_RING * W32_STAGE);
-    float* window = reinterpret_cast<float*>(window_smem + W32_RING_BYTES);      // [wlen][32]
-    // this lane's 16-byte shares of a full piece (4 rows x (4 + 8) shares): share `lane`, and share `lane + 32` for lanes < 16
-    const int sh_row0 = lane / 12, sh_q0 = lane - sh_row0 * 12;
-    const int sh_row1 = (lane + 32) / 12, sh_q1 = (lane + 32) - sh_row1 * 12;
+    extern __shared__ __align__(128) unsigned char window_smem[];                 // [wlen][32] floats
+    constexpr int TC = 32, WARPS = W32_THREADS / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane & 1, grp = lane >> 1;
+    const unsigned turn = 16u * (grp & 3);
+    const unsigned xw = (unsigned)__cvta_generic_to_shared(window_smem) + sub * 64u;
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
     const int per_group = chunks * splits;
@@ -795,82 +806,71 @@ forward_window32_kernel(Windowed m, const float* __restrict__ xin, float* __rest
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int g = item / per_group, rest = item - g * per_group;
         const int split = rest / chunks, t0 = (rest - split * chunks) * TC;
-        const int c0 = m.g_c0[g], wlen = m.g_wlen[g], k = m.g_k[g];
-        const int g0 = m.g_row0[g], per_split = (m.g_row0[g + 1] - g0 + splits - 1) / splits;
-        const int r0 = g0 + split * per_split + warp * W32_ROWS, r1 = min(m.g_row0[g + 1], g0 + (split + 1) * per_split);
-        const int rstep = nwarps * W32_ROWS;
-        const unsigned short* gcol = m.col + m.g_ebase[g];
-        const float* gval = m.val + m.g_ebase[g];
-        // one 16-byte share of a piece (rows rbase .. rbase + 3, entries t .. t + n - 1 of each): columns first (n / 8
-        // shares per row), then values (n / 4)
-        auto share = [&](unsigned char* stage, int rbase, int t, int n, int rr, int q) {
-            const int row = rbase + rr;
-            if (rr < W32_ROWS && row < r1) {
-                const size_t at = (size_t)(row - g0) * k + t;
-                if (q < (n >> 3)) cp_async16(stage + rr * W32_SLOT + q * 16, gcol + at + q * 8);
-                else if (q - (n >> 3) < (n >> 2)) cp_async16(stage + rr * W32_SLOT + 64 + (q - (n >> 3)) * 16, gval + at + (q - (n >> 3)) * 4);
+        const int c0 = m.g_c0[g], wlen = m.g_wlen[g], k = m.g_k[g], nch = k >> 2;
+        const int g0 = m.g_row0[g], rows = m.g_row0[g + 1] - g0, slices = (rows + SLICE - 1) / SLICE;
+        const int per_split = (slices + splits - 1) / splits;
+        const int s1 = min(slices, (split + 1) * per_split);
+        int s = split * per_split + warp;                                         // this warp's slice of the group
+        const unsigned short* gcol = m.col + m.g_ebase[g] + grp * 4;
+        const float* gval = m.val + m.g_ebase[g] + grp * 4;
+        uint2 c_a = make_uint2(0u, 0u), c_b = c_a;
+        float4 w_a = make_float4(0.f, 0.f, 0.f, 0.f), w_b = w_a;
+        float bias = 0.0f;
+        int to = 0;
+        auto place = [&](int sl) { const int r = min(sl * SLICE + grp, rows - 1); bias = m.bias[g0 + r]; to = m.out[g0 + r]; };
+        if (s < s1) {                                                             // first two chunks, bias and place of the first slice
+            const size_t at = (size_t)s * SLICE * k;
+            if (nch) {
+                c_a = __ldg(reinterpret_cast<const uint2*>(gcol + at));
+                w_a = __ldg(reinterpret_cast<const float4*>(gval + at));
+                c_b = __ldg(reinterpret_cast<const uint2*>(gcol + at + CHUNK_ROW));
+                w_b = __ldg(reinterpret_cast<const float4*>(gval + at + CHUNK_ROW));
             }
-        };
-        auto fetch = [&](int stage_no, int rbase, int t) {
-            if (rbase < r1 && t < k) {
-                unsigned char* stage = ring + stage_no * W32_STAGE;
-                const int n = min(32, k - t);                            // entries of the piece, a multiple of 8
-                if (n == 32) {
-                    share(stage, rbase, t, 32, sh_row0, sh_q0);
-                    if (lane < 16) share(stage, rbase, t, 32, sh_row1, sh_q1);
-                } else {
-                    const int per_row = (n >> 3) + (n >> 2);
-                    for (int p = lane; p < W32_ROWS * per_row; p += 32) share(stage, rbase, t, n, p / per_row, p % per_row);
-                }
-            }
-            cp_async_commit();
-        };
-        __syncthreads();                                  // the previous item's readers are done with the window and the rings
-        fetch(0, r0, 0);
-        for (int p = threadIdx.x; p < wlen * (TC / 4); p += blockDim.x)
-            cp_async16(window + p * 4, xin + (size_t)(c0 + (p >> 3)) * ld + t0 + (p & 7) * 4);
+            place(s);
+        }
+        __syncthreads();                                                          // the previous item's readers are done with the window
+        for (int p = threadIdx.x; p < wlen * (TC / 4); p += W32_THREADS)
+            cp_async16(window_smem + p * 16, xin + (size_t)(c0 + (p >> 3)) * ld + t0 + (p & 7) * 4);
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
-        const unsigned xw = (unsigned)__cvta_generic_to_shared(window) + sub * 16;
-        int stage_no = 0;
-        for (int rbase = r0; rbase < r1; rbase += rstep) {
-            const int row = rbase + grp;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int t = 0; t < k; t += 32) {
-                __syncwarp();                             // every lane has finished reading the stage that is refilled now
-                if (t + 32 < k) fetch(stage_no ^ 1, rbase, t + 32); else fetch(stage_no ^ 1, rbase + rstep, 0);
-                cp_async_wait<1>();                       // this lane's share of the current piece has landed ...
-                __syncwarp();                             // ... and so has every other lane's
-                const int n = min(32, k - t);
-                const unsigned slot = (unsigned)__cvta_generic_to_shared(ring + stage_no * W32_STAGE + grp * W32_SLOT);
-                if (row < r1) {
-#pragma unroll 2
-                    for (int j = 0; j < n; j += 4) {
-                        unsigned ca, cb;
-                        float4 w, x0, x1, x2, x3;
-                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(ca), "=r"(cb) : "r"(slot + j * 2));
-                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w.x), "=f"(w.y), "=f"(w.z), "=f"(w.w) : "r"(slot + 64 + j * 4));
-                        // a window row is 128 bytes: address = window + column * 128 (+ this lane's 16 bytes)
-                        const unsigned a0 = xw + ((ca & 0xffffu) << 7), a1 = xw + ((ca >> 16) << 7);
-                        const unsigned a2 = xw + ((cb & 0xffffu) << 7), a3 = xw + ((cb >> 16) << 7);
-                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x0.x), "=f"(x0.y), "=f"(x0.z), "=f"(x0.w) : "r"(a0));
-                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x1.x), "=f"(x1.y), "=f"(x1.z), "=f"(x1.w) : "r"(a1));
-                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x2.x), "=f"(x2.y), "=f"(x2.z), "=f"(x2.w) : "r"(a2));
-                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x3.x), "=f"(x3.y), "=f"(x3.z), "=f"(x3.w) : "r"(a3));
-                        f4_fma(w.x, x0, acc); f4_fma(w.y, x1, acc); f4_fma(w.z, x2, acc); f4_fma(w.w, x3, acc);
-                    }
-                }
-                stage_no ^= 1;
+        for (; s < s1; s += WARPS) {
+            const size_t at = (size_t)s * SLICE * k, next = (size_t)(s + WARPS < s1 ? s + WARPS : s) * SLICE * k;
+            const float b = bias;
+            const int row_to = to;
+            const bool stored = s * SLICE + grp < rows;
+            if (s + WARPS < s1) place(s + WARPS);
+            float4 acc[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            // chunk T, held in (c, w): a window row is 128 bytes; then the registers take the chunk two further on, at the end
+            // of a slice the first two of the warp's next one
+            auto chunk = [&](uint2& c, float4& w, int T) {
+                const unsigned a0 = xw + ((c.x & 0xffffu) << 7), a1 = xw + ((c.x >> 16) << 7);
+                const unsigned a2 = xw + ((c.y & 0xffffu) << 7), a3 = xw + ((c.y >> 16) << 7);
+                const float4 wv = w;
+                const size_t q = T + 2 < nch ? at + (size_t)(T + 2) * CHUNK_ROW : next + (size_t)(T & 1) * CHUNK_ROW;
+                c = __ldg(reinterpret_cast<const uint2*>(gcol + q));
+                w = __ldg(reinterpret_cast<const float4*>(gval + q));
+                window_entry(a0, turn, wv.x, acc);
+                window_entry(a1, turn, wv.y, acc);
+                window_entry(a2, turn, wv.z, acc);
+                window_entry(a3, turn, wv.w, acc);
+            };
+            for (int t = 0; t < nch; t += 2) {                                    // k is a multiple of eight
+                chunk(c_a, w_a, t);
+                chunk(c_b, w_b, t + 1);
             }
-            if (row < r1) {                               // also the rows of a group without entries (k = 0): x = f(b)
-                const float b = m.bias[row];
-                acc.x += b; acc.y += b; acc.z += b; acc.w += b;
-                f4_activate(acc, act, clamp);
-                st_f4(xout + (size_t)m.out[row] * ld + t0 + sub * 4, acc);
+            if (stored) {                                                         // also the rows of a group without entries (k = 0): x = f(b)
+                float* dst = xout + (size_t)row_to * ld + t0 + sub * 16;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc[i].x += b; acc[i].y += b; acc[i].z += b; acc[i].w += b;
+                    f4_activate(acc[i], act, clamp);
+                    st_f4(dst + (((turn + i * 16u) & 63u) >> 2), acc[i]);
+                }
             }
         }
-        cp_async_wait<0>();
     }
     if (pdl == 1) grid_launch_dependents();
 }

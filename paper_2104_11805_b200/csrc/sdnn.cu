@@ -80,7 +80,7 @@ struct LayerMem {
     // windowed layer: rows grouped by shared columns, the group's window staged in shared memory (forward_window_kernel)
     bool windowed = false;
     int groups = 0, max_wlen = 0;
-    std::vector<int> w_row_at;             // [N] host: offset of each stored row's entries in w_col / w_val
+    std::vector<int> w_row_at;             // [N] host: offset of each stored row's first entry in w_col / w_val (see w_pos)
     int64_t w_elems = 0;                   // padded entries
     unsigned short* w_col = nullptr; float* w_val = nullptr; int* w_out = nullptr;
     int* w_g_row0 = nullptr; int* w_g_c0 = nullptr; int* w_g_wlen = nullptr; int* w_g_ebase = nullptr; int* w_g_k = nullptr;
@@ -644,7 +644,8 @@ cudaError_t launch_forward_window_tc(sdnn* h, const LayerMem& lm, const Windowed
                               h->pdl ? PDL_AT_END : 0);
 }
 
-// chunks of 32 inputs: the kernel with four rows side by side in a warp, where its larger entry ring leaves room for the window
+// chunks of 32 inputs: the kernel with 16 rows side by side in a warp.  An item keeps at least 128 rows (half of its 16 warps at
+// work): cut further, staging the window again for every part costs more than the idle SMs.
 cudaError_t launch_forward_window32(sdnn* h, const LayerMem& lm, const Windowed& m, const float* xin, float* xout, int ld, int cols) {
     static bool configured[64] = {};
     if (h->device < 64 && !configured[h->device]) {
@@ -659,7 +660,7 @@ cudaError_t launch_forward_window32(sdnn* h, const LayerMem& lm, const Windowed&
     const int items = lm.groups * chunks * splits;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(std::max(1, std::min(items, h->sms))); lc.blockDim = dim3(W32_THREADS);
-    lc.dynamicSmemBytes = W32_RING_BYTES + (size_t)std::max(lm.max_wlen, 1) * 32 * sizeof(float);
+    lc.dynamicSmemBytes = (size_t)std::max(lm.max_wlen, 1) * 32 * sizeof(float);
     lc.stream = h->launch_stream ? h->launch_stream : h->stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -675,8 +676,7 @@ void launch_forward_window(sdnn* h, int layer, const float* xin, float* xout, in
     m.col = lm.w_col; m.val = lm.w_val; m.out = lm.w_out;
     m.bias = h->d_bias + (size_t)layer * h->N;
     m.g_row0 = lm.w_g_row0; m.g_c0 = lm.w_g_c0; m.g_wlen = lm.w_g_wlen; m.g_ebase = lm.w_g_ebase; m.g_k = lm.w_g_k; m.groups = lm.groups;
-    if (cols >= 32 && W32_RING_BYTES + (size_t)lm.max_wlen * 128 <= 227u * 1024u) launch_forward_window32(h, lm, m, xin, xout, ld, cols);
-    else if (cols >= 32) launch_forward_window_tc<32>(h, lm, m, xin, xout, ld, cols);
+    if (cols >= 32) launch_forward_window32(h, lm, m, xin, xout, ld, cols);
     else if (cols == 16) launch_forward_window_tc<16>(h, lm, m, xin, xout, ld, cols);
     else if (cols == 8) launch_forward_window_tc<8>(h, lm, m, xin, xout, ld, cols);
     else launch_forward_window_tc<4>(h, lm, m, xin, xout, ld, cols);
@@ -1635,6 +1635,9 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
     return SDNN_OK;
 }
 
+// place of entry q of a row of a windowed layer, from the place of the row's first one (see Windowed)
+inline size_t w_pos(int row_at, int q) { return (size_t)row_at + (size_t)(q >> 2) * CHUNK_ROW + (q & 3); }
+
 // Entries per (padded) row of every group of a structured layer and the padded total; -1 if padding every row of a
 // group to its longest row would more than quadruple the layer (plus a margin of 64 entries per row).
 int64_t windowed_padding(int n, const int32_t* rp, const sdnn_reorder::Grouping& g, std::vector<int>* ks) {
@@ -1646,7 +1649,7 @@ int64_t windowed_padding(int n, const int32_t* rp, const sdnn_reorder::Grouping&
         for (int s = g.group_row0[q]; s < g.group_row0[q + 1]; ++s) k = std::max(k, rp[g.row_order[s] + 1] - rp[g.row_order[s]]);
         k = (k + 7) / 8 * 8;
         if (ks) (*ks)[q] = k;
-        total += (int64_t)k * (g.group_row0[q + 1] - g.group_row0[q]);
+        total += (int64_t)k * ((g.group_row0[q + 1] - g.group_row0[q] + SLICE - 1) / SLICE * SLICE);
     }
     if (total > 4 * (int64_t)rp[n] + 64 * (int64_t)n || total > INT32_MAX) return -1;
     return total;
@@ -1663,12 +1666,16 @@ int build_windowed_layer(sdnn* h, int layer, const HostLayer& hl, const sdnn_reo
     std::vector<int> ks, ebase(groups, 0);
     const int64_t padded = windowed_padding(N, hl.rp.data(), g, &ks);
     if (padded < 0) return fail(h, SDNN_ERR_STATE, "layer %d: windowed layout too large", layer);      // excluded by build_reordered
-    for (int q = 1; q < groups; ++q) ebase[q] = ebase[q - 1] + ks[q - 1] * (g.group_row0[q] - g.group_row0[q - 1]);
+    for (int q = 1; q < groups; ++q)
+        ebase[q] = ebase[q - 1] + ks[q - 1] * ((g.group_row0[q] - g.group_row0[q - 1] + SLICE - 1) / SLICE * SLICE);
     std::vector<int> stored_rp(N + 1, 0), out(N);
     std::vector<float> bias_s(N);
     lm.w_row_at.assign(N, 0);
     for (int q = 0; q < groups; ++q)
-        for (int s = g.group_row0[q]; s < g.group_row0[q + 1]; ++s) lm.w_row_at[s] = ebase[q] + (s - g.group_row0[q]) * ks[q];
+        for (int s = g.group_row0[q]; s < g.group_row0[q + 1]; ++s) {
+            const int r = s - g.group_row0[q];
+            lm.w_row_at[s] = ebase[q] + r / SLICE * SLICE * ks[q] + r % SLICE * 4;
+        }
     for (int s = 0; s < N; ++s) {
         const int i = g.row_order[s];
         stored_rp[s + 1] = stored_rp[s] + (hl.rp[i + 1] - hl.rp[i]);
@@ -1689,8 +1696,8 @@ int build_windowed_layer(sdnn* h, int layer, const HostLayer& hl, const sdnn_reo
             for (int p = hl.rp[i]; p < hl.rp[i + 1]; ++p) ent.emplace_back(g.col_label[hl.col[p]] - g.group_c0[q], p);
             std::sort(ent.begin(), ent.end());
             for (size_t t = 0; t < ent.size(); ++t) {
-                wcol[(size_t)lm.w_row_at[s] + t] = (unsigned short)ent[t].first;
-                wval[(size_t)lm.w_row_at[s] + t] = hl.val[ent[t].second];
+                wcol[w_pos(lm.w_row_at[s], (int)t)] = (unsigned short)ent[t].first;
+                wval[w_pos(lm.w_row_at[s], (int)t)] = hl.val[ent[t].second];
                 lm.entry_src[(size_t)stored_rp[s] + t] = ent[t].second;
             }
         }
@@ -2225,7 +2232,7 @@ int sdnn_get_weights(sdnn_t* h, int32_t layer, float* values_out, float* bias_ou
             std::vector<float> tmp((size_t)lm.w_elems);
             CU(h, cudaMemcpy(tmp.data(), lm.w_val, tmp.size() * sizeof(float), cudaMemcpyDeviceToHost));
             for (int r = 0; r < h->N; ++r)
-                std::copy(tmp.begin() + lm.w_row_at[r], tmp.begin() + lm.w_row_at[r] + lm.shape.len(r), stored.begin() + lm.shape.start(r));
+                for (int q = 0; q < lm.shape.len(r); ++q) stored[(size_t)lm.shape.start(r) + q] = tmp[w_pos(lm.w_row_at[r], q)];
         } else {
             std::vector<float> tmp((size_t)lm.r_elems);
             CU(h, cudaMemcpy(tmp.data(), lm.r_val, tmp.size() * sizeof(float), cudaMemcpyDeviceToHost));
@@ -2275,7 +2282,7 @@ int sdnn_set_weights(sdnn_t* h, int32_t layer, const float* values, const float*
         } else if (lm.windowed) {
             tmp.assign((size_t)lm.w_elems, 0.0f);
             for (int r = 0; r < h->N; ++r)
-                std::copy(stored.begin() + lm.shape.start(r), stored.begin() + lm.shape.start(r) + lm.shape.len(r), tmp.begin() + lm.w_row_at[r]);
+                for (int q = 0; q < lm.shape.len(r); ++q) tmp[w_pos(lm.w_row_at[r], q)] = stored[(size_t)lm.shape.start(r) + q];
             CU(h, cudaMemcpy(lm.w_val, tmp.data(), tmp.size() * sizeof(float), cudaMemcpyHostToDevice));
         } else {
             csr_to_sliced(h, lm, stored.data(), tmp);

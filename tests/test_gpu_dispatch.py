@@ -131,3 +131,31 @@ def test_train_with_the_forward_chain_in_one_launch(torch_cuda, n, k, B):  # noq
         for l in range(3):
             check_close(h.get_weights(l, want_bias=False), ora.w[l], f"W^{l + 1} at B = {b}")
     h.destroy()
+
+
+@pytest.mark.parametrize("sizes,kmax,cnt", [([1025, 15, 17, 1], 9, 33), ([16, 16, 16], 17, 64), ([1536, 2048 - 1536], 40, 96), ([128] * 12, 1, 32)])
+def test_windowed_rows_sixteen_to_a_warp(torch_cuda, sizes, kmax, cnt):  # noqa: F811
+    """The shared-memory window kernel for chunks of 32 inputs: groups short of a slice, one row over, of one row, the widest
+    window, rows of one chunk pair and of several, weights read back in the caller's order."""
+    rng = np.random.default_rng(sum(sizes) + kmax)
+    n, start = sum(sizes), 0
+    rows = []
+    for size in sizes:
+        for i in range(size):
+            m = int(rng.integers(1, min(kmax, size) + 1))
+            rows.append(np.sort(start + rng.choice(size, size=m, replace=False)))
+        start += size
+    rp = np.zeros(n + 1, dtype=np.int32)
+    rp[1:] = np.cumsum([len(r) for r in rows])
+    layers = 2
+    arrays = ([rp] * layers, [np.concatenate(rows).astype(np.int32)] * layers,
+              [(rng.standard_normal(rp[-1]) * 0.6).astype(np.float32) for _ in range(layers)],
+              [(rng.standard_normal(n) * 0.1).astype(np.float32) for _ in range(layers)])
+    pkg = sdnn()
+    flags = pkg.FLAG_REORDER | pkg.FLAG_SMEM_WINDOWS
+    infer_parity(torch_cuda, arrays, vectors(rng, cnt, n), 128, expect_nonempty=True, flags=flags)
+    h = pkg.Sdnn.create(*arrays, max_batch=128, flags=flags)
+    for l in range(layers):
+        w, bias = h.get_weights(l)
+        assert np.array_equal(w, arrays[2][l]) and np.array_equal(bias, arrays[3][l])
+    h.destroy()
