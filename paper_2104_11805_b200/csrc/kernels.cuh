@@ -771,7 +771,8 @@ forward_window_kernel(Windowed m, const float* __restrict__ xin, float* __restri
 
 // ---------------------------------------------------------------------------------------------
 // The same layer for chunks of 32 inputs with 16 rows side by side in a warp, two lanes a row, 16 inputs a lane: a window row is
-// read with four 128-bit loads per lane, and the four rows of a phase (eight lanes) start with different quarters of their
+// read with four 128-bit loads per lane (a row's two lanes take the halves of one 32-byte sector, the unit the output is stored
+// in), and the four rows of a phase (eight lanes) start with different quarters of their
 // 128 bytes, so that a phase never meets in a bank.  What bounds the kernel is the shared-memory pipe, one wavefront per stored
 // entry and 32 inputs.  A warp's entries come straight from global memory (128 contiguous bytes of columns, 256 of values per four
 // entries of 16 rows), two chunks ahead, under the shared-memory reads of the two chunks before them.
@@ -779,13 +780,13 @@ forward_window_kernel(Windowed m, const float* __restrict__ xin, float* __restri
 // blocks, six layers of 4096 inputs with the copies in and out 9.83 -> 8.42 ms; 4096 neurons, 24 layers, 256 inputs 261 -> 209 us.
 constexpr int W32_THREADS = 512;
 
-// acc += w * (the lane's 64 bytes of a window row), in 16-byte pieces from `turn` on
+// acc += w * (the lane's 64 bytes of a window row: every other 16-byte piece), from the piece at `turn` on
 __device__ __forceinline__ void window_entry(unsigned row, unsigned turn, float w, float4 (&acc)[4]) {
     float4 x[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[i].x), "=f"(x[i].y), "=f"(x[i].z), "=f"(x[i].w)
-                     : "r"(row + ((turn + i * 16u) & 63u)));
+                     : "r"(row + ((turn + i * 32u) & 127u)));
 #pragma unroll
     for (int i = 0; i < 4; ++i) f4_fma(w, x[i], acc[i]);
 }
@@ -797,8 +798,8 @@ forward_window32_kernel(Windowed m, const float* __restrict__ xin, float* __rest
     constexpr int TC = 32, WARPS = W32_THREADS / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane & 1, grp = lane >> 1;
-    const unsigned turn = 16u * (grp & 3);
-    const unsigned xw = (unsigned)__cvta_generic_to_shared(window_smem) + sub * 64u;
+    const unsigned turn = 32u * (grp & 3);
+    const unsigned xw = (unsigned)__cvta_generic_to_shared(window_smem) + sub * 16u;
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
     const int per_group = chunks * splits;
@@ -862,12 +863,12 @@ forward_window32_kernel(Windowed m, const float* __restrict__ xin, float* __rest
                 chunk(c_b, w_b, t + 1);
             }
             if (stored) {                                                         // also the rows of a group without entries (k = 0): x = f(b)
-                float* dst = xout + (size_t)row_to * ld + t0 + sub * 16;
+                float* dst = xout + (size_t)row_to * ld + t0 + sub * 4;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     acc[i].x += b; acc[i].y += b; acc[i].z += b; acc[i].w += b;
                     f4_activate(acc[i], act, clamp);
-                    st_f4(dst + (((turn + i * 16u) & 63u) >> 2), acc[i]);
+                    st_f4(dst + (((turn + i * 32u) & 127u) >> 2), acc[i]);
                 }
             }
         }
