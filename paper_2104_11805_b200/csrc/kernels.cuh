@@ -777,7 +777,8 @@ forward_window_kernel(Windowed m, const float* __restrict__ xin, float* __restri
 // entry and 32 inputs.  A warp's entries come straight from global memory (128 contiguous bytes of columns, 256 of values per four
 // entries of 16 rows), two chunks ahead, under the shared-memory reads of the two chunks before them.
 // Four rows in a warp and the entries passed through a ring in shared memory cost a fifth of that pipe on top: 65536 neurons in 64
-// blocks, six layers of 4096 inputs with the copies in and out 9.83 -> 8.42 ms; 4096 neurons, 24 layers, 256 inputs 261 -> 209 us.
+// blocks, six layers of 4096 inputs with the copies in and out 9.83 -> 8.19 ms (8.42 with each lane on its own half of the row); 4096 neurons, 24 layers, 256
+// inputs 260 -> 204 us.
 constexpr int W32_THREADS = 512;
 
 // acc += w * (the lane's 64 bytes of a window row: every other 16-byte piece), from the piece at `turn` on
