@@ -419,7 +419,7 @@ template <int G, int V, int STEP>
 __global__ void __launch_bounds__(256)
 forward_csr_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ val,
                    const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
-                   int n, int ld, float clamp, unsigned long long* __restrict__ bad_columns) {
+                   int n, int ld, int last, float clamp, unsigned long long* __restrict__ bad_columns) {
     constexpr int RPW = 32 / G, OWN = (STEP + G - 1) / G;      // entries of a step that a lane fetches (G > STEP: only the first STEP lanes do)
     const int lane = threadIdx.x & 31;
     const int sub = lane % G, lead = lane - sub;
@@ -428,7 +428,7 @@ forward_csr_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
     float b = 0.0f;
     if (row < n) { p = row_ptr[row]; e = row_ptr[row + 1]; b = bias[row]; }
     const int boff = blockIdx.y * (V * G) + sub * V;
-    const float* xg = xin + boff;
+    const float* xg = xin + min(boff, last);      // lanes of nothing but padding gather what the last lane with inputs does (no sector more)
     const unsigned pitch = (unsigned)ld * 4u;
     unsigned bad = 0;
     int c[OWN];
@@ -562,12 +562,15 @@ __device__ __forceinline__ void prefetch_unit(const Sliced& m, int u, int rpw, i
 // While it works on a unit a warp asks for the entries of its next unit to be brought into L2.
 // CG: the gathers go past L1 (64-byte rows of a layer without padding entries).
 // SPAN: a CTA takes a run of `span` consecutive units instead of walking the units in a grid-wide stride.
+// last: offset of the last lane that holds inputs.  Lanes of nothing but padding gather what that lane gathers (what they store is
+// multiplied by the zeros of delta's padding or never read), which adds no sector to a request: rows wider than 64 bytes cost by
+// their bytes (40000 neurons, 8 layers, 90 inputs: 319 -> 299 us).
 // TRACK (dropping dead inputs): one grid for all chunks, whose warps walk the units of the chunks that still hold live inputs
 // (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.
 template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false, bool TRACK = false>
 __global__ void __launch_bounds__(256, CPS > 2 ? 1 : 2)
 forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
-               int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span) {
+               int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span, int last) {
     constexpr int RPW = 32 / G;
     constexpr int UPS = (RPW >= SLICE) ? 1 : SLICE / RPW;      // units per slice
     const int lane = threadIdx.x & 31;
@@ -612,7 +615,7 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         Lane<V> acc;
         lane_fill(acc, b);
         const float* vp = val + base;
-        const float* xg = xin + boff;
+        const float* xg = xin + (TRACK || G <= 2 ? boff : min(boff, last));
         for (int t = 0; t < nch; t += CPS) {
             float4 w[CPS];
             Lane<V> x[4 * CPS];
@@ -694,7 +697,7 @@ template <int TC>
 __global__ void __launch_bounds__(WINDOW_THREADS, 1)
 forward_window_kernel(Windowed m, const float* __restrict__ xin, float* __restrict__ xout, int ld, int chunks, int splits,
                       float clamp, int act, int pdl) {
-    extern __shared__ __align__(16) unsigned char window_smem[];
+    extern __shared__ __align__(128) unsigned char window_smem[];
     constexpr int PPR = TC / 4;                           // 16-byte pieces per window row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     unsigned char* ring = window_smem + warp * (WINDOW_RING * WINDOW_PIECE_BYTES);
@@ -1000,7 +1003,9 @@ struct BackwardArgs {
     unsigned warm_bytes;      // because it was written a whole forward pass ago and has left the cache
 };
 
-// Column units of the transposed realisation.
+// Column units of the transposed realisation.  (Lanes of nothing but padding gather their zeros: sending them to the last lane with
+// inputs, as the forward kernel does, costs registers that this kernel does not have; 16384 neurons: 2 to 3 % faster at 37
+// inputs, 1 to 2 % slower at 64.)
 template <int G, int V, int CPS, bool I16>
 __device__ __forceinline__ void backward_col_units(const Sliced m, const float* __restrict__ xprev, const float* __restrict__ dk,
                                                    float* __restrict__ dprev, int n, float clamp, int act, float step, float inv_b,
@@ -1017,9 +1022,11 @@ __device__ __forceinline__ void backward_col_units(const Sliced m, const float* 
     const float* dg = dk + boff;
 
     // The columns come by descending length.  alternate: a warp that takes several units takes them from alternating ends of
-    // its rounds, so that every warp gets long and short columns (two units each, no row units beside them: 18.3 -> 17.3 us per
-    // layer at 65536 neurons and 16 inputs, 13.4 -> 12.8 at 16384 and 64; row units fill the tail as well and gain nothing by it)
-    int u = first, item, base, nch, round = 0;
+    // its rounds (its hops add up to two strides), so that every warp gets long and short columns (two units each, no row units
+    // beside them: 13.4 -> 12.8 us per layer at 16384 neurons and 64 inputs; row units fill the tail as well and gain nothing
+    // by it).  Tiles of at least 32 inputs only: narrower ones never ask for it, and the registers it takes cost them 0.7 %.
+    int u = first, item, base, nch;
+    int hop = G > 2 && alternate ? 2 * (stride - first) - 1 : stride;
     SDNN_UNIT_SHAPE(m, u, nunits, item, base, nch)
     if (u < nunits && lane == 0) prefetch_unit(m, u, RPW, n, UPS);
     int len = 0, j = 0;
@@ -1036,8 +1043,8 @@ __device__ __forceinline__ void backward_col_units(const Sliced m, const float* 
     if (pdl == 2) grid_launch_dependents();
 
     while (u < nunits) {
-        ++round;
-        const int nu = round * stride + ((alternate & round & 1) ? stride - 1 - first : first);
+        const int nu = u + hop;
+        if (G > 2) hop = 2 * stride - hop;
         int nitem, nbase, nnch, nlen = 0, nj = 0;
         SDNN_UNIT_SHAPE(m, nu, nunits, nitem, nbase, nnch)
         if (nitem < n) { nlen = m.len[nitem]; nj = m.order[nitem]; }

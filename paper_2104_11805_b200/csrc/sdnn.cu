@@ -144,7 +144,8 @@ struct sdnn {
     StepParams* d_sp_batch = nullptr;   // the real batch, while d_sp describes the single backpropagated vector
     const float* bwd_acts = nullptr;    // activations the backward launches read (NULL: d_acts)
     cudaGraphExec_t graph = nullptr, graph_avg = nullptr;
-    int graph_ld = 0, graph_avg_ld = 0, graph_v = 0, graph_avg_v = 0;
+    int graph_ld = 0, graph_avg_ld = 0, graph_v = 0, graph_avg_v = 0, graph_used = 0, graph_avg_used = 0;
+    int used = 0;                       // tile columns of the step being enqueued that hold inputs, rounded up to a lane's eight
     int64_t graph_launches = 0, graph_avg_launches = 0;   // kernel nodes of the captured steps
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};   // before forward chain, between, after backward chain
 
@@ -516,7 +517,7 @@ cudaError_t launch_k(sdnn* h, void (*kernel)(KArgs...), dim3 grid, dim3 block, b
 }
 
 template <bool I16, int G, int V, int CPS = 2>
-void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld, int chunks) {
+void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld, int chunks, int last) {
     constexpr int RPW = 32 / G;
     const int units = (h->N + RPW - 1) / RPW;
     const float* bias = h->d_bias + (size_t)layer * h->N;
@@ -538,7 +539,7 @@ void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld
 #define SDNN_FWD(CG_, SPAN_)                                                                                                   \
     launch_k(h, forward_kernel<G, V, CPS, I16, CG_, SPAN_>, dim3(plan.first, chunks), dim3(plan.second), h->pdl, rows_of(h, layer), \
              bias, xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,                              \
-             (const int*)nullptr, (int*)nullptr, span)
+             (const int*)nullptr, (int*)nullptr, span, last)
     // the grid-stride instantiation is the one the wide inference tiles take: it carries nothing of the other walk
     if (cg) { if (span > 0) SDNN_FWD((G == 2 && V == 8 && CPS == 2), true); else SDNN_FWD((G == 2 && V == 8 && CPS == 2), false); }
     else if (span > 0) SDNN_FWD(false, true);
@@ -556,7 +557,7 @@ void launch_forward_tracked(sdnn* h, int layer, const float* xin, float* xout, i
     auto plan = plan_grid(h, (const void*)forward_kernel<G, V, 2, I16, false, false, true>, units * chunks, 1);
     launch_k(h, forward_kernel<G, V, 2, I16, false, false, true>, dim3(plan.first), dim3(plan.second), h->pdl, rows_of(h, layer),
              (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,
-             (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0);
+             (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0, 0);
     count_launch(h);
 }
 template <bool I16>
@@ -577,38 +578,38 @@ bool entry_parallel(const sdnn* h, int ld) {
 }
 
 template <bool I16>
-void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw) {
+void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used) {
     const Geometry q = geometry(cw);
-    const int chunks = cols / cw;
+    const int chunks = cols / cw, last = (used - 1) / q.v * q.v;
     if (q.v == 4 && entry_parallel(h, ld)) {
         const int wf = h->NS <= h->sms ? 1 : 4;      // few slices: one per CTA, so that they spread over as many SMs
         launch_k(h, forward_ep_kernel<I16>, dim3((h->NS + wf - 1) / wf), dim3(32 * wf), h->pdl, rows_of(h, layer),
                  (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0);
-    } else if (q.v == 4) launch_forward_gv<I16, 1, 4>(h, layer, xin, xout, ld, chunks);
+    } else if (q.v == 4) launch_forward_gv<I16, 1, 4>(h, layer, xin, xout, ld, chunks, last);
     else switch (q.g) {
-        case 1: launch_forward_gv<I16, 1, 8>(h, layer, xin, xout, ld, chunks); break;
-        case 2: launch_forward_gv<I16, 2, 8>(h, layer, xin, xout, ld, chunks); break;
-        case 4: launch_forward_gv<I16, 4, 8>(h, layer, xin, xout, ld, chunks); break;
-        case 8: launch_forward_gv<I16, 8, 8>(h, layer, xin, xout, ld, chunks); break;
-        case 16: launch_forward_gv<I16, 16, 8>(h, layer, xin, xout, ld, chunks); break;
+        case 1: launch_forward_gv<I16, 1, 8>(h, layer, xin, xout, ld, chunks, last); break;
+        case 2: launch_forward_gv<I16, 2, 8>(h, layer, xin, xout, ld, chunks, last); break;
+        case 4: launch_forward_gv<I16, 4, 8>(h, layer, xin, xout, ld, chunks, last); break;
+        case 8: launch_forward_gv<I16, 8, 8>(h, layer, xin, xout, ld, chunks, last); break;
+        case 16: launch_forward_gv<I16, 16, 8>(h, layer, xin, xout, ld, chunks, last); break;
         default:
             // a launch of at most one warp-row per resident slot is bound by its chain of round trips: four chunks (16
             // entries) of a row in flight per step instead of two, where every slice has whole steps of that size
             if (h->lay[layer].r_chunks_mult4 && (int64_t)h->N * chunks <= (int64_t)h->sms * 8)
-                launch_forward_gv<I16, 32, 8, 4>(h, layer, xin, xout, ld, chunks);
-            else launch_forward_gv<I16, 32, 8>(h, layer, xin, xout, ld, chunks);
+                launch_forward_gv<I16, 32, 8, 4>(h, layer, xin, xout, ld, chunks, last);
+            else launch_forward_gv<I16, 32, 8>(h, layer, xin, xout, ld, chunks, last);
             break;
     }
     count_launch(h);
 }
 
-// the kernels are instantiated for both index widths of the sliced copies
-void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, bool track = false) {
+// the kernels are instantiated for both index widths of the sliced copies; used: columns that hold inputs
+void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used, bool track = false) {
     if (track) {
         if (h->idx16) launch_forward_tracked_i<true>(h, layer, xin, xout, ld, cols);
         else launch_forward_tracked_i<false>(h, layer, xin, xout, ld, cols);
-    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, cw);
-    else launch_forward_i<false>(h, layer, xin, xout, ld, cols, cw);
+    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, cw, used);
+    else launch_forward_i<false>(h, layer, xin, xout, ld, cols, cw, used);
 }
 
 // Windowed layers (rows grouped by shared columns at set-up): the group's window of the input tile is staged in shared
@@ -1020,7 +1021,7 @@ void enqueue_step_body(sdnn* h, int ld, int v, unsigned flags, bool averaged) {
         if (v) forward_vector(h, v);
         else for (int k = 0; k < h->L; ++k) {
             NvtxRange pass("forward layer", k + 1);
-            launch_forward(h, k, h->d_acts + (size_t)k * tile, h->d_acts + (size_t)(k + 1) * tile, ld, ld, ld);
+            launch_forward(h, k, h->d_acts + (size_t)k * tile, h->d_acts + (size_t)(k + 1) * tile, ld, ld, ld, h->used);
         }
     }
     cudaEventRecordWithFlags(h->ev[1], h->stream, flags);
@@ -1049,6 +1050,7 @@ void enqueue_step_body(sdnn* h, int ld, int v, unsigned flags, bool averaged) {
 int train_step_device(sdnn* h, const float* x0, const float* target, int B, float eta, float* loss_out, bool averaged = false) {
     NvtxRange call(averaged ? "sdnn_train_step_averaged" : "sdnn_train_step");
     const int ld = padded_width(B), v = train_vector_width(h, B);      // v: the forward chain as one launch for v inputs (0: a launch per layer)
+    h->used = std::min((B + 7) / 8 * 8, ld);
     if (const int rc = vector_check(h)) return rc;
     h->fwd_pdl = PDL_EARLY;
     if (averaged) {
@@ -1068,8 +1070,10 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
         cudaGraphExec_t& graph = averaged ? h->graph_avg : h->graph;
         int& graph_ld = averaged ? h->graph_avg_ld : h->graph_ld;
         int& graph_v = averaged ? h->graph_avg_v : h->graph_v;
+        int& graph_used = averaged ? h->graph_avg_used : h->graph_used;
         int64_t& graph_launches = averaged ? h->graph_avg_launches : h->graph_launches;
-        if (!graph || graph_ld != ld || graph_v != v) {
+        // a graph made for more inputs of the same padded width serves fewer as well (the short batch at the end of an epoch)
+        if (!graph || graph_ld != ld || graph_v != v || graph_used < h->used) {
             if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
             cudaGraph_t g = nullptr;
             const int64_t before = h->launches;
@@ -1082,7 +1086,7 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
             e = cudaGraphInstantiate(&graph, g, 0);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) { graph = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
-            graph_ld = ld; graph_v = v;
+            graph_ld = ld; graph_v = v; graph_used = h->used;
         }
         CU(h, cudaGraphLaunch(graph, h->stream));
         count_launch(h, (int)graph_launches);
@@ -1143,11 +1147,11 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
 // being dropped: nobody knows what is left of those.
 constexpr int64_t GRAPH_WORK = 32 << 20;      // stored elements x inputs per layer: about 7 us
 template <typename Layers>
-int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, bool track, const Layers& layers) {
+int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int cnt, bool track, const Layers& layers) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (h->infer_calls < 2 || h->L < 4 || (!track && h->lay[0].r_elems * cols > GRAPH_WORK) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
         capturing != cudaStreamCaptureStatusNone) {
-        layers();
+        layers(cnt);
         return SDNN_OK;
     }
     TileGraph* g = &ln.graphs[0];
@@ -1160,7 +1164,7 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, bool track, const L
         cudaGraph_t graph = nullptr;
         const int64_t before = h->launches;
         CU(h, cudaStreamBeginCapture(ln.stream, cudaStreamCaptureModeThreadLocal));
-        layers();
+        layers(cols);      // the graph serves every tile of this padded width
         cudaError_t e = cudaStreamEndCapture(ln.stream, &graph);
         g->launches = h->launches - before;
         h->launches = before;
@@ -1192,14 +1196,14 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     const int cw = shape.cw, cols = shape.cols;
     launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     if (consumed) CU(h, cudaEventRecord(consumed, st));
-    auto layers = [&]() {
+    auto layers = [&](int used) {
         int cur = 0;
         if (track) {
             const int chunk = std::min(cols, TRACK_CHUNK);
             const int rows_grid = std::min((h->N + 7) / 8, h->sms * 8);
             cudaMemsetAsync(ln.cs.flags, 0, (size_t)h->L * ld * sizeof(int), st);
             for (int k = 0; k < h->L; ++k) {
-                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, true);
+                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, cols, true);
                 cur ^= 1;
                 // dropping what has died: after each of the first layers, where most do, then at growing distances (after 1, 2, 3, 4,
                 // 6, 8, 12, 16, 24, ... layers)
@@ -1217,7 +1221,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
             for (int k = 0; k < h->L; ++k) {
                 NvtxRange pass("forward layer", k + 1);
                 if (h->lay[k].windowed) launch_forward_window(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
-                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw);
+                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, used);
                 cur ^= 1;
             }
         }
@@ -1229,7 +1233,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
         h->live_lane = (int)(&ln - h->lane);
     }
     {
-        const int rc = enqueue_layers(h, ln, cw, cols, track, layers);
+        const int rc = enqueue_layers(h, ln, cw, cols, cnt, track, layers);
         if (rc) return rc;
     }
     const int cur = (h->L + (track ? 1 : 0)) & 1;
@@ -2997,7 +3001,7 @@ int noalloc_scratch(float** out, unsigned long long** bad_out) {
 // a layer may start its prologue (its rows' places, first entries) under the tail of the one before
 template <int G, int V, int STEP = 8>
 void noalloc_forward_g(cudaStream_t st, const int* rp, const int* col, const float* val, const float* bias,
-                       const float* xin, float* xout, int n, int ld, int chunks, float clamp, unsigned long long* bad) {
+                       const float* xin, float* xout, int n, int ld, int chunks, int n_inputs, float clamp, unsigned long long* bad) {
     const int warps = (n + 32 / G - 1) / (32 / G), wpb = warps * chunks < 4096 ? 2 : 4;      // small CTAs: more SMs, finer tails
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((warps + wpb - 1) / wpb, chunks); lc.blockDim = dim3(32 * wpb); lc.stream = st;
@@ -3005,7 +3009,7 @@ void noalloc_forward_g(cudaStream_t st, const int* rp, const int* col, const flo
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at; lc.numAttrs = 1;
-    cudaLaunchKernelEx(&lc, forward_csr_kernel<G, V, STEP>, rp, col, val, bias, xin, xout, n, ld, clamp, bad);
+    cudaLaunchKernelEx(&lc, forward_csr_kernel<G, V, STEP>, rp, col, val, bias, xin, xout, n, ld, (n_inputs - 1) / V * V, clamp, bad);
 }
 
 }  // namespace
@@ -3049,7 +3053,7 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
         const int* col = col_idx + layer_offset[l];
         const float* val = values + layer_offset[l];
         const float* b = bias + (size_t)l * n_neurons;
-#define SDNN_NOALLOC(...) noalloc_forward_g<__VA_ARGS__>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, chunks, clamp, bad)
+#define SDNN_NOALLOC(...) noalloc_forward_g<__VA_ARGS__>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, chunks, n_inputs, clamp, bad)
         // up to 32 inputs a row has few lanes, so that 16 of its entries in flight per step still fit the registers
         switch (ld / chunks) {
             case 4: SDNN_NOALLOC(1, 4, 16); break;

@@ -159,3 +159,30 @@ def test_windowed_rows_sixteen_to_a_warp(torch_cuda, sizes, kmax, cnt):  # noqa:
         w, bias = h.get_weights(l)
         assert np.array_equal(w, arrays[2][l]) and np.array_equal(bias, arrays[3][l])
     h.destroy()
+
+
+@pytest.mark.parametrize("mode", sorted(BWD_MODES))
+@pytest.mark.parametrize("batches", [(17, 24, 25, 32), (40, 37, 33, 64, 56), (100, 65, 121, 128)])
+def test_lanes_of_nothing_but_padding(torch_cuda, batches, mode):  # noqa: F811
+    """Batches that leave whole lanes of a padded tile row empty, one handle for all of them: growing ones, smaller ones that run
+    in the graph of a larger one, full ones.  The sigmoid's padding is not zero, so anything it reached would show."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(batches[0])
+    n = 530
+    arrays = ragged_net(rng, n=n, layers=3, kmax=40, scale=0.3)
+    h = pkg.Sdnn.create(*arrays, max_batch=max(batches), train=True, update_bias=True, activation=pkg.ACT_SIGMOID, flags=BWD_MODES[mode])
+    ora = OracleNet(*arrays, update_bias=True, activation="sigmoid")
+    for b in batches:
+        ora.quantize_state()
+        for l in range(3):
+            h.set_weights(l, ora.w[l], ora.bias[l])
+        x0, y = vectors(rng, b, n), vectors(rng, b, n)
+        h.train_step(torch.from_numpy(x0).cuda(), torch.from_numpy(y).cuda(), b, 0.5)
+        ora.train_step(x0, y, 0.5, keep=())
+        for l in range(3):
+            w, bias = h.get_weights(l)
+            check_close(w, ora.w[l], f"W^{l + 1} at B = {b}")
+            check_close(bias, ora.bias[l], f"b^{l + 1} at B = {b}")
+    h.destroy()
+    for cnt in batches:
+        infer_parity(torch_cuda, arrays, vectors(rng, cnt, n), max(batches), expect_nonempty=True)
