@@ -998,14 +998,14 @@ int train_vector_width(const sdnn* h, int B) {
     return B <= 4 && h->split && h->N < VECTOR_TRAIN_WORK && h->N * v <= VECTOR_TRAIN_WORK && takes_vector(h, B) ? v : 0;
 }
 int forward_vector(sdnn* h, int v) {
-    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, h->vector_kpad, 0, nullptr, v, nullptr, nullptr, h->d_acts, h->vector_status, h->cfg.clamp, h->cfg.activation};
+    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, vector_ctas(h->N), h->vector_kpad, 0, nullptr, v, nullptr, nullptr, h->d_acts, h->vector_status, h->cfg.clamp, h->cfg.activation};
     return v == 1 ? launch_vector<1>(h, a) : v == 2 ? launch_vector<2>(h, a) : launch_vector<4>(h, a);
 }
 
 // All layers for one to four inputs: x0 [cnt][N] -> y and nonzero counts (either may be NULL).
 int infer_vector(sdnn* h, const float* x0, int cnt, float* y, int* nz_count) {
     NvtxRange call("sdnn whole-network inference");
-    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, h->vector_kpad, 0, x0, cnt, y, nz_count, nullptr, h->vector_status, h->cfg.clamp, h->cfg.activation};
+    const VectorArgs a{h->d_vector, h->d_bias, h->N, h->L, vector_ctas(h->N), h->vector_kpad, 0, x0, cnt, y, nz_count, nullptr, h->vector_status, h->cfg.clamp, h->cfg.activation};
     return cnt == 1 ? launch_vector<1>(h, a) : cnt == 2 ? launch_vector<2>(h, a) : launch_vector<4>(h, a);
 }
 

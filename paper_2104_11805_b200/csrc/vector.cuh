@@ -7,7 +7,10 @@
 // each, which counts its bytes down on the receiver's mbarrier.  A CTA goes on to the next layer when all n values have
 // arrived: no cluster-wide barrier in the chain.  Two buffers are enough: a CTA sends layer k + 1 after it has received all of layer
 // k, and a CTA sends its part of layer k after its last read of layer k - 1.  What bounds a layer is that chain: read, add,
-// collect, send, arrive.  The entries are off it: a CTA's part of a layer is one contiguous stretch of the sliced copy, and
+// collect, send, arrive.  The argument needs every CTA that is sent to to send as well: a CTA that sent nothing would be waited for by
+// nobody, and the others could be two layers ahead of it, counting on a barrier whose last phase it has not seen the end of.  A
+// net of at most 960 neurons leaves CTAs without rows: they take no part in the exchange (vector_ctas).
+// The entries are off the chain: a CTA's part of a layer is one contiguous stretch of the sliced copy, and
 // bulk copies bring it into a ring of shared-memory stages several layers ahead.  (Prefetched into registers two layers ahead
 // instead, a layer took 1.0 us: loads of different ages share a scoreboard, so that waiting for the older ones waits for
 // the younger ones too.)
@@ -15,11 +18,13 @@
 // CTA leaves the cluster before the last, nor with a copy of its own under way that has not failed to arrive in time).
 #pragma once
 #include "kernels.cuh"
+#include "plan.h"
 
 namespace sdnn_kernels {
 
-constexpr int VECTOR_CTAS = 16, VECTOR_THREADS = 256, VECTOR_WARPS = VECTOR_THREADS / 32;
-constexpr int VECTOR_BLOCK = VECTOR_WARPS * 8;               // rows a CTA works on at once
+using namespace sdnn_plan;
+constexpr int VECTOR_THREADS = 256, VECTOR_WARPS = VECTOR_THREADS / 32;
+static_assert(VECTOR_BLOCK == VECTOR_WARPS * 8 && VECTOR_CTAS == 2 * VECTOR_WARPS, "eight rows a warp; a warp sends to two CTAs");
 constexpr int VECTOR_STAGES = 8;                             // most stages of the ring of entries
 constexpr unsigned VECTOR_WAIT_LIMIT = 1u << 20;
 
@@ -31,6 +36,7 @@ struct VectorArgs {
     const VectorLayer* layers;      // [depth]
     const float* bias;              // [depth][n]
     int n, depth;
+    int ctas;                       // CTAs that have rows (vector_ctas): the others only hold their place in the cluster
     int kpad;                       // entries per row of every slice of every layer (a multiple of 8)
     int stages;                     // of the ring of entries
     const float* x;                 // [cnt][n]
@@ -113,7 +119,8 @@ vector_infer_kernel(const VectorArgs a) {
 #pragma unroll
         for (int b = 0; b < V; ++b)
             reinterpret_cast<float*>(vector_smem)[i * V + b] = a.acts ? a.acts[i * 4 + b] : b < a.cnt ? a.x[(size_t)b * n + i] : 0.0f;
-    // receivers: warp w sends to CTAs w and w + 8
+    const unsigned ctas = (unsigned)a.ctas;
+    // receivers: warp w sends to CTAs w and w + 8, those of them that have rows
     const unsigned my_x = x0 + rank * (VECTOR_BLOCK * PITCH);
     const unsigned to_x[2] = {cluster_addr(my_x, warp), cluster_addr(my_x, warp + VECTOR_WARPS)};
     const unsigned to_bar[2] = {cluster_addr(bar0, warp), cluster_addr(bar0, warp + VECTOR_WARPS)};
@@ -138,7 +145,7 @@ vector_infer_kernel(const VectorArgs a) {
             }
         }
     };
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0 && rank < ctas)
         for (int k = 0; k < min(a.stages, a.depth); ++k) load(k);
 
     const int row0 = (int)rank * VECTOR_BLOCK + warp * 8 + (lane & 7);                    // this lane's row in block 0
@@ -151,6 +158,7 @@ vector_infer_kernel(const VectorArgs a) {
     };
     next_bias(0);
     cluster_barrier();
+    if (rank >= ctas) { cluster_barrier(); return; }                                      // no rows: nobody sends to it, it waits for nothing
     if (threadIdx.x == 0) mbar_expect_tx(bar0 + 8u, x_bytes);
 
     bool ok = true;
@@ -208,8 +216,8 @@ vector_infer_kernel(const VectorArgs a) {
                 const int rows = min(VECTOR_BLOCK, n - ((int)rank * VECTOR_BLOCK + s * STRIDE));
                 if (rows <= 0) break;
                 const unsigned bytes = ((unsigned)rows * PITCH + 15u) & ~15u, off = out_off + (unsigned)(s * STRIDE) * PITCH;
-                send_bulk(to_x[0] + off, send + (unsigned)(s * VECTOR_BLOCK) * PITCH, bytes, to_bar[0] + bar_off);
-                send_bulk(to_x[1] + off, send + (unsigned)(s * VECTOR_BLOCK) * PITCH, bytes, to_bar[1] + bar_off);
+                if (warp < ctas) send_bulk(to_x[0] + off, send + (unsigned)(s * VECTOR_BLOCK) * PITCH, bytes, to_bar[0] + bar_off);
+                if (warp + VECTOR_WARPS < ctas) send_bulk(to_x[1] + off, send + (unsigned)(s * VECTOR_BLOCK) * PITCH, bytes, to_bar[1] + bar_off);
             }
             if (warp == 0 && k + a.stages < a.depth) load(k + a.stages);                  // every warp has read this layer's stage
         }
@@ -226,7 +234,7 @@ vector_infer_kernel(const VectorArgs a) {
 
     const float* x = reinterpret_cast<const float*>(vector_smem + ((a.depth & 1) ? x_bytes : 0u));
     if (a.y)
-        for (int i = (int)rank * VECTOR_THREADS + threadIdx.x; i < n; i += VECTOR_CTAS * VECTOR_THREADS)
+        for (int i = (int)rank * VECTOR_THREADS + threadIdx.x; i < n; i += a.ctas * VECTOR_THREADS)
 #pragma unroll
             for (int b = 0; b < V; ++b) if (b < a.cnt) a.y[(size_t)b * n + i] = x[i * V + b];
     if (a.nz_count && rank == 0) {

@@ -87,6 +87,36 @@ def test_whole_network_launch(torch_cuda, n, k, layers, cnt, act):  # noqa: F811
     h.destroy()
 
 
+@pytest.mark.parametrize("n,layers", [(40, 120), (600, 120), (960, 40), (961, 40)])
+@pytest.mark.parametrize("cnt", [1, 2, 4])
+def test_whole_network_launch_with_ctas_that_have_no_rows(torch_cuda, n, layers, cnt):  # noqa: F811
+    """Nets of at most 960 neurons leave some CTAs of the cluster without rows; deep enough, and called often enough, that a CTA
+    that got ahead of the others would be noticed: every call the same bits, and the oracle's numbers.  Training runs its forward chain
+    the same way."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    k = 32
+    rp = [np.arange(n + 1, dtype=np.int32) * k] * layers
+    cols = [np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for _ in range(n)]).astype(np.int32) for _ in range(layers)]
+    vals = [rng.uniform(-1, 1, size=n * k).astype(np.float32) for _ in range(layers)]
+    bias = [(rng.standard_normal(n) * 0.1).astype(np.float32) for _ in range(layers)]
+    x0 = vectors(rng, cnt, n)
+    want = OracleNet(rp, cols, vals, bias, activation="sigmoid").infer(x0)
+    for train in (False, True):
+        h = pkg.Sdnn.create(rp, cols, vals, bias, max_batch=4, train=train, activation=pkg.ACT_SIGMOID)
+        x, outs = torch.from_numpy(x0).cuda(), []
+        for _ in range(50):
+            if train:
+                h.train_step(x, torch.zeros_like(x), cnt, 0.0)      # a step of no length: only the activations matter here
+            else:
+                outs.append(torch.full((cnt, n), -1.0, device="cuda"))
+                h.infer_batch(x, cnt, outs[-1])
+        got = h.get_activations(layers, cnt) if train else outs[0].cpu().numpy()
+        check_close(got, want, "x^L")
+        assert all(torch.equal(y, outs[0]) for y in outs)
+        h.destroy()
+
+
 @pytest.mark.parametrize("cnt", [65, 129, 150, 300, 449, 513])
 def test_tile_widths_between_powers_of_two(torch_cuda, cnt):  # noqa: F811
     """Layers large enough for tiles cut into chunks of 64 or 128 inputs: widths just above a chunk, a few chunks, and one that
