@@ -14,8 +14,10 @@
 // bulk copies bring it into a ring of shared-memory stages several layers ahead.  (Prefetched into registers two layers ahead
 // instead, a layer took 1.0 us: loads of different ages share a scoreboard, so that waiting for the older ones waits for
 // the younger ones too.)
-// Every wait is bounded: after VECTOR_WAIT_LIMIT polls the thread raises *status, waits no more and ends with the others (no
-// CTA leaves the cluster before the last, nor with a copy of its own under way that has not failed to arrive in time).
+// Every wait is bounded: after VECTOR_WAIT_LIMIT polls the thread raises *status, waits no more and ends with the others.  From then
+// on it sends nothing, loads nothing and arms no barrier: a barrier whose phase it has not seen the end of must not be counted
+// on again, and every copy it has issued is older than the wait that it gave up.  CTAs that miss what it would have sent give up
+// in their turn.  Nor does it gather: indices that have not arrived could point anywhere.  No CTA leaves the cluster before the last.
 #pragma once
 #include "kernels.cuh"
 #include "plan.h"
@@ -186,7 +188,7 @@ vector_infer_kernel(const VectorArgs a) {
                 for (int b = 0; b < V; ++b)
                     acc.a[b] = fmaf(w.a[3], g3.a[b], fmaf(w.a[2], g2.a[b], fmaf(w.a[1], g1.a[b], fmaf(w.a[0], g0.a[b], acc.a[b]))));
             };
-            const int mine = row0 + d * STRIDE < n ? nch : 0;                             // the stage holds nothing for rows beyond the last one
+            const int mine = ok && row0 + d * STRIDE < n ? nch : 0;                       // the stage holds nothing for rows beyond the last one
             int t = 0;
             for (; t + 4 + e < mine; t += 8) { chunk(acc0, t); chunk(acc1, t + 4); }
             if (t + e < mine) chunk(acc0, t);
@@ -210,7 +212,7 @@ vector_infer_kernel(const VectorArgs a) {
             }
         }
         __syncthreads();
-        if (lane == 0) {
+        if (lane == 0 && ok) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             for (int s = 0; s < per_layer; ++s) {
                 const int rows = min(VECTOR_BLOCK, n - ((int)rank * VECTOR_BLOCK + s * STRIDE));
@@ -229,7 +231,7 @@ vector_infer_kernel(const VectorArgs a) {
         if (bar_off == 8u) { bar_off = 0u; out_off = 0u; send += s_bytes; }
         else { bar_off = 8u; out_off = x_bytes; send -= s_bytes; phase ^= 1u; }           // both barriers have completed once more
         // this barrier's last phase is over: it counts the next layer
-        if (threadIdx.x == 0 && k + 1 < a.depth) mbar_expect_tx(bar0 + bar_off, x_bytes);
+        if (threadIdx.x == 0 && ok && k + 1 < a.depth) mbar_expect_tx(bar0 + bar_off, x_bytes);
     }
 
     const float* x = reinterpret_cast<const float*>(vector_smem + ((a.depth & 1) ? x_bytes : 0u));

@@ -29,10 +29,13 @@ class Fault(Exception):
     pass
 
 
-def exchange(owners, ctas, depth, rng):
+def exchange(owners, ctas, depth, rng, mute=None, careless=False):
     """The exchange of vector_infer_kernel as its comments state it, under a random schedule: `ctas` CTAs run the layers, the first
     `owners` of them have rows and send them.  A CTA's barrier (k % 2) counts layer k: armed for all of the layer, completed when
-    `owners` messages are in.  Raises Fault where a message meets a barrier or a buffer that is not ready for it."""
+    `owners` messages are in.  Raises Fault where a message meets a barrier or a buffer that is not ready for it.
+    mute: (CTA, layer) whose messages are lost, so that waits run out; careless: a CTA that gave up goes on sending and arming.
+    Returns the CTAs that gave up."""
+    gave_up = set()
     step = [("send", 0)] * ctas                 # what each CTA does next
     armed = [[1, 0] for _ in range(ctas)]       # layers that each barrier has been armed for (layer 0 before the loop)
     done = [[0, 0] for _ in range(ctas)]        # ... and has completed
@@ -49,10 +52,14 @@ def exchange(owners, ctas, depth, rng):
     while flying or any(s is not None for s in step):
         moves = [("message", i) for i in range(len(flying))]
         for r in range(ctas):
-            if step[r] and (step[r][0] == "send" or done[r][step[r][1] % 2] > step[r][1] // 2):
+            if step[r] and (step[r][0] == "send" or r in gave_up or done[r][step[r][1] % 2] > step[r][1] // 2):
                 moves.append(("cta", r))
-        if not moves:
-            raise Fault("everybody waits")
+        if not moves:                           # a wait runs out only where nothing else can happen
+            if mute is None:
+                raise Fault("everybody waits")
+            i = rng.choice([r for r in range(ctas) if step[r]])
+            gave_up.add(i)
+            moves = [("cta", i)]
         rest = [m for m in moves if m != ("cta", slow)]
         kind, i = rng.choice(rest if rest and rng.random() < 0.98 else moves)
         if kind == "message":
@@ -67,18 +74,23 @@ def exchange(owners, ctas, depth, rng):
         what, k = step[i]
         if what == "send":
             read[i] = k
-            if i < owners:
+            if i < owners and (careless or i not in gave_up):
                 if any(f[0] == i and f[2] == k - 2 for f in flying):
                     raise Fault("layer %d written over a copy under way" % k)
-                flying += [(i, r, k) for r in range(ctas)]
+                flying += [(i, r, k) for r in range(ctas) if (i, k) != mute]
             step[i] = ("wait", k)
         else:
             if k + 1 < depth:
-                armed[i][(k + 1) % 2] += 1
-                settle(i, (k + 1) % 2)
+                if careless or i not in gave_up:
+                    b = (k + 1) % 2
+                    if armed[i][b] > done[i][b]:
+                        raise Fault("armed for layer %d with the last phase still open" % (k + 1))
+                    armed[i][b] += 1
+                    settle(i, b)
                 step[i] = ("send", k + 1)
             else:
                 step[i] = None
+    return gave_up
 
 
 def test_whole_network_exchange_stays_in_step(plan):
@@ -92,3 +104,17 @@ def test_whole_network_exchange_stays_in_step(plan):
     with pytest.raises(Fault):
         for seed in range(25):
             exchange((600 + block - 1) // block, cluster, 6, random.Random(seed))
+
+
+def test_whole_network_exchange_ends_when_a_message_is_lost(plan):
+    """A layer's part that never arrives: every CTA that needs it gives up in its turn, and none counts on a barrier again whose
+    phase it has not seen the end of (which going on as if nothing had happened would)."""
+    for n in [100, 600, 1024]:
+        ctas = plan.ctas(n)
+        for seed in range(25):
+            rng = random.Random(seed)
+            lost = (rng.randrange(ctas), rng.randrange(5))
+            assert exchange(ctas, ctas, 6, rng, mute=lost) == set(range(ctas))
+    with pytest.raises(Fault):
+        for seed in range(25):
+            exchange(10, 10, 6, random.Random(seed), mute=(3, 2), careless=True)
