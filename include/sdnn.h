@@ -33,6 +33,10 @@
  *  - Calls are issued on cfg->cuda_stream; a call that returns a scalar to the host
  *    (loss_out, nz_total_out) or uses host buffers synchronises that stream before
  *    returning, otherwise it returns after enqueueing.
+ *  - Narrow nets run one to four inputs as one launch whose CTAs wait for one another, each wait with a limit.  If one
+ *    runs out (SDNN_ERR_CUDA), the results of that call are not valid.  It is reported once: by the call itself where
+ *    that waits for the stream, else by the handle's next call that launches such work or waits for the stream
+ *    (sdnn_get_weights(h, 0, NULL, NULL) does nothing else); sdnn_set_weights then changes nothing.
  *  - A handle is not thread-safe.  There is no CPU fallback: without a CUDA device
  *    creation fails with SDNN_ERR_CUDA.
  */
@@ -374,6 +378,10 @@ int64_t sdnn_device_bytes(const sdnn_t* h);
  * launches, bwd_ms the L backward+update launches.  Synchronises the stream.  SDNN_ERR_STATE if no
  * step has run. */
 int sdnn_get_phase_times(sdnn_t* h, float* fwd_ms, float* bwd_ms);
+
+/* For tests of a caller's error handling: raises, on the host, the word that a whole-network launch raises when a wait
+ * in it runs out (see the conventions above).  SDNN_ERR_STATE for handles without such launches. */
+int sdnn_inject_wait_failure(sdnn_t* h);
 
 /* Per-layer liveness of the most recent inference tile run with SDNN_FLAG_SKIP_DEAD in effect (see the flag):
  * live_inputs_out host int32[L] = inputs of that tile whose activation vector is not all zero after each layer.

@@ -62,6 +62,7 @@ _PROTOS = {
     "sdnn_probe_mixed_gather": (ctypes.c_int, [_i32, _i64, _i32, _i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double)]),
     "sdnn_probe_word_rate": (ctypes.c_int, [_i32, _i64, ctypes.POINTER(ctypes.c_double)]),
     "sdnn_probe_smem_gather_rate": (ctypes.c_int, [_i32, _i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(_i32)]),
+    "sdnn_inject_wait_failure": (ctypes.c_int, [_vp]),
     "sdnn_get_phase_times": (ctypes.c_int, [_vp, ctypes.POINTER(_f32), ctypes.POINTER(_f32)]),
     "sdnn_get_liveness": (ctypes.c_int, [_vp, _vp]),
     "sdnn_infer_noalloc": (ctypes.c_int, [_i32, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _i32, _vp, _f32, _vp]),
@@ -356,6 +357,10 @@ class Sdnn:
         a, b = ctypes.c_float(0.0), ctypes.c_float(0.0)
         self._check(self._lib.sdnn_get_phase_times(self._h, ctypes.byref(a), ctypes.byref(b)))
         return a.value, b.value
+
+    def inject_wait_failure(self):
+        """Raises the word that a whole-network launch raises when a wait in it runs out (tests of error handling)."""
+        self._check(self._lib.sdnn_inject_wait_failure(self._h))
 
     def get_liveness(self):
         out = np.empty(self.n_layers, dtype=np.int32)

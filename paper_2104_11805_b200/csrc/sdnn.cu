@@ -943,6 +943,7 @@ int build_vector(sdnn* h) {
     return SDNN_OK;
 }
 
+// Whether a whole-network launch that has ended gave up; asked wherever the host has waited for the stream, and before new work
 int vector_check(sdnn* h) {
     if (!h->vector_status || !*h->vector_status) return SDNN_OK;
     *h->vector_status = 0;
@@ -2112,7 +2113,7 @@ int sdnn_train_step_host(sdnn_t* h, const float* x0, const float* target, int32_
     rc = train_step_device(h, h->d_stage_a, h->d_stage_b, B, eta, loss_out);
     if (rc) return rc;
     CU(h, cudaStreamSynchronize(h->stream));
-    return SDNN_OK;
+    return vector_check(h);
 }
 
 int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out, int32_t* nz_count_out,
@@ -2140,6 +2141,7 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
         long long total = 0;
         CU(h, cudaMemcpyAsync(&total, h->d_running, sizeof total, cudaMemcpyDeviceToHost, h->stream));
         CU(h, cudaStreamSynchronize(h->stream));
+        if ((rc = vector_check(h))) return rc;
         if (nz_total_out) *nz_total_out = total;
         if (nz_index_out && total > nz_index_capacity)
             return fail(h, SDNN_ERR_INVALID_ARG, "nz_index_capacity %lld too small, %lld ids needed", (long long)nz_index_capacity, total);
@@ -2152,7 +2154,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     int rc = check_infer_args(h, x0, n_inputs, nz_index_out, nz_index_capacity);
     if (rc) return rc;
     CU(h, cudaSetDevice(h->device));
-    if ((rc = ensure_stage(h))) return rc;
+    if ((rc = vector_check(h)) || (rc = ensure_stage(h))) return rc;
     if (nz_index_out && nz_index_capacity > h->stage_idx_cap) {
         if ((rc = dev_alloc(h, &h->d_stage_idx, (size_t)nz_index_capacity, false))) return rc;   // grows; old block freed at destroy
         h->stage_idx_cap = nz_index_capacity;
@@ -2204,6 +2206,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     long long total = 0;
     if (want_sets) CU(h, cudaMemcpyAsync(&total, h->d_running, sizeof total, cudaMemcpyDeviceToHost, h->stream));
     CU(h, cudaStreamSynchronize(h->stream));
+    if ((rc = vector_check(h))) return rc;
     if (nz_total_out) *nz_total_out = total;
     if (nz_index_out) {
         const long long m = total < nz_index_capacity ? total : nz_index_capacity;
@@ -2256,8 +2259,8 @@ int sdnn_get_weights(sdnn_t* h, int32_t layer, float* values_out, float* bias_ou
             for (int r = 0; r < h->N; ++r) bias_out[lm.row_src[r]] = tmp[r];
         }
     }
-    if (!values_out && !bias_out) CU(h, cudaStreamSynchronize(h->stream));
-    return SDNN_OK;
+    if (!bias_out && !(values_out && nnz)) CU(h, cudaStreamSynchronize(h->stream));      // else the copies have waited
+    return vector_check(h);
 }
 
 int sdnn_set_weights(sdnn_t* h, int32_t layer, const float* values, const float* bias) {
@@ -2272,6 +2275,7 @@ int sdnn_set_weights(sdnn_t* h, int32_t layer, const float* values, const float*
             if (!std::isfinite(bias[i])) return fail(h, SDNN_ERR_BAD_CSR, "layer %d: non-finite bias at row %d", layer, i);
     CU(h, cudaSetDevice(h->device));
     CU(h, cudaStreamSynchronize(h->stream));
+    if (const int rc = vector_check(h)) return rc;
     const LayerMem& lm = h->lay[layer];
     const int64_t nnz = h->nnz[layer];
     if (values && nnz) {
@@ -2327,7 +2331,7 @@ int sdnn_mirror_mismatches(sdnn_t* h, int32_t layer, int64_t* count_out) {
     CU(h, cudaMemcpyAsync(&v, h->d_mismatch, sizeof v, cudaMemcpyDeviceToHost, h->stream));
     CU(h, cudaStreamSynchronize(h->stream));
     *count_out = (int64_t)v;
-    return SDNN_OK;
+    return vector_check(h);
 }
 
 static int fetch_tile(sdnn_t* h, const float* tile, float* out, int B, int ld, int boundary) {
@@ -2340,7 +2344,7 @@ static int fetch_tile(sdnn_t* h, const float* tile, float* out, int B, int ld, i
     CU(h, cudaMemcpy(tmp.data(), tile, tmp.size() * sizeof(float), cudaMemcpyDeviceToHost));
     for (int b = 0; b < B; ++b)
         for (int i = 0; i < N; ++i) out[(size_t)b * N + i] = tmp[(size_t)(lab ? (*lab)[i] : i) * ld + b];
-    return SDNN_OK;
+    return vector_check(h);
 }
 
 int sdnn_get_activations(sdnn_t* h, int32_t layer, float* out) {
@@ -2371,7 +2375,7 @@ int sdnn_get_gradient(sdnn_t* h, int32_t layer, float* out) {
         sliced_to_csr(h, lm, tmp, stored.data());
         stored_to_caller(lm, stored, out, h->nnz[layer - 1]);
     }
-    return SDNN_OK;
+    return vector_check(h);
 }
 
 int sdnn_get_phase_times(sdnn_t* h, float* fwd_ms, float* bwd_ms) {
@@ -2384,6 +2388,13 @@ int sdnn_get_phase_times(sdnn_t* h, float* fwd_ms, float* bwd_ms) {
     CU(h, cudaEventElapsedTime(&b, h->ev[1], h->ev[2]));
     if (fwd_ms) *fwd_ms = a;
     if (bwd_ms) *bwd_ms = b;
+    return vector_check(h);
+}
+
+int sdnn_inject_wait_failure(sdnn_t* h) {
+    if (!h) return SDNN_ERR_INVALID_ARG;
+    if (!h->vector_status) return fail(h, SDNN_ERR_STATE, "this handle has no whole-network launches");
+    *h->vector_status = 1;
     return SDNN_OK;
 }
 

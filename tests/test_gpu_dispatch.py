@@ -117,6 +117,46 @@ def test_whole_network_launch_with_ctas_that_have_no_rows(torch_cuda, n, layers,
         h.destroy()
 
 
+def test_a_wait_that_ran_out_is_reported_by_the_next_call_that_looks(torch_cuda):  # noqa: F811
+    """The word that a whole-network launch raises, raised from the host: every call that launches such work or waits for the stream
+    reports it, once; sdnn_set_weights leaves the weights as they are; handles without such launches have no word."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(3)
+    n, k, layers = 600, 16, 3
+    arrays = ([np.arange(n + 1, dtype=np.int32) * k] * layers,
+              [np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for _ in range(n)]).astype(np.int32)] * layers,
+              [(rng.standard_normal(n * k) * 0.3).astype(np.float32)] * layers, [np.zeros(n, dtype=np.float32)] * layers)
+    h = pkg.Sdnn.create(*arrays, max_batch=4, train=True, activation=pkg.ACT_SIGMOID, flags=pkg.FLAG_KEEP_DEBUG)
+    x0 = vectors(rng, 4, n)
+    x, y, host_y, ids = torch.from_numpy(x0).cuda(), torch.zeros(4, n, device="cuda"), np.zeros((4, n), np.float32), torch.zeros(4 * n, dtype=torch.int32, device="cuda")
+    h.train_step(x, x, 4, 0.1, want_loss=True)
+    kept = h.get_weights(1)
+    calls = {
+        "train_step": lambda: h.train_step(x, x, 2, 0.1), "train_step with its loss": lambda: h.train_step(x, x, 2, 0.1, want_loss=True),
+        "train_step_averaged": lambda: h.train_step(x, x, 4, 0.1, averaged=True), "train_step_host": lambda: h.train_step(x0, x0, 2, 0.1, host=True),
+        "infer_batch": lambda: h.infer_batch(x, 1, y), "infer_batch with ids": lambda: h.infer_batch(x, 4, y, None, ids, 4 * n, want_total=True),
+        "infer_batch of a tile": lambda: h.infer_batch(x, 4, y, want_total=True), "infer_batch_host": lambda: h.infer_batch(x0, 4, host_y, host=True),
+        "get_weights": lambda: h.get_weights(0), "values alone": lambda: h.get_weights(0, want_bias=False),
+        "set_weights": lambda: h.set_weights(1, np.ones_like(kept[0]), np.ones_like(kept[1])), "get_activations": lambda: h.get_activations(1, 4),
+        "get_delta": lambda: h.get_delta(1, 4), "get_gradient": lambda: h.get_gradient(1), "mirror_mismatches": lambda: h.mirror_mismatches(1),
+        "get_phase_times": h.get_phase_times}
+    for name, call in calls.items():
+        before = h.get_weights(1)
+        h.inject_wait_failure()
+        with pytest.raises(pkg.SdnnError) as e:
+            call()
+        assert e.value.code == -4 and "gave up" in e.value.message, name
+        if name == "set_weights":
+            assert all(np.array_equal(a, b) for a, b in zip(h.get_weights(1), before))
+        call()                                                  # reported once
+    h.destroy()
+    h = pkg.Sdnn.create(*ragged_net(rng, n=n, layers=2, kmax=40, scale=0.3), max_batch=4)
+    with pytest.raises(pkg.SdnnError) as e:
+        h.inject_wait_failure()
+    assert e.value.code == -5
+    h.destroy()
+
+
 @pytest.mark.parametrize("cnt", [65, 129, 150, 300, 449, 513])
 def test_tile_widths_between_powers_of_two(torch_cuda, cnt):  # noqa: F811
     """Layers large enough for tiles cut into chunks of 64 or 128 inputs: widths just above a chunk, a few chunks, and one that
