@@ -4,6 +4,7 @@
 // arithmetic step runs in the kernels of kernels.cuh.
 #include "../../include/sdnn.h"
 #include "kernels.cuh"
+#include "plan.h"
 #include "vector.cuh"
 #include "reorder.h"
 
@@ -164,6 +165,7 @@ struct sdnn {
     int* d_in_label = nullptr;          // [N] tile row of input neuron i (NULL: identity)
     std::vector<std::vector<int>> labels;   // [L + 1] host: tile row of neuron i at boundary k (x^k, delta^k); empty = identity
     int windowed_layers = 0;
+    int64_t mean_elems = 0;             // stored elements per layer, padding included
     VectorLayer* d_vector = nullptr;    // [L] table of vector_infer_kernel (NULL: the net is not for it)
     int vector_kpad = 0;                // entries per row of every slice of every layer (the same everywhere, or no table)
     int* vector_status = nullptr;       // pinned: raised by a whole-network kernel whose wait for its neighbours ran out
@@ -263,37 +265,11 @@ int dev_alloc(sdnn* h, T** out, size_t count, bool zero) {
 // then stand in their way (N = 16384, B = 1: 6 % slower).
 constexpr int PDL_AT_END = 1, PDL_EARLY = 2;
 
-// padded batch width: 4, 8, .., 256, then multiples of 256
-int padded_width(int b) {
-    if (b <= 4) return 4;
-    if (b <= 256) { int w = 4; while (w < b) w <<= 1; return w; }
-    return (b + 255) / 256 * 256;
-}
-
 // lanes per row group (g) and batch entries per lane (v) for a chunk of cw inputs (a power of two up to 256)
 struct Geometry { int g; int v; };
 Geometry geometry(int cw) {
     if (cw <= 4) return {1, 4};
     return {cw / 8, 8};
-}
-
-// How the columns of an inference tile of `cnt` inputs are padded and cut: chunks of cw inputs, cols of them in all.  One chunk up
-// to 256 inputs and chunks of 256 beyond, unless chunks of 128 or 64 save more padding than the 5 or 10 % they may cost, in
-// layers that are bound by their gathers: 4096 neurons, 300 inputs are 320 columns, not 512 (960 -> 681 us for 60 layers),
-// 16384 neurons, 150 inputs 192, not 256 (631 -> 434 us for 20).  Smaller layers are bound by their chain of round trips, which
-// padding does not lengthen and more chunks do (1024 neurons, 300 inputs: 517 -> 555 us for 120).
-constexpr int64_t SHAPE_WORK = 32 << 20;      // stored elements x inputs per layer
-struct TileShape { int cw, cols; };
-TileShape tile_shape(int cnt, int64_t elems) {
-    TileShape best{std::min(padded_width(cnt), 256), padded_width(cnt)};
-    if (cnt <= 64 || elems * cnt < SHAPE_WORK) return best;
-    double least = best.cols;
-    for (int cw = 128; cw >= 64; cw /= 2) {
-        const int cols = (cnt + cw - 1) / cw * cw;
-        const double work = cols * (cw == 64 ? 1.10 : 1.05);
-        if (work < least) { least = work; best = {cw, cols}; }
-    }
-    return best;
 }
 
 int validate_cfg(const sdnn_config* cfg) {
@@ -1140,17 +1116,11 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     return SDNN_OK;
 }
 
-// The launches of a tile's layers, as a graph from a handle's second call on: one launch of the host's instead of one per
-// layer, which take 2.2 us each and which a layer of a narrow net does not outlast (1024 neurons x 120 layers, 256 inputs, three
-// handles in turn: 300 us a call of launches).  The first call launches directly, so that a net that is asked once does not pay for
-// the graph.  A lane keeps four, for as many tile widths.  Layers that outlast their launch calls several times over are
-// launched directly (4096 neurons, tiles of 1024: 27 us a layer, 1 % slower as graphs on two streams), unless dead inputs are
-// being dropped: nobody knows what is left of those.
-constexpr int64_t GRAPH_WORK = 32 << 20;      // stored elements x inputs per layer: about 7 us
+// The launches of a tile's layers, as a graph where tile_as_graph says so.  A lane keeps four, for as many tile widths.
 template <typename Layers>
 int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int cnt, bool track, const Layers& layers) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (h->infer_calls < 2 || h->L < 4 || (!track && h->lay[0].r_elems * cols > GRAPH_WORK) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
+    if (h->infer_calls < 2 || !tile_as_graph(h->L, h->mean_elems, cols, track) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
         capturing != cudaStreamCaptureStatusNone) {
         layers(cnt);
         return SDNN_OK;
@@ -1193,7 +1163,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     bool track = h->compaction && h->cfg.activation == SDNN_ACT_CLAMPED_RELU;      // sigmoid(b) is never 0: nothing ever dies
     for (int l = 0; l < h->L && track; ++l) track = h->bias_nonpositive[l] != 0;     // the zero vector must be a fixed point
     // dropping dead inputs works on chunks of 64 whatever the padding
-    const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->lay[0].r_elems);
+    const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->mean_elems, h->windowed_layers == h->L);
     const int cw = shape.cw, cols = shape.cols;
     launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     if (consumed) CU(h, cudaEventRecord(consumed, st));
@@ -2055,6 +2025,9 @@ int sdnn_finalize(sdnn_t* h) {
         int rc = build_vector(h);
         if (rc) return rc;
     }
+    int64_t elems = 0;
+    for (const LayerMem& lm : h->lay) elems += lm.windowed ? lm.w_elems : lm.r_elems;
+    h->mean_elems = elems / h->L;
     CU(h, cudaStreamSynchronize(h->stream));
     h->finalized = true;
     return SDNN_OK;

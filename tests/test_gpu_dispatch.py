@@ -231,6 +231,32 @@ def test_windowed_rows_sixteen_to_a_warp(torch_cuda, sizes, kmax, cnt):  # noqa:
     h.destroy()
 
 
+@pytest.mark.parametrize("cnt", [17, 33, 70, 96, 100, 300])
+def test_windowed_tiles_of_whole_chunks(torch_cuda, cnt):  # noqa: F811
+    """Nets with all their operands in shared memory: tiles padded to the next 32 columns, on a handle that has seen a wider one, in
+    the first call and in later ones."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(cnt)
+    n, size, layers, k = 1536, 512, 5, 24
+    rp = np.arange(n + 1, dtype=np.int32) * k
+    cols = [np.concatenate([np.sort(i // size * size + rng.choice(size, size=k, replace=False)) for i in range(n)]).astype(np.int32) for _ in range(layers)]
+    vals = [(rng.standard_normal(n * k) * (2.0 / k) ** 0.5).astype(np.float32) for _ in range(layers)]
+    bias = [(rng.standard_normal(n) * 0.1).astype(np.float32) for _ in range(layers)]
+    h = pkg.Sdnn.create([rp] * layers, cols, vals, bias, max_batch=300, flags=pkg.FLAG_REORDER | pkg.FLAG_SMEM_WINDOWS)
+    assert h.windowed_layers() == layers
+    ora = OracleNet([rp] * layers, cols, vals, bias)
+    wide = torch.from_numpy(vectors(rng, 300, n) + 5.0).cuda()
+    h.infer_batch(wide, 300, torch.zeros(300, n, device="cuda"))
+    for _ in range(3):
+        x0 = vectors(rng, cnt, n)
+        y, c = torch.full((cnt, n), -1.0, device="cuda"), torch.zeros(cnt, dtype=torch.int32, device="cuda")
+        h.infer_batch(torch.from_numpy(x0).cuda(), cnt, y, c)
+        got = y.cpu().numpy()
+        check_close(got, ora.infer(x0), "x^L")
+        assert np.array_equal(c.cpu().numpy(), np.count_nonzero(got, axis=1))
+    h.destroy()
+
+
 @pytest.mark.parametrize("mode", sorted(BWD_MODES))
 @pytest.mark.parametrize("batches", [(17, 24, 25, 32), (40, 37, 33, 64, 56), (100, 65, 121, 128)])
 def test_lanes_of_nothing_but_padding(torch_cuda, batches, mode):  # noqa: F811

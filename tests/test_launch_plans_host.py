@@ -13,6 +13,9 @@ WRAPPER = """
 #include "plan.h"
 using namespace sdnn_plan;
 extern "C" int ctas(int n) { return vector_ctas(n); }
+extern "C" int cols(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cols; }
+extern "C" int chunk(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cw; }
+extern "C" int graph(int layers, long long elems, int cols, int track) { return tile_as_graph(layers, elems, cols, track); }
 """
 
 
@@ -22,7 +25,31 @@ def plan(tmp_path_factory):
     src, lib = d / "plan.cpp", d / "libplan.so"
     src.write_text(WRAPPER)
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)])
-    return ctypes.CDLL(str(lib))
+    lib = ctypes.CDLL(str(lib))
+    for f in (lib.cols, lib.chunk):
+        f.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+    lib.graph.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    return lib
+
+
+def test_tile_shapes(plan):
+    """Every tile holds its inputs in whole chunks within the widest tile its width stands for; narrow layers keep one chunk; nets with
+    their operands in shared memory pad to 32 columns whatever their layers hold."""
+    for cnt in list(range(1, 700)) + [1000, 1024, 1025, 4000]:
+        widest = plan.cols(cnt, 0, 0)
+        for elems in (0, 1 << 15, 1 << 17, 1 << 21, 1 << 28):
+            cw, cols = plan.chunk(cnt, elems, 0), plan.cols(cnt, elems, 0)
+            assert cnt <= cols <= widest and cols % cw == 0
+            if elems * cnt < 32 << 20:
+                assert cols == widest
+            assert plan.cols(cnt, elems, 1) == (widest if cnt <= 32 else (cnt + 31) // 32 * 32)
+    assert plan.cols(300, 131072, 0) == 512 - 192 and plan.cols(150, 524288, 0) == 192
+
+
+def test_layers_that_outlast_their_launch_call_are_launched_directly(plan):
+    """The line is drawn by what a layer holds, at 32 M stored elements x columns, for any layout."""
+    assert plan.graph(120, 1 << 17, 256, 0) and not plan.graph(120, (1 << 17) + 1, 256, 0)
+    assert plan.graph(120, 1 << 21, 1024, 1) and not plan.graph(3, 1, 4, 0)
 
 
 class Fault(Exception):
