@@ -44,6 +44,32 @@ inline TileShape tile_shape(int cnt, int64_t elems, bool windows) {
 constexpr int64_t GRAPH_WORK = 32 << 20;      // stored elements x columns per layer: about 7 us
 inline bool tile_as_graph(int layers, int64_t elems, int cols, bool track) { return layers >= 4 && (track || elems * cols <= GRAPH_WORK); }
 
+// Which of the `n` graphs that a lane keeps a tile takes.  `used` columns of its `cols` hold inputs (rounded up to a lane's eight: the
+// launches gather no padding beyond those), and a graph made for more of them serves fewer, for the price of their padding.  A graph
+// of its own, then, while there is room (4096 neurons x 60, 72 of 128 columns: 204 -> 189 us, 100 of them 197); else the narrowest that serves; else
+// the one not asked for longest makes room for one that serves any tile of this shape.  So batches that vary at will make a lane
+// fill its places, and after that one graph per shape (as long as there are no more shapes than places).
+// Returns the place; `make` is set where the graph has to be made first, with want.used columns (which may have been raised).
+struct GraphKey { int cw = 0, cols = 0, used = 0, pdl = 0; bool track = false; };
+inline int pick_graph(const GraphKey* have, const int64_t* asked, int n, GraphKey& want, bool& make) {      // asked[q] = 0: empty
+    int room = -1, serves = -1, oldest = 0;
+    make = false;
+    for (int q = 0; q < n; ++q) {
+        if (!asked[q]) { if (room < 0) room = q; continue; }
+        const GraphKey& g = have[q];
+        if (g.cw == want.cw && g.cols == want.cols && g.pdl == want.pdl && g.track == want.track && g.used >= want.used) {
+            if (g.used == want.used) return q;
+            if (serves < 0 || g.used < have[serves].used) serves = q;
+        }
+        if (asked[q] < asked[oldest]) oldest = q;
+    }
+    if (room < 0 && serves >= 0) return serves;
+    make = true;
+    if (room >= 0) return room;
+    want.used = want.cols;
+    return oldest;
+}
+
 // Whole networks in one launch (vector.cuh): CTAs of the cluster, and rows a CTA works on at once; CTA r has the rows r * VECTOR_BLOCK
 // .. of every VECTOR_CTAS * VECTOR_BLOCK.
 constexpr int VECTOR_CTAS = 16, VECTOR_BLOCK = 64;

@@ -43,7 +43,8 @@ struct RowShape {
 // Buffers of one inference tile in flight.  Tiles are independent of one another (so are the inputs), and a
 // handle may work on two at a time, each on its own stream, so that the ramp and tail of one tile's launches are
 // filled by the other's.
-struct TileGraph { int cw = 0, cols = 0, pdl = 0; bool track = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0, used = 0; };
+constexpr int TILE_GRAPHS = 4;
+struct TileGraph { cudaGraphExec_t exec = nullptr; int64_t launches = 0; };
 
 struct InferLane {
     cudaStream_t stream = nullptr;         // lane 0: the handle's stream
@@ -56,7 +57,9 @@ struct InferLane {
     int* live_hist = nullptr;              // [L] live inputs after each layer of this lane's most recent tile
     float* stage_out = nullptr;            // host entry point: staged x^L and counts of this lane's tile
     int* stage_cnt = nullptr;
-    TileGraph graphs[4];                   // captured layer chains of this lane's tiles, by width
+    TileGraph graphs[TILE_GRAPHS];         // captured layer chains of this lane's tiles,
+    GraphKey graph_key[TILE_GRAPHS];       // what each was made for,
+    int64_t graph_asked[TILE_GRAPHS] = {}; // and the call that asked for it last (0: none made)
     cudaEvent_t ev_scan = nullptr;         // this lane's last scan of the running id total is done
     cudaEvent_t ev_done = nullptr;         // everything this lane was given in the current call is done
     bool ready = false;
@@ -1116,38 +1119,38 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     return SDNN_OK;
 }
 
-// The launches of a tile's layers, as a graph where tile_as_graph says so.  A lane keeps four, for as many tile widths.
+// The launches of a tile's layers, as a graph where tile_as_graph says so; used: columns that the launches gather for.
 template <typename Layers>
-int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int cnt, bool track, const Layers& layers) {
+int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, bool track, const Layers& layers) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (h->infer_calls < 2 || !tile_as_graph(h->L, h->mean_elems, cols, track) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
         capturing != cudaStreamCaptureStatusNone) {
-        layers(cnt);
+        layers(used);
         return SDNN_OK;
     }
-    TileGraph* g = &ln.graphs[0];
-    for (TileGraph& q : ln.graphs) {
-        if (q.exec && q.cw == cw && q.cols == cols && q.track == track && q.pdl == h->fwd_pdl) { g = &q; break; }
-        if (g->exec && (!q.exec || q.used < g->used)) g = &q;      // the one not used for longest
-    }
-    if (!g->exec || g->cw != cw || g->cols != cols || g->track != track || g->pdl != h->fwd_pdl) {
-        if (g->exec) { cudaGraphExecDestroy(g->exec); g->exec = nullptr; }
+    GraphKey key;
+    key.cw = cw; key.cols = cols; key.used = used; key.pdl = h->fwd_pdl; key.track = track;
+    bool make = false;
+    const int q = pick_graph(ln.graph_key, ln.graph_asked, TILE_GRAPHS, key, make);
+    TileGraph& g = ln.graphs[q];
+    if (make) {
+        if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; ln.graph_asked[q] = 0; }
         cudaGraph_t graph = nullptr;
         const int64_t before = h->launches;
         CU(h, cudaStreamBeginCapture(ln.stream, cudaStreamCaptureModeThreadLocal));
-        layers(cols);      // the graph serves every tile of this padded width
+        layers(key.used);
         cudaError_t e = cudaStreamEndCapture(ln.stream, &graph);
-        g->launches = h->launches - before;
+        g.launches = h->launches - before;
         h->launches = before;
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&g->exec, graph, 0);
+        e = cudaGraphInstantiate(&g.exec, graph, 0);
         cudaGraphDestroy(graph);
-        if (e != cudaSuccess) { g->exec = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
-        g->cw = cw; g->cols = cols; g->track = track; g->pdl = h->fwd_pdl;
+        if (e != cudaSuccess) { g.exec = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
+        ln.graph_key[q] = key;
     }
-    g->used = h->infer_calls;
-    CU(h, cudaGraphLaunch(g->exec, ln.stream));
-    h->launches += g->launches;
+    ln.graph_asked[q] = h->infer_calls;
+    CU(h, cudaGraphLaunch(g.exec, ln.stream));
+    h->launches += g.launches;
     return SDNN_OK;
 }
 
@@ -1167,7 +1170,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     const int cw = shape.cw, cols = shape.cols;
     launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     if (consumed) CU(h, cudaEventRecord(consumed, st));
-    auto layers = [&](int used) {
+    auto layers = [&](int used) {      // used: columns to gather for, a multiple of a lane's
         int cur = 0;
         if (track) {
             const int chunk = std::min(cols, TRACK_CHUNK);
@@ -1204,7 +1207,9 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
         h->live_lane = (int)(&ln - h->lane);
     }
     {
-        const int rc = enqueue_layers(h, ln, cw, cols, cnt, track, layers);
+        // of the columns the tracked and the windowed kernels take whole chunks
+        const int used = track || h->windowed_layers == h->L ? cols : std::min((cnt + 7) / 8 * 8, cols);
+        const int rc = enqueue_layers(h, ln, cw, cols, used, track, layers);
         if (rc) return rc;
     }
     const int cur = (h->L + (track ? 1 : 0)) & 1;

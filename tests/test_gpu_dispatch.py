@@ -231,6 +231,25 @@ def test_windowed_rows_sixteen_to_a_warp(torch_cuda, sizes, kmax, cnt):  # noqa:
     h.destroy()
 
 
+@pytest.mark.parametrize("flags", ["", "NO_PDL", "IDX32"])
+def test_graphs_for_tiles_of_one_padded_width(torch_cuda, flags):  # noqa: F811
+    """A handle asked for batches of many sizes: graphs that gather for exactly their inputs, graphs of more inputs that serve fewer, one
+    that replaces another, two lanes of two tiles.  The sigmoid's padding is not zero, so anything it reached would show."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(8)
+    n = 530
+    arrays = ragged_net(rng, n=n, layers=5, kmax=40, scale=0.3)
+    h = pkg.Sdnn.create(*arrays, max_batch=128, activation=pkg.ACT_SIGMOID, flags=getattr(pkg, "FLAG_" + flags) if flags else 0)
+    ora = OracleNet(*arrays, activation="sigmoid")
+    x0 = vectors(rng, 256, n)
+    want, x = ora.infer(x0), torch.from_numpy(x0).cuda()
+    for cnt in (128, 65, 72, 100, 128, 65, 3, 17, 80, 104, 127, 73, 128, 9, 200, 250, 193, 66, 256, 4):
+        y = torch.full((cnt, n), -1.0, device="cuda")
+        h.infer_batch(x, cnt, y)
+        check_close(y.cpu().numpy(), want[:cnt], f"{cnt} inputs")
+    h.destroy()
+
+
 @pytest.mark.parametrize("cnt", [17, 33, 70, 96, 100, 300])
 def test_windowed_tiles_of_whole_chunks(torch_cuda, cnt):  # noqa: F811
     """Nets with all their operands in shared memory: tiles padded to the next 32 columns, on a handle that has seen a wider one, in

@@ -16,6 +16,21 @@ extern "C" int ctas(int n) { return vector_ctas(n); }
 extern "C" int cols(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cols; }
 extern "C" int chunk(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cw; }
 extern "C" int graph(int layers, long long elems, int cols, int track) { return tile_as_graph(layers, elems, cols, track); }
+extern "C" int graphs_made(const int* cols, const int* used, int calls, int* served_with) {
+    GraphKey have[4];
+    int64_t asked[4] = {};
+    int made = 0;
+    for (int i = 0; i < calls; ++i) {
+        GraphKey want;
+        want.cw = want.cols = cols[i]; want.used = used[i];
+        bool make = false;
+        const int q = pick_graph(have, asked, 4, want, make);
+        if (make) { have[q] = want; ++made; }
+        asked[q] = i + 2;
+        served_with[i] = have[q].cols == cols[i] ? have[q].used : -1;
+    }
+    return made;
+}
 """
 
 
@@ -50,6 +65,33 @@ def test_layers_that_outlast_their_launch_call_are_launched_directly(plan):
     """The line is drawn by what a layer holds, at 32 M stored elements x columns, for any layout."""
     assert plan.graph(120, 1 << 17, 256, 0) and not plan.graph(120, (1 << 17) + 1, 256, 0)
     assert plan.graph(120, 1 << 21, 1024, 1) and not plan.graph(3, 1, 4, 0)
+
+
+def graphs_made(plan, tiles):
+    n = len(tiles)
+    arrays = [(ctypes.c_int * n)(*[t[q] for t in tiles]) for q in range(2)]
+    out = (ctypes.c_int * n)()
+    made = plan.graphs_made(*arrays, n, out)
+    assert all(used <= got <= cols for (cols, used), got in zip(tiles, out))
+    return made, list(out)
+
+
+def test_graphs_gather_no_more_padding_than_they_have_to(plan):
+    """Up to four kinds of tile each have a graph of their own, as wide as their inputs; sizes that vary at will fill the four places and
+    then make one per shape; tiles of as many shapes as places settle."""
+    kinds = [(128, 72), (128, 104), (256, 136), (8, 8)]
+    made, got = graphs_made(plan, kinds * 5)
+    assert made == 4 and got == [used for _, used in kinds] * 5
+    rng = random.Random(1)
+    made, _ = graphs_made(plan, [(128, rng.randrange(72, 129, 8)) for _ in range(500)])
+    assert made <= 5
+    for shapes in (2, 4):
+        tiles = []
+        for i in range(2000):
+            cols = 64 << i % shapes
+            tiles.append((cols, rng.randrange(cols // 2 + 8, cols + 1, 8)))
+        early, _ = graphs_made(plan, tiles[:1000])
+        assert graphs_made(plan, tiles)[0] == early <= 4 + 2 * shapes
 
 
 class Fault(Exception):
