@@ -1464,30 +1464,59 @@ merge_values_kernel(Move m, const float* __restrict__ T, float* __restrict__ rva
     __syncthreads();
     for (int q = threadIdx.x * 4; q < cnt; q += MOVE_THREADS * 4) __stcs(reinterpret_cast<float4*>(rval + lo + q), ld_f4(move_smem + q));
 }
-// Set-up of a Move, from `from` (place in the transposed copy of each element of the row-major copy, -1: padding): run
-// lengths, run starts (each block of the transposed copy begins at a multiple of 4 in T), places.
+// Set-up of a Move, from `from` (place in the transposed copy of each element of the row-major copy, -1: padding): run lengths, the
+// room of each block of the transposed copy in T (it begins at a multiple of 4), run starts, places.
 __global__ void move_count_kernel(const int* __restrict__ from, int r_elems, int block, int nb, int* __restrict__ count) {
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < r_elems; e += gridDim.x * blockDim.x)
         if (from[e] >= 0) atomicAdd(count + (from[e] / block) * nb + e / block, 1);
 }
-__global__ void __launch_bounds__(1024) move_starts_kernel(int* __restrict__ count, int nb, int* __restrict__ start, int2* __restrict__ runs) {
-    __shared__ int first[1025];
-    const int cb = threadIdx.x;                                                         // nb <= 1024
-    int total = 0;
-    if (cb < nb) for (int rb = 0; rb < nb; ++rb) total += count[cb * nb + rb];
-    if (cb < nb) first[cb + 1] = (total + 3) / 4 * 4;
+constexpr int MOVE_SCAN = 256;
+// sum over the CTA of v, in every thread; the CTA's threads all call it
+__device__ __forceinline__ int move_sum(int v) {
+    __shared__ int part[MOVE_SCAN / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     __syncthreads();
-    if (cb == 0) { first[0] = 0; for (int q = 1; q <= nb; ++q) first[q] += first[q - 1]; }
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (cb >= nb) return;
-    int at = first[cb];
-    for (int rb = 0; rb < nb; ++rb) {
-        const int c = count[cb * nb + rb];
-        start[cb * (nb + 1) + rb] = at; runs[(size_t)rb * nb + cb] = make_int2(at, c);
-        count[cb * nb + rb] = at;                                                       // from here on: cursor of the run
-        at += c;
+    int sum = 0;
+#pragma unroll
+    for (int q = 0; q < MOVE_SCAN / 32; ++q) sum += part[q];
+    return sum;
+}
+__global__ void __launch_bounds__(MOVE_SCAN) move_room_kernel(const int* __restrict__ count, int nb, int* __restrict__ room) {
+    int c = 0;
+    for (int rb = threadIdx.x; rb < nb; rb += MOVE_SCAN) c += count[blockIdx.x * nb + rb];
+    c = move_sum(c);
+    if (threadIdx.x == 0) room[blockIdx.x] = (c + 3) / 4 * 4;
+}
+// a CTA per block of the transposed copy; count: from here on the cursor of each run
+__global__ void __launch_bounds__(MOVE_SCAN) move_starts_kernel(int* __restrict__ count, const int* __restrict__ room, int nb, int* __restrict__ start,
+                                                                int2* __restrict__ runs) {
+    __shared__ int warp_sum[MOVE_SCAN / 32];
+    const int cb = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int at = 0;
+    for (int q = threadIdx.x; q < cb; q += MOVE_SCAN) at += room[q];
+    at = move_sum(at);
+    for (int rb0 = 0; rb0 < nb; rb0 += MOVE_SCAN) {
+        const int rb = rb0 + threadIdx.x, c = rb < nb ? count[cb * nb + rb] : 0;
+        int upto = c;                                                                   // inclusive prefix within the warp
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, upto, o); if (lane >= o) upto += v; }
+        __syncthreads();
+        if (lane == 31) warp_sum[warp] = upto;
+        __syncthreads();
+        int before = at, all = 0;
+#pragma unroll
+        for (int q = 0; q < MOVE_SCAN / 32; ++q) { before += q < warp ? warp_sum[q] : 0; all += warp_sum[q]; }
+        if (rb < nb) {
+            const int first = before + upto - c;
+            start[cb * (nb + 1) + rb] = first; runs[(size_t)rb * nb + cb] = make_int2(first, c);
+            count[cb * nb + rb] = first;
+        }
+        at += all;
     }
-    start[cb * (nb + 1) + nb] = at;
+    if (threadIdx.x == 0) start[cb * (nb + 1) + nb] = at;
 }
 __global__ void move_places_kernel(const int* __restrict__ from, int r_elems, int block, int nb, int* __restrict__ cursor,
                                    unsigned short* __restrict__ pos_a, unsigned short* __restrict__ pos_b) {

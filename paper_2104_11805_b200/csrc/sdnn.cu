@@ -132,7 +132,6 @@ struct sdnn {
     cudaEvent_t ev_side_join[MAX_SIDE] = {};
     int n_side = 0;
     float* d_move[MAX_SIDE] = {};       // T of split_values_kernel / merge_values_kernel
-    size_t move_elems[MAX_SIDE] = {};
     cudaStream_t launch_stream = nullptr;     // where launch_k currently enqueues (NULL = stream)
     std::vector<cudaEvent_t> ev_delta;  // [L] delta^k (0-based layer) complete
     cudaEvent_t ev_fork = nullptr;
@@ -1436,42 +1435,73 @@ int upload_indices(sdnn* h, int* dst, const std::vector<int>& src) {      // syn
     return SDNN_OK;
 }
 
-// Fills the transposed copy's values and, where the row-major copy is to be updated from them (see Move), lays down the
-// maps for that.  Blocks of 2^k elements (256 .. 8192: at most 32 KB of shared memory) so that a run has about 32 entries.
-// Not with the gradient kept for inspection, which the row units record; and not beyond 1024 blocks (8 M stored elements a
-// layer), where runs would get long tables: there the row units compute the update themselves.
-int build_move(sdnn* h, int layer) {
-    LayerMem& lm = h->lay[layer];
+// How the row-major copy of a layer is cut to be updated from the transposed one (see Move): blocks of 2^k elements (256 .. 8192: at
+// most 32 KB of shared memory) so that a run has about 32 entries.  nb = 0: row units compute the update themselves.  So it is
+// with the gradient kept for inspection, which the row units record, and beyond 1024 blocks (8 M stored elements a layer), where
+// runs would get long tables.
+struct MoveShape { int nb = 0, block = 256; size_t t_elems = 0; };
+MoveShape move_shape(const sdnn* h, int layer) {
+    const LayerMem& lm = h->lay[layer];
+    MoveShape m;
+    if (!h->split || layer == 0 || lm.r_grad || !moves(lm, h->ld_max)) return m;
     const int64_t most = std::max(lm.r_elems, lm.c_elems);
-    int block = 256;
-    while (block < 8192 && (int64_t)block * block < 24 * most) block *= 2;
-    const int nb = (int)((most + block - 1) / block);
-    if (!h->split || lm.r_grad || !moves(lm, h->ld_max) || nb < 1 || nb > 1024) return refresh_mirror(h, layer, nullptr);
+    while (m.block < 8192 && (int64_t)m.block * m.block < 24 * most) m.block *= 2;
+    const int64_t nb = (most + m.block - 1) / m.block;
+    if (nb < 1 || nb > 1024) return m;
+    m.nb = (int)nb;
+    m.t_elems = ((size_t)h->nnz[layer] + 4 * (size_t)nb + 7) / 8 * 8;
+    return m;
+}
+
+// Lays down the maps of all layers that have them, and with them fills those layers' transposed copies (called by sdnn_finalize).  One
+// piece of device memory for all maps and staging arrays, one scratch for all layers: allocated, and given back with a wait, layer by
+// layer, the scratch alone took 25 to 40 ms of the 150 that 24 layers of 16384 neurons take to set up; all of this takes 3.3.
+int build_moves(sdnn* h) {
+    std::vector<MoveShape> shape(h->L);
+    size_t bytes = 0, scratch_ints = 0, most = 0;
+    auto room = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    for (int k = 0; k < h->L; ++k) {
+        const MoveShape m = shape[k] = move_shape(h, k);
+        if (!m.nb) continue;
+        const size_t nb = (size_t)m.nb;
+        bytes += room(nb * (nb + 1) * sizeof(int)) + room(nb * nb * sizeof(int2)) + 2 * room(m.t_elems * sizeof(unsigned short));
+        scratch_ints = std::max(scratch_ints, (size_t)h->lay[k].r_elems + nb * nb + nb);
+        most = std::max(most, m.t_elems);
+    }
+    if (!most) return SDNN_OK;
+    bytes += h->n_side * room(most * sizeof(float));
+    char* at = nullptr;
     int rc;
-    int *from = nullptr, *start = nullptr;
-    int2* runs = nullptr;
-    unsigned short* pos[2] = {nullptr, nullptr};
-    const size_t t_elems = (size_t)h->nnz[layer] + 4 * (size_t)nb;
-    if ((rc = dev_alloc(h, &start, (size_t)nb * (nb + 1), false)) || (rc = dev_alloc(h, &runs, (size_t)nb * nb, false)) ||
-        (rc = dev_alloc(h, &pos[0], t_elems, true)) || (rc = dev_alloc(h, &pos[1], t_elems, true))) return rc;
-    for (int q = 0; q < h->n_side; ++q)
-        if (t_elems > h->move_elems[q]) {      // one T per side stream, grown to the largest layer
-            if ((rc = dev_alloc(h, &h->d_move[q], t_elems, false))) return rc;
-            h->move_elems[q] = t_elems;
-        }
-    CU(h, cudaMallocAsync((void**)&from, (size_t)(lm.r_elems + (int64_t)nb * nb) * sizeof(int), h->stream));
-    int* count = from + lm.r_elems;
-    CU(h, cudaMemsetAsync(from, 0xff, (size_t)lm.r_elems * sizeof(int), h->stream));
-    CU(h, cudaMemsetAsync(count, 0, (size_t)nb * nb * sizeof(int), h->stream));
-    if ((rc = refresh_mirror(h, layer, nullptr, from))) return rc;
-    const int grid = (int)std::min<int64_t>((lm.r_elems + 255) / 256, 8 * (int64_t)h->sms);
-    move_count_kernel<<<grid, 256, 0, h->stream>>>(from, (int)lm.r_elems, block, nb, count);
-    move_starts_kernel<<<1, 1024, 0, h->stream>>>(count, nb, start, runs);
-    move_places_kernel<<<grid, 256, 0, h->stream>>>(from, (int)lm.r_elems, block, nb, count, pos[0], pos[1]);
-    CU(h, cudaFreeAsync(from, h->stream));
-    CU(h, cudaGetLastError());
-    lm.move = Move{start, runs, pos[0], pos[1], nb, block};
-    return SDNN_OK;
+    if ((rc = dev_alloc(h, &at, bytes, true))) return rc;
+    auto take = [&](size_t b) { char* p = at; at += room(b); return p; };
+    int* scratch = nullptr;
+    CU(h, cudaMalloc((void**)&scratch, scratch_ints * sizeof(int)));
+    for (int q = 0; q < h->n_side; ++q) h->d_move[q] = reinterpret_cast<float*>(take(most * sizeof(float)));
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < h->L && !rc && e == cudaSuccess; ++k) {
+        const MoveShape& m = shape[k];
+        if (!m.nb) continue;
+        LayerMem& lm = h->lay[k];
+        const size_t nb = (size_t)m.nb;
+        int* start = reinterpret_cast<int*>(take(nb * (nb + 1) * sizeof(int)));
+        int2* runs = reinterpret_cast<int2*>(take(nb * nb * sizeof(int2)));
+        unsigned short* pos[2];
+        for (unsigned short*& p : pos) p = reinterpret_cast<unsigned short*>(take(m.t_elems * sizeof(unsigned short)));
+        int *from = scratch, *count = from + lm.r_elems, *per_block = count + nb * nb;
+        cudaMemsetAsync(from, 0xff, (size_t)lm.r_elems * sizeof(int), h->stream);
+        cudaMemsetAsync(count, 0, nb * nb * sizeof(int), h->stream);
+        rc = refresh_mirror(h, k, nullptr, from);
+        const int grid = (int)std::min<int64_t>((lm.r_elems + 255) / 256, 8 * (int64_t)h->sms);
+        move_count_kernel<<<grid, 256, 0, h->stream>>>(from, (int)lm.r_elems, m.block, m.nb, count);
+        move_room_kernel<<<m.nb, MOVE_SCAN, 0, h->stream>>>(count, m.nb, per_block);
+        move_starts_kernel<<<m.nb, MOVE_SCAN, 0, h->stream>>>(count, per_block, m.nb, start, runs);
+        move_places_kernel<<<grid, 256, 0, h->stream>>>(from, (int)lm.r_elems, m.block, m.nb, count, pos[0], pos[1]);
+        e = cudaGetLastError();
+        lm.move = Move{start, runs, pos[0], pos[1], m.nb, m.block};
+    }
+    cudaFree(scratch);      // waits for its last reader
+    if (e != cudaSuccess) return cuda_fail(h, e, "set-up of the move maps");
+    return rc;
 }
 
 // Lays out one validated layer (caller's or reordered CSR, host arrays) in the kernels' sliced format and uploads it.
@@ -1594,7 +1624,7 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
         CU(h, cudaMemcpyAsync(h->d_c_len + (size_t)layer * N, c_len.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         CU(h, cudaMemcpyAsync(h->d_c_order + (size_t)layer * N, order.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         if (lm.c_elems && (rc = upload_indices(h, lm.c_idx, c_idx))) return rc;
-        if ((rc = build_move(h, layer))) return rc;      // fills the transposed copy's values too
+        if (!move_shape(h, layer).nb && (rc = refresh_mirror(h, layer, nullptr))) return rc;      // else with its maps, in sdnn_finalize
     }
     CU(h, cudaStreamSynchronize(h->stream));   // the host vectors above go out of scope; the caller may reuse its arrays
     {
@@ -2027,8 +2057,8 @@ int sdnn_finalize(sdnn_t* h) {
         if (rc) return rc;
     }
     {
-        int rc = build_vector(h);
-        if (rc) return rc;
+        int rc;
+        if ((rc = build_moves(h)) || (rc = build_vector(h))) return rc;
     }
     int64_t elems = 0;
     for (const LayerMem& lm : h->lay) elems += lm.windowed ? lm.w_elems : lm.r_elems;

@@ -26,10 +26,10 @@ def test_ragged_rows_stored_by_length(torch_cuda, n, B):  # noqa: F811
     infer_parity(torch_cuda, arrays, vectors(rng, 3 * B, n), 2 * B, expect_nonempty=True)
 
 
-@pytest.mark.parametrize("n,k,B", [(4097, 48, 100), (1500, 300, 33), (8200, 32, 33)])
+@pytest.mark.parametrize("n,k,B", [(4097, 48, 100), (1500, 300, 33), (8200, 32, 33), (16400, 140, 33)])
 def test_row_major_copy_moved_from_the_transposed_one(torch_cuda, n, k, B):  # noqa: F811
-    """Layers large enough to have their row-major copy filled from the transposed one after an update (blocks of 2048 to 4096
-    elements, the last one partial, ragged rows and columns), two steps of one handle at the full batch and one at a batch
+    """Layers large enough to have their row-major copy filled from the transposed one after an update (blocks of 2048 to
+    8192 elements, up to 300 of them, the last one partial, ragged rows and columns), two steps of one handle at the full batch and one at a batch
     narrow enough for row units, against the oracle; both copies hold the same bits."""
     torch, pkg = torch_cuda, sdnn()
     rng = np.random.default_rng(n)
