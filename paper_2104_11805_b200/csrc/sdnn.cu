@@ -237,10 +237,16 @@ int dev_alloc(sdnn* h, T** out, size_t count, bool zero) {
     const size_t padded = (bytes + 255) & ~(size_t)255;
     if (padded <= ((size_t)8 << 20)) {
         if (padded > h->block_left) {
-            const size_t want = std::max(padded, h->block_next);
-            cudaError_t e = cudaMalloc((void**)&h->block, want);
-            if (e != cudaSuccess) { cudaGetLastError(); h->block_left = 0; return cuda_fail(h, e, "cudaMalloc"); }
-            h->allocs.push_back(h->block);
+            size_t want = std::max(padded, h->block_next);
+            cudaError_t e = cudaMalloc(&p, want);
+            while (e == cudaErrorMemoryAllocation && want > padded) {      // little is left: a smaller block may still fit
+                cudaGetLastError();
+                want = std::max(padded, want / 2);
+                e = cudaMalloc(&p, want);
+            }
+            if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(h, e, "cudaMalloc"); }
+            h->block = static_cast<char*>(p);
+            h->allocs.push_back(p);
             h->dev_bytes += (int64_t)want;
             h->block_left = want;
             h->block_next = std::min(2 * want, (size_t)64 << 20);

@@ -59,6 +59,46 @@ def test_row_major_copy_moved_from_the_transposed_one(torch_cuda, n, k, B):  # n
     h.destroy()
 
 
+def uniform_net(rng, n, k, layers):
+    """Layers of k entries per row anywhere, made quickly."""
+    cols = [(np.sort(rng.integers(0, n - k + 1, size=(n, k)), axis=1) + np.arange(k)).astype(np.int32).ravel() for _ in range(layers)]
+    vals = [rng.uniform(-1, 1, size=n * k).astype(np.float32) for _ in range(layers)]
+    return [np.arange(n + 1, dtype=np.int32) * k] * layers, cols, vals, [np.zeros(n, dtype=np.float32)] * layers
+
+
+@pytest.fixture
+def all_but(torch_cuda):  # noqa: F811
+    """all_but(bytes): takes the device's free memory but for so many bytes until the test is over."""
+    torch, held = torch_cuda, []
+
+    def take(room):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        held.append(torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda"))
+    yield take
+    held.clear()
+    torch.cuda.empty_cache()
+
+
+def test_small_arrays_take_what_is_left(torch_cuda, all_but):  # noqa: F811
+    """Small arrays are cut from blocks that double: with less left than the next block, a handle that fits is made all the same."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(0)
+    arrays = uniform_net(rng, 4096, 32, 80)                       # 0.79 MB a layer: blocks of 2, 4, .. 32 MB, then 64 MB for the last few layers
+    x = torch.from_numpy(vectors(rng, 8, 4096)).cuda()
+    outs, taken = [torch.zeros(8, 4096, device="cuda") for _ in range(2)], []
+    for y in outs:
+        if taken:
+            all_but(72 << 20)
+        h = pkg.Sdnn.create(*arrays, max_batch=8, activation=pkg.ACT_SIGMOID)
+        h.infer_batch(x, 8, y)
+        torch.cuda.synchronize()
+        taken.append(h.device_bytes())
+        h.destroy()
+    assert taken[1] <= 72 << 20 < taken[0]
+    assert torch.equal(outs[0], outs[1])
+
+
 @pytest.mark.parametrize("n,k,layers", [(9, 3, 2), (64, 5, 3), (1000, 32, 4), (1024, 33, 9), (1025, 32, 5), (2047, 8, 12), (4096, 16, 3)])
 @pytest.mark.parametrize("cnt", [1, 2, 3])
 @pytest.mark.parametrize("act", ["clamped_relu", "sigmoid"])
