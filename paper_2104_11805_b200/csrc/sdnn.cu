@@ -1476,12 +1476,28 @@ int build_moves(sdnn* h) {
     }
     if (!most) return SDNN_OK;
     bytes += h->n_side * room(most * sizeof(float));
-    char* at = nullptr;
-    int rc;
-    if ((rc = dev_alloc(h, &at, bytes, true))) return rc;
-    auto take = [&](size_t b) { char* p = at; at += room(b); return p; };
+    // The maps save time, they are not needed: where they would take what later calls allocate (staging of host batches, a second
+    // inference lane, the means of the averaged step, values in the caller's order, graphs), or do not fit at all, row units update
+    // the row-major copies.
+    const size_t tile = (size_t)h->N * h->ld_max * sizeof(float);
+    const size_t later = 4 * tile + (size_t)(h->L + 1) * h->N * 4 * sizeof(float) + (size_t)*std::max_element(h->nnz.begin(), h->nnz.end()) * sizeof(float) + ((size_t)64 << 20);
+    size_t left = 0, whole = 0;
     int* scratch = nullptr;
-    CU(h, cudaMalloc((void**)&scratch, scratch_ints * sizeof(int)));
+    char* at = nullptr;
+    int rc = SDNN_OK;
+    CU(h, cudaMemGetInfo(&left, &whole));
+    bool fits = bytes + scratch_ints * sizeof(int) + later <= left && cudaMalloc((void**)&scratch, scratch_ints * sizeof(int)) == cudaSuccess;
+    if (fits && (rc = dev_alloc(h, &at, bytes, true)) != SDNN_OK) {
+        cudaFree(scratch);
+        if (rc != SDNN_ERR_OOM) return rc;
+        fits = false;
+    }
+    if (!fits) {
+        cudaGetLastError();
+        for (int k = 0; k < h->L; ++k) if (shape[k].nb && (rc = refresh_mirror(h, k, nullptr))) return rc;
+        return SDNN_OK;
+    }
+    auto take = [&](size_t b) { char* p = at; at += room(b); return p; };
     for (int q = 0; q < h->n_side; ++q) h->d_move[q] = reinterpret_cast<float*>(take(most * sizeof(float)));
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < h->L && !rc && e == cudaSuccess; ++k) {

@@ -99,6 +99,29 @@ def test_small_arrays_take_what_is_left(torch_cuda, all_but):  # noqa: F811
     assert torch.equal(outs[0], outs[1])
 
 
+def test_a_training_net_that_just_fits_does_without_the_move_maps(torch_cuda, all_but):  # noqa: F811
+    """With room for the net but not for the maps that move its row-major values (60 MB here), row units update them: the same
+    launches as for a narrow batch, and the same bits."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(1)
+    n, layers, B = 16384, 24, 64
+    arrays = uniform_net(rng, n, 32, layers)
+    x, y = (torch.from_numpy(vectors(rng, B, n)).cuda() for _ in range(2))
+    taken, launches, weights = [], [], []
+    for _ in range(2):
+        if taken:
+            all_but(taken[0] - (30 << 20))
+        h = pkg.Sdnn.create(*arrays, max_batch=B, train=True, activation=pkg.ACT_SIGMOID)
+        taken.append(h.device_bytes())
+        h.train_step(x, y, B, 0.5)
+        launches.append(h.kernel_launches())
+        weights.append([h.get_weights(l, want_bias=False) for l in range(layers)])
+        assert h.mirror_mismatches(layers - 1) == 0
+        h.destroy()
+    assert taken[1] <= taken[0] - (50 << 20) and launches[1] == launches[0] - (layers - 1)
+    assert all(np.array_equal(a, b) for a, b in zip(*weights))
+
+
 @pytest.mark.parametrize("n,k,layers", [(9, 3, 2), (64, 5, 3), (1000, 32, 4), (1024, 33, 9), (1025, 32, 5), (2047, 8, 12), (4096, 16, 3)])
 @pytest.mark.parametrize("cnt", [1, 2, 3])
 @pytest.mark.parametrize("act", ["clamped_relu", "sigmoid"])
