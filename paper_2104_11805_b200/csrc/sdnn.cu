@@ -192,7 +192,7 @@ struct sdnn {
     int64_t stage_idx_cap = 0;
 
     std::map<std::tuple<const void*, int, int>, std::pair<int, int>> plans;   // (kernel, units, chunks) -> (grid.x, block)
-    std::map<const void*, bool> carved;                                       // kernels given the shared-memory split of the move kernels
+    std::map<const void*, bool> configured;                                   // kernels given what a launch of theirs needs (launch_vector)
     std::map<std::pair<const void*, int>, int> occupancy;                     // (kernel, block) -> resident CTAs per SM
 
     int64_t launches = 0;
@@ -479,25 +479,31 @@ Sliced cols_of(sdnn* h, int layer) {
     return m;
 }
 
-// Gives a kernel that runs beside the move kernels their split of an SM's memory between L1 and shared memory: an SM changes
-// the split only when it is empty, so that kernels with different ones take turns instead of running side by side (65536
-// neurons, 64 inputs: backward 60 us per layer without this, 52 with it; the gathers do not miss the L1).
+// A launch on the stream the handle works for.  beside_moves: the launch runs beside the move kernels and asks for their split of
+// an SM's memory between L1 and shared memory: an SM changes the split only when it is empty, so that kernels with different ones
+// take turns instead of running side by side (65536 neurons, 64 inputs: backward 60 us per layer without this, 52 with it; the
+// gathers do not miss the L1).  Asked for launch by launch: the kernel's own preference is one for the whole process, and
+// would take L1 away from every other handle's launches of it.
 constexpr int MOVE_SMEM_KB = 100;
-void carve(sdnn* h, const void* kernel) {
-    if (h->carved[kernel]) return;
-    h->carved[kernel] = true;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, MOVE_SMEM_KB * 100 / 228) != cudaSuccess) cudaGetLastError();
+template <typename... KArgs, typename... Args>
+cudaError_t launch_on(sdnn* h, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, bool pdl, bool beside_moves, Args... args) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid; lc.blockDim = block; lc.dynamicSmemBytes = smem; lc.stream = h->launch_stream ? h->launch_stream : h->stream;
+    cudaLaunchAttribute at[2];
+    lc.attrs = at;
+    if (pdl) {
+        at[lc.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[lc.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (beside_moves) {
+        at[lc.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[lc.numAttrs++].val.sharedMemCarveout = MOVE_SMEM_KB * 100 / 228;
+    }
+    return cudaLaunchKernelEx(&lc, kernel, KArgs(args)...);
 }
-
 template <typename... KArgs, typename... Args>
 cudaError_t launch_k(sdnn* h, void (*kernel)(KArgs...), dim3 grid, dim3 block, bool pdl, Args... args) {
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = grid; lc.blockDim = block; lc.dynamicSmemBytes = 0; lc.stream = h->launch_stream ? h->launch_stream : h->stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at; lc.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, kernel, KArgs(args)...);
+    return launch_on(h, kernel, grid, block, 0, pdl, false, args...);
 }
 
 template <bool I16, int G, int V, int CPS = 2>
@@ -676,6 +682,7 @@ void launch_forward_window(sdnn* h, int layer, const float* xin, float* xout, in
 constexpr int MOVE_WIDTH = 32;
 constexpr int64_t MOVE_WORK = 8 << 20;      // stored elements x padded batch
 bool moves(const LayerMem& lm, int ld) { return ld >= MOVE_WIDTH && lm.r_elems * ld >= MOVE_WORK; }
+bool moved(const LayerMem& lm, int ld) { return lm.move.nb > 0 && moves(lm, ld); }
 
 // delta tile of layer `layer` (0-based; the paper's delta^{layer+1}) in the transposed realisation
 float* delta_tile(sdnn* h, int layer, size_t tile) {
@@ -712,6 +719,7 @@ void launch_backward_gvc(sdnn* h, int layer, int ld, int part) {
     // and 9 % (config 3) faster than two persistent grids sharing the SMs.  Alone on the device (forward, one launch per
     // layer) the persistent grid is the faster one.
     const int os_ = (h->split && part != 0) ? 1 : 0;
+    const bool beside = part != 0 && moved(h->lay[layer], ld);
 #define SDNN_BWD(FROM_S, SCAT, MIR)                                                            \
     do {                                                                                       \
         if (a.dbg_grad) {                                                                      \
@@ -721,8 +729,7 @@ void launch_backward_gvc(sdnn* h, int layer, int ld, int part) {
         } else {                                                                               \
             auto plan = plan_grid(h, (const void*)backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>, units, 1, os_);  \
             if (a.pdl && (plan.first <= h->sms || MIR)) a.pdl = PDL_EARLY;                     \
-            if (part != 0 && h->lay[layer].move.nb > 0) carve(h, (const void*)backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>); \
-            launch_k(h, backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>, dim3(plan.first), dim3(plan.second), a.pdl != 0, a); \
+            launch_on(h, backward_kernel<G, V, CPS, I16, FROM_S, SCAT, MIR, false>, dim3(plan.first), dim3(plan.second), 0, a.pdl != 0, beside, a); \
         }                                                                                      \
     } while (0)
     if (h->mirror) {
@@ -731,7 +738,7 @@ void launch_backward_gvc(sdnn* h, int layer, int ld, int part) {
             a.cols = cols_of(h, layer);
             a.dprev = delta_tile(h, layer - 1, tile);
             a.cols_only = part == 1 ? 1 : 0;
-            a.alternate = a.cols_only && h->lay[layer].move.nb > 0 && moves(h->lay[layer], ld) ? 1 : 0;
+            a.alternate = a.cols_only && moved(h->lay[layer], ld) ? 1 : 0;
             SDNN_BWD(false, false, true);
         } else if (part != 1) {
             if (part == 2) { a.pdl = 0; a.warm = nullptr; }
@@ -803,10 +810,8 @@ void launch_move(sdnn* h, int layer, int ld, int side) {
     const LayerMem& lm = h->lay[layer];
     const Move& m = lm.move;
     const size_t smem = (size_t)m.block * sizeof(float);
-    carve(h, (const void*)split_values_kernel);
-    carve(h, (const void*)merge_values_kernel);
-    split_values_kernel<<<m.nb, MOVE_THREADS, smem, h->launch_stream>>>(m, (const float*)lm.c_val, (int)lm.c_elems, h->d_move[side]);
-    merge_values_kernel<<<m.nb, MOVE_THREADS, smem + (size_t)m.nb * sizeof(int2), h->launch_stream>>>(m, (const float*)h->d_move[side], lm.r_val, (int)lm.r_elems);
+    launch_on(h, split_values_kernel, dim3(m.nb), dim3(MOVE_THREADS), smem, false, true, m, (const float*)lm.c_val, (int)lm.c_elems, h->d_move[side]);
+    launch_on(h, merge_values_kernel, dim3(m.nb), dim3(MOVE_THREADS), smem + (size_t)m.nb * sizeof(int2), false, true, m, (const float*)h->d_move[side], lm.r_val, (int)lm.r_elems);
     count_launch(h, 2);
     if (h->cfg.update_bias) {
         update_bias_kernel<<<(h->N + 255) / 256, 256, 0, h->launch_stream>>>(h->d_bias + (size_t)layer * h->N, (const float*)delta_tile(h, layer, (size_t)h->N * ld),
@@ -849,7 +854,7 @@ void enqueue_backward_chain(sdnn* h, int ld) {
         cudaEventRecord(h->ev_delta[h->L - 1], h->stream);
         for (int k = h->L - 1; k >= 0; --k) {
             NvtxRange pass("backward layer", k + 1);
-            const bool move = h->lay[k].move.nb > 0 && moves(h->lay[k], ld);
+            const bool move = moved(h->lay[k], ld);
             const int q = k % (move ? h->n_side : sdnn::ROW_SIDE);
             if (k > 0) {
                 launch_backward(h, k, ld, 1);
@@ -954,10 +959,10 @@ int launch_vector(sdnn* h, VectorArgs a) {
     const size_t base = vector_smem(h, V, &stage), smem = base + vector_stages(h, V) * stage;
     a.stages = vector_stages(h, V);
     const void* kernel = (const void*)vector_infer_kernel<V>;
-    if (!h->carved[kernel]) {
+    if (!h->configured[kernel]) {
         CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VECTOR_SMEM));
         CU(h, cudaFuncSetAttribute(vector_infer_kernel<V>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        h->carved[kernel] = true;
+        h->configured[kernel] = true;
     }
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(VECTOR_CTAS); lc.blockDim = dim3(VECTOR_THREADS); lc.dynamicSmemBytes = smem; lc.stream = h->stream;

@@ -94,6 +94,13 @@ def test_graphs_gather_no_more_padding_than_they_have_to(plan):
         assert graphs_made(plan, tiles)[0] == early <= 4 + 2 * shapes
 
 
+def test_no_kernel_is_given_a_memory_split_for_the_whole_process():
+    """The split between L1 and shared memory is asked for launch by launch: set on a kernel it would hold for every handle."""
+    for name in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, name)) as f:
+            assert "cudaFuncAttributePreferredSharedMemoryCarveout" not in f.read(), name
+
+
 class Fault(Exception):
     pass
 
