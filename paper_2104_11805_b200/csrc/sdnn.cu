@@ -185,9 +185,8 @@ struct sdnn {
     int* d_stage_cnt = nullptr;
     int* d_stage_cnt2 = nullptr;
     float* d_stage_w = nullptr;         // one layer's values in the caller's order (sdnn_get/set_weights)
-    static constexpr int PINS = 4;      // pinned pieces that results for pageable memory travel through
-    char* pin[PINS] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t ev_pin[PINS] = {nullptr, nullptr, nullptr, nullptr};
+    bool uses_pins = false;             // has a share in pin_pool()
+    cudaEvent_t ev_pin[4] = {};         // [PinPool::PIECES]
     int* d_stage_idx = nullptr;
     int64_t stage_idx_cap = 0;
 
@@ -1354,49 +1353,84 @@ void sliced_to_csr(const sdnn* h, const LayerMem& lm, const std::vector<float>& 
     }
 }
 
+// Pinned pieces that results for pageable memory travel through, the same for all handles: pinning four of its own took every
+// handle's first sdnn_get_weights 3 to 13 ms.  Made when a copy first needs them, given back when the last handle goes that used
+// them.  A copy has the pieces to itself; one that finds them taken does without and does not wait for another handle's stream.
+struct PinPool {
+    static constexpr int PIECES = 4;
+    static constexpr size_t BYTES = 1 << 20;      // of a piece
+    std::mutex busy, mutex;
+    char* piece[PIECES] = {};
+    int users = 0;
+    bool make(int pieces) {                       // with `busy` held; for the handles of every device
+        for (int q = 0; q < pieces; ++q)
+            if (!piece[q] && cudaHostAlloc((void**)&piece[q], BYTES, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); piece[q] = nullptr; return false; }
+        return true;
+    }
+    void join() { std::lock_guard<std::mutex> lock(mutex); ++users; }
+    void leave() {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (--users) return;                      // no user left: nobody holds `busy`
+        for (char*& p : piece) if (p) { cudaFreeHost(p); p = nullptr; }
+    }
+};
+PinPool& pin_pool() { static PinPool pool; return pool; }
+
+// The pieces for a copy of the handle's: owns them while it lives, or owns nothing (taken, or no pinned memory to be had).
+struct Pins {
+    std::unique_lock<std::mutex> lock;
+    Pins(sdnn* h, int pieces) : lock(pin_pool().busy, std::defer_lock) {
+        for (cudaEvent_t& ev : h->ev_pin)
+            if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); ev = nullptr; return; }
+        if (!h->uses_pins) { pin_pool().join(); h->uses_pins = true; }
+        if (lock.try_lock() && !pin_pool().make(pieces)) lock.unlock();
+    }
+    bool owned() const { return lock.owns_lock(); }
+};
+
 // Device memory -> the caller's host memory, behind what the handle's stream has been given; returns when it is there.
 // Pinned memory takes one copy.  Pageable memory (a fresh numpy array) goes through four pinned pieces of 1 MB: the copy
 // engine fills some while the host cores empty the others, so that the page faults of a fresh array are taken by several
 // cores and under the transfer (sdnn_get_weights of 2 M entries, 8 MB: 3.7 -> 0.7 ms; of 0.5 M entries: 0.7 -> 0.13 ms).
-constexpr size_t PIN_BYTES = 1 << 20;
-int ensure_pin(sdnn* h, int q) {
-    if (h->pin[q]) return SDNN_OK;
-    CU(h, cudaMallocHost((void**)&h->pin[q], PIN_BYTES));
-    CU(h, cudaEventCreateWithFlags(&h->ev_pin[q], cudaEventDisableTiming));
-    return SDNN_OK;
-}
 int copy_to_caller(sdnn* h, void* dst, const void* src, size_t bytes) {
     cudaPointerAttributes at{};
     const bool pageable = cudaPointerGetAttributes(&at, dst) != cudaSuccess || at.type == cudaMemoryTypeUnregistered;
-    if (!pageable) {
+    cudaGetLastError();
+    auto whole = [&]() -> int {
         CU(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, h->stream));
         CU(h, cudaStreamSynchronize(h->stream));
         return SDNN_OK;
-    }
-    cudaGetLastError();
-    const int64_t pieces = (int64_t)((bytes + PIN_BYTES - 1) / PIN_BYTES);
+    };
+    if (!pageable) return whole();
+    constexpr int PIECES = PinPool::PIECES;
+    constexpr size_t PIECE = PinPool::BYTES;
+    const int64_t pieces = (int64_t)((bytes + PIECE - 1) / PIECE);
+    const Pins pins(h, (int)std::min<int64_t>(pieces, PIECES));
+    if (!pins.owned()) return whole();
+    char* const* piece = pin_pool().piece;
     auto issue = [&](int64_t p) -> int {
-        const int q = (int)(p % sdnn::PINS);
-        if (const int rc_pin = ensure_pin(h, q)) return rc_pin;
-        const size_t lo = (size_t)p * PIN_BYTES;
-        CU(h, cudaMemcpyAsync(h->pin[q], static_cast<const char*>(src) + lo, std::min(PIN_BYTES, bytes - lo), cudaMemcpyDeviceToHost, h->stream));
+        const int q = (int)(p % PIECES);
+        const size_t lo = (size_t)p * PIECE;
+        CU(h, cudaMemcpyAsync(piece[q], static_cast<const char*>(src) + lo, std::min(PIECE, bytes - lo), cudaMemcpyDeviceToHost, h->stream));
         CU(h, cudaEventRecord(h->ev_pin[q], h->stream));
         return SDNN_OK;
     };
-    int rc;
-    for (int64_t p = 0; p < std::min<int64_t>(pieces, sdnn::PINS); ++p) if ((rc = issue(p))) return rc;
-    for (int64_t p = 0; p < pieces; ++p) {
-        const int q = (int)(p % sdnn::PINS);
-        CU(h, cudaEventSynchronize(h->ev_pin[q]));
-        const size_t lo = (size_t)p * PIN_BYTES, len = std::min(PIN_BYTES, bytes - lo);
+    int rc = SDNN_OK;
+    for (int64_t p = 0; p < std::min<int64_t>(pieces, PIECES) && !rc; ++p) rc = issue(p);
+    for (int64_t p = 0; p < pieces && !rc; ++p) {
+        const int q = (int)(p % PIECES);
+        const cudaError_t e = cudaEventSynchronize(h->ev_pin[q]);
+        if (e != cudaSuccess) { rc = cuda_fail(h, e, "cudaEventSynchronize"); break; }
+        const size_t lo = (size_t)p * PIECE, len = std::min(PIECE, bytes - lo);
         constexpr size_t GRAIN = 128 << 10;
         const int parts = (int)((len + GRAIN - 1) / GRAIN);
 #pragma omp parallel for schedule(static, 1) num_threads(parts) if (parts > 1)
         for (int k = 0; k < parts; ++k)
-            memcpy(static_cast<char*>(dst) + lo + k * GRAIN, h->pin[q] + k * GRAIN, std::min(GRAIN, len - k * GRAIN));
-        if (p + sdnn::PINS < pieces && (rc = issue(p + sdnn::PINS))) return rc;
+            memcpy(static_cast<char*>(dst) + lo + k * GRAIN, piece[q] + k * GRAIN, std::min(GRAIN, len - k * GRAIN));
+        if (p + PIECES < pieces) rc = issue(p + PIECES);
     }
-    return SDNN_OK;
+    if (rc) cudaStreamSynchronize(h->stream);      // the pieces go to another handle: nothing may still be on its way to them
+    return rc;
 }
 
 int ensure_stage_w(sdnn* h) {
@@ -1941,10 +1975,8 @@ void sdnn_destroy(sdnn_t* h) {
     for (cudaEvent_t e : h->ev_copied) if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev_consumed) if (e) cudaEventDestroy(e);
     if (h->copy_stream) { cudaStreamSynchronize(h->copy_stream); cudaStreamDestroy(h->copy_stream); }
-    for (int q = 0; q < sdnn::PINS; ++q) {
-        if (h->ev_pin[q]) cudaEventDestroy(h->ev_pin[q]);
-        if (h->pin[q]) cudaFreeHost(h->pin[q]);
-    }
+    for (cudaEvent_t e : h->ev_pin) if (e) cudaEventDestroy(e);
+    if (h->uses_pins) pin_pool().leave();
     if (h->vector_status) status_page().put(h->vector_status);
     for (void* p : h->allocs) cudaFree(p);
     if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -2262,11 +2294,17 @@ int sdnn_get_weights(sdnn_t* h, int32_t layer, float* values_out, float* bias_ou
     if (values_out && nnz && lm.entry_src.empty()) {
         int rc;
         const size_t bytes = (size_t)nnz * sizeof(float);
-        if (bytes <= PIN_BYTES / 4) {      // a small layer: the kernel writes to pinned memory itself, one launch and one wait
-            if ((rc = ensure_pin(h, 0)) || (rc = convert_values<true>(h, layer, reinterpret_cast<float*>(h->pin[0])))) return rc;
-            CU(h, cudaStreamSynchronize(h->stream));
-            memcpy(values_out, h->pin[0], bytes);
-        } else if ((rc = ensure_stage_w(h)) || (rc = convert_values<true>(h, layer, h->d_stage_w)) || (rc = copy_to_caller(h, values_out, h->d_stage_w, bytes))) return rc;
+        bool done = false;
+        if (bytes <= PinPool::BYTES / 4) {      // a small layer: the kernel writes to pinned memory itself, one launch and one wait
+            const Pins pins(h, 1);
+            if (pins.owned()) {
+                if ((rc = convert_values<true>(h, layer, reinterpret_cast<float*>(pin_pool().piece[0])))) return rc;
+                CU(h, cudaStreamSynchronize(h->stream));
+                memcpy(values_out, pin_pool().piece[0], bytes);
+                done = true;
+            }
+        }
+        if (!done && ((rc = ensure_stage_w(h)) || (rc = convert_values<true>(h, layer, h->d_stage_w)) || (rc = copy_to_caller(h, values_out, h->d_stage_w, bytes)))) return rc;
     } else if (values_out && nnz) {      // entries in another order than the caller's (SDNN_FLAG_REORDER)
         CU(h, cudaStreamSynchronize(h->stream));
         std::vector<float> stored((size_t)nnz);

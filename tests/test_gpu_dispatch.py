@@ -122,6 +122,29 @@ def test_a_training_net_that_just_fits_does_without_the_move_maps(torch_cuda, al
     assert all(np.array_equal(a, b) for a, b in zip(*weights))
 
 
+def test_weights_of_several_handles_read_from_several_threads(torch_cuda):  # noqa: F811
+    """Handles share the pinned pieces that weights travel through: small layers, layers of several pieces and biases, read by a thread
+    per handle, while handles come and go."""
+    from concurrent.futures import ThreadPoolExecutor
+    pkg = sdnn()
+
+    def one(seed):
+        rng = np.random.default_rng(seed)
+        n, k = ((700, 16), (9000, 100), (30000, 61), (4096, 32))[seed % 4]
+        rp, cols, vals, _ = uniform_net(rng, n, k, 2)
+        bias = [rng.standard_normal(n).astype(np.float32) for _ in range(2)]
+        for _ in range(3):
+            h = pkg.Sdnn.create(rp, cols, vals, bias, max_batch=4)
+            for _ in range(4):
+                for l in range(2):
+                    w, b = h.get_weights(l)
+                    assert np.array_equal(w, vals[l]) and np.array_equal(b, bias[l])
+            h.destroy()
+        return True
+    with ThreadPoolExecutor(4) as pool:
+        assert all(pool.map(one, range(8)))
+
+
 @pytest.mark.parametrize("n,k,layers", [(9, 3, 2), (64, 5, 3), (1000, 32, 4), (1024, 33, 9), (1025, 32, 5), (2047, 8, 12), (4096, 16, 3)])
 @pytest.mark.parametrize("cnt", [1, 2, 3])
 @pytest.mark.parametrize("act", ["clamped_relu", "sigmoid"])
