@@ -1525,9 +1525,9 @@ int build_moves(sdnn* h) {
     char* at = nullptr;
     int rc = SDNN_OK;
     CU(h, cudaMemGetInfo(&left, &whole));
-    bool fits = bytes + scratch_ints * sizeof(int) + later <= left && cudaMalloc((void**)&scratch, scratch_ints * sizeof(int)) == cudaSuccess;
+    bool fits = bytes + scratch_ints * sizeof(int) + later <= left && cudaMallocAsync((void**)&scratch, scratch_ints * sizeof(int), h->stream) == cudaSuccess;
     if (fits && (rc = dev_alloc(h, &at, bytes, true)) != SDNN_OK) {
-        cudaFree(scratch);
+        cudaFreeAsync(scratch, h->stream);
         if (rc != SDNN_ERR_OOM) return rc;
         fits = false;
     }
@@ -1560,7 +1560,7 @@ int build_moves(sdnn* h) {
         e = cudaGetLastError();
         lm.move = Move{start, runs, pos[0], pos[1], m.nb, m.block};
     }
-    cudaFree(scratch);      // waits for its last reader
+    cudaFreeAsync(scratch, h->stream);      // given back to the device at sdnn_finalize's wait
     if (e != cudaSuccess) return cuda_fail(h, e, "set-up of the move maps");
     return rc;
 }
