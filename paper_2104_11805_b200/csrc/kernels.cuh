@@ -1398,8 +1398,10 @@ backward_row_ep_kernel(Sliced m, float* __restrict__ bias, const float* __restri
 //                  block size is chosen for that) and writes it
 // pos_a[t] / pos_b[t]: place of T's element t within its block of the transposed / row-major copy.  Nothing is scattered in
 // global memory: fetching each value by its 4-byte address instead costs a request per entry (about one per clock and SM,
-// 7 us for 2 M entries, and slower than the row units it would replace).  CTAs of 128 threads and at most 32 registers a
-// thread take the place of one one-warp CTA of the column units, beside which they run.
+// 7 us for 2 M entries, and slower than the row units it would replace).  Per stored entry 20 bytes, all of it in order: split
+// reads 4 + 2 (value, place) and writes 4, merge the same; the maps take 4 bytes an entry and the tables of runs some 0.4.  Alone
+// on the device the two take 5.5 and 7.4 us for 0.5 M entries, two short launches of mostly round trips (143 CTAs of 256 threads at
+// 32 and 64 registers, load pipe 5 and 12 % busy), which is why they run on four side streams beside the column units.
 struct Move {
     const int* start;             // [nb * (nb + 1)] first element of run (block of the transposed copy, block of the row-major copy) in T
     const int2* runs;             // [nb * nb] the same by row-major block: (first element, length)

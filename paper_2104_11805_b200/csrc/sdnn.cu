@@ -882,7 +882,7 @@ void enqueue_backward_chain(sdnn* h, int ld) {
 // Whole networks in one launch for one to four inputs (vector.cuh): nets whose rows all have the same padded length, up to 4096
 // neurons x (padded) inputs.  120 layers of 1024 neurons, one launch per layer / one launch: 1 input 255 / 121 us, 4 inputs 252 /
 // 176; 60 layers of 2048: 1 input 143 / 98, 4 inputs 142 / 159; of 4096: 1 input 149 / 156, 2 inputs 149 / 195.  And it leaves 132
-// SMs to other handles: three of them asked in turn answer an input in 47 us each instead of 240 (1024 x 120).
+// SMs to other handles: three of them asked in turn answer an input in 42 us each instead of 237 (1024 x 120).
 constexpr int VECTOR_WORK = 4096, VECTOR_DEPTH = 2048;
 
 // Status words that kernels raise and the host reads without waiting: one page of pinned memory for all handles (pinning one
@@ -3086,7 +3086,9 @@ int noalloc_scratch(float** out, unsigned long long** bad_out) {
 template <int G, int V, int STEP = 8>
 void noalloc_forward_g(cudaStream_t st, const int* rp, const int* col, const float* val, const float* bias,
                        const float* xin, float* xout, int n, int ld, int chunks, int n_inputs, float clamp, unsigned long long* bad) {
-    const int warps = (n + 32 / G - 1) / (32 / G), wpb = warps * chunks < 4096 ? 2 : 4;      // small CTAs: more SMs, finer tails
+    // small CTAs spread a narrow layer over more SMs and end in finer tails (1024 uniform rows, 4 inputs, 32 warps: 4.2 us a layer
+    // with CTAs of two warps, 4.5 of four, 5.7 of eight); from 4096 warps on two and four are within 1 % (16384 x 64: 12.18 / 12.24)
+    const int warps = (n + 32 / G - 1) / (32 / G), wpb = warps * chunks < 4096 ? 2 : 4;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((warps + wpb - 1) / wpb, chunks); lc.blockDim = dim3(32 * wpb); lc.stream = st;
     cudaLaunchAttribute at[1];
@@ -3138,7 +3140,13 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
         const float* val = values + layer_offset[l];
         const float* b = bias + (size_t)l * n_neurons;
 #define SDNN_NOALLOC(...) noalloc_forward_g<__VA_ARGS__>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, chunks, n_inputs, clamp, bad)
-        // up to 32 inputs a row has few lanes, so that 16 of its entries in flight per step still fit the registers
+        // Lanes per row, inputs per lane, entries of a row in flight per step.  At 4, 16 and 32 inputs the gathers of a row fit
+        // the registers 16 at a time, in lanes of four inputs; from 64 on a row has lanes enough, and 16 lose on the wider nets.  At 8 a
+        // lane a row is the better one only for the widest nets: two lanes are the variant to take for the others, not taken yet.
+        // us per layer of 24, rows of 8 to 56 entries, 4096 neurons (16384 in brackets), this / the other: 4 inputs <1,4,8> 6.9 / 7.2
+        // (8.6 / 9.0); 8 inputs <2,4,16> 7.9 / 5.8 (9.7 / 7.6; 65536 neurons 18.4 / 19.6); 16 inputs <4,4,8> 5.2 / 5.6 (7.9 / 7.6),
+        // <2,8,8> 5.2 / 8.6 (7.9 / 10.5); 32 inputs <8,4,8> 5.0 / 5.7 (11.9 / 12.1), <4,8,8> 5.0 / 6.9 (11.9 / 10.2); 64 inputs
+        // <16,4,16> 6.9 / 6.6 (16.2 / 20.0); 128 inputs <32,4,16> 8.3 / 10.7, <32,4,8> 8.3 / 7.9.
         switch (ld / chunks) {
             case 4: SDNN_NOALLOC(1, 4, 16); break;
             case 8: SDNN_NOALLOC(1, 8); break;

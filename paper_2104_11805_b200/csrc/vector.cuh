@@ -12,8 +12,9 @@
 // net of at most 960 neurons leaves CTAs without rows: they take no part in the exchange (vector_ctas).
 // The entries are off the chain: a CTA's part of a layer is one contiguous stretch of the sliced copy, and
 // bulk copies bring it into a ring of shared-memory stages several layers ahead.  (Prefetched into registers two layers ahead
-// instead, a layer took 1.0 us: loads of different ages share a scoreboard, so that waiting for the older ones waits for
-// the younger ones too.)
+// instead, a layer takes 1.0 us as well: either way the entries are not what it waits for, and the ring needs no registers for them.)
+// The launch: 16 CTAs of 256 threads, 80 registers; under ncu 132 us for 120 layers of 1024, the issue slots of its 16 SMs 27 % busy,
+// shared-memory wavefronts 20 % of what those SMs could do, 43 % of them bank conflicts of the random reads: latency, not a pipe.
 // Every wait is bounded: after VECTOR_WAIT_LIMIT polls the thread raises *status, waits no more and ends with the others.  From then
 // on it sends nothing, loads nothing and arms no barrier: a barrier whose phase it has not seen the end of must not be counted
 // on again, and every copy it has issued is older than the wait that it gave up.  CTAs that miss what it would have sent give up

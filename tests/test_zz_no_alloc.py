@@ -6,8 +6,8 @@ it), so this entry point keeps its activation scratch in a fixed array inside th
 network as the caller's own device arrays.  The test calls it through the C ABI twice in a row (the
 second call with a smaller batch, so stale scratch contents from the first would show) and compares
 with the handle-based entry point and with the float64 oracle; a second test runs nets whose rows have any
-length (rows that do not start on a multiple of four entries take the kernel's one-entry-at-a-time path)
-and batches of one to a few inputs.  This file is collected last on purpose.
+length (the lanes of a row fetch its entries as vectors only where it starts on a multiple of four) and batches
+of every padded width from 4 to two chunks of 128.  This file is collected last on purpose.
 """
 import numpy as np
 import pytest
@@ -55,9 +55,9 @@ def test_noalloc_inference_matches_handle_inference_twice_in_a_row():
     h.destroy()
 
 
-@pytest.mark.parametrize("cnt", [1, 3, 5, 20, 150])
+@pytest.mark.parametrize("cnt", [1, 3, 5, 12, 20, 40, 100, 150])
 def test_noalloc_inference_on_ragged_rows_and_tiny_batches_matches_the_oracle(cnt):
-    """Rows of 0..11 entries, so that most rows start off a multiple of four; each layer's entries start on one
+    """Widths of 4, 8, 16, 32, 64, 128 and two times 128.  Rows of 0..11 entries, so that most rows start off a multiple of four; each layer's entries start on one
     (the entry point's rule), which leaves up to three unused slots between layers."""
     torch = pytest.importorskip("torch")
     assert torch.cuda.is_available()
