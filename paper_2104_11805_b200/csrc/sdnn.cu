@@ -2111,6 +2111,7 @@ int sdnn_finalize(sdnn_t* h) {
     if (h->finalized) return fail(h, SDNN_ERR_STATE, "handle already finalized");
     for (int l = 0; l < h->L; ++l)
         if (!h->loaded[l]) return fail(h, SDNN_ERR_STATE, "layer %d was never loaded", l);
+    CU(h, cudaSetDevice(h->device));      // the caller may have gone to another one since the last layer
     if (h->reorder) {
         int rc = build_reordered(h);
         if (rc) return rc;
