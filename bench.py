@@ -63,7 +63,7 @@ def setup_of(spec):
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under profiles/
 # (training kernels: captured on a 48-layer slice of the same net, per-launch traffic does not depend on the depth)
 NCU_TRAFFIC = {("cfg5", "backward_kernel"): 21.26e6 + 27.10e6, ("cfg5", "forward_kernel"): 17.07e6,      # backward: both launches of a layer
-               ("cfg3", "backward_kernel"): 11.62e6 + 16.24e6, ("cfg3", "forward_kernel"): 7.42e6}
+               ("cfg3", "backward_kernel"): 16.24e6 + 3.41e6 + 3.32e6, ("cfg3", "forward_kernel"): 7.42e6}
 
 
 def measured_peaks():
@@ -653,10 +653,17 @@ def main():
         ep = not (args.flags & 0x81)
         names = ("backward_col_ep_kernel<4 or 8>", "backward_row_ep_kernel") if ep and ld_bwd == 4 else \
                 ("backward_kernel<..,1,..>", "backward_kernel<..,0,..>")
-        extra = {"backward_launches": f"per layer one column-unit launch ({names[0]}) on the main stream and one "
-                                      f"row-unit launch ({names[1]}) on a side stream, running beside each other; "
-                                      "launch_ms is the backward chain's time per layer, bytes and gathers are those of both",
-                 "kernel_names": {"forward": "forward_ep_kernel" if ep and ld == 4 else "forward_kernel", "backward": list(names)},
+        # what the step's launches say about it: 3L + 1 with a launch per layer forward and two backward; from 32 inputs on the
+        # row-major values of all layers but the first are moved (two launches); narrow nets run all layers forward as one
+        per_step = launches / args.steps
+        moved, one_forward = ep and per_step == 4 * L, ep and per_step == 2 * L + 2
+        beside = "two launches on a side stream that move the row-major values (split_values_kernel, merge_values_kernel)" if moved else \
+                 f"one row-unit launch ({names[1]}) on a side stream"
+        gathers_bwd = 1 if moved else 2
+        extra = {"backward_launches": f"per layer one column-unit launch ({names[0]}) on the main stream and {beside}, running "
+                                      "beside each other; launch_ms is the backward chain's time per layer, bytes and gathers are those of all",
+                 "kernel_names": {"forward": "vector_infer_kernel" if one_forward else "forward_ep_kernel" if ep and ld == 4 else "forward_kernel",
+                                  "backward": [names[0], "split_values_kernel", "merge_values_kernel"] if moved else list(names)},
                  "fwd_ms_per_step": fwd_ms, "bwd_ms_per_step": bwd_ms,
                  "fwd_GBps": fwd_bytes * L / (fwd_ms * 1e-3) / 1e9 if fwd_ms else None,
                  "bwd_GBps": bwd_bytes * L / (bwd_ms * 1e-3) / 1e9 if bwd_ms else None,
@@ -677,7 +684,7 @@ def main():
                           "launch, not one launch's start-to-end duration" if in_flight > 1 else "")}
     # what bounds these launches instead of HBM: random gathers of tile rows out of L2 (measured now, on this device)
     if kind == "train":
-        row_bytes, gathers = 4 * (ld_bwd if dom == "backward_kernel" else ld), (2 if dom == "backward_kernel" else 1) * nnz_l
+        row_bytes, gathers = 4 * (ld_bwd if dom == "backward_kernel" else ld), (gathers_bwd if dom == "backward_kernel" else 1) * nnz_l
         table_rows = 1 << (N - 1).bit_length()
     else:
         row_bytes = min(1024, 4 * (1 << (min(batch, n_inputs) - 1).bit_length()))      # one chunk of a tile row
@@ -694,7 +701,7 @@ def main():
         if kind == "train":      # both chains of the step against the floor of their own gathers
             fwd_rate = gather_rate if ld == ld_bwd else pkg.probe_gather_rate(4 * ld, table_rows)
             bwd_rate = gather_rate if dom == "backward_kernel" else pkg.probe_gather_rate(4 * ld_bwd, table_rows)
-            f_floor, b_floor = nnz_l * L / fwd_rate * 1e3, 2 * nnz_l * L / bwd_rate * 1e3
+            f_floor, b_floor = nnz_l * L / fwd_rate * 1e3, gathers_bwd * nnz_l * L / bwd_rate * 1e3
             extra["gather_bound"].update({"forward_chain_floor_ms": f_floor, "forward_chain_frac_of_floor": f_floor / fwd_ms if fwd_ms else None,
                                           "backward_chain_floor_ms": b_floor, "backward_chain_frac_of_floor": b_floor / bwd_ms if bwd_ms else None,
                                           "step_floor_ms": f_floor + b_floor,
