@@ -1,0 +1,185 @@
+// Plan of the kernel that keeps a whole network's activations in shared memory (resident.cuh): which nets and batches it takes, how
+// its memory is cut, and in which order the entries of eight rows are read.  Plain code, so that it can be looked at without a device.
+#pragma once
+#include <stdint.h>
+
+#include <algorithm>
+
+#ifdef __CUDACC__
+#define SDNN_HD __host__ __device__ __forceinline__
+#else
+#define SDNN_HD inline
+#endif
+
+namespace sdnn_plan {
+
+constexpr int RES_UNIT = 32;              // rows of a unit: one per lane of a warp
+constexpr int RES_CLASSES = 8;            // 16-byte columns of shared memory: slots s and t meet in a bank where s = t modulo 8
+constexpr int RES_WARPS = 16;
+constexpr int RES_BLOCK = 1024;           // rows among which groups of eight are chosen
+constexpr int RES_MAX_ROW = 248;          // entries of a row: counts and places are kept in bytes
+constexpr int RES_SMEM = 226 * 1024;
+
+// One step of a group of eight rows, of `left` that are left: which class each row reads from.  have: byte c = mask of the rows that
+// still have an entry of class c; total[c]: entries of class c that the group still has; must: rows that have to read now (no step to
+// spare).  Returns a class per row, four bits each, 15 = the row waits.
+// While no class has more entries than there are steps, the rows read eight different ones (the rest can then always be read that
+// way: a bipartite graph of rows and classes falls apart into as many matchings as its largest degree).  Else one or more classes have
+// to be read twice in some step, which costs that step a second wavefront whatever else is read twice in it: so this step reads
+// as many entries twice as bring the classes to the number of steps that will be left.  With rows of equal length the steps
+// that take two wavefronts are as few as the group's counts allow: the largest distance of a class from the mean.
+// A largest matching of classes (twice: and of second copies of classes) with rows by augmenting paths, the fullest classes first.
+SDNN_HD uint32_t resident_step(uint64_t have, const int (&total)[RES_CLASSES], uint32_t must, int left) {
+    int key[RES_CLASSES];
+    for (int c = 0; c < RES_CLASSES; ++c) key[c] = total[c] * RES_CLASSES + c;
+#define SDNN_ORDER(A, B) { const int hi_ = key[A] > key[B] ? key[A] : key[B], lo_ = key[A] > key[B] ? key[B] : key[A]; key[A] = hi_; key[B] = lo_; }
+    SDNN_ORDER(0, 2) SDNN_ORDER(1, 3) SDNN_ORDER(4, 6) SDNN_ORDER(5, 7)
+    SDNN_ORDER(0, 4) SDNN_ORDER(1, 5) SDNN_ORDER(2, 6) SDNN_ORDER(3, 7)
+    SDNN_ORDER(0, 1) SDNN_ORDER(2, 3) SDNN_ORDER(4, 5) SDNN_ORDER(6, 7)
+    SDNN_ORDER(2, 4) SDNN_ORDER(3, 5)
+    SDNN_ORDER(1, 4) SDNN_ORDER(3, 6)
+    SDNN_ORDER(1, 2) SDNN_ORDER(3, 4) SDNN_ORDER(5, 6)
+#undef SDNN_ORDER
+    // nodes in the order they are matched: class, or class + 8 for the second copy
+    uint64_t order = 0;
+    int nodes = 0;
+    const bool twice = key[0] / RES_CLASSES > left;
+    for (int i = 0; i < RES_CLASSES; ++i)
+        if (!twice || key[i] / RES_CLASSES >= left) order |= (uint64_t)(key[i] & 7) << (4 * nodes++);
+    if (twice) {
+        for (int i = 0; i < RES_CLASSES; ++i)
+            if (key[i] / RES_CLASSES > left) order |= (uint64_t)((key[i] & 7) | 8) << (4 * nodes++);
+        for (int i = 0; i < RES_CLASSES; ++i)
+            if (key[i] / RES_CLASSES < left) order |= (uint64_t)(key[i] & 7) << (4 * nodes++);
+    }
+    uint64_t of_node = 0;                 // row of each matched node, node of each matched row: four bits each
+    uint32_t of_row = 0, rows_set = 0, nodes_set = 0;
+    for (int i = 0; i < nodes && rows_set != 0xffu; ++i) {
+        uint64_t queue = (order >> (4 * i)) & 15u;
+        uint32_t from = 0, seen = 0;      // node each row was reached from
+        int head = 0, tail = 1, end = -1;
+        while (head < tail && end < 0) {
+            const uint32_t q = (uint32_t)(queue >> (4 * head++)) & 15u;
+            uint32_t rows = (uint32_t)(have >> (8 * (q & 7u))) & 0xffu & ~seen;
+            for (int r = 0; r < RES_CLASSES && rows >> r; ++r) {
+                if (!((rows >> r) & 1u)) continue;
+                seen |= 1u << r;
+                from = (from & ~(15u << (4 * r))) | q << (4 * r);
+                if (!((rows_set >> r) & 1u)) { end = r; break; }
+                queue |= (uint64_t)((of_row >> (4 * r)) & 15u) << (4 * tail++);
+            }
+        }
+        if (end < 0) continue;
+        rows_set |= 1u << end;
+        for (int r = end;;) {             // hand the rows of the path on to the node each was reached from
+            const uint32_t q = (from >> (4 * r)) & 15u;
+            const bool had = (nodes_set >> q) & 1u;
+            const int before = (int)((of_node >> (4 * q)) & 15u);
+            of_row = (of_row & ~(15u << (4 * r))) | q << (4 * r);
+            of_node = (of_node & ~((uint64_t)15u << (4 * q))) | (uint64_t)r << (4 * q);
+            nodes_set |= 1u << q;
+            if (!had) break;
+            r = before;
+        }
+    }
+    uint32_t read = 0, load = 0;          // class of each row; rows reading each class, four bits each
+    for (int r = 0; r < RES_CLASSES; ++r) {
+        const uint32_t c = (of_row >> (4 * r)) & 7u;
+        if ((rows_set >> r) & 1u) { read |= c << (4 * r); load += 1u << (4 * c); }
+        else read |= 15u << (4 * r);
+    }
+    for (int r = 0; r < RES_CLASSES; ++r) {      // rows of different lengths: one may be left over that cannot wait
+        if (!((must >> r) & 1u) || ((rows_set >> r) & 1u)) continue;
+        int best = -1, best_key = 0;
+        for (int c = 0; c < RES_CLASSES; ++c) {
+            if (!((have >> (8 * c + r)) & 1u)) continue;
+            const int k = (int)((load >> (4 * c)) & 15u) * 65536 - total[c];
+            if (best < 0 || k < best_key) { best = c; best_key = k; }
+        }
+        if (best >= 0) {
+            read = (read & ~(15u << (4 * r))) | (uint32_t)best << (4 * r);
+            load += 1u << (4 * best);
+        }
+    }
+    return read;
+}
+
+// Class of the zeros that a waiting row reads: the rows that wait share out the classes that nobody reads.
+SDNN_HD int resident_idle_class(uint32_t of_row, int row) {
+    uint32_t read = 0;
+    int before = 0;
+    for (int r = 0; r < RES_CLASSES; ++r) {
+        const uint32_t c = (of_row >> (4 * r)) & 15u;
+        if (c != 15u) read |= 1u << c;
+        else if (r < row) ++before;
+    }
+    for (int c = 0; c < RES_CLASSES; ++c)
+        if (!((read >> c) & 1u) && before-- == 0) return c;
+    return 0;
+}
+
+// How the kernel holds a net of n neurons with 4 p inputs to a CTA.  A layer's activations are `slots` slots of 16 p bytes; outputs go
+// to the free slots of a ring of `cap`, and what does not fit stays in the registers of the warps' last `held` units until the
+// layer has been read.  ok = false: it does not fit at all.
+struct ResidentShape { bool ok; int units, slots, cap, held; };
+SDNN_HD ResidentShape resident_shape(int n, int p) {
+    ResidentShape s{};
+    s.units = (n + RES_UNIT - 1) / RES_UNIT;
+    s.slots = s.units * RES_UNIT + RES_CLASSES;      // the last eight hold zeros, one of each class
+    const int fit = RES_SMEM / (16 * p) / RES_CLASSES * RES_CLASSES, rounds = (s.units + RES_WARPS - 1) / RES_WARPS;
+    if (2 * s.slots <= fit) { s.ok = true; s.cap = 2 * s.slots; return s; }
+    if (s.slots > fit) return s;
+    s.cap = fit;
+    const int free_rounds = (fit - s.slots) / RES_UNIT / RES_WARPS, most = p <= 2 ? 4 : 2;      // registers: 4 p numbers a held unit
+    s.held = rounds - free_rounds <= 2 ? 2 : 4;
+    s.ok = rounds - free_rounds <= most && rounds >= s.held;
+    return s;
+}
+
+// How a batch is cut into CTAs.  Rounds of 4 p inputs on every SM as long as they are whole; what is left, less than a round, is one more
+// round of CTAs that take as few inputs as that needs: the launch of each width q <= p looks whether the rest is its own.
+// Where the number of inputs is known only on the device, all these launches are made, and all but one find nothing.
+SDNN_HD int resident_rest_width(int rest, int sms) { return rest ? (rest + 4 * sms - 1) / (4 * sms) : 0; }
+// inputs [begin, end) of `total` that the launch of width q takes
+SDNN_HD void resident_share(int total, int sms, int p, int q, int* begin, int* end) {
+    const int main = total / (4 * p * sms) * (4 * p * sms), rest = total - main;
+    const bool own = resident_rest_width(rest, sms) == q;
+    *begin = q == p ? 0 : main;
+    *end = own ? total : q == p ? main : *begin;
+}
+// The width for `inputs` inputs, 0 where the layer launches, in tiles of `tile` inputs, are faster.  Clocks per layer, fitted to both
+// over 640 .. 8000 neurons and 32 .. 4000 inputs (24 layers; us per layer, layer launches / this kernel):
+//   neurons   256 inputs      400             592             1184            2368            4000
+//     640     3.49 / 3.83     4.59 / 3.88     4.75 / 3.90     7.71 / 5.22     13.5 / 8.2      18.7 / 14.8
+//    1024     3.50 / 4.75     4.72 / 4.75     6.85 / 4.79     9.52 / 6.84     18.5 / 11.4     27.2 / 20.5
+//    2048     4.86 / 8.35     7.96 / 8.39     11.0 / 8.45     17.3 / 12.7     34.9 / 22.3     54.0 / 39.6
+//    4096     8.75 / 15.5     17.4 / 15.5     19.9 / 15.6     33.4 / 24.9     67.0 / 50.0     109 / 90.7
+//    8000     17.0 / 33.2     27.1 / 33.8     38.4 / 34.7     66.2 / 70.4     131 / 134
+// A CTA: wavefronts of operands (1.06 for eight of them), entries (6 bytes each) and outputs; a single piece of 4 inputs leaves the
+// pipe waiting for entries, units held in registers cost addresses; 2500 clocks for the ends of a layer.  The layer launches:
+// 66 bytes of operands per clock and SM, and the round trips at the ends of a launch, which a second tile in flight fills.
+inline double resident_clocks(int n, double elems, int p) {
+    const double pipe = elems * (p * 1.06 / 8 + 6.0 / 128) + n * p / 4.0;
+    const int held = resident_shape(n, p).held;
+    return pipe * (p == 1 ? 1.10 : 1.0) * (held == 4 ? 1.18 : held ? 1.04 : 1.0) + 2500;
+}
+// drop: dead inputs are dropped.  A third is taken to be left after a few layers, and the layer launches to take 1.8 times as long for what
+// is left (a tile of 1024 inputs is then a tile of 340, with what finding and moving them costs: 4096 x 120, 5000 inputs, us a layer:
+// 80 / 47; 1024 x 120, 3000: 15.9 / 8.1; 1465 x 120, 449: 6.9 / 7.1).
+inline int resident_width(int n, double elems, int64_t inputs, int sms, int tile, bool drop) {
+    int best = 0;
+    if (inputs <= 256) return best;      // a single chunk of inputs: the table's first column
+    if (drop) inputs = (inputs + 2) / 3;
+    const double gathers = elems * (double)inputs * 4.0 / (66.0 * sms);
+    double least = drop ? 1.8 * std::max(6300.0, gathers + 2800) : inputs > tile ? gathers : std::max(8700.0, gathers + 4500);
+    for (int p = 1; p <= 4; ++p) {
+        if (!resident_shape(n, p).ok) break;      // nor does a wider one
+        const int64_t round = (int64_t)4 * p * sms;
+        const int q = resident_rest_width((int)(inputs % round), sms);
+        const double all = (double)(inputs / round) * resident_clocks(n, elems, p) + (q ? resident_clocks(n, elems, q) : 0.0);
+        if (all < least) { least = all; best = p; }
+    }
+    return best;
+}
+
+}  // namespace sdnn_plan

@@ -6,6 +6,7 @@
 #include "kernels.cuh"
 #include "plan.h"
 #include "vector.cuh"
+#include "resident.cuh"
 #include "reorder.h"
 
 #include <nvtx3/nvToolsExt.h>
@@ -62,6 +63,7 @@ struct InferLane {
     int64_t graph_asked[TILE_GRAPHS] = {}; // and the call that asked for it last (0: none made)
     cudaEvent_t ev_scan = nullptr;         // this lane's last scan of the running id total is done
     cudaEvent_t ev_done = nullptr;         // everything this lane was given in the current call is done
+    int* res_list = nullptr;               // whole networks in shared memory: [2][resident_piece] inputs that are alive, [2] how many, [resident_piece] counts
     bool ready = false;
 };
 
@@ -80,6 +82,7 @@ struct LayerMem {
     int* r_start = nullptr;                // ... the same on the device (ragged layers whose entries keep the caller's order; else NULL)
     std::vector<int> entry_src;            // [nnz] entry in stored order (stored rows, their entries in stored order) -> caller's position
     int* r_out = nullptr;                  // rows not stored in neuron order: tile row each stored row writes (device, [N])
+    unsigned char* r_order = nullptr;      // which of a row's entries is stored at each place (NULL: in the caller's order; see resident_reorder_kernel)
     int* r_row_of = nullptr;               // ... and its inverse: stored row that holds neuron (tile row) i (device, [N])
     // windowed layer: rows grouped by shared columns, the group's window staged in shared memory (forward_window_kernel)
     bool windowed = false;
@@ -171,6 +174,9 @@ struct sdnn {
     VectorLayer* d_vector = nullptr;    // [L] table of vector_infer_kernel (NULL: the net is not for it)
     int vector_kpad = 0;                // entries per row of every slice of every layer (the same everywhere, or no table)
     int* vector_status = nullptr;       // pinned: raised by a whole-network kernel whose wait for its neighbours ran out
+    Resident resident{};                // the net as resident_infer_kernel reads it (units = 0: it does not)
+    ResidentSetup resident_setup{};
+    double resident_elems = 0;          // stored elements per layer there, padding included
     bool compaction = false;            // SDNN_FLAG_SKIP_DEAD asked for; effective while no bias is positive
     std::vector<char> bias_nonpositive; // per layer
     bool live_valid = false;
@@ -1103,6 +1109,15 @@ int check_train_args(sdnn* h, const float* x0, const float* target, int B, float
     return SDNN_OK;
 }
 
+int resident_piece(const sdnn* h);
+
+// whether inference drops dead inputs: the zero vector must be a fixed point of every layer (sigmoid(b) is never 0: nothing ever dies)
+bool drops_dead(const sdnn* h) {
+    bool track = h->compaction && h->cfg.activation == SDNN_ACT_CLAMPED_RELU;
+    for (int l = 0; l < h->L && track; ++l) track = h->bias_nonpositive[l] != 0;
+    return track;
+}
+
 int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
     if (ln.ready) return SDNN_OK;
     const size_t N = (size_t)h->N, tile = N * (size_t)h->ld_max, nseg = (N + NZ_SEG - 1) / NZ_SEG;
@@ -1124,6 +1139,7 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
         ln.cs.ncols = blk + (2 + (size_t)h->L) * (size_t)h->ld_max; ln.cs.old_ncols = ln.cs.ncols + 1; ln.cs.do_compact = ln.cs.ncols + 2;
         if ((rc = dev_alloc(h, &ln.live_hist, (size_t)h->L, true))) return rc;
     }
+    if (h->resident.units && (rc = dev_alloc(h, &ln.res_list, 3 * (size_t)resident_piece(h) + 2, false))) return rc;
     ln.ready = true;
     return SDNN_OK;
 }
@@ -1172,8 +1188,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     cudaStream_t st = ln.stream;
     h->cur = &ln;
     h->launch_stream = st;
-    bool track = h->compaction && h->cfg.activation == SDNN_ACT_CLAMPED_RELU;      // sigmoid(b) is never 0: nothing ever dies
-    for (int l = 0; l < h->L && track; ++l) track = h->bias_nonpositive[l] != 0;     // the zero vector must be a fixed point
+    const bool track = drops_dead(h);
     // dropping dead inputs works on chunks of 64 whatever the padding
     const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->mean_elems, h->windowed_layers == h->L);
     const int cw = shape.cw, cols = shape.cols;
@@ -1312,6 +1327,218 @@ int lanes_end(sdnn* h, int lanes) {
     return SDNN_OK;
 }
 
+// ---------------------------------------------------------------------------------------------
+// Whole networks in shared memory (resident.cuh)
+
+// Inputs per turn: a multiple of the tile width, so that "the most recent tile" (sdnn_get_liveness) lies in one
+int resident_piece(const sdnn* h) {
+    const int T = infer_tile_width(h);
+    return std::max(1, 16384 / T) * T;
+}
+
+// Lays the net out for resident_infer_kernel where batches of max_batch inputs would go through it, or where the handle is for
+// large batches and larger ones would (called by sdnn_finalize).
+int build_resident(sdnn* h) {
+    if (h->cfg.train || h->reorder || h->N > 65536 - 2 * RES_UNIT || !resident_shape(h->N, 1).ok) return SDNN_OK;
+    const int N = h->N, L = h->L, units = resident_shape(N, 1).units;
+    int longest = 0;
+    bool uniform = true;
+    for (const LayerMem& lm : h->lay) {
+        uniform = uniform && lm.shape.uniform_k >= 0;
+        if (lm.shape.uniform_k >= 0) longest = std::max(longest, lm.shape.uniform_k);
+        else for (int i = 0; i < N; ++i) longest = std::max(longest, lm.shape.len(i));
+    }
+    if (longest > RES_MAX_ROW) return SDNN_OK;
+    // rows by descending length in chunks, so that a unit's rows are of one length or nearly; rows change places only with their like
+    std::vector<unsigned short> row0, place0;
+    std::vector<int> unit_at((size_t)L * units + 1);
+    if (!uniform) { row0.resize((size_t)L * N); place0.resize((size_t)L * N); }
+    int64_t run = 0;
+    for (int k = 0; k < L; ++k) {
+        const LayerMem& lm = h->lay[k];
+        auto chunks = [&](int row) { return std::max(1, (lm.shape.len(row) + 3) / 4); };
+        unsigned short* at = uniform ? nullptr : row0.data() + (size_t)k * N;
+        if (at) {
+            std::vector<int> bucket(RES_MAX_ROW / 4 + 2, 0);
+            for (int i = 0; i < N; ++i) ++bucket[RES_MAX_ROW / 4 - chunks(i) + 1];
+            for (size_t d = 1; d < bucket.size(); ++d) bucket[d] += bucket[d - 1];
+            for (int i = 0; i < N; ++i) at[bucket[RES_MAX_ROW / 4 - chunks(i)]++] = (unsigned short)i;
+            for (int p = 0; p < N; ++p) place0[(size_t)k * N + (lm.row_src.empty() ? at[p] : lm.row_src[at[p]])] = (unsigned short)p;
+        }
+        for (int u = 0; u < units; ++u) {
+            unit_at[(size_t)k * units + u] = (int)run;
+            run += chunks(at ? at[u * RES_UNIT] : u * RES_UNIT);
+        }
+        if (run > INT32_MAX / 128) return SDNN_OK;
+    }
+    unit_at[(size_t)L * units] = (int)run;
+    const double elems = 128.0 * run / L;
+    auto takes = [&](int64_t inputs) { return resident_width(N, elems, inputs, h->sms, infer_tile_width(h), drops_dead(h)) != 0; };
+    if (!takes(h->cfg.max_batch) && !(h->cfg.max_batch >= 512 && takes(10 * (int64_t)h->cfg.max_batch))) return SDNN_OK;
+
+    auto room = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t rows = (size_t)L * units * RES_UNIT, entries = (size_t)run * 128;
+    int64_t elems_stored = 0;
+    for (const LayerMem& lm : h->lay) elems_stored += lm.r_elems;
+    const size_t sizes[] = {entries * sizeof(unsigned short), entries * sizeof(float), rows * sizeof(float), unit_at.size() * sizeof(int),
+                            (size_t)L * N * sizeof(unsigned short), rows * sizeof(int), L * sizeof(Sliced), L * sizeof(float*),
+                            row0.size() * sizeof(unsigned short), place0.size() * sizeof(unsigned short), L * sizeof(unsigned char*), (size_t)elems_stored};
+    size_t bytes = 0, left = 0, whole = 0;
+    for (size_t b : sizes) bytes += room(b);
+    // it saves time and is not needed: not where it would take what later calls allocate (a second lane, staging of host batches)
+    CU(h, cudaMemGetInfo(&left, &whole));
+    if (bytes + 6 * (size_t)N * h->ld_max * sizeof(float) + ((size_t)64 << 20) > left) return SDNN_OK;
+    char* at = nullptr;
+    int rc = dev_alloc(h, &at, bytes, false);
+    if (rc) return rc == SDNN_ERR_OOM ? SDNN_OK : rc;
+    constexpr int PARTS = sizeof sizes / sizeof sizes[0];
+    char* part[PARTS];
+    for (int i = 0; i < PARTS; ++i) { part[i] = at; at += room(sizes[i]); }
+    Resident net{};
+    net.col = reinterpret_cast<unsigned short*>(part[0]); net.val = reinterpret_cast<float*>(part[1]); net.bias = reinterpret_cast<float*>(part[2]);
+    net.unit_at = reinterpret_cast<int*>(part[3]); net.slot_of = reinterpret_cast<unsigned short*>(part[4]); net.row_at = reinterpret_cast<int*>(part[5]);
+    net.n = N; net.units = units;
+    std::vector<Sliced> tables(L);
+    std::vector<const float*> biases(L);
+    std::vector<unsigned char*> orders(L);
+    for (int k = 0; k < L; ++k) {
+        tables[k] = rows_of(h, k); biases[k] = h->d_bias + (size_t)k * N;
+        orders[k] = k ? orders[k - 1] + h->lay[k - 1].r_elems : reinterpret_cast<unsigned char*>(part[11]);
+    }
+    ResidentSetup set{};
+    set.rows = reinterpret_cast<const Sliced*>(part[6]); set.bias = reinterpret_cast<const float* const*>(part[7]);
+    if (!uniform) { set.row0 = reinterpret_cast<const unsigned short*>(part[8]); set.place0 = reinterpret_cast<const unsigned short*>(part[9]); }
+    set.order = reinterpret_cast<unsigned char* const*>(part[10]);
+    const void* from[] = {unit_at.data(), tables.data(), biases.data(), row0.data(), place0.data(), orders.data()};
+    const int to[] = {3, 6, 7, 8, 9, 10};
+    for (int i = 0; i < 6; ++i) if (sizes[to[i]]) CU(h, cudaMemcpyAsync(part[to[i]], from[i], sizes[to[i]], cudaMemcpyHostToDevice, h->stream));
+    for (int k = 0; k < L; k += 32768) {      // a grid has at most 65535 rows of blocks
+        set.layer0 = k;
+        const int layers = std::min(L - k, 32768);
+        resident_order_kernel<<<dim3((units * RES_UNIT + RES_BLOCK - 1) / RES_BLOCK, layers), RES_BLOCK, 0, h->stream>>>(net, set);
+    }
+    for (int k = 0; k < L; k += 32768) {
+        set.layer0 = k;
+        const int layers = std::min(L - k, 32768), pitch = std::max(4, (longest + 3) / 4 * 4);
+        resident_fill_kernel<<<dim3(units, layers), 32, 32 * pitch, h->stream>>>(net, set, pitch);
+        resident_reorder_kernel<<<dim3((N + 7) / 8, layers), 256, 0, h->stream>>>(set, N);
+    }
+    CU(h, cudaGetLastError());
+    CU(h, cudaStreamSynchronize(h->stream));
+    for (int k = 0; k < L; ++k) h->lay[k].r_order = orders[k];
+    h->resident = net; h->resident_setup = set; h->resident_elems = elems;
+    return dev_alloc(h, &h->lane[0].res_list, 3 * (size_t)resident_piece(h) + 2, false);
+}
+
+// values or biases of a layer have changed: its entries keep their places
+int refresh_resident(sdnn* h, int layer) {
+    if (!h->resident.units) return SDNN_OK;
+    h->resident_setup.layer0 = layer;
+    resident_refill_kernel<<<h->resident.units, 32, 0, h->stream>>>(h->resident, h->resident_setup);
+    CU(h, cudaGetLastError());
+    CU(h, cudaStreamSynchronize(h->stream));
+    return SDNN_OK;
+}
+
+template <int P, int HELD>
+int launch_resident(sdnn* h, const ResidentArgs& a, int ctas, cudaStream_t st) {
+    const void* kernel = (const void*)resident_infer_kernel<P, HELD>;
+    if (!h->configured[kernel]) {
+        CU(h, cudaFuncSetAttribute(resident_infer_kernel<P, HELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
+        h->configured[kernel] = true;
+    }
+    resident_infer_kernel<P, HELD><<<ctas, RES_THREADS, (size_t)a.cap * 16 * P, st>>>(a);
+    count_launch(h);
+    CU(h, cudaGetLastError());
+    return SDNN_OK;
+}
+// the launches that share out a.inputs inputs, or *a.count of them, of width p and narrower
+int launch_resident(sdnn* h, ResidentArgs a, int p, cudaStream_t st) {
+    a.net = h->resident; a.clamp = h->cfg.clamp; a.act = h->cfg.activation;
+    a.sms = h->sms; a.width = p;
+    for (int q = p; q >= 1; --q) {
+        int begin, end;
+        resident_share(a.inputs, h->sms, p, q, &begin, &end);
+        if (a.count) { begin = 0; end = q == p ? a.inputs : std::min(a.inputs, 4 * q * h->sms); }
+        const int ctas = (end - begin + 4 * q - 1) / (4 * q);
+        if (!ctas) continue;
+        const ResidentShape s = resident_shape(h->N, q);
+        a.slots = s.slots; a.cap = s.cap;
+        int rc;
+        if (q == 1) rc = s.held == 0 ? launch_resident<1, 0>(h, a, ctas, st) : s.held == 2 ? launch_resident<1, 2>(h, a, ctas, st) : launch_resident<1, 4>(h, a, ctas, st);
+        else if (q == 2) rc = s.held == 0 ? launch_resident<2, 0>(h, a, ctas, st) : s.held == 2 ? launch_resident<2, 2>(h, a, ctas, st) : launch_resident<2, 4>(h, a, ctas, st);
+        else if (q == 3) rc = s.held == 0 ? launch_resident<3, 0>(h, a, ctas, st) : launch_resident<3, 2>(h, a, ctas, st);
+        else rc = s.held == 0 ? launch_resident<4, 0>(h, a, ctas, st) : launch_resident<4, 2>(h, a, ctas, st);
+        if (rc) return rc;
+    }
+    return SDNN_OK;
+}
+
+// Width for a call's inputs, 0 if they go through the layer launches.  The ids of nonzero outputs are found in the outputs: without
+// those the tiles do it.
+int takes_resident(const sdnn* h, int64_t inputs, bool outputs) {
+    return h->resident.units && outputs ? resident_width(h->N, h->resident_elems, inputs, h->sms, infer_tile_width(h), drops_dead(h)) : 0;
+}
+
+// All layers for `inputs` inputs on lane `ln`; arguments as for infer_tile.  total: the running total of ids is wanted.
+int infer_resident(sdnn* h, InferLane& ln, int p, const float* x0, int64_t inputs, float* y, int* cnt_out, int* idx_out, long long capacity,
+                   bool want_sets, bool total, cudaEvent_t consumed = nullptr) {
+    NvtxRange call("sdnn whole-network inference");
+    const int piece = resident_piece(h), T = infer_tile_width(h);
+    cudaStream_t st = ln.stream;
+    int* list[2] = {ln.res_list, ln.res_list + piece};
+    int* count = ln.res_list + 2 * (size_t)piece;
+    int* nz = count + 2;
+    const bool track = drops_dead(h);
+    if (track) {
+        CU(h, cudaMemsetAsync(ln.live_hist, 0, (size_t)h->L * sizeof(int), st));
+        h->live_valid = true;
+        h->live_lane = (int)(&ln - h->lane);
+    }
+    int rc;
+    for (int64_t at = 0; at < inputs; at += piece) {
+        const int cnt = (int)std::min<int64_t>(piece, inputs - at);
+        int* counts = want_sets ? (cnt_out ? cnt_out + at : nz) : nullptr;
+        ResidentArgs a{};
+        a.x = x0 + (size_t)at * h->N; a.y = y + (size_t)at * h->N; a.nz_count = counts;
+        a.from = 0; a.to = h->L; a.inputs = cnt;
+        if (!track) {
+            if ((rc = launch_resident(h, a, p, st))) return rc;
+        } else {
+            // in stages, between which the inputs that are left move together; what is on its way waits in y
+            a.live_hist = ln.live_hist;
+            a.live_first = (int)std::min<int64_t>((inputs - 1) / T * T - at, INT32_MAX);      // the most recent tile is the last one
+            int q = 0;
+            for (int from = 0; from < h->L; q ^= 1) {      // after 3, 12, 48, .. layers (4096 x 120, 5000 inputs, a third survive: 5.68 ms; 4, 12, 36, ..: 5.74; 2, 4, 8, ..: 5.70)
+                const int to = std::min(h->L, from ? 4 * from : 3);
+                CU(h, cudaMemsetAsync(count + q, 0, sizeof(int), st));
+                a.from = from; a.to = to;
+                a.left = to < h->L ? list[q] : nullptr; a.n_left = count + q;
+                if ((rc = launch_resident(h, a, p, st))) return rc;
+                a.list = list[q]; a.count = count + q;
+                a.x = a.y;
+                from = to;
+            }
+        }
+        if (consumed) CU(h, cudaEventRecord(consumed, st));
+        if (total || idx_out)
+            for (int t0 = 0; t0 < cnt; t0 += T) {
+                const int some = std::min(T, cnt - t0);
+                if (h->last_scan_ev && h->last_scan_ev != ln.ev_scan) CU(h, cudaStreamWaitEvent(st, h->last_scan_ev, 0));
+                nz_scan_inputs_kernel<<<1, 1024, 0, st>>>(counts + t0, ln.offs, h->d_running, nullptr, some);
+                CU(h, cudaEventRecord(ln.ev_scan, st));
+                h->last_scan_ev = ln.ev_scan;
+                count_launch(h);
+                if (idx_out) {
+                    nz_fill_rows_kernel<<<some, 256, 0, st>>>(y + ((size_t)at + t0) * h->N, ln.offs, idx_out, capacity, h->N);
+                    count_launch(h);
+                }
+            }
+    }
+    CU(h, cudaGetLastError());
+    return SDNN_OK;
+}
+
 int check_infer_args(sdnn* h, const float* x0, int64_t n_inputs, int32_t* idx, int64_t cap) {
     if (!h) return SDNN_ERR_INVALID_ARG;
     if (!h->finalized) return fail(h, SDNN_ERR_STATE, "handle is not finalized");
@@ -1443,7 +1670,7 @@ int ensure_stage_w(sdnn* h) {
 template <bool TO_CSR>
 int convert_values(sdnn* h, int layer, float* csr) {
     const LayerMem& lm = h->lay[layer];
-    sliced_csr_kernel<TO_CSR><<<(h->N + 15) / 16, 512, 0, h->stream>>>(rows_of(h, layer), csr, (const int*)lm.r_start, lm.shape.uniform_k, h->N);
+    sliced_csr_kernel<TO_CSR><<<(h->N + 15) / 16, 512, 0, h->stream>>>(rows_of(h, layer), csr, (const int*)lm.r_start, lm.shape.uniform_k, h->N, (const unsigned char*)lm.r_order);
     count_launch(h);
     CU(h, cudaGetLastError());
     return SDNN_OK;
@@ -2118,7 +2345,7 @@ int sdnn_finalize(sdnn_t* h) {
     }
     {
         int rc;
-        if ((rc = build_moves(h)) || (rc = build_vector(h))) return rc;
+        if ((rc = build_moves(h)) || (rc = build_vector(h)) || (rc = build_resident(h))) return rc;
     }
     int64_t elems = 0;
     for (const LayerMem& lm : h->lay) elems += lm.windowed ? lm.w_elems : lm.r_elems;
@@ -2194,10 +2421,12 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
     const bool want_sets = nz_count_out || nz_index_out || nz_total_out;
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     const int T = infer_tile_width(h);
-    const int lanes = n_inputs > T ? infer_lanes(h, T) : 1;
+    const int width = takes_resident(h, n_inputs, y_out != nullptr);
+    const int lanes = n_inputs > T && !width ? infer_lanes(h, T) : 1;
     if ((rc = lanes_begin(h, lanes))) return rc;
+    if (width && (rc = infer_resident(h, h->lane[0], width, x0, n_inputs, y_out, nz_count_out, nz_index_out, nz_index_capacity, want_sets, nz_index_out || nz_total_out))) return rc;
     int64_t tile_no = 0;
-    for (int64_t t0 = 0; t0 < n_inputs; t0 += T, ++tile_no) {
+    for (int64_t t0 = 0; t0 < n_inputs && !width; t0 += T, ++tile_no) {
         const int cnt = (int)((n_inputs - t0 < T) ? (n_inputs - t0) : T);
         rc = infer_tile(h, h->lane[tile_no % lanes], x0 + (size_t)t0 * h->N, cnt, y_out ? y_out + (size_t)t0 * h->N : nullptr,
                         nz_count_out ? nz_count_out + t0 : nullptr, nz_index_out, nz_index_capacity, want_sets);
@@ -2263,8 +2492,11 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         CU(h, cudaMemcpyAsync(stage[q], x0 + (size_t)t0 * h->N, bytes, cudaMemcpyHostToDevice, h->copy_stream));
         CU(h, cudaEventRecord(h->ev_copied[q], h->copy_stream));
         CU(h, cudaStreamWaitEvent(ln.stream, h->ev_copied[q], 0));
-        rc = infer_tile(h, ln, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
-                        nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity, want_sets, h->ev_consumed[q]);
+        if (const int width = takes_resident(h, cnt, y_out != nullptr))
+            rc = infer_resident(h, ln, width, stage[q], cnt, ln.stage_out, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
+                                want_sets, want_sets, h->ev_consumed[q]);
+        else rc = infer_tile(h, ln, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
+                             nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity, want_sets, h->ev_consumed[q]);
         if (rc) break;
         if (y_out) CU(h, cudaMemcpyAsync(y_out + (size_t)t0 * h->N, ln.stage_out, bytes, cudaMemcpyDeviceToHost, ln.stream));
         if (nz_count_out) CU(h, cudaMemcpyAsync(nz_count_out + t0, ln.stage_cnt, (size_t)cnt * sizeof(int), cudaMemcpyDeviceToHost, ln.stream));
@@ -2388,7 +2620,7 @@ int sdnn_set_weights(sdnn_t* h, int32_t layer, const float* values, const float*
         for (int i = 0; i < h->N && nonpos; ++i) nonpos = !(bias[i] > 0.0f);
         h->bias_nonpositive[layer] = nonpos ? 1 : 0;
     }
-    return SDNN_OK;
+    return refresh_resident(h, layer);
 }
 
 int sdnn_mirror_mismatches(sdnn_t* h, int32_t layer, int64_t* count_out) {

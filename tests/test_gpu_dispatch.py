@@ -387,3 +387,116 @@ def test_lanes_of_nothing_but_padding(torch_cuda, batches, mode):  # noqa: F811
     h.destroy()
     for cnt in batches:
         infer_parity(torch_cuda, arrays, vectors(rng, cnt, n), max(batches), expect_nonempty=True)
+
+
+def rowwise(rp, cols, vals, bias, x, act):
+    """A layer in float64, entry by entry, so that what an entry does not read does not matter; NaN clamps to 0 as on the device."""
+    out = np.empty((len(x), len(rp) - 1))
+    for i in range(len(rp) - 1):
+        with np.errstate(invalid="ignore"):
+            z = bias[i] + (vals[rp[i]:rp[i + 1]].astype(np.float64) * x[:, cols[rp[i]:rp[i + 1]]]).sum(axis=1)
+        out[:, i] = 1.0 / (1.0 + np.exp(-z)) if act == "sigmoid" else np.where(np.isnan(z), 0.0, np.clip(z, 0.0, 32.0))
+    return out
+
+
+@pytest.mark.parametrize("n,cnt,ragged", [(640, 1500, False), (1000, 590, True), (1024, 2400, False), (1025, 7105, True), (2047, 591, False), (2048, 1777, True),
+                                          (2700, 3000, False), (3585, 2368, True), (4096, 1777, False), (4608, 1184, False), (7200, 591, True), (8192, 592, False)])
+def test_networks_held_in_shared_memory(torch_cuda, n, cnt, ragged):  # noqa: F811
+    """Batches that go through whole networks in one launch (or two, for a last round of another width): 4 to 16 inputs a CTA, outputs
+    that fit beside the inputs and outputs that wait in registers, last units and groups of eight of a few rows, empty rows, rows of 56; outputs
+    and counts, ids, host buffers, and new weights.  The layer launches add up in the same order."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n)
+    layers, act = 3, "clamped_relu" if n % 2 else "sigmoid"
+    if ragged:
+        rps, cols = [], []
+        for _ in range(layers):
+            length = rng.integers(0, 57, size=n)
+            rps.append(np.concatenate([[0], np.cumsum(length)]).astype(np.int32))
+            cols.append(np.concatenate([np.sort(rng.choice(n, size=m, replace=False)) for m in length]).astype(np.int32))
+    else:
+        rps, cols, _, _ = uniform_net(rng, n, 32, layers)
+    vals = [(rng.standard_normal(len(c)) * 0.25).astype(np.float32) for c in cols]
+    bias = [(rng.standard_normal(n) * 0.1).astype(np.float32) for _ in range(layers)]
+    h = pkg.Sdnn.create(rps, cols, vals, bias, max_batch=min(cnt, 1024), activation=pkg.ACT_SIGMOID if act == "sigmoid" else pkg.ACT_CLAMPED_RELU)
+    ora = OracleNet(rps, cols, vals, bias, activation=act)
+    x0 = vectors(rng, cnt, n)
+    x = torch.from_numpy(x0).cuda()
+    pick = np.unique(np.concatenate([[0, cnt - 1], rng.integers(0, cnt, size=30)]))
+
+    def call(**kw):
+        y, c = torch.full((cnt, n), -1.0, device="cuda"), torch.full((cnt,), -1, dtype=torch.int32, device="cuda")
+        before = h.kernel_launches()
+        total = h.infer_batch(x, cnt, y, c, **kw)
+        torch.cuda.synchronize()
+        return y.cpu().numpy(), c.cpu().numpy(), total, h.kernel_launches() - before
+    y, c, _, launches = call()
+    assert launches <= 2, "one launch for whole rounds of CTAs, one for what is left"
+    check_close(y[pick], ora.infer(x0[pick]), "x^L")
+    assert np.array_equal(c, np.count_nonzero(y, axis=1))
+
+    ids = torch.full((cnt * n,), -1, dtype=torch.int32, device="cuda")
+    y2, c2, total, _ = call(nz_index_out=ids, nz_index_capacity=cnt * n, want_total=True)
+    assert np.array_equal(y, y2) and np.array_equal(c, c2) and total == c.sum()
+    ids = ids.cpu().numpy()
+    assert np.array_equal(ids[:total], np.nonzero(y)[1]) and (ids[total:] == -1).all()
+
+    yh = np.empty((cnt, n), dtype=np.float32)
+    h.infer_batch(x0, cnt, yh, None, host=True)
+    few = torch.full((200, n), -1.0, device="cuda")
+    h.infer_batch(x, 200, few)                                     # through the layer launches
+    assert np.array_equal(yh, y) and np.array_equal(few.cpu().numpy(), y[:200]), "an input's outputs do not depend on its batch"
+    for l in range(layers):
+        w, b = h.get_weights(l)
+        assert np.array_equal(w, vals[l]) and np.array_equal(b, bias[l])
+
+    vals = [(rng.standard_normal(len(c)) * 0.25).astype(np.float32) for c in cols]
+    bias = [(rng.standard_normal(n) * 0.1).astype(np.float32) for _ in range(layers)]
+    for l in range(layers):
+        h.set_weights(l, vals[l], bias[l])
+    y, c, _, _ = call()
+    check_close(y[pick], OracleNet(rps, cols, vals, bias, activation=act).infer(x0[pick]), "x^L with new weights")
+
+    # what no entry reads does not reach a row: infinities and NaN in some inputs' neurons
+    x0[pick[1], :8] = np.inf
+    x0[pick[2], n // 2] = np.nan
+    x0[pick[3], n - 9:] = -np.inf
+    x = torch.from_numpy(x0).cuda()
+    y, c, _, _ = call()
+    want = x0[pick[:5]].astype(np.float64)
+    for l in range(layers):
+        want = rowwise(rps[l], cols[l], vals[l], bias[l], want, act)
+    assert np.array_equal(np.isnan(y[pick[:5]]), np.isnan(want))
+    check_close(np.nan_to_num(y[pick[:5]]), np.nan_to_num(want), "x^L of inputs that are not finite")
+    h.destroy()
+
+
+@pytest.mark.parametrize("n,cnt,tile", [(640, 2000, 1024), (1024, 1000, 1000), (2048, 1500, 600), (4096, 2500, 1024), (4096, 592, 592)])
+def test_dead_inputs_dropped_from_networks_held_in_shared_memory(torch_cuda, n, cnt, tile):  # noqa: F811
+    """Inputs that die at once, after some layers, or not at all: the same bits as without dropping them, and the live inputs of the last tile
+    after each layer; all inputs dead; none."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    layers, k = 14, 32
+    rp, cols, _, _ = uniform_net(rng, n, k, layers)
+    vals = [np.full(n * k, 1.0 / 16.0, dtype=np.float32)] * layers
+    bias = [np.full(n, -0.35, dtype=np.float32)] * layers
+    dense, drop = (pkg.Sdnn.create(rp, cols, vals, bias, max_batch=tile, flags=f) for f in (0, pkg.FLAG_SKIP_DEAD))
+    mixed = (rng.random((cnt, n)) < rng.uniform(0.05, 0.5, size=(cnt, 1))).astype(np.float32)
+    for x0 in (mixed, np.zeros_like(mixed), np.ones_like(mixed)):
+        x, outs = torch.from_numpy(x0).cuda(), []
+        for h in (dense, drop):
+            y, c = torch.full((cnt, n), -1.0, device="cuda"), torch.full((cnt,), -1, dtype=torch.int32, device="cuda")
+            ids = torch.full((cnt * n,), -1, dtype=torch.int32, device="cuda")
+            total = h.infer_batch(x, cnt, y, c, ids, cnt * n, want_total=True)
+            torch.cuda.synchronize()
+            outs.append((y.cpu().numpy(), c.cpu().numpy(), ids.cpu().numpy(), total))
+        assert all(np.array_equal(a, b) for a, b in zip(*outs))
+        last = (cnt - 1) // drop.infer_tile_width() * drop.infer_tile_width()
+        live, want = x0[last:], []
+        for l in range(layers):
+            live = np.clip(live[:, cols[l].reshape(n, k)].sum(axis=2) / 16.0 - 0.35, 0.0, 32.0)      # multiples of 1/16 from the 0/1 inputs of the first layer on
+            want.append(int(live.any(axis=1).sum()))
+            assert abs(int(drop.get_liveness()[l]) - want[-1]) <= 1, l      # rounding may keep the last neuron of an input alive
+    dense.destroy()
+    drop.destroy()

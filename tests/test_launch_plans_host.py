@@ -194,3 +194,114 @@ def test_whole_network_exchange_ends_when_a_message_is_lost(plan):
     with pytest.raises(Fault):
         for seed in range(25):
             exchange(10, 10, 6, random.Random(seed), mute=(3, 2), careless=True)
+
+
+RESIDENT = """
+#include "resident.h"
+using namespace sdnn_plan;
+extern "C" int width(int n, double elems, long long inputs, int sms, int tile, int drop) { return resident_width(n, elems, inputs, sms, tile, drop != 0); }
+extern "C" void shape(int n, int p, int* out) {
+    const ResidentShape s = resident_shape(n, p);
+    out[0] = s.ok; out[1] = s.units; out[2] = s.slots; out[3] = s.cap; out[4] = s.held;
+}
+extern "C" void share(int total, int sms, int p, int q, int* out) { resident_share(total, sms, p, q, out, out + 1); }
+// steps of a group: left[row][class] entries; read[step][row] = class, 8 + class of the zeros for a row that waits
+extern "C" void steps(int* left, int steps, int* read) {
+    int total[8] = {};
+    for (int r = 0; r < 8; ++r) for (int c = 0; c < 8; ++c) total[c] += left[r * 8 + c];
+    for (int t = 0; t < steps; ++t) {
+        uint64_t have = 0;
+        uint32_t must = 0;
+        for (int r = 0; r < 8; ++r) {
+            int togo = 0;
+            for (int c = 0; c < 8; ++c) { togo += left[r * 8 + c]; if (left[r * 8 + c]) have |= (uint64_t)1 << (8 * c + r); }
+            if (togo && togo >= steps - t) must |= 1u << r;
+        }
+        const uint32_t row = resident_step(have, total, must, steps - t);
+        for (int r = 0; r < 8; ++r) {
+            const int c = (row >> (4 * r)) & 15;
+            read[t * 8 + r] = c == 15 ? 8 + resident_idle_class(row, r) : c;
+            if (c != 15) { --left[r * 8 + c]; --total[c]; }
+        }
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def resident(tmp_path_factory):
+    d = tmp_path_factory.mktemp("resident")
+    src, lib = d / "resident.cpp", d / "libresident.so"
+    src.write_text(RESIDENT)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)])
+    lib = ctypes.CDLL(str(lib))
+    lib.width.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_longlong, ctypes.c_int, ctypes.c_int, ctypes.c_int]
+    return lib
+
+
+def test_shapes_of_networks_held_in_shared_memory(resident):
+    """Inputs, free slots and the units held in registers make room for a layer's outputs, within 226 KB; wider needs more room."""
+    out = (ctypes.c_int * 5)()
+    for n in list(range(1, 300)) + list(range(300, 9000, 37)) + [1024, 2048, 4096, 4608, 4609, 8192, 8193, 20000, 65536]:
+        fitted = True
+        for p in range(1, 5):
+            resident.shape(n, p, out)
+            ok, units, slots, cap, held = out
+            assert units * 32 >= n > (units - 1) * 32 and slots == units * 32 + 8
+            if not ok:
+                fitted = False
+                continue
+            assert fitted and cap * 16 * p <= 226 * 1024 and cap % 8 == 0 and slots <= cap
+            rounds = (units + 15) // 16
+            assert rounds >= held and (held or cap >= 2 * slots)
+            assert min(units, (rounds - held) * 16) * 32 <= cap - slots      # what is stored at once overwrites no input
+            assert held <= (4 if p <= 2 else 2)
+        if n > 8192:
+            assert not fitted and resident.width(n, 32.0 * n, 10000, 148, 1024, 0) == 0
+
+
+def test_shares_of_networks_held_in_shared_memory(resident):
+    """The launches of all widths take every input once; the last round is as narrow as it can be."""
+    out = (ctypes.c_int * 2)()
+    for sms in (1, 148):
+        for p in range(1, 5):
+            for total in list(range(0, 60)) + [4 * sms * q + d for q in range(1, 13) for d in (-1, 0, 1)] + [10000, 16384]:
+                taken = []
+                for q in range(p, 0, -1):
+                    resident.share(total, sms, p, q, out)
+                    taken += list(range(out[0], out[1]))
+                    if q < p:
+                        assert out[1] - out[0] <= 4 * q * sms
+                assert taken == list(range(total))
+
+
+@pytest.mark.parametrize("spread", [0, 1, 5])
+def test_steps_of_eight_rows(resident, spread):
+    """Every entry is read once, in as few wavefronts as the group's counts allow where the rows are of one length (the largest distance of a
+    class from the mean on top of one per step); rows that wait read zeros of a class that nobody else reads in that step."""
+    rng = random.Random(spread)
+    for case in range(200):
+        steps = rng.choice([4, 8, 32, 56, 248])
+        lens = [max(0, steps - rng.randint(0, spread)) if spread else steps for _ in range(8)]
+        skew = rng.choice([1, 1, 1, 4])
+        counts = (ctypes.c_int * 64)()
+        for r in range(8):
+            for _ in range(lens[r]):
+                counts[r * 8 + min(rng.randrange(8 * skew), 7)] += 1
+        before = list(counts)
+        total = [sum(before[c::8]) for c in range(8)]
+        read = (ctypes.c_int * (8 * steps))()
+        resident.steps(counts, steps, read)
+        assert not any(counts)
+        waves, seen = 0, [0] * 64
+        for t in range(steps):
+            row = list(read[t * 8:t * 8 + 8])
+            for r, c in enumerate(row):
+                if c < 8:
+                    seen[r * 8 + c] += 1
+            waits = [c - 8 for c in row if c >= 8]
+            assert len(set(waits)) == len(waits) and not set(waits) & {c for c in row if c < 8}
+            waves += max(row.count(c) for c in set(row))
+        assert seen == before
+        if not spread and skew == 1:
+            assert waves == steps + max(abs(c - steps) for c in total)
