@@ -1209,6 +1209,155 @@ backward_kernel(const BackwardArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------
+// Layers that do not fill the device (train steps; see sdnn_plan::split_units).  A launch of fewer row groups than warps fit is over when its
+// longest row is: 7 dependent round trips of 8 gathers for a row of 56 entries, while the short rows' warps have ended and the request
+// path idles.  Here the steps of a long row are dealt to 2, 4, .. groups of G lanes of a warp, whose partial sums meet in shuffles, as
+// far as all units still fit the device in one round: `units` lists, for every warp, its first row * 8 + log2(groups per row).
+// us a layer, as it was / split: 6007 neurons, rows of 8 to 56 entries, 37 inputs: forward 7.17 / 5.12, backward 8.37 / 7.01; 3000 neurons,
+// 32 a row, 12 inputs: 3.92 / 2.56, 5.11 / 3.92; 700 neurons, 64 inputs: 3.58 / 2.21, 4.77 / 3.24.
+struct SplitUnit { int row, part, parts; };
+template <int G>
+__device__ __forceinline__ SplitUnit split_unit(const unsigned* units, int u, int nunits, int grp) {
+    const unsigned d = u < nunits ? units[u] : 0xffffffffu;
+    const int ls = d & 7u;
+    if (d == 0xffffffffu) return SplitUnit{0x7fffffff, 0, 1};
+    return SplitUnit{(int)(d >> 3) + (grp >> ls), grp & ((1 << ls) - 1), 1 << ls};
+}
+template <int G, int V>
+__device__ __forceinline__ void split_join(Lane<V>& acc, int parts) {      // all lanes of the warp
+    for (int o = G; o < G * parts; o <<= 1) {
+        acc.a.x += __shfl_xor_sync(0xffffffffu, acc.a.x, o); acc.a.y += __shfl_xor_sync(0xffffffffu, acc.a.y, o);
+        acc.a.z += __shfl_xor_sync(0xffffffffu, acc.a.z, o); acc.a.w += __shfl_xor_sync(0xffffffffu, acc.a.w, o);
+        acc.b.x += __shfl_xor_sync(0xffffffffu, acc.b.x, o); acc.b.y += __shfl_xor_sync(0xffffffffu, acc.b.y, o);
+        acc.b.z += __shfl_xor_sync(0xffffffffu, acc.b.z, o); acc.b.w += __shfl_xor_sync(0xffffffffu, acc.b.w, o);
+    }
+}
+
+constexpr int SPLIT_WARPS = 4;      // of a forward CTA
+template <int G, bool I16>
+__global__ void __launch_bounds__(32 * SPLIT_WARPS, 16 / SPLIT_WARPS)
+forward_split_kernel(Sliced m, const unsigned* __restrict__ units, int nunits, const float* __restrict__ bias, const float* __restrict__ xin,
+                     float* __restrict__ xout, int n, float clamp, int act, int pdl, int last) {
+    constexpr int V = 8, CPS = 2;
+    constexpr unsigned pitch = 4u * V * G;
+    const int lane = threadIdx.x & 31, sub = lane % G;
+    const SplitUnit s = split_unit<G>(units, blockIdx.x * SPLIT_WARPS + (threadIdx.x >> 5), nunits, lane / G);
+    int nch = 0, base = 0, to = 0;
+    float b = 0.0f;
+    IdxChunk<I16> c[CPS];
+    if (s.row < n) {
+        const int so = m.slice_off[s.row / SLICE];
+        nch = (m.slice_off[s.row / SLICE + 1] - so) / CHUNK_ROW;
+        base = so + (s.row % SLICE) * 4;
+        to = m.out ? m.out[s.row] : s.row;
+        if (s.part == 0) b = bias[s.row];
+        if (s.part * CPS < nch) load_idx<CPS, I16>(c, m, base + s.part * CPS * CHUNK_ROW);
+    }
+    if (pdl) grid_dependency_wait();
+    if (pdl == 2) grid_launch_dependents();
+    Lane<V> acc;
+    lane_fill(acc, b);
+    const float* vp = m.val + base;
+    const float* xg = xin + min(sub * V, last);
+    for (int t = s.part * CPS; t < nch; t += s.parts * CPS) {
+        float4 w[CPS];
+        Lane<V> x[4 * CPS];
+#pragma unroll
+        for (int i = 0; i < CPS; ++i) w[i] = __ldcs(reinterpret_cast<const float4*>(vp + (t + i) * CHUNK_ROW));
+#pragma unroll
+        for (int i = 0; i < CPS; ++i) { SDNN_GATHER_CHUNK(x, i, c[i], xg, pitch) }
+        if (t + s.parts * CPS < nch) load_idx<CPS, I16>(c, m, base + (t + s.parts * CPS) * CHUNK_ROW);
+#pragma unroll
+        for (int i = 0; i < CPS; ++i) {
+            lane_fma(w[i].x, x[4 * i + 0], acc); lane_fma(w[i].y, x[4 * i + 1], acc);
+            lane_fma(w[i].z, x[4 * i + 2], acc); lane_fma(w[i].w, x[4 * i + 3], acc);
+        }
+    }
+    __syncwarp();
+    split_join<G, V>(acc, s.parts);
+    if (s.row < n && s.part == 0) {
+        lane_activate(acc, act, clamp);
+        lane_store(tile_row(xout + sub * V, to, pitch), acc);
+    }
+    if (pdl == 1) grid_launch_dependents();
+}
+
+// Column units: as backward_col_units, per entry the same arithmetic.  CTAs of one warp, like the launches they run beside.
+template <int G, bool I16>
+__global__ void __launch_bounds__(32, 16)
+backward_split_kernel(Sliced m, const unsigned* __restrict__ units, int nunits, const float* __restrict__ xprev, const float* __restrict__ dk,
+                      float* __restrict__ dprev, int n, float clamp, int act, const StepParams* __restrict__ sp, int pdl,
+                      const float* __restrict__ warm, unsigned warm_bytes) {
+    constexpr int V = 8, CPS = 2;
+    constexpr unsigned pitch = 4u * V * G;
+    const int lane = threadIdx.x, sub = lane % G;
+    if (warm && lane == 0) {
+        const unsigned pieces = (warm_bytes + 4095u) >> 12;
+        for (unsigned q = blockIdx.x; q < pieces; q += gridDim.x) {
+            const unsigned lo = q << 12, len = min(4096u, warm_bytes - lo);
+            prefetch_l2(reinterpret_cast<const char*>(warm) + lo, len & ~15u);
+        }
+    }
+    const float inv_b = sp->inv_b, step = sp->eta * inv_b;
+    const SplitUnit s = split_unit<G>(units, blockIdx.x, nunits, lane / G);
+    int nch = 0, base = 0, len = 0, j = 0;
+    IdxChunk<I16> c[CPS];
+#pragma unroll
+    for (int i = 0; i < CPS; ++i) idx_zero(c[i]);
+    Lane<V> xj, acc;
+    lane_fill(xj, 0.0f);
+    lane_fill(acc, 0.0f);
+    if (s.row < n) {
+        const int so = m.slice_off[s.row / SLICE];
+        nch = (m.slice_off[s.row / SLICE + 1] - so) / CHUNK_ROW;
+        base = so + (s.row % SLICE) * 4;
+        len = m.len[s.row]; j = m.order[s.row];
+        if (s.part * CPS < nch) load_idx<CPS, I16>(c, m, base + s.part * CPS * CHUNK_ROW);
+        lane_load(xj, tile_row(xprev + sub * V, j, pitch));
+    }
+    if (pdl) grid_dependency_wait();
+    if (pdl == 2) grid_launch_dependents();
+    float* vp = m.val + base;
+    const float* dg = dk + sub * V;
+    const int lim = len - ((G >= 4) ? (sub & 3) : (G == 2) ? 2 * sub : 0);
+    // rows of a slice take the same number of steps; a group beyond its last one goes through the shuffles with the others
+    const int most = __reduce_max_sync(0xffffffffu, nch);
+    for (int t0 = 0; t0 < most; t0 += s.parts * CPS) {
+        const int t = t0 + s.part * CPS;
+        float4 w[CPS];
+        Lane<V> d[4 * CPS];
+        if (t < nch) {
+#pragma unroll
+            for (int i = 0; i < CPS; ++i) w[i] = __ldcs(reinterpret_cast<const float4*>(vp + (t + i) * CHUNK_ROW));
+#pragma unroll
+            for (int i = 0; i < CPS; ++i) { SDNN_GATHER_CHUNK(d, i, c[i], dg, pitch) }
+            if (t + s.parts * CPS < nch) load_idx<CPS, I16>(c, m, base + (t + s.parts * CPS) * CHUNK_ROW);
+        } else {
+#pragma unroll
+            for (int i = 0; i < CPS; ++i) {
+                w[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                lane_fill(d[4 * i], 0.f); lane_fill(d[4 * i + 1], 0.f); lane_fill(d[4 * i + 2], 0.f); lane_fill(d[4 * i + 3], 0.f);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < CPS; ++i) {
+            lane_fma(w[i].x, d[4 * i + 0], acc); lane_fma(w[i].y, d[4 * i + 1], acc);
+            lane_fma(w[i].z, d[4 * i + 2], acc); lane_fma(w[i].w, d[4 * i + 3], acc);
+            float p0 = lane_dot(d[4 * i + 0], xj), p1 = lane_dot(d[4 * i + 1], xj), p2 = lane_dot(d[4 * i + 2], xj), p3 = lane_dot(d[4 * i + 3], xj);
+            chunk_sums<G>(p0, p1, p2, p3, sub, 0xffffffffu);
+            chunk_update<G, false>(vp + (t + i) * CHUNK_ROW, nullptr, w[i], p0, p1, p2, p3, sub, (t + i) * 4, lim, step, inv_b);
+        }
+    }
+    split_join<G, V>(acc, s.parts);
+    if (s.row < n && s.part == 0) {
+        lane_mask(acc, xj, act, clamp);
+        lane_store(tile_row(dprev + sub * V, j, pitch), acc);
+    }
+    if (pdl == 1) grid_launch_dependents();
+}
+
+// ---------------------------------------------------------------------------------------------
 // Layer kernels for tiles of padded width 4 (B <= 4: per-input SGD as in Algorithm 1, single vectors).
 // With so few batch entries a row's work is its entries, not its batch: a lane per row (the mapping above) leaves a
 // 1024-neuron layer to 32 warps that each walk 32 entries in four dependent steps.  Here a warp takes one SLICE of 16
@@ -1409,11 +1558,24 @@ struct Move {
     const unsigned short* pos_b;
     int nb, block;
 };
+// Trained biases: b^k -= step * sum over the batch of delta^k (one more column of W^k whose input is the constant 1), a thread per
+// stored row, in CTAs of the split launch behind those of the move: a launch of their own, which did not ask for the same split of an
+// SM's memory, kept the column units waiting (6007 neurons, 37 inputs: 9.4 -> 7.8 us a layer).  n = 0: frozen.  The padding columns of delta are zero.
+struct BiasUpdate { float* bias; const float* dk; const int* out; int n, ld; const StepParams* sp; };
 constexpr int MOVE_THREADS = 256;
 __global__ void __launch_bounds__(MOVE_THREADS, 4)
-split_values_kernel(Move m, const float* __restrict__ cval, int c_elems, float* __restrict__ T) {
+split_values_kernel(Move m, const float* __restrict__ cval, int c_elems, float* __restrict__ T, BiasUpdate u) {
     extern __shared__ __align__(16) float move_smem[];
     constexpr int AHEAD = 4;
+    if ((int)blockIdx.x >= m.nb) {
+        const int row = ((int)blockIdx.x - m.nb) * MOVE_THREADS + threadIdx.x;
+        if (row >= u.n) return;
+        const float* d = u.dk + (size_t)(u.out ? u.out[row] : row) * u.ld;
+        float s = 0.0f;
+        for (int b = 0; b < u.ld; b += 4) { const float4 v = ld_f4(d + b); s += (v.x + v.y) + (v.z + v.w); }
+        u.bias[row] -= u.sp->eta * u.sp->inv_b * s;
+        return;
+    }
     const int cb = blockIdx.x, lo = cb * m.block, cnt = min(m.block, c_elems - lo);      // both multiples of 4
     for (int q = threadIdx.x * 4; q < cnt; q += MOVE_THREADS * 4) cp_async16(move_smem + q, cval + lo + q);
     cp_async_commit();
@@ -1528,19 +1690,6 @@ __global__ void move_places_kernel(const int* __restrict__ from, int r_elems, in
         const int t = atomicAdd(cursor + (p / block) * nb + e / block, 1);
         pos_a[t] = (unsigned short)(p % block); pos_b[t] = (unsigned short)(e % block);
     }
-}
-
-// b^k -= step * sum over the batch of delta^k (biases trained: read as one more column of W^k whose input is the constant 1).
-// A thread per stored row; the padding columns of delta are zero.
-__global__ void __launch_bounds__(256)
-update_bias_kernel(float* __restrict__ bias, const float* __restrict__ dk, const int* __restrict__ out, int n, int ld,
-                   const StepParams* __restrict__ sp) {
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= n) return;
-    const float* d = dk + (size_t)(out ? out[row] : row) * ld;
-    float s = 0.0f;
-    for (int b = 0; b < ld; b += 4) { const float4 v = ld_f4(d + b); s += (v.x + v.y) + (v.z + v.w); }
-    bias[row] -= sp->eta * sp->inv_b * s;
 }
 
 // ---------------------------------------------------------------------------------------------

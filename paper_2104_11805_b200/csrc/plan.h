@@ -3,6 +3,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <vector>
 
 namespace sdnn_plan {
 
@@ -75,5 +76,46 @@ inline int pick_graph(const GraphKey* have, const int64_t* asked, int n, GraphKe
 constexpr int VECTOR_CTAS = 16, VECTOR_BLOCK = 64;
 // CTAs that have rows of a net of n neurons.  Only these exchange activations: see vector.cuh.
 constexpr int vector_ctas(int n) { return n > (VECTOR_CTAS - 1) * VECTOR_BLOCK ? VECTOR_CTAS : (n + VECTOR_BLOCK - 1) / VECTOR_BLOCK; }
+
+// Units of a layer that does not fill the device, one per warp (see forward_split_kernel): first row * 8 + log2 of the groups of
+// lanes that share a row.  off: offsets of the slices of 16 rows; a step is 8 entries of a row; `rows`: rows a warp works on at once with
+// a group each; `slots`: warps that fit the device.  A slice's rows are split into as many parts as bring its steps down to the fewest
+// that all units together leave room for.  Empty: nothing to gain by it.  So it is where the gathers of a launch (0.72, 0.57, 0.31 and
+// 0.15 rows of up to 64, 128, 256 and 512 bytes per clock and SM) outlast the round trips of its longest row (0.77 us each; 0.9 backward, where
+// the update of the other copy goes over the same path): 30000 neurons, 6 inputs, 4 steps forward 6.82 us as it is, 7.00 split, 16384: 4.77 and
+// 4.43; 16384, 28 inputs, backward 8.89 and 9.42, 10000: 8.03 and 7.01.
+inline std::vector<unsigned> split_units(const std::vector<int>& off, int n, int rows, int row_bytes, int sms, int64_t slots, bool backward) {
+    const int slices = (n + 15) / 16;
+    int longest = 0;
+    auto steps = [&](int s) { return (off[s + 1] - off[s]) / 128; };
+    for (int s = 0; s < slices; ++s) longest = std::max(longest, steps(s));
+    auto log_parts = [&](int s, int most) {
+        int ls = rows > 16 ? 1 : 0;
+        while ((rows >> (ls + 1)) >= 1 && ((steps(s) + (1 << ls) - 1) >> ls) > most) ++ls;
+        return ls;
+    };
+    auto units_of = [&](int s, int ls) { return (std::min(16, n - s * 16) + (rows >> ls) - 1) / (rows >> ls); };
+    const double rows_per_us = (row_bytes <= 64 ? 0.72 : row_bytes <= 128 ? 0.57 : row_bytes <= 256 ? 0.31 : 0.15) * 1900.0 * sms;
+    if (longest * (backward ? 0.9 : 0.77) < (backward ? 2.0 : 1.0) * off[slices] / rows_per_us) return {};
+    int pick = longest;
+    for (int most = longest - 1; most >= 1; --most) {
+        int64_t units = 0;
+        bool reached = true;
+        for (int s = 0; s < slices && reached; ++s) {
+            const int ls = log_parts(s, most);
+            reached = ((steps(s) + (1 << ls) - 1) >> ls) <= most;
+            units += units_of(s, ls);
+        }
+        if (!reached || units > slots) break;
+        pick = most;
+    }
+    std::vector<unsigned> list;
+    if (pick == longest) return list;
+    for (int s = 0; s < slices; ++s) {
+        const int ls = log_parts(s, pick);
+        for (int u = 0; u < units_of(s, ls); ++u) list.push_back((unsigned)(s * 16 + u * (rows >> ls)) << 3 | (unsigned)ls);
+    }
+    return list;
+}
 
 }  // namespace sdnn_plan

@@ -73,6 +73,8 @@ struct LayerMem {
     bool r_chunks_mult4 = false;           // every slice of the row-major copy has a multiple of 4 chunks
     int* r_idx = nullptr; float* r_val = nullptr; float* r_grad = nullptr;
     int* c_idx = nullptr; float* c_val = nullptr;
+    unsigned *r_units = nullptr, *c_units = nullptr;      // split_units of the two copies, for tiles of the handle's widest (NULL: none)
+    int r_nunits = 0, c_nunits = 0;
     Move move{};                           // how r_val is filled from c_val after an update (nb = 0: row units compute theirs)
     std::vector<int> r_slice_off;          // host copy of the row-major slice offsets
     RowShape shape;
@@ -572,10 +574,70 @@ bool entry_parallel(const sdnn* h, int ld) {
     return ld == 4 && !(h->cfg.flags & (SDNN_FLAG_BWD_ATOMICS | SDNN_FLAG_BWD_ONE_LAUNCH));
 }
 
+bool moved(const LayerMem& lm, int ld);
+float* delta_tile(sdnn* h, int layer, size_t tile);
+
+// Layers of a training handle that do not fill the device, at the width of its minibatches: units with long rows split
+template <int G, bool I16>
+void launch_forward_split(sdnn* h, int layer, const float* xin, float* xout, int last) {
+    const LayerMem& lm = h->lay[layer];
+    launch_k(h, forward_split_kernel<G, I16>, dim3((lm.r_nunits + SPLIT_WARPS - 1) / SPLIT_WARPS), dim3(32 * SPLIT_WARPS), h->pdl, rows_of(h, layer),
+             (const unsigned*)lm.r_units, lm.r_nunits, (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, h->cfg.clamp, h->cfg.activation,
+             h->pdl ? h->fwd_pdl : 0, last);
+    count_launch(h);
+}
+template <int G, bool I16>
+void launch_backward_split(sdnn* h, int layer, int ld) {
+    const LayerMem& lm = h->lay[layer];
+    const size_t tile = (size_t)h->N * ld;
+    const float* acts = h->bwd_acts ? h->bwd_acts : h->d_acts;
+    launch_on(h, backward_split_kernel<G, I16>, dim3(lm.c_nunits), dim3(32), 0, h->pdl, moved(lm, ld), cols_of(h, layer), (const unsigned*)lm.c_units, lm.c_nunits,
+              acts + (size_t)layer * tile, (const float*)delta_tile(h, layer, tile), delta_tile(h, layer - 1, tile), h->N, h->cfg.clamp, h->cfg.activation,
+              (const StepParams*)h->d_sp, h->pdl ? PDL_EARLY : 0, acts + (size_t)(layer - 1) * tile, (unsigned)(tile * sizeof(float)));
+    count_launch(h);
+}
+#define SDNN_BY_WIDTH(FN, ...)                            \
+    switch (h->ld_max) {                                  \
+        case 8: FN<1, I16>(__VA_ARGS__); break;           \
+        case 16: FN<2, I16>(__VA_ARGS__); break;          \
+        case 32: FN<4, I16>(__VA_ARGS__); break;          \
+        case 64: FN<8, I16>(__VA_ARGS__); break;          \
+        default: FN<16, I16>(__VA_ARGS__); break;         \
+    }
+
+// Lists the units of one copy of a layer for them (off: its slice offsets).  beside_rows: the launch shares the device with row units,
+// which are done later when it takes all of it (us per backward layer, none split / 70 % / 100 % of the warps that fit: 6007 neurons, 28
+// inputs 5.62 / 5.12 / 5.79, ragged 6.13 / 5.46 / 6.48; 16384, 12, ragged 9.40 / 8.36 / 9.38); moves leave it all (6007, 37: 8.37 / 7.34 / 7.01).
+template <bool I16>
+int build_units(sdnn* h, const std::vector<int>& off, bool backward, bool beside_rows, unsigned** units, int* nunits) {
+    if (!h->split || h->ld_max < 8 || h->ld_max > 128) return SDNN_OK;
+    const int block = backward ? 32 : 32 * SPLIT_WARPS;
+    const void* kernel = nullptr;
+#define SDNN_KERNEL(G_) backward ? (const void*)backward_split_kernel<G_, I16> : (const void*)forward_split_kernel<G_, I16>
+    switch (h->ld_max) {
+        case 8: kernel = SDNN_KERNEL(1); break;
+        case 16: kernel = SDNN_KERNEL(2); break;
+        case 32: kernel = SDNN_KERNEL(4); break;
+        case 64: kernel = SDNN_KERNEL(8); break;
+        default: kernel = SDNN_KERNEL(16); break;
+    }
+#undef SDNN_KERNEL
+    const int64_t slots = (int64_t)h->sms * resident_ctas(h, kernel, block) * (block / 32);
+    const std::vector<unsigned> list = split_units(off, h->N, 32 / (h->ld_max / 8), h->ld_max * 4, h->sms, beside_rows ? slots * 7 / 10 : slots, backward);
+    if (list.empty()) return SDNN_OK;
+    int rc;
+    if ((rc = dev_alloc(h, units, list.size(), false))) return rc;
+    CU(h, cudaMemcpyAsync(*units, list.data(), list.size() * sizeof(unsigned), cudaMemcpyHostToDevice, h->stream));
+    CU(h, cudaStreamSynchronize(h->stream));
+    *nunits = (int)list.size();
+    return SDNN_OK;
+}
+
 template <bool I16>
 void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used) {
     const Geometry q = geometry(cw);
     const int chunks = cols / cw, last = (used - 1) / q.v * q.v;
+    if (h->lay[layer].r_nunits && ld == h->ld_max && cols == ld) { SDNN_BY_WIDTH(launch_forward_split, h, layer, xin, xout, last) return; }
     if (q.v == 4 && entry_parallel(h, ld)) {
         const int wf = h->NS <= h->sms ? 1 : 4;      // few slices: one per CTA, so that they spread over as many SMs
         launch_k(h, forward_ep_kernel<I16>, dim3((h->NS + wf - 1) / wf), dim3(32 * wf), h->pdl, rows_of(h, layer),
@@ -798,6 +860,7 @@ void launch_backward_ep(sdnn* h, int layer, int part) {
 template <bool I16>
 void launch_backward_i(sdnn* h, int layer, int ld, int part) {
     const Geometry q = geometry(ld);
+    if (part == 1 && ld == h->ld_max && h->lay[layer].c_nunits) { SDNN_BY_WIDTH(launch_backward_split, h, layer, ld) return; }
     if (q.v == 4 && h->split && part != 0 && entry_parallel(h, ld)) launch_backward_ep<I16>(h, layer, part);
     else if (q.v == 4) launch_backward_gv<I16, 1, 4>(h, layer, ld, part);
     else switch (q.g) {
@@ -815,14 +878,10 @@ void launch_move(sdnn* h, int layer, int ld, int side) {
     const LayerMem& lm = h->lay[layer];
     const Move& m = lm.move;
     const size_t smem = (size_t)m.block * sizeof(float);
-    launch_on(h, split_values_kernel, dim3(m.nb), dim3(MOVE_THREADS), smem, false, true, m, (const float*)lm.c_val, (int)lm.c_elems, h->d_move[side]);
+    const BiasUpdate bias{h->d_bias + (size_t)layer * h->N, (const float*)delta_tile(h, layer, (size_t)h->N * ld), (const int*)lm.r_out, h->cfg.update_bias ? h->N : 0, ld, (const StepParams*)h->d_sp};
+    launch_on(h, split_values_kernel, dim3(m.nb + (bias.n + MOVE_THREADS - 1) / MOVE_THREADS), dim3(MOVE_THREADS), smem, false, true, m, (const float*)lm.c_val, (int)lm.c_elems, h->d_move[side], bias);
     launch_on(h, merge_values_kernel, dim3(m.nb), dim3(MOVE_THREADS), smem + (size_t)m.nb * sizeof(int2), false, true, m, (const float*)h->d_move[side], lm.r_val, (int)lm.r_elems);
     count_launch(h, 2);
-    if (h->cfg.update_bias) {
-        update_bias_kernel<<<(h->N + 255) / 256, 256, 0, h->launch_stream>>>(h->d_bias + (size_t)layer * h->N, (const float*)delta_tile(h, layer, (size_t)h->N * ld),
-                                                                           (const int*)lm.r_out, h->N, ld, (const StepParams*)h->d_sp);
-        count_launch(h);
-    }
 }
 
 void launch_backward(sdnn* h, int layer, int ld, int part = 0) {
@@ -1845,6 +1904,7 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
         if ((rc = dev_alloc(h, &lm.r_grad, (size_t)lm.r_elems, true))) return rc;
     CU(h, cudaMemcpyAsync(h->d_r_slice_off + (size_t)layer * (NS + 1), lm.r_slice_off.data(), (size_t)(NS + 1) * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CU(h, cudaMemcpyAsync(h->d_r_len + (size_t)layer * N, r_len.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    if ((rc = h->idx16 ? build_units<true>(h, lm.r_slice_off, false, false, &lm.r_units, &lm.r_nunits) : build_units<false>(h, lm.r_slice_off, false, false, &lm.r_units, &lm.r_nunits))) return rc;
     std::vector<float> bias_s;            // bias in stored order
     if (!perm.empty()) { bias_s.resize(N); for (int s = 0; s < N; ++s) bias_s[s] = bias[perm[s]]; }
     CU(h, cudaMemcpyAsync(h->d_bias + (size_t)layer * N, perm.empty() ? bias : bias_s.data(), (size_t)N * sizeof(float), cudaMemcpyHostToDevice, h->stream));
@@ -1906,6 +1966,7 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
                     c_idx[(size_t)sliced_pos(c_off.data(), place[j], q)] = out_label ? out_label[i] : i;      // the delta tile's row
                 }
         }
+        if ((rc = h->idx16 ? build_units<true>(h, c_off, true, !moves(lm, h->ld_max), &lm.c_units, &lm.c_nunits) : build_units<false>(h, c_off, true, !moves(lm, h->ld_max), &lm.c_units, &lm.c_nunits))) return rc;
         if ((rc = alloc_indices(h, &lm.c_idx, (size_t)lm.c_elems))) return rc;
         if ((rc = dev_alloc(h, &lm.c_val, (size_t)lm.c_elems, true))) return rc;
         CU(h, cudaMemcpyAsync(h->d_c_slice_off + (size_t)layer * (NS + 1), c_off.data(), (size_t)(NS + 1) * sizeof(int), cudaMemcpyHostToDevice, h->stream));

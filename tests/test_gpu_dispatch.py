@@ -500,3 +500,17 @@ def test_dead_inputs_dropped_from_networks_held_in_shared_memory(torch_cuda, n, 
             assert abs(int(drop.get_liveness()[l]) - want[-1]) <= 1, l      # rounding may keep the last neuron of an input alive
     dense.destroy()
     drop.destroy()
+
+
+@pytest.mark.parametrize("n,B", [(17, 8), (700, 6), (700, 100), (1500, 33), (3001, 16), (6007, 37), (9000, 20)])
+@pytest.mark.parametrize("ragged", [False, True])
+def test_layers_that_do_not_fill_the_device(torch_cuda, n, B, ragged):  # noqa: F811
+    """Train steps whose long rows and columns are split between groups of lanes (two, four, all of a warp's), trained and frozen biases."""
+    rng = np.random.default_rng(n + B)
+    if ragged:
+        arrays = ragged_net(rng, n=n, layers=3, kmax=min(n, 60), scale=0.3)
+    else:
+        arrays = uniform_net(rng, n, min(n // 2, 32), 3)
+    data = [(vectors(rng, B, n), vectors(rng, B, n)) for _ in range(2)]
+    train_parity(torch_cuda, arrays, data, eta=0.02, update_bias=True, activation="sigmoid", expect_live=True)
+    train_parity(torch_cuda, arrays, data[:1], eta=0.02, expect_live=True)

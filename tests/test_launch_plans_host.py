@@ -16,6 +16,11 @@ extern "C" int ctas(int n) { return vector_ctas(n); }
 extern "C" int cols(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cols; }
 extern "C" int chunk(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cw; }
 extern "C" int graph(int layers, long long elems, int cols, int track) { return tile_as_graph(layers, elems, cols, track); }
+extern "C" int units(const int* off, int n, int rows, int bytes, long long slots, int backward, unsigned* out) {
+    const std::vector<unsigned> list = split_units(std::vector<int>(off, off + (n + 15) / 16 + 1), n, rows, bytes, 148, slots, backward != 0);
+    std::copy(list.begin(), list.end(), out);
+    return (int)list.size();
+}
 extern "C" int graphs_made(const int* cols, const int* used, int calls, int* served_with) {
     GraphKey have[4];
     int64_t asked[4] = {};
@@ -45,6 +50,34 @@ def plan(tmp_path_factory):
         f.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
     lib.graph.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
     return lib
+
+
+@pytest.mark.parametrize("width", [8, 16, 32, 64, 128])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 700, 1500, 6007])
+def test_units_of_layers_that_do_not_fill_the_device(plan, width, n):
+    """Every row once, in units within a slice and with as many rows as groups of lanes are left for; no more units than fit; where there
+    are units, the longest chain is shorter than it was."""
+    plan.units.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_void_p]
+    rng = random.Random(n * width)
+    rows, slices = 32 // (width // 8), (n + 15) // 16
+    for steps in ([4] * slices, [rng.randint(0, 7) for _ in range(slices)], sorted((rng.randint(1, 9) for _ in range(slices)), reverse=True), [0] * slices):
+        off = [0]
+        for s in steps:
+            off.append(off[-1] + 128 * s)
+        arr, out = (ctypes.c_int * len(off))(*off), (ctypes.c_uint * (32 * slices + 32))()
+        for slots in (16, 1184, 2368):
+            for backward in (0, 1):
+                got = [out[i] for i in range(plan.units(arr, n, rows, 4 * width, slots, backward, out))]
+                if not got:
+                    continue
+                assert len(got) <= slots
+                taken, longest = [], 0
+                for d in got:
+                    row, parts = d >> 3, 1 << (d & 7)
+                    assert parts <= rows and row // 16 == (row + rows // parts - 1) // 16
+                    taken += [r for r in range(row, row + rows // parts) if r < n]
+                    longest = max(longest, -(-steps[row // 16] // parts))
+                assert taken == list(range(n)) and longest < max(steps)
 
 
 def test_tile_shapes(plan):
