@@ -194,6 +194,14 @@ __device__ __forceinline__ void lane_activate(Lane<8>& v, int act, float c) { f4
 __device__ __forceinline__ float lane_sum(const Lane<4>& v) { return v.a.x + v.a.y + v.a.z + v.a.w; }
 __device__ __forceinline__ float lane_sum(const Lane<8>& v) { return (v.a.x + v.a.y + v.a.z + v.a.w) + (v.b.x + v.b.y + v.b.z + v.b.w); }
 
+// acc += that of the lane whose number differs in bit(s) o; all lanes of the warp
+__device__ __forceinline__ void f4_join(float4& v, int o) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o); v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    v.z += __shfl_xor_sync(0xffffffffu, v.z, o); v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
+}
+__device__ __forceinline__ void lane_join(Lane<4>& v, int o) { f4_join(v.a, o); }
+__device__ __forceinline__ void lane_join(Lane<8>& v, int o) { f4_join(v.a, o); f4_join(v.b, o); }
+
 __device__ __forceinline__ bool f4_any(const float4& v) { return !(v.x == 0.0f && v.y == 0.0f && v.z == 0.0f && v.w == 0.0f); }
 __device__ __forceinline__ bool lane_any(const Lane<4>& v) { return f4_any(v.a); }
 __device__ __forceinline__ bool lane_any(const Lane<8>& v) { return f4_any(v.a) || f4_any(v.b); }
@@ -411,29 +419,35 @@ start_step_kernel(const float* __restrict__ x0, float* __restrict__ x_tile, cons
 // belong to the caller and cannot be re-laid out (sdnn_infer_noalloc).
 // The arrays are the caller's and were never validated on the host: a column index outside [0, n) is not followed
 // (its entry contributes nothing) and is counted in *bad_columns, which the host can read afterwards.
-// G lanes share a row, V inputs each.  Rows start anywhere, so the lanes of a row fetch the entries of a step (each lane OWN of
+// G lanes hold V inputs each, and S groups of G lanes share a row: group s takes STEP entries of every STEP * S, and the groups' sums meet in
+// shuffles.  Rows start anywhere, so the lanes of a group fetch the entries of a step (each lane OWN of
 // them side by side, one step ahead; as vectors where the row starts at a multiple of four), check their columns once and hand them
-// round by shuffles: STEP gathers of every row are in flight whatever the row's alignment (rows of 8 .. 56 entries, 4096
+// round by shuffles: STEP gathers of every group are in flight whatever the row's alignment (rows of 8 .. 56 entries, 4096
 // neurons, 100 inputs: 14.7 -> 8.5 us per layer, where rows off a multiple of four had taken their entries one at a time).
-template <int G, int V, int STEP>
+template <int G, int V, int STEP, int S>
 __global__ void __launch_bounds__(256)
 forward_csr_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ val,
                    const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
                    int n, int ld, int last, float clamp, unsigned long long* __restrict__ bad_columns) {
-    constexpr int RPW = 32 / G, OWN = (STEP + G - 1) / G;      // entries of a step that a lane fetches (G > STEP: only the first STEP lanes do)
+    constexpr int RPW = 32 / (G * S), OWN = (STEP + G - 1) / G;      // entries of a step that a lane fetches (G > STEP: only the first STEP lanes do)
     const int lane = threadIdx.x & 31;
-    const int sub = lane % G, lead = lane - sub;
-    const int row = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RPW + lane / G;
+    const int sub = lane % G, lead = lane - sub, part = lane / G % S;
+    const int row = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RPW + lane / (G * S);
     int p = 0, e = 0;
     float b = 0.0f;
-    if (row < n) { p = row_ptr[row]; e = row_ptr[row + 1]; b = bias[row]; }
+    if (row < n) { p = row_ptr[row]; e = row_ptr[row + 1]; if (part == 0) b = bias[row]; }
+    // the rows of a warp take as many steps as its longest: the shuffles want all lanes
+    int steps = (e - p + STEP * S - 1) / (STEP * S);
+#pragma unroll
+    for (int o = G * S; o < 32; o <<= 1) steps = max(steps, __shfl_xor_sync(0xffffffffu, steps, o));
+    const bool aligned = (p & 3) == 0;
+    p += part * STEP;
     const int boff = blockIdx.y * (V * G) + sub * V;
     const float* xg = xin + min(boff, last);      // lanes of nothing but padding gather what the last lane with inputs does (no sector more)
     const unsigned pitch = (unsigned)ld * 4u;
     unsigned bad = 0;
     int c[OWN];
     float w[OWN];
-    const bool aligned = (p & 3) == 0;
     auto fetch = [&](int at) {
         const int first = at + sub * OWN;
         if (OWN >= 4 && aligned && first + OWN <= e) {
@@ -461,11 +475,7 @@ forward_csr_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
     grid_launch_dependents();
     Lane<V> acc;
     lane_fill(acc, b);
-    // the rows of a warp take as many steps as its longest: the shuffles want all lanes
-    int steps = (e - p + STEP - 1) / STEP;
-#pragma unroll
-    for (int o = G; o < 32; o <<= 1) steps = max(steps, __shfl_xor_sync(0xffffffffu, steps, o));
-    for (int t = 0; t < steps; ++t, p += STEP) {
+    for (int t = 0; t < steps; ++t, p += STEP * S) {
         Lane<V> x[STEP];
         float ww[STEP];
 #pragma unroll
@@ -474,12 +484,14 @@ forward_csr_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
             ww[j] = __shfl_sync(0xffffffffu, w[j % OWN], lead + j / OWN);
             if (p + j < e) lane_gather(x[j], tile_row(xg, cc, pitch)); else lane_fill(x[j], 0.0f);
         }
-        fetch(p + STEP);
+        fetch(p + STEP * S);
 #pragma unroll
         for (int j = 0; j < STEP; ++j) if (p + j < e) lane_fma(ww[j], x[j], acc);
     }
+#pragma unroll
+    for (int o = G; o < G * S; o <<= 1) lane_join(acc, o);
     if (bad) atomicAdd(bad_columns, (unsigned long long)bad);
-    if (row < n) {
+    if (row < n && part == 0) {
         lane_activate(acc, ACT_CLAMPED_RELU, clamp);
         lane_store(tile_row(xout + boff, row, pitch), acc);
     }
@@ -1223,15 +1235,6 @@ __device__ __forceinline__ SplitUnit split_unit(const unsigned* units, int u, in
     if (d == 0xffffffffu) return SplitUnit{0x7fffffff, 0, 1};
     return SplitUnit{(int)(d >> 3) + (grp >> ls), grp & ((1 << ls) - 1), 1 << ls};
 }
-template <int G, int V>
-__device__ __forceinline__ void split_join(Lane<V>& acc, int parts) {      // all lanes of the warp
-    for (int o = G; o < G * parts; o <<= 1) {
-        acc.a.x += __shfl_xor_sync(0xffffffffu, acc.a.x, o); acc.a.y += __shfl_xor_sync(0xffffffffu, acc.a.y, o);
-        acc.a.z += __shfl_xor_sync(0xffffffffu, acc.a.z, o); acc.a.w += __shfl_xor_sync(0xffffffffu, acc.a.w, o);
-        acc.b.x += __shfl_xor_sync(0xffffffffu, acc.b.x, o); acc.b.y += __shfl_xor_sync(0xffffffffu, acc.b.y, o);
-        acc.b.z += __shfl_xor_sync(0xffffffffu, acc.b.z, o); acc.b.w += __shfl_xor_sync(0xffffffffu, acc.b.w, o);
-    }
-}
 
 constexpr int SPLIT_WARPS = 4;      // of a forward CTA
 template <int G, bool I16>
@@ -1274,7 +1277,7 @@ forward_split_kernel(Sliced m, const unsigned* __restrict__ units, int nunits, c
         }
     }
     __syncwarp();
-    split_join<G, V>(acc, s.parts);
+    for (int o = G; o < G * s.parts; o <<= 1) lane_join(acc, o);
     if (s.row < n && s.part == 0) {
         lane_activate(acc, act, clamp);
         lane_store(tile_row(xout + sub * V, to, pitch), acc);
@@ -1349,7 +1352,7 @@ backward_split_kernel(Sliced m, const unsigned* __restrict__ units, int nunits, 
             chunk_update<G, false>(vp + (t + i) * CHUNK_ROW, nullptr, w[i], p0, p1, p2, p3, sub, (t + i) * 4, lim, step, inv_b);
         }
     }
-    split_join<G, V>(acc, s.parts);
+    for (int o = G; o < G * s.parts; o <<= 1) lane_join(acc, o);
     if (s.row < n && s.part == 0) {
         lane_mask(acc, xj, act, clamp);
         lane_store(tile_row(dprev + sub * V, j, pitch), acc);

@@ -3377,19 +3377,19 @@ int noalloc_scratch(float** out, unsigned long long** bad_out) {
 }
 
 // a layer may start its prologue (its rows' places, first entries) under the tail of the one before
-template <int G, int V, int STEP = 8>
+template <int G, int V, int STEP, int S>
 void noalloc_forward_g(cudaStream_t st, const int* rp, const int* col, const float* val, const float* bias,
                        const float* xin, float* xout, int n, int ld, int chunks, int n_inputs, float clamp, unsigned long long* bad) {
     // small CTAs spread a narrow layer over more SMs and end in finer tails (1024 uniform rows, 4 inputs, 32 warps: 4.2 us a layer
     // with CTAs of two warps, 4.5 of four, 5.7 of eight); from 4096 warps on two and four are within 1 % (16384 x 64: 12.18 / 12.24)
-    const int warps = (n + 32 / G - 1) / (32 / G), wpb = warps * chunks < 4096 ? 2 : 4;
+    const int warps = (n + 32 / (G * S) - 1) / (32 / (G * S)), wpb = warps * chunks < 4096 ? 2 : 4;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((warps + wpb - 1) / wpb, chunks); lc.blockDim = dim3(32 * wpb); lc.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at; lc.numAttrs = 1;
-    cudaLaunchKernelEx(&lc, forward_csr_kernel<G, V, STEP>, rp, col, val, bias, xin, xout, n, ld, (n_inputs - 1) / V * V, clamp, bad);
+    cudaLaunchKernelEx(&lc, forward_csr_kernel<G, V, STEP, S>, rp, col, val, bias, xin, xout, n, ld, (n_inputs - 1) / V * V, clamp, bad);
 }
 
 }  // namespace
@@ -3434,20 +3434,21 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
         const float* val = values + layer_offset[l];
         const float* b = bias + (size_t)l * n_neurons;
 #define SDNN_NOALLOC(...) noalloc_forward_g<__VA_ARGS__>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, chunks, n_inputs, clamp, bad)
-        // Lanes per row, inputs per lane, entries of a row in flight per step.  At 4, 16 and 32 inputs the gathers of a row fit
-        // the registers 16 at a time, in lanes of four inputs; from 64 on a row has lanes enough, and 16 lose on the wider nets.  At 8 a
-        // lane a row is the better one only for the widest nets: two lanes are the variant to take for the others, not taken yet.
-        // us per layer of 24, rows of 8 to 56 entries, 4096 neurons (16384 in brackets), this / the other: 4 inputs <1,4,8> 6.9 / 7.2
-        // (8.6 / 9.0); 8 inputs <2,4,16> 7.9 / 5.8 (9.7 / 7.6; 65536 neurons 18.4 / 19.6); 16 inputs <4,4,8> 5.2 / 5.6 (7.9 / 7.6),
-        // <2,8,8> 5.2 / 8.6 (7.9 / 10.5); 32 inputs <8,4,8> 5.0 / 5.7 (11.9 / 12.1), <4,8,8> 5.0 / 6.9 (11.9 / 10.2); 64 inputs
-        // <16,4,16> 6.9 / 6.6 (16.2 / 20.0); 128 inputs <32,4,16> 8.3 / 10.7, <32,4,8> 8.3 / 7.9.
+        // Lanes per group, inputs per lane, entries of a group in flight per step, groups per row.  A launch of few rows is over when its
+        // longest row is: the row goes to as many groups as 2048 warps (the device's fill) leave room for; with one lane a group four
+        // pay at any size, eight up to 5000 rows.  us per layer of 24, 4096 rows of 8 to 56 entries (of 32 in brackets), one group / this:
+        // 4 inputs 6.9 / 2.8 (4.5 / 2.8), 8 inputs 7.8 / 3.0 (5.1 / 3.1), 16 inputs 5.3 / 3.4 (3.7 / 3.4), 32 inputs 5.2 / 4.2
+        // (3.9 / 3.4), 64 inputs 7.1 / 5.8 (5.4 / 4.4); 700 rows, 128 inputs 6.3 / 4.5 (4.9 / 3.4), 8 inputs 7.3 / 2.5.  More rows than that:
+        // 128 inputs, 4096 rows 8.5 with one group, 9.0 with two; 16 inputs, 16000 rows lanes of four inputs 8.2, two groups 8.4.
+        const int fill = 2048 * 32;      // lanes
+        const int groups = (int)std::min<int64_t>(8, fill / std::max<int64_t>(1, (int64_t)n_neurons * std::max(1, ld / chunks / 8)));
         switch (ld / chunks) {
-            case 4: SDNN_NOALLOC(1, 4, 16); break;
-            case 8: SDNN_NOALLOC(1, 8); break;
-            case 16: SDNN_NOALLOC(4, 4, 16); break;
-            case 32: SDNN_NOALLOC(8, 4, 16); break;
-            case 64: SDNN_NOALLOC(8, 8); break;
-            default: SDNN_NOALLOC(16, 8); break;
+            case 4: if (n_neurons <= 5120) SDNN_NOALLOC(1, 4, 8, 8); else SDNN_NOALLOC(1, 4, 8, 4); break;
+            case 8: if (n_neurons <= 5120) SDNN_NOALLOC(1, 8, 8, 8); else SDNN_NOALLOC(1, 8, 8, 4); break;
+            case 16: if (groups >= 8) SDNN_NOALLOC(2, 8, 8, 8); else if (groups >= 4) SDNN_NOALLOC(2, 8, 8, 4); else SDNN_NOALLOC(4, 4, 16, 1); break;
+            case 32: if (groups >= 8) SDNN_NOALLOC(4, 8, 8, 8); else if (groups >= 4) SDNN_NOALLOC(4, 8, 8, 4); else if (groups >= 2) SDNN_NOALLOC(4, 8, 8, 2); else SDNN_NOALLOC(4, 8, 8, 1); break;
+            case 64: if (groups >= 4) SDNN_NOALLOC(8, 8, 8, 4); else if (groups >= 2) SDNN_NOALLOC(8, 8, 8, 2); else SDNN_NOALLOC(8, 8, 8, 1); break;
+            default: if (groups >= 2) SDNN_NOALLOC(16, 8, 8, 2); else SDNN_NOALLOC(16, 8, 8, 1); break;
         }
 #undef SDNN_NOALLOC
         cur ^= 1;

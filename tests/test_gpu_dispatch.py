@@ -514,3 +514,30 @@ def test_layers_that_do_not_fill_the_device(torch_cuda, n, B, ragged):  # noqa: 
     data = [(vectors(rng, B, n), vectors(rng, B, n)) for _ in range(2)]
     train_parity(torch_cuda, arrays, data, eta=0.02, update_bias=True, activation="sigmoid", expect_live=True)
     train_parity(torch_cuda, arrays, data[:1], eta=0.02, expect_live=True)
+
+
+@pytest.mark.parametrize("n,cnt", [(5120, 3), (5121, 4), (5000, 7), (6001, 5), (4096, 12), (8192, 16), (8193, 9), (2048, 28), (4097, 20), (8000, 32), (17001, 28),
+                                   (2048, 50), (4001, 64), (4097, 33), (2048, 100), (2049, 100), (1500, 250)])
+def test_allocation_free_call_with_rows_shared_by_groups_of_lanes(torch_cuda, n, cnt):  # noqa: F811
+    """One, two, four and eight groups of lanes to a row of the caller's CSR arrays, on either side of each rule; rows of 0 to 150 entries
+    from any alignment, so that some take several steps of all groups and some not one."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    rp, cols, vals, bias = ragged_net(rng, n=n, layers=2, kmax=40, scale=0.3)
+    for l in range(2):                                       # some rows much longer than the others
+        length = np.diff(rp[l])
+        length[rng.integers(0, n, size=20)] = 150
+        rp[l] = np.concatenate([[0], np.cumsum(length)]).astype(np.int32)
+        cols[l] = np.concatenate([np.sort(rng.choice(n, size=m, replace=False)) for m in length]).astype(np.int32)
+        vals[l] = (rng.standard_normal(rp[l][-1]) * 0.3).astype(np.float32)
+    at = [0, (len(cols[0]) + 3) // 4 * 4]
+    col, val = np.zeros(at[1] + len(cols[1]), dtype=np.int32), np.zeros(at[1] + len(cols[1]), dtype=np.float32)
+    for l in range(2):
+        col[at[l]:at[l] + len(cols[l])] = cols[l]
+        val[at[l]:at[l] + len(vals[l])] = vals[l]
+    x0 = vectors(rng, cnt, n)
+    got = torch.full((cnt, n), -1.0, device="cuda")
+    pkg.infer_noalloc(2, n, *(torch.from_numpy(a).cuda() for a in (np.stack(rp), col, val)), np.asarray(at, dtype=np.int64),
+                      torch.from_numpy(np.stack(bias)).cuda(), torch.from_numpy(x0).cuda(), cnt, got)
+    torch.cuda.synchronize()
+    check_close(got.cpu().numpy(), OracleNet(rp, cols, vals, bias).infer(x0), f"{n} neurons, {cnt} inputs")
