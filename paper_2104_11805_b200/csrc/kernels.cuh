@@ -1735,21 +1735,18 @@ __global__ void mirror_values_kernel(Sliced rows, Sliced cols, int n, unsigned l
 // its len[s] entries at start[s] .. of the caller's array (start NULL: at s * k, every row k long).  A warp takes a row: its
 // side of the CSR array is contiguous, and the 16-byte pieces of the sliced side share their lines with the 15 other rows
 // of the slice, which the warps of the same CTA read (both sides together run at HBM rate, 4 us for 2 M entries; what the
-// calls wait for is the copy over PCIe).  TO_CSR false: CSR -> sliced.  order (or NULL): which of a row's entries is stored at each
-// place, for rows whose entries are not in the caller's order (resident.cuh).
+// calls wait for is the copy over PCIe).  TO_CSR false: CSR -> sliced.
 template <bool TO_CSR>
 __global__ void __launch_bounds__(512)
-sliced_csr_kernel(Sliced m, float* __restrict__ csr, const int* __restrict__ start, int k, int n, const unsigned char* __restrict__ order) {
+sliced_csr_kernel(Sliced m, float* __restrict__ csr, const int* __restrict__ start, int k, int n) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= n) return;
     const int len = m.len[row];
     const size_t at = start ? (size_t)start[row] : (size_t)row * k;
-    const int base = m.slice_off[row / SLICE] + (row % SLICE) * 4;
+    float* v = m.val + m.slice_off[row / SLICE] + (row % SLICE) * 4;
     for (int q = threadIdx.x & 31; q < len; q += 32) {
-        const int p = base + (q >> 2) * CHUNK_ROW + (q & 3);
-        float& w = m.val[p];
-        float& c = csr[at + (order ? order[p] : q)];
-        if (TO_CSR) c = w; else w = c;
+        float& w = v[(q >> 2) * CHUNK_ROW + (q & 3)];
+        if (TO_CSR) csr[at + q] = w; else w = csr[at + q];
     }
 }
 

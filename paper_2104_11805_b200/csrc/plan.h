@@ -51,14 +51,14 @@ inline bool tile_as_graph(int layers, int64_t elems, int cols, bool track) { ret
 // the one not asked for longest makes room for one that serves any tile of this shape.  So batches that vary at will make a lane
 // fill its places, and after that one graph per shape (as long as there are no more shapes than places).
 // Returns the place; `make` is set where the graph has to be made first, with want.used columns (which may have been raised).
-struct GraphKey { int cw = 0, cols = 0, used = 0, pdl = 0; bool track = false; };
+struct GraphKey { int cw = 0, cols = 0, used = 0, pdl = 0; bool track = false, other = false; };      // other: of the reordered copies
 inline int pick_graph(const GraphKey* have, const int64_t* asked, int n, GraphKey& want, bool& make) {      // asked[q] = 0: empty
     int room = -1, serves = -1, oldest = 0;
     make = false;
     for (int q = 0; q < n; ++q) {
         if (!asked[q]) { if (room < 0) room = q; continue; }
         const GraphKey& g = have[q];
-        if (g.cw == want.cw && g.cols == want.cols && g.pdl == want.pdl && g.track == want.track && g.used >= want.used) {
+        if (g.cw == want.cw && g.cols == want.cols && g.pdl == want.pdl && g.track == want.track && g.other == want.other && g.used >= want.used) {
             if (g.used == want.used) return q;
             if (serves < 0 || g.used < have[serves].used) serves = q;
         }

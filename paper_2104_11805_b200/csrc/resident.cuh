@@ -10,8 +10,9 @@
 // 8.  Random columns meet (2.5 wavefronts where one would do).  So the rows of a unit of 32 are chosen, and the order in which
 // each reads its entries laid down, when the net is loaded: resident_order_kernel picks groups of eight rows whose columns
 // spread evenly over the eight classes, resident_fill_kernel orders their entries step by step (resident.h).  1.06 wavefronts per
-// eight entries are left at 32 random columns a row.  The order of a row's sum is all that this changes; the layer launches take
-// over the same order (resident_reorder_kernel), so results do not depend on how a batch is cut.  A row that has nothing to read in a step reads one of eight slots of zeros.
+// eight entries are left at 32 random columns a row.  The order of a row's sum is all that this changes; it is the same for every
+// width, so results do not depend on how a batch is cut into CTAs.  The layer launches keep the ascending order (in this one their gathers
+// find less in L1: 4096 neurons, 128 inputs 4.91 -> 5.25 us a layer).  A row that has nothing to read in a step reads one of eight slots of zeros.
 //
 // Neurons are numbered by the place that their row was given: outputs are stored side by side, and columns name slots.
 // Memory: a ring of slots.  A layer's outputs go behind its inputs; where both do not fit (4096 neurons, 8 inputs: 128 KB of
@@ -344,7 +345,7 @@ struct ResidentSetup {
     const float* const* bias;           // [layers] in stored order
     const unsigned short* row0;         // [layers][n] stored row at each place, or NULL: identity
     const unsigned short* place0;       // [layers][n] place of each neuron, or NULL: identity
-    unsigned char* const* order;        // [layers] which of a row's entries is read at each place of the sliced copy
+    unsigned char* const* order;        // [layers] which of a row's entries (by their places in the sliced copy) is read at each place
     int layer0;                         // first layer of the launch
 };
 
@@ -501,36 +502,24 @@ resident_fill_kernel(Resident net, ResidentSetup s, int pitch) {
     }
 }
 
-// The sliced copies' rows in the same order (a warp a row), so that the layer launches add up a row's entries as this kernel does: an
-// input's outputs have the same bits whichever way its batch goes.
+// The sliced copies once more with their rows' entries in that order (a warp a row), for handles that drop dead inputs: where a batch is
+// too small to be dropped this way but goes this way without dropping, the layer launches read these, so that dropping changes no bit.
 __global__ void __launch_bounds__(256)
-resident_reorder_kernel(ResidentSetup s, int n) {
-    const int k = s.layer0 + blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+resident_reorder_kernel(ResidentSetup s, int n, int* const* idx, float* const* val) {
+    const int k = s.layer0 + blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (row >= n) return;
     const Sliced m = s.rows[k];
     const int len = m.len[row], at = m.slice_off[row / SLICE] + (row % SLICE) * 4;
     auto entry = [&](int q) { return at + (q >> 2) * CHUNK_ROW + (q & 3); };
-    constexpr int MOST = (RES_MAX_ROW + 31) / 32;
-    int col[MOST];
-    float val[MOST];
-#pragma unroll
-    for (int i = 0; i < MOST; ++i) {
-        const int q = i * 32 + lane, from = q < len ? entry(s.order[k][entry(q)]) : 0;
-        col[i] = q < len ? load_idx1(m, from) : 0;
-        val[i] = q < len ? m.val[from] : 0.0f;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < MOST; ++i) {
-        const int q = i * 32 + lane;
-        if (q >= len) continue;
-        if (m.idx16) reinterpret_cast<unsigned short*>(const_cast<int*>(m.idx))[entry(q)] = (unsigned short)col[i];
-        else const_cast<int*>(m.idx)[entry(q)] = col[i];
-        m.val[entry(q)] = val[i];
+    for (int q = threadIdx.x & 31; q < len; q += 32) {
+        const int from = entry(s.order[k][entry(q)]);
+        if (m.idx16) reinterpret_cast<unsigned short*>(idx[k])[entry(q)] = (unsigned short)load_idx1(m, from);
+        else idx[k][entry(q)] = load_idx1(m, from);
+        val[k][entry(q)] = m.val[from];
     }
 }
 
-// New values and biases, from the sliced copy: a unit per block of one warp.  A row's entries stand in the order in which it reads them.
+// New values and biases, from the sliced copy: a unit per block of one warp.
 __global__ void __launch_bounds__(32)
 resident_refill_kernel(Resident net, ResidentSetup s) {
     const int k = s.layer0, u = blockIdx.x, lane = threadIdx.x, place = u * RES_UNIT + lane;
@@ -543,7 +532,8 @@ resident_refill_kernel(Resident net, ResidentSetup s) {
     for (int t = 0, q = 0; t < steps; ++t) {
         const size_t o = ((size_t)(q0 + (t >> 2)) * 32 + lane) * 4 + (t & 3);
         if (net.col[o] >= net.units * RES_UNIT) continue;      // a step in which the row waits
-        net.val[o] = m.val[at + (q >> 2) * CHUNK_ROW + (q & 3)];
+        const int from = s.order[k][at + (q >> 2) * CHUNK_ROW + (q & 3)];
+        net.val[o] = m.val[at + (from >> 2) * CHUNK_ROW + (from & 3)];
         ++q;
     }
 }

@@ -182,4 +182,14 @@ inline int resident_width(int n, double elems, int64_t inputs, int sms, int tile
     return best;
 }
 
+// A batch from host memory that is one tile goes in two pieces, so that one's copies run under the other's layers.  Halves of 4 inputs a
+// CTA whose CTAs fit the device together cost no round of their own (us, layer launches / halves: 3000 x 40, 592 inputs 952 / 717, rows of 8 to
+// 56 entries 957 / 829; 1500 x 60 738 / 521; 700 x 60, 300 inputs 344 / 292).  Not where the copies weigh as much as the layers (4096 x 40, 592
+// inputs 1003 / 974 and 1082 / 1150), nor as 8 and 4 inputs a CTA beyond that (3000 x 40, 700 inputs 927 / 931, 4096 x 40, 900 1434 / 1487): there both
+// halves go through the layer launches, which fill each other's gaps.  Returns the inputs of the first half, 0: not this way.
+constexpr int RES_HALVES = 3072;      // most neurons
+inline int resident_half(int n, int64_t inputs, int sms) {
+    return n <= RES_HALVES && inputs >= 8 && (inputs + 3) / 4 <= sms ? (int)((inputs + 7) / 8) * 4 : 0;
+}
+
 }  // namespace sdnn_plan

@@ -84,7 +84,7 @@ struct LayerMem {
     int* r_start = nullptr;                // ... the same on the device (ragged layers whose entries keep the caller's order; else NULL)
     std::vector<int> entry_src;            // [nnz] entry in stored order (stored rows, their entries in stored order) -> caller's position
     int* r_out = nullptr;                  // rows not stored in neuron order: tile row each stored row writes (device, [N])
-    unsigned char* r_order = nullptr;      // which of a row's entries is stored at each place (NULL: in the caller's order; see resident_reorder_kernel)
+    int* r_idx2 = nullptr; float* r_val2 = nullptr;      // the row-major copy with rows in resident_infer_kernel's order (see resident_reorder_kernel)
     int* r_row_of = nullptr;               // ... and its inverse: stored row that holds neuron (tile row) i (device, [N])
     // windowed layer: rows grouped by shared columns, the group's window staged in shared memory (forward_window_kernel)
     bool windowed = false;
@@ -179,6 +179,8 @@ struct sdnn {
     Resident resident{};                // the net as resident_infer_kernel reads it (units = 0: it does not)
     ResidentSetup resident_setup{};
     double resident_elems = 0;          // stored elements per layer there, padding included
+    int* const* resident_idx2 = nullptr; float* const* resident_val2 = nullptr;      // device: [L] r_idx2, r_val2 (NULL: none)
+    bool other_rows = false;            // the launch helpers currently read those
     bool compaction = false;            // SDNN_FLAG_SKIP_DEAD asked for; effective while no bias is positive
     std::vector<char> bias_nonpositive; // per layer
     bool live_valid = false;
@@ -552,7 +554,9 @@ template <bool I16, int G, int V>
 void launch_forward_tracked(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
     const int units = (h->N + 32 / G - 1) / (32 / G), chunks = cols / (V * G);
     auto plan = plan_grid(h, (const void*)forward_kernel<G, V, 2, I16, false, false, true>, units * chunks, 1);
-    launch_k(h, forward_kernel<G, V, 2, I16, false, false, true>, dim3(plan.first), dim3(plan.second), h->pdl, rows_of(h, layer),
+    Sliced m = rows_of(h, layer);
+    if (h->other_rows) { m.idx = h->lay[layer].r_idx2; m.val = h->lay[layer].r_val2; }
+    launch_k(h, forward_kernel<G, V, 2, I16, false, false, true>, dim3(plan.first), dim3(plan.second), h->pdl, m,
              (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,
              (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0, 0);
     count_launch(h);
@@ -1213,7 +1217,7 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, bool trac
         return SDNN_OK;
     }
     GraphKey key;
-    key.cw = cw; key.cols = cols; key.used = used; key.pdl = h->fwd_pdl; key.track = track;
+    key.cw = cw; key.cols = cols; key.used = used; key.pdl = h->fwd_pdl; key.track = track; key.other = h->other_rows;
     bool make = false;
     const int q = pick_graph(ln.graph_key, ln.graph_asked, TILE_GRAPHS, key, make);
     TileGraph& g = ln.graphs[q];
@@ -1395,6 +1399,13 @@ int resident_piece(const sdnn* h) {
     return std::max(1, 16384 / T) * T;
 }
 
+// fills the reordered copies of some layers
+void reorder_rows(sdnn* h, int layer, int layers) {
+    ResidentSetup set = h->resident_setup;
+    set.layer0 = layer;
+    resident_reorder_kernel<<<dim3((h->N + 7) / 8, layers), 256, 0, h->stream>>>(set, h->N, h->resident_idx2, h->resident_val2);
+}
+
 // Lays the net out for resident_infer_kernel where batches of max_batch inputs would go through it, or where the handle is for
 // large batches and larger ones would (called by sdnn_finalize).
 int build_resident(sdnn* h) {
@@ -1432,7 +1443,7 @@ int build_resident(sdnn* h) {
     }
     unit_at[(size_t)L * units] = (int)run;
     const double elems = 128.0 * run / L;
-    auto takes = [&](int64_t inputs) { return resident_width(N, elems, inputs, h->sms, infer_tile_width(h), drops_dead(h)) != 0; };
+    auto takes = [&](int64_t inputs) { return resident_width(N, elems, inputs, h->sms, infer_tile_width(h), false) != 0; };
     if (!takes(h->cfg.max_batch) && !(h->cfg.max_batch >= 512 && takes(10 * (int64_t)h->cfg.max_batch))) return SDNN_OK;
 
     auto room = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -1441,7 +1452,8 @@ int build_resident(sdnn* h) {
     for (const LayerMem& lm : h->lay) elems_stored += lm.r_elems;
     const size_t sizes[] = {entries * sizeof(unsigned short), entries * sizeof(float), rows * sizeof(float), unit_at.size() * sizeof(int),
                             (size_t)L * N * sizeof(unsigned short), rows * sizeof(int), L * sizeof(Sliced), L * sizeof(float*),
-                            row0.size() * sizeof(unsigned short), place0.size() * sizeof(unsigned short), L * sizeof(unsigned char*), (size_t)elems_stored};
+                            row0.size() * sizeof(unsigned short), place0.size() * sizeof(unsigned short), L * sizeof(unsigned char*), (size_t)elems_stored,
+                            h->compaction ? (size_t)elems_stored * (h->idx16 ? 2 : 4) : 0, h->compaction ? (size_t)elems_stored * sizeof(float) : 0, L * sizeof(int*), L * sizeof(float*)};
     size_t bytes = 0, left = 0, whole = 0;
     for (size_t b : sizes) bytes += room(b);
     // it saves time and is not needed: not where it would take what later calls allocate (a second lane, staging of host batches)
@@ -1460,17 +1472,22 @@ int build_resident(sdnn* h) {
     std::vector<Sliced> tables(L);
     std::vector<const float*> biases(L);
     std::vector<unsigned char*> orders(L);
+    std::vector<int*> idx2(L);
+    std::vector<float*> val2(L);
     for (int k = 0; k < L; ++k) {
         tables[k] = rows_of(h, k); biases[k] = h->d_bias + (size_t)k * N;
-        orders[k] = k ? orders[k - 1] + h->lay[k - 1].r_elems : reinterpret_cast<unsigned char*>(part[11]);
+        const size_t before = k ? (size_t)(orders[k - 1] - reinterpret_cast<unsigned char*>(part[11])) + (size_t)h->lay[k - 1].r_elems : 0;      // multiples of 128
+        orders[k] = reinterpret_cast<unsigned char*>(part[11]) + before;
+        idx2[k] = reinterpret_cast<int*>(part[12] + before * (h->idx16 ? 2 : 4));
+        val2[k] = reinterpret_cast<float*>(part[13]) + before;
     }
     ResidentSetup set{};
     set.rows = reinterpret_cast<const Sliced*>(part[6]); set.bias = reinterpret_cast<const float* const*>(part[7]);
     if (!uniform) { set.row0 = reinterpret_cast<const unsigned short*>(part[8]); set.place0 = reinterpret_cast<const unsigned short*>(part[9]); }
     set.order = reinterpret_cast<unsigned char* const*>(part[10]);
-    const void* from[] = {unit_at.data(), tables.data(), biases.data(), row0.data(), place0.data(), orders.data()};
-    const int to[] = {3, 6, 7, 8, 9, 10};
-    for (int i = 0; i < 6; ++i) if (sizes[to[i]]) CU(h, cudaMemcpyAsync(part[to[i]], from[i], sizes[to[i]], cudaMemcpyHostToDevice, h->stream));
+    const void* from[] = {unit_at.data(), tables.data(), biases.data(), row0.data(), place0.data(), orders.data(), idx2.data(), val2.data()};
+    const int to[] = {3, 6, 7, 8, 9, 10, 14, 15};
+    for (int i = 0; i < 8; ++i) if (sizes[to[i]]) CU(h, cudaMemcpyAsync(part[to[i]], from[i], sizes[to[i]], cudaMemcpyHostToDevice, h->stream));
     for (int k = 0; k < L; k += 32768) {      // a grid has at most 65535 rows of blocks
         set.layer0 = k;
         const int layers = std::min(L - k, 32768);
@@ -1480,12 +1497,18 @@ int build_resident(sdnn* h) {
         set.layer0 = k;
         const int layers = std::min(L - k, 32768), pitch = std::max(4, (longest + 3) / 4 * 4);
         resident_fill_kernel<<<dim3(units, layers), 32, 32 * pitch, h->stream>>>(net, set, pitch);
-        resident_reorder_kernel<<<dim3((N + 7) / 8, layers), 256, 0, h->stream>>>(set, N);
     }
     CU(h, cudaGetLastError());
     CU(h, cudaStreamSynchronize(h->stream));
-    for (int k = 0; k < L; ++k) h->lay[k].r_order = orders[k];
     h->resident = net; h->resident_setup = set; h->resident_elems = elems;
+    if (h->compaction) {
+        CU(h, cudaMemsetAsync(part[12], 0, sizes[12], h->stream));      // padding: index 0, value 0
+        CU(h, cudaMemsetAsync(part[13], 0, sizes[13], h->stream));
+        for (int k = 0; k < L; ++k) { h->lay[k].r_idx2 = idx2[k]; h->lay[k].r_val2 = val2[k]; }
+        h->resident_idx2 = reinterpret_cast<int* const*>(part[14]); h->resident_val2 = reinterpret_cast<float* const*>(part[15]);
+        for (int k = 0; k < L; k += 32768) reorder_rows(h, k, std::min(L - k, 32768));
+        CU(h, cudaGetLastError());
+    }
     return dev_alloc(h, &h->lane[0].res_list, 3 * (size_t)resident_piece(h) + 2, false);
 }
 
@@ -1493,6 +1516,7 @@ int build_resident(sdnn* h) {
 int refresh_resident(sdnn* h, int layer) {
     if (!h->resident.units) return SDNN_OK;
     h->resident_setup.layer0 = layer;
+    if (h->resident_idx2) reorder_rows(h, layer, 1);
     resident_refill_kernel<<<h->resident.units, 32, 0, h->stream>>>(h->resident, h->resident_setup);
     CU(h, cudaGetLastError());
     CU(h, cudaStreamSynchronize(h->stream));
@@ -1533,10 +1557,17 @@ int launch_resident(sdnn* h, ResidentArgs a, int p, cudaStream_t st) {
     return SDNN_OK;
 }
 
-// Width for a call's inputs, 0 if they go through the layer launches.  The ids of nonzero outputs are found in the outputs: without
-// those the tiles do it.
-int takes_resident(const sdnn* h, int64_t inputs, bool outputs) {
-    return h->resident.units && outputs ? resident_width(h->N, h->resident_elems, inputs, h->sms, infer_tile_width(h), drops_dead(h)) : 0;
+// How a call's inputs go: the width of resident_infer_kernel's CTAs, or 0 for the layer launches, which then read the reordered copies
+// (other) where the kernel would have taken the inputs had none of them been expected to die: with dead inputs dropped or not, the
+// bits are the same.  The ids of nonzero outputs are found in the outputs: without those the tiles do it.
+struct Route { int width = 0; bool other = false; };
+Route route_of(const sdnn* h, int64_t inputs, bool outputs) {
+    Route r;
+    if (!h->resident.units || !outputs) return r;
+    const int tile = infer_tile_width(h), dense = resident_width(h->N, h->resident_elems, inputs, h->sms, tile, false);
+    r.width = dense && drops_dead(h) ? resident_width(h->N, h->resident_elems, inputs, h->sms, tile, true) : dense;
+    r.other = dense && !r.width;
+    return r;
 }
 
 // All layers for `inputs` inputs on lane `ln`; arguments as for infer_tile.  total: the running total of ids is wanted.
@@ -1729,7 +1760,7 @@ int ensure_stage_w(sdnn* h) {
 template <bool TO_CSR>
 int convert_values(sdnn* h, int layer, float* csr) {
     const LayerMem& lm = h->lay[layer];
-    sliced_csr_kernel<TO_CSR><<<(h->N + 15) / 16, 512, 0, h->stream>>>(rows_of(h, layer), csr, (const int*)lm.r_start, lm.shape.uniform_k, h->N, (const unsigned char*)lm.r_order);
+    sliced_csr_kernel<TO_CSR><<<(h->N + 15) / 16, 512, 0, h->stream>>>(rows_of(h, layer), csr, (const int*)lm.r_start, lm.shape.uniform_k, h->N);
     count_launch(h);
     CU(h, cudaGetLastError());
     return SDNN_OK;
@@ -2482,10 +2513,11 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
     const bool want_sets = nz_count_out || nz_index_out || nz_total_out;
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     const int T = infer_tile_width(h);
-    const int width = takes_resident(h, n_inputs, y_out != nullptr);
-    const int lanes = n_inputs > T && !width ? infer_lanes(h, T) : 1;
+    const Route route = route_of(h, n_inputs, y_out != nullptr);
+    const int width = route.width, lanes = n_inputs > T && !width ? infer_lanes(h, T) : 1;
     if ((rc = lanes_begin(h, lanes))) return rc;
     if (width && (rc = infer_resident(h, h->lane[0], width, x0, n_inputs, y_out, nz_count_out, nz_index_out, nz_index_capacity, want_sets, nz_index_out || nz_total_out))) return rc;
+    h->other_rows = route.other;
     int64_t tile_no = 0;
     for (int64_t t0 = 0; t0 < n_inputs && !width; t0 += T, ++tile_no) {
         const int cnt = (int)((n_inputs - t0 < T) ? (n_inputs - t0) : T);
@@ -2493,6 +2525,7 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
                         nz_count_out ? nz_count_out + t0 : nullptr, nz_index_out, nz_index_capacity, want_sets);
         if (rc) break;
     }
+    h->other_rows = false;
     const int rc_end = lanes_end(h, lanes);
     if (rc || rc_end) return rc ? rc : rc_end;
     if (nz_total_out || nz_index_out) {
@@ -2522,6 +2555,10 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     // two input stages and a copy stream: the copy of tile t+1 runs under the layers of tile t
     const int T = host_tile_width(h, n_inputs);
     const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // the two halves share the stages of one tile
+    const int first = halved ? resident_half(h->N, n_inputs, h->sms) : 0;  // inputs of the first half, where both go through whole networks
+    Route route;                                                           // of both halves
+    if (first) route = route_of(h, n_inputs, y_out != nullptr);
+    const int64_t half = route.width ? first : T;
     if (!h->copy_stream) {
         CU(h, cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
         for (int q = 0; q < 2; ++q) {
@@ -2530,7 +2567,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         }
     }
     if (!halved && !h->d_stage_a2 && (rc = dev_alloc(h, &h->d_stage_a2, (size_t)h->cfg.max_batch * h->N, false))) return rc;
-    float* stage[2] = {h->d_stage_a, halved ? h->d_stage_a + (size_t)T * h->N : h->d_stage_a2};
+    float* stage[2] = {h->d_stage_a, halved ? h->d_stage_a + (size_t)half * h->N : h->d_stage_a2};
     CU(h, cudaEventRecord(h->ev_consumed[0], h->stream));       // the stages may still be read by earlier work on the stream
     CU(h, cudaEventRecord(h->ev_consumed[1], h->stream));
     const int lanes = n_inputs > T ? infer_lanes(h, T) : 1;
@@ -2541,11 +2578,12 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     }
     h->lane[0].stage_out = h->d_stage_b;
     h->lane[0].stage_cnt = h->d_stage_cnt;
-    h->lane[1].stage_out = halved ? h->d_stage_b + (size_t)T * h->N : h->d_stage_b2;
-    h->lane[1].stage_cnt = halved ? h->d_stage_cnt + T : h->d_stage_cnt2;
+    h->lane[1].stage_out = halved ? h->d_stage_b + (size_t)half * h->N : h->d_stage_b2;
+    h->lane[1].stage_cnt = halved ? h->d_stage_cnt + half : h->d_stage_cnt2;
     int64_t tile_no = 0;
-    for (int64_t t0 = 0; t0 < n_inputs; t0 += T, ++tile_no) {
-        const int cnt = (int)((n_inputs - t0 < T) ? (n_inputs - t0) : T);
+    for (int64_t t0 = 0, t1; t0 < n_inputs; t0 = t1, ++tile_no) {
+        t1 = halved ? (tile_no ? n_inputs : half) : std::min<int64_t>(n_inputs, t0 + T);
+        const int cnt = (int)(t1 - t0);
         const size_t bytes = (size_t)cnt * h->N * sizeof(float);
         const int q = (int)(tile_no & 1);
         InferLane& ln = h->lane[tile_no % lanes];
@@ -2553,11 +2591,14 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         CU(h, cudaMemcpyAsync(stage[q], x0 + (size_t)t0 * h->N, bytes, cudaMemcpyHostToDevice, h->copy_stream));
         CU(h, cudaEventRecord(h->ev_copied[q], h->copy_stream));
         CU(h, cudaStreamWaitEvent(ln.stream, h->ev_copied[q], 0));
-        if (const int width = takes_resident(h, cnt, y_out != nullptr))
-            rc = infer_resident(h, ln, width, stage[q], cnt, ln.stage_out, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
+        if (!halved) route = route_of(h, cnt, y_out != nullptr);
+        h->other_rows = route.other;
+        if (route.width)
+            rc = infer_resident(h, ln, halved ? 1 : route.width, stage[q], cnt, ln.stage_out, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
                                 want_sets, want_sets, h->ev_consumed[q]);
         else rc = infer_tile(h, ln, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
                              nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity, want_sets, h->ev_consumed[q]);
+        h->other_rows = false;
         if (rc) break;
         if (y_out) CU(h, cudaMemcpyAsync(y_out + (size_t)t0 * h->N, ln.stage_out, bytes, cudaMemcpyDeviceToHost, ln.stream));
         if (nz_count_out) CU(h, cudaMemcpyAsync(nz_count_out + t0, ln.stage_cnt, (size_t)cnt * sizeof(int), cudaMemcpyDeviceToHost, ln.stream));

@@ -238,6 +238,7 @@ extern "C" void shape(int n, int p, int* out) {
     out[0] = s.ok; out[1] = s.units; out[2] = s.slots; out[3] = s.cap; out[4] = s.held;
 }
 extern "C" void share(int total, int sms, int p, int q, int* out) { resident_share(total, sms, p, q, out, out + 1); }
+extern "C" int half(int n, long long inputs, int sms) { return resident_half(n, inputs, sms); }
 // steps of a group: left[row][class] entries; read[step][row] = class, 8 + class of the zeros for a row that waits
 extern "C" void steps(int* left, int steps, int* read) {
     int total[8] = {};
@@ -306,6 +307,19 @@ def test_shares_of_networks_held_in_shared_memory(resident):
                     if q < p:
                         assert out[1] - out[0] <= 4 * q * sms
                 assert taken == list(range(total))
+
+
+def test_halves_of_a_batch_from_host_memory(resident):
+    """Both halves hold inputs, and their CTAs fit the device side by side."""
+    resident.half.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+    for sms in (4, 148):
+        for inputs in range(0, 5 * sms):
+            first = resident.half(3000, inputs, sms)
+            if first:
+                assert 0 < first < inputs and first % 4 == 0 and first // 4 + (inputs - first + 3) // 4 <= sms
+            else:
+                assert inputs < 8 or inputs > 4 * sms
+            assert resident.half(4000, inputs, sms) == 0
 
 
 @pytest.mark.parametrize("spread", [0, 1, 5])
