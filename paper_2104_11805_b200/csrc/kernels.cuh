@@ -578,15 +578,17 @@ __device__ __forceinline__ void prefetch_unit(const Sliced& m, int u, int rpw, i
 // multiplied by the zeros of delta's padding or never read), which adds no sector to a request: rows wider than 64 bytes cost by
 // their bytes (40000 neurons, 8 layers, 90 inputs: 319 -> 299 us).
 // TRACK (dropping dead inputs): one grid for all chunks, whose warps walk the units of the chunks that still hold live inputs
-// (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.
+// (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.  ls: 2^ls groups of
+// lanes share a row, as in forward_split_kernel, which runs the same layers when nothing is dropped.
 template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false, bool TRACK = false>
 __global__ void __launch_bounds__(256, CPS > 2 ? 1 : 2)
 forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
-               int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span, int last) {
-    constexpr int RPW = 32 / G;
-    constexpr int UPS = (RPW >= SLICE) ? 1 : SLICE / RPW;      // units per slice
+               int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span, int last, int ls) {
+    const int RPW = 32 / G >> (TRACK ? ls : 0);
+    const int UPS = (RPW >= SLICE) ? 1 : SLICE / RPW;      // units per slice
     const int lane = threadIdx.x & 31;
-    const int sub = lane % G, grp = lane / G;
+    const int sub = lane % G, grp = lane / G >> (TRACK ? ls : 0);
+    const int part = TRACK ? (lane / G) & ((1 << ls) - 1) : 0, hop = TRACK ? CPS << ls : CPS, skip = part * CPS;      // this group's steps of its row
     const int wpb = blockDim.x >> 5;
     const int all_units = (n + RPW - 1) / RPW;
     const int nunits = SPAN ? min(all_units, ((int)blockIdx.x + 1) * span) : all_units;
@@ -602,13 +604,13 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
     // prologue that does not depend on the previous layer: shape of the first row, its entries on their way to L2
     int row, base, nch;
     SDNN_UNIT_SHAPE(m, unit, nunits, row, base, nch)
-    float b = (row < n) ? bias[row] : 0.0f;
+    float b = (row < n && part == 0) ? bias[row] : 0.0f;
     int to = (m.out && row < n) ? m.out[row] : row;       // tile row this row writes
     if (unit < nunits && lane == 0) prefetch_unit(m, unit, RPW, n, UPS);
     IdxChunk<I16> c[CPS];
 #pragma unroll
     for (int i = 0; i < CPS; ++i) idx_zero(c[i]);
-    if (nch > 0) load_idx<CPS, I16>(c, m, base);
+    if (nch > skip) load_idx<CPS, I16>(c, m, base + skip * CHUNK_ROW);
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
     if (TRACK) chunks_left += (*ncols_dev + V * G - 1) / (V * G) - 0x7fffffff;
@@ -620,7 +622,7 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         SDNN_WRAP(nunit, nboff, nleft)
         int nrow, nbase, nnch;
         SDNN_UNIT_SHAPE(m, nunit, nunits, nrow, nbase, nnch)
-        const float nb = (nrow < n) ? bias[nrow] : 0.0f;
+        const float nb = (nrow < n && part == 0) ? bias[nrow] : 0.0f;
         const int nto = (m.out && nrow < n) ? m.out[nrow] : nrow;
         if (nunit < nunits && lane == 0) prefetch_unit(m, nunit, RPW, n, UPS);
 
@@ -628,23 +630,27 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
         lane_fill(acc, b);
         const float* vp = val + base;
         const float* xg = xin + (TRACK || G <= 2 ? boff : min(boff, last));
-        for (int t = 0; t < nch; t += CPS) {
+        for (int t = skip; t < nch; t += hop) {
             float4 w[CPS];
             Lane<V> x[4 * CPS];
 #pragma unroll
             for (int i = 0; i < CPS; ++i) w[i] = __ldcs(reinterpret_cast<const float4*>(vp + (t + i) * CHUNK_ROW));
 #pragma unroll
             for (int i = 0; i < CPS; ++i) { SDNN_GATHER_CHUNK_SEL(CG, x, i, c[i], xg, pitch) }
-            if (t + CPS < nch) load_idx<CPS, I16>(c, m, base + (t + CPS) * CHUNK_ROW);
-            else if (nnch > 0) load_idx<CPS, I16>(c, m, nbase);
+            if (t + hop < nch) load_idx<CPS, I16>(c, m, base + (t + hop) * CHUNK_ROW);
+            else if (nnch > skip) load_idx<CPS, I16>(c, m, nbase + skip * CHUNK_ROW);
 #pragma unroll
             for (int i = 0; i < CPS; ++i) {
                 lane_fma(w[i].x, x[4 * i + 0], acc); lane_fma(w[i].y, x[4 * i + 1], acc);
                 lane_fma(w[i].z, x[4 * i + 2], acc); lane_fma(w[i].w, x[4 * i + 3], acc);
             }
         }
-        if (nch == 0 && nnch > 0) load_idx<CPS, I16>(c, m, nbase);      // empty slice: nothing prefetched across the boundary yet
-        if (row < n) {
+        if (nch <= skip && nnch > skip) load_idx<CPS, I16>(c, m, nbase + skip * CHUNK_ROW);      // no step: nothing prefetched across the boundary yet
+        if (TRACK) {
+            __syncwarp();
+            for (int o = G; o < G << ls; o <<= 1) lane_join(acc, o);
+        }
+        if (row < n && part == 0) {
             lane_activate(acc, act, clamp);
             lane_store(tile_row(xout + boff, to, pitch), acc);
             if (TRACK) live |= lane_nonzero_bits(acc);
@@ -1221,30 +1227,31 @@ backward_kernel(const BackwardArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Layers that do not fill the device (train steps; see sdnn_plan::split_units).  A launch of fewer row groups than warps fit is over when its
+// Layers that do not fill the device (train steps: see sdnn_plan::split_units; inference: sdnn_plan::split_rows).  A launch of fewer row groups than warps fit is over when its
 // longest row is: 7 dependent round trips of 8 gathers for a row of 56 entries, while the short rows' warps have ended and the request
 // path idles.  Here the steps of a long row are dealt to 2, 4, .. groups of G lanes of a warp, whose partial sums meet in shuffles, as
 // far as all units still fit the device in one round: `units` lists, for every warp, its first row * 8 + log2(groups per row).
 // us a layer, as it was / split: 6007 neurons, rows of 8 to 56 entries, 37 inputs: forward 7.17 / 5.12, backward 8.37 / 7.01; 3000 neurons,
 // 32 a row, 12 inputs: 3.92 / 2.56, 5.11 / 3.92; 700 neurons, 64 inputs: 3.58 / 2.21, 4.77 / 3.24.
 struct SplitUnit { int row, part, parts; };
+// units NULL: every row is split into 2^ls parts
 template <int G>
-__device__ __forceinline__ SplitUnit split_unit(const unsigned* units, int u, int nunits, int grp) {
-    const unsigned d = u < nunits ? units[u] : 0xffffffffu;
-    const int ls = d & 7u;
-    if (d == 0xffffffffu) return SplitUnit{0x7fffffff, 0, 1};
+__device__ __forceinline__ SplitUnit split_unit(const unsigned* units, int ls, int u, int nunits, int grp) {
+    if (u >= nunits) return SplitUnit{0x7fffffff, 0, 1};
+    const unsigned d = units ? units[u] : (unsigned)(u * (32 / G >> ls)) << 3 | (unsigned)ls;
+    ls = d & 7u;
     return SplitUnit{(int)(d >> 3) + (grp >> ls), grp & ((1 << ls) - 1), 1 << ls};
 }
 
 constexpr int SPLIT_WARPS = 4;      // of a forward CTA
 template <int G, bool I16>
 __global__ void __launch_bounds__(32 * SPLIT_WARPS, 16 / SPLIT_WARPS)
-forward_split_kernel(Sliced m, const unsigned* __restrict__ units, int nunits, const float* __restrict__ bias, const float* __restrict__ xin,
-                     float* __restrict__ xout, int n, float clamp, int act, int pdl, int last) {
+forward_split_kernel(Sliced m, const unsigned* __restrict__ units, int ls, int nunits, const float* __restrict__ bias, const float* __restrict__ xin,
+                     float* __restrict__ xout, int n, int ld, float clamp, int act, int pdl, int last) {
     constexpr int V = 8, CPS = 2;
-    constexpr unsigned pitch = 4u * V * G;
+    const unsigned pitch = 4u * ld;
     const int lane = threadIdx.x & 31, sub = lane % G;
-    const SplitUnit s = split_unit<G>(units, blockIdx.x * SPLIT_WARPS + (threadIdx.x >> 5), nunits, lane / G);
+    const SplitUnit s = split_unit<G>(units, ls, blockIdx.x * SPLIT_WARPS + (threadIdx.x >> 5), nunits, lane / G);
     int nch = 0, base = 0, to = 0;
     float b = 0.0f;
     IdxChunk<I16> c[CPS];
@@ -1302,7 +1309,7 @@ backward_split_kernel(Sliced m, const unsigned* __restrict__ units, int nunits, 
         }
     }
     const float inv_b = sp->inv_b, step = sp->eta * inv_b;
-    const SplitUnit s = split_unit<G>(units, blockIdx.x, nunits, lane / G);
+    const SplitUnit s = split_unit<G>(units, 0, blockIdx.x, nunits, lane / G);
     int nch = 0, base = 0, len = 0, j = 0;
     IdxChunk<I16> c[CPS];
 #pragma unroll

@@ -77,11 +77,27 @@ constexpr int VECTOR_CTAS = 16, VECTOR_BLOCK = 64;
 // CTAs that have rows of a net of n neurons.  Only these exchange activations: see vector.cuh.
 constexpr int vector_ctas(int n) { return n > (VECTOR_CTAS - 1) * VECTOR_BLOCK ? VECTOR_CTAS : (n + VECTOR_BLOCK - 1) / VECTOR_BLOCK; }
 
+// Rows gathered per us: 0.72, 0.57, 0.31 and 0.15 rows of up to 64, 128, 256 and 512 bytes per clock and SM
+inline double gathers_per_us(int row_bytes, int sms) { return (row_bytes <= 64 ? 0.72 : row_bytes <= 128 ? 0.57 : row_bytes <= 256 ? 0.31 : 0.15) * 1900.0 * sms; }
+
+// Inference: log2 of the groups of lanes that share a row, the same for every row: as many as leave no more units than 2048 warps, the
+// device's fill, and no more than a row has steps of 8 entries in the mean; none where a layer's gathers take long beside the round
+// trips of a row (0.77 us a step).  A function of the net and the tile's chunk alone, so that
+// the kernels that drop dead inputs, in narrower chunks, add up in the same order.  us a layer, one group / this: 700 neurons of 32 entries,
+// 6 inputs 3.63 / 2.26, 50 inputs 3.20 / 2.18, 100 inputs 3.22 / 2.62; 3000, 12 inputs 3.88 / 2.60, 50 inputs 3.80 / 3.46; 6000, 12 inputs 4.06 / 3.65;
+// left alone: 6000, 28 inputs, rows of 8 to 56 entries 5.34 / 5.46; 16384, 12 inputs 4.91 / 4.99; 30000, 6 inputs 6.79 / 7.04.
+inline int split_rows(int n, int64_t elems, int cw, int sms) {
+    int ls = 0;
+    if (cw < 8 || cw > 128 || 2.6 * elems / gathers_per_us(4 * cw, sms) > 0.77 * elems / (8.0 * n)) return 0;
+    const int lanes = cw / 8;      // of a group
+    while ((lanes << (ls + 1)) <= 32 && (((int64_t)n * lanes) << (ls + 1)) <= 2048 * 32 && (int64_t)n * 8 << (ls + 1) <= elems) ++ls;
+    return ls;
+}
+
 // Units of a layer that does not fill the device, one per warp (see forward_split_kernel): first row * 8 + log2 of the groups of
 // lanes that share a row.  off: offsets of the slices of 16 rows; a step is 8 entries of a row; `rows`: rows a warp works on at once with
 // a group each; `slots`: warps that fit the device.  A slice's rows are split into as many parts as bring its steps down to the fewest
-// that all units together leave room for.  Empty: nothing to gain by it.  So it is where the gathers of a launch (0.72, 0.57, 0.31 and
-// 0.15 rows of up to 64, 128, 256 and 512 bytes per clock and SM) outlast the round trips of its longest row (0.77 us each; 0.9 backward, where
+// that all units together leave room for.  Empty: nothing to gain by it.  So it is where the gathers of a launch outlast the round trips of its longest row (0.77 us each; 0.9 backward, where
 // the update of the other copy goes over the same path): 30000 neurons, 6 inputs, 4 steps forward 6.82 us as it is, 7.00 split, 16384: 4.77 and
 // 4.43; 16384, 28 inputs, backward 8.89 and 9.42, 10000: 8.03 and 7.01.
 inline std::vector<unsigned> split_units(const std::vector<int>& off, int n, int rows, int row_bytes, int sms, int64_t slots, bool backward) {
@@ -95,8 +111,7 @@ inline std::vector<unsigned> split_units(const std::vector<int>& off, int n, int
         return ls;
     };
     auto units_of = [&](int s, int ls) { return (std::min(16, n - s * 16) + (rows >> ls) - 1) / (rows >> ls); };
-    const double rows_per_us = (row_bytes <= 64 ? 0.72 : row_bytes <= 128 ? 0.57 : row_bytes <= 256 ? 0.31 : 0.15) * 1900.0 * sms;
-    if (longest * (backward ? 0.9 : 0.77) < (backward ? 2.0 : 1.0) * off[slices] / rows_per_us) return {};
+    if (longest * (backward ? 0.9 : 0.77) < (backward ? 2.0 : 1.0) * off[slices] / gathers_per_us(row_bytes, sms)) return {};
     int pick = longest;
     for (int most = longest - 1; most >= 1; --most) {
         int64_t units = 0;

@@ -538,7 +538,7 @@ void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld
 #define SDNN_FWD(CG_, SPAN_)                                                                                                   \
     launch_k(h, forward_kernel<G, V, CPS, I16, CG_, SPAN_>, dim3(plan.first, chunks), dim3(plan.second), h->pdl, rows_of(h, layer), \
              bias, xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,                              \
-             (const int*)nullptr, (int*)nullptr, span, last)
+             (const int*)nullptr, (int*)nullptr, span, last, 0)
     // the grid-stride instantiation is the one the wide inference tiles take: it carries nothing of the other walk
     if (cg) { if (span > 0) SDNN_FWD((G == 2 && V == 8 && CPS == 2), true); else SDNN_FWD((G == 2 && V == 8 && CPS == 2), false); }
     else if (span > 0) SDNN_FWD(false, true);
@@ -551,24 +551,24 @@ void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld
 // of 256), only the live ones, and each column that stays live marked.
 constexpr int TRACK_CHUNK = 64;
 template <bool I16, int G, int V>
-void launch_forward_tracked(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
-    const int units = (h->N + 32 / G - 1) / (32 / G), chunks = cols / (V * G);
+void launch_forward_tracked(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int ls) {
+    const int rows = 32 / G >> ls, units = (h->N + rows - 1) / rows, chunks = cols / (V * G);
     auto plan = plan_grid(h, (const void*)forward_kernel<G, V, 2, I16, false, false, true>, units * chunks, 1);
     Sliced m = rows_of(h, layer);
     if (h->other_rows) { m.idx = h->lay[layer].r_idx2; m.val = h->lay[layer].r_val2; }
     launch_k(h, forward_kernel<G, V, 2, I16, false, false, true>, dim3(plan.first), dim3(plan.second), h->pdl, m,
              (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,
-             (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0, 0);
+             (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0, 0, ls);
     count_launch(h);
 }
 template <bool I16>
-void launch_forward_tracked_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols) {
+void launch_forward_tracked_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int ls) {
     switch (std::min(cols, TRACK_CHUNK)) {
-        case 4: launch_forward_tracked<I16, 1, 4>(h, layer, xin, xout, ld, cols); break;
-        case 8: launch_forward_tracked<I16, 1, 8>(h, layer, xin, xout, ld, cols); break;
-        case 16: launch_forward_tracked<I16, 2, 8>(h, layer, xin, xout, ld, cols); break;
-        case 32: launch_forward_tracked<I16, 4, 8>(h, layer, xin, xout, ld, cols); break;
-        default: launch_forward_tracked<I16, 8, 8>(h, layer, xin, xout, ld, cols); break;
+        case 4: launch_forward_tracked<I16, 1, 4>(h, layer, xin, xout, ld, cols, ls); break;
+        case 8: launch_forward_tracked<I16, 1, 8>(h, layer, xin, xout, ld, cols, ls); break;
+        case 16: launch_forward_tracked<I16, 2, 8>(h, layer, xin, xout, ld, cols, ls); break;
+        case 32: launch_forward_tracked<I16, 4, 8>(h, layer, xin, xout, ld, cols, ls); break;
+        default: launch_forward_tracked<I16, 8, 8>(h, layer, xin, xout, ld, cols, ls); break;
     }
 }
 
@@ -581,13 +581,14 @@ bool entry_parallel(const sdnn* h, int ld) {
 bool moved(const LayerMem& lm, int ld);
 float* delta_tile(sdnn* h, int layer, size_t tile);
 
-// Layers of a training handle that do not fill the device, at the width of its minibatches: units with long rows split
+// Layers that do not fill the device.  ls = 0: of a training handle, at the width of its minibatches, by its list of units; else every row is split.
 template <int G, bool I16>
-void launch_forward_split(sdnn* h, int layer, const float* xin, float* xout, int last) {
+void launch_forward_split(sdnn* h, int layer, const float* xin, float* xout, int ld, int ls, int last) {
     const LayerMem& lm = h->lay[layer];
-    launch_k(h, forward_split_kernel<G, I16>, dim3((lm.r_nunits + SPLIT_WARPS - 1) / SPLIT_WARPS), dim3(32 * SPLIT_WARPS), h->pdl, rows_of(h, layer),
-             (const unsigned*)lm.r_units, lm.r_nunits, (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, h->cfg.clamp, h->cfg.activation,
-             h->pdl ? h->fwd_pdl : 0, last);
+    const int rows = 32 / G >> ls, nunits = ls ? (h->N + rows - 1) / rows : lm.r_nunits;
+    launch_k(h, forward_split_kernel<G, I16>, dim3((nunits + SPLIT_WARPS - 1) / SPLIT_WARPS), dim3(32 * SPLIT_WARPS), h->pdl, rows_of(h, layer),
+             ls ? (const unsigned*)nullptr : (const unsigned*)lm.r_units, ls, nunits, (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp,
+             h->cfg.activation, h->pdl ? h->fwd_pdl : 0, last);
     count_launch(h);
 }
 template <int G, bool I16>
@@ -600,8 +601,8 @@ void launch_backward_split(sdnn* h, int layer, int ld) {
               (const StepParams*)h->d_sp, h->pdl ? PDL_EARLY : 0, acts + (size_t)(layer - 1) * tile, (unsigned)(tile * sizeof(float)));
     count_launch(h);
 }
-#define SDNN_BY_WIDTH(FN, ...)                            \
-    switch (h->ld_max) {                                  \
+#define SDNN_BY_WIDTH(WIDTH, FN, ...)                     \
+    switch (WIDTH) {                                      \
         case 8: FN<1, I16>(__VA_ARGS__); break;           \
         case 16: FN<2, I16>(__VA_ARGS__); break;          \
         case 32: FN<4, I16>(__VA_ARGS__); break;          \
@@ -638,10 +639,11 @@ int build_units(sdnn* h, const std::vector<int>& off, bool backward, bool beside
 }
 
 template <bool I16>
-void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used) {
+void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used, int ls) {
     const Geometry q = geometry(cw);
     const int chunks = cols / cw, last = (used - 1) / q.v * q.v;
-    if (h->lay[layer].r_nunits && ld == h->ld_max && cols == ld) { SDNN_BY_WIDTH(launch_forward_split, h, layer, xin, xout, last) return; }
+    if (ls < 0 && h->lay[layer].r_nunits && ld == h->ld_max) { SDNN_BY_WIDTH(ld, launch_forward_split, h, layer, xin, xout, ld, 0, last) return; }
+    if (ls > 0 && chunks == 1) { SDNN_BY_WIDTH(cw, launch_forward_split, h, layer, xin, xout, ld, ls, last) return; }
     if (q.v == 4 && entry_parallel(h, ld)) {
         const int wf = h->NS <= h->sms ? 1 : 4;      // few slices: one per CTA, so that they spread over as many SMs
         launch_k(h, forward_ep_kernel<I16>, dim3((h->NS + wf - 1) / wf), dim3(32 * wf), h->pdl, rows_of(h, layer),
@@ -664,13 +666,13 @@ void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld,
     count_launch(h);
 }
 
-// the kernels are instantiated for both index widths of the sliced copies; used: columns that hold inputs
-void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used, bool track = false) {
+// the kernels are instantiated for both index widths of the sliced copies; used: columns that hold inputs; ls: see split_rows, -1 in a train step
+void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used, bool track = false, int ls = -1) {
     if (track) {
-        if (h->idx16) launch_forward_tracked_i<true>(h, layer, xin, xout, ld, cols);
-        else launch_forward_tracked_i<false>(h, layer, xin, xout, ld, cols);
-    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, cw, used);
-    else launch_forward_i<false>(h, layer, xin, xout, ld, cols, cw, used);
+        if (h->idx16) launch_forward_tracked_i<true>(h, layer, xin, xout, ld, cols, ls);
+        else launch_forward_tracked_i<false>(h, layer, xin, xout, ld, cols, ls);
+    } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, cw, used, ls);
+    else launch_forward_i<false>(h, layer, xin, xout, ld, cols, cw, used, ls);
 }
 
 // Windowed layers (rows grouped by shared columns at set-up): the group's window of the input tile is staged in shared
@@ -864,7 +866,7 @@ void launch_backward_ep(sdnn* h, int layer, int part) {
 template <bool I16>
 void launch_backward_i(sdnn* h, int layer, int ld, int part) {
     const Geometry q = geometry(ld);
-    if (part == 1 && ld == h->ld_max && h->lay[layer].c_nunits) { SDNN_BY_WIDTH(launch_backward_split, h, layer, ld) return; }
+    if (part == 1 && ld == h->ld_max && h->lay[layer].c_nunits) { SDNN_BY_WIDTH(ld, launch_backward_split, h, layer, ld) return; }
     if (q.v == 4 && h->split && part != 0 && entry_parallel(h, ld)) launch_backward_ep<I16>(h, layer, part);
     else if (q.v == 4) launch_backward_gv<I16, 1, 4>(h, layer, ld, part);
     else switch (q.g) {
@@ -1255,6 +1257,9 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     // dropping dead inputs works on chunks of 64 whatever the padding
     const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->mean_elems, h->windowed_layers == h->L);
     const int cw = shape.cw, cols = shape.cols;
+    // by the shape that the tile has without dropping; tiles of several chunks are not split, nor what stands in for whole networks
+    const TileShape dense = tile_shape(cnt, h->mean_elems, false);
+    const int ls = dense.cw == dense.cols && !h->other_rows ? split_rows(h->N, h->mean_elems, dense.cw, h->sms) : 0;
     launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     if (consumed) CU(h, cudaEventRecord(consumed, st));
     auto layers = [&](int used) {      // used: columns to gather for, a multiple of a lane's
@@ -1264,7 +1269,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
             const int rows_grid = std::min((h->N + 7) / 8, h->sms * 8);
             cudaMemsetAsync(ln.cs.flags, 0, (size_t)h->L * ld * sizeof(int), st);
             for (int k = 0; k < h->L; ++k) {
-                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, cols, true);
+                launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, cols, true, ls);
                 cur ^= 1;
                 // dropping what has died: after each of the first layers, where most do, then at growing distances (after 1, 2, 3, 4,
                 // 6, 8, 12, 16, 24, ... layers)
@@ -1282,7 +1287,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
             for (int k = 0; k < h->L; ++k) {
                 NvtxRange pass("forward layer", k + 1);
                 if (h->lay[k].windowed) launch_forward_window(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols);
-                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, used);
+                else launch_forward(h, k, ln.tile[cur], ln.tile[cur ^ 1], ld, cols, cw, used, false, ls);
                 cur ^= 1;
             }
         }

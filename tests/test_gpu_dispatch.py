@@ -470,7 +470,7 @@ def test_networks_held_in_shared_memory(torch_cuda, n, cnt, ragged):  # noqa: F8
 
 
 @pytest.mark.parametrize("n,cnt,tile", [(640, 2000, 1024), (1024, 1000, 1000), (2048, 1500, 600), (4096, 2500, 1024), (4096, 592, 592),
-                                        (1465, 449, 449), (1465, 200, 600)])
+                                        (1465, 449, 449), (1465, 200, 600), (700, 60, 100), (1500, 120, 128), (2000, 7, 40), (900, 1030, 1000)])
 def test_dead_inputs_dropped_from_networks_held_in_shared_memory(torch_cuda, n, cnt, tile):  # noqa: F811
     """Inputs that die at once, after some layers, or not at all, dropped that way or, fewer of them, by the layer launches: the same bits as without dropping them, and the live inputs of the last tile
     after each layer; all inputs dead; none."""
@@ -540,3 +540,24 @@ def test_allocation_free_call_with_rows_shared_by_groups_of_lanes(torch_cuda, n,
                       torch.from_numpy(np.stack(bias)).cuda(), torch.from_numpy(x0).cuda(), cnt, got)
     torch.cuda.synchronize()
     check_close(got.cpu().numpy(), OracleNet(rp, cols, vals, bias).infer(x0), f"{n} neurons, {cnt} inputs")
+
+
+@pytest.mark.parametrize("n,cnt", [(17, 8), (700, 6), (700, 100), (1500, 33), (3001, 16), (6007, 40), (9000, 20), (16000, 5), (17000, 64)])
+@pytest.mark.parametrize("ragged", [False, True])
+def test_inference_with_rows_shared_by_groups_of_lanes(torch_cuda, n, cnt, ragged):  # noqa: F811
+    """Small batches through layers that do not fill the device, from the first call's launches and the later ones' graph, in a handle for just
+    as many inputs and in one for more, with either index width."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    arrays = ragged_net(rng, n=n, layers=5, kmax=min(n, 60), scale=0.3) if ragged else uniform_net(rng, n, min(n // 2, 32), 5)
+    x0 = vectors(rng, cnt, n)
+    want, outs = OracleNet(*arrays).infer(x0), []
+    for batch, flags in ((cnt, 0), (300, 0), (cnt, pkg.FLAG_IDX32)):
+        h = pkg.Sdnn.create(*arrays, max_batch=batch, flags=flags)
+        for _ in range(3):
+            outs.append(torch.full((cnt, n), -1.0, device="cuda"))
+            h.infer_batch(torch.from_numpy(x0).cuda(), cnt, outs[-1])
+        torch.cuda.synchronize()
+        h.destroy()
+    check_close(outs[0].cpu().numpy(), want, "x^L")
+    assert all(torch.equal(y, outs[0]) for y in outs)

@@ -16,6 +16,7 @@ extern "C" int ctas(int n) { return vector_ctas(n); }
 extern "C" int cols(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cols; }
 extern "C" int chunk(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cw; }
 extern "C" int graph(int layers, long long elems, int cols, int track) { return tile_as_graph(layers, elems, cols, track); }
+extern "C" int rows_log(int n, long long elems, int cw) { return split_rows(n, elems, cw, 148); }
 extern "C" int units(const int* off, int n, int rows, int bytes, long long slots, int backward, unsigned* out) {
     const std::vector<unsigned> list = split_units(std::vector<int>(off, off + (n + 15) / 16 + 1), n, rows, bytes, 148, slots, backward != 0);
     std::copy(list.begin(), list.end(), out);
@@ -78,6 +79,18 @@ def test_units_of_layers_that_do_not_fill_the_device(plan, width, n):
                     taken += [r for r in range(row, row + rows // parts) if r < n]
                     longest = max(longest, -(-steps[row // 16] // parts))
                 assert taken == list(range(n)) and longest < max(steps)
+
+
+def test_rows_shared_in_inference(plan):
+    """A group of lanes fits a warp as often as a row is shared, the launch fits the device, and no part of a row is without a step."""
+    plan.rows_log.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+    for n in (1, 17, 700, 1024, 4096, 6007, 16384, 70000):
+        for per_row in (0, 8, 32, 56, 300):
+            assert plan.rows_log(n, n * per_row, 4) == plan.rows_log(n, n * per_row, 256) == 0
+            for cw in (8, 16, 32, 64, 128):
+                parts = 1 << plan.rows_log(n, n * per_row, cw)
+                assert parts == 1 or (cw // 8 * parts <= 32 and n * (cw // 8) * parts <= 65536 and parts * 8 <= per_row)
+    assert plan.rows_log(700, 700 * 32, 64) == 2 and plan.rows_log(16384, 16384 * 32, 64) == 0
 
 
 def test_tile_shapes(plan):
