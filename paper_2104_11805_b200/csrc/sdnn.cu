@@ -1564,11 +1564,11 @@ int launch_resident(sdnn* h, ResidentArgs a, int p, cudaStream_t st) {
 
 // How a call's inputs go: the width of resident_infer_kernel's CTAs, or 0 for the layer launches, which then read the reordered copies
 // (other) where the kernel would have taken the inputs had none of them been expected to die: with dead inputs dropped or not, the
-// bits are the same.  The ids of nonzero outputs are found in the outputs: without those the tiles do it.
+// bits are the same.
 struct Route { int width = 0; bool other = false; };
-Route route_of(const sdnn* h, int64_t inputs, bool outputs) {
+Route route_of(const sdnn* h, int64_t inputs) {
     Route r;
-    if (!h->resident.units || !outputs) return r;
+    if (!h->resident.units) return r;
     const int tile = infer_tile_width(h), dense = resident_width(h->N, h->resident_elems, inputs, h->sms, tile, false);
     r.width = dense && drops_dead(h) ? resident_width(h->N, h->resident_elems, inputs, h->sms, tile, true) : dense;
     r.other = dense && !r.width;
@@ -1579,12 +1579,15 @@ Route route_of(const sdnn* h, int64_t inputs, bool outputs) {
 int infer_resident(sdnn* h, InferLane& ln, int p, const float* x0, int64_t inputs, float* y, int* cnt_out, int* idx_out, long long capacity,
                    bool want_sets, bool total, cudaEvent_t consumed = nullptr) {
     NvtxRange call("sdnn whole-network inference");
-    const int piece = resident_piece(h), T = infer_tile_width(h);
+    const int room = resident_piece(h), T = infer_tile_width(h);
     cudaStream_t st = ln.stream;
-    int* list[2] = {ln.res_list, ln.res_list + piece};
-    int* count = ln.res_list + 2 * (size_t)piece;
+    int* list[2] = {ln.res_list, ln.res_list + room};
+    int* count = ln.res_list + 2 * (size_t)room;
     int* nz = count + 2;
     const bool track = drops_dead(h);
+    // what is on its way between stages, and what ids are found in, waits in the outputs; where the caller wants none, in the lane's tiles
+    float* const held = y || (!track && !idx_out) ? nullptr : ln.tile[0];
+    const int piece = held ? std::min(room, 2 * h->ld_max / T * T) : room;
     if (track) {
         CU(h, cudaMemsetAsync(ln.live_hist, 0, (size_t)h->L * sizeof(int), st));
         h->live_valid = true;
@@ -1595,7 +1598,8 @@ int infer_resident(sdnn* h, InferLane& ln, int p, const float* x0, int64_t input
         const int cnt = (int)std::min<int64_t>(piece, inputs - at);
         int* counts = want_sets ? (cnt_out ? cnt_out + at : nz) : nullptr;
         ResidentArgs a{};
-        a.x = x0 + (size_t)at * h->N; a.y = y + (size_t)at * h->N; a.nz_count = counts;
+        a.x = x0 + (size_t)at * h->N; a.y = y ? y + (size_t)at * h->N : held; a.nz_count = counts;
+        const float* const out = a.y;
         a.from = 0; a.to = h->L; a.inputs = cnt;
         if (!track) {
             if ((rc = launch_resident(h, a, p, st))) return rc;
@@ -1625,7 +1629,7 @@ int infer_resident(sdnn* h, InferLane& ln, int p, const float* x0, int64_t input
                 h->last_scan_ev = ln.ev_scan;
                 count_launch(h);
                 if (idx_out) {
-                    nz_fill_rows_kernel<<<some, 256, 0, st>>>(y + ((size_t)at + t0) * h->N, ln.offs, idx_out, capacity, h->N);
+                    nz_fill_rows_kernel<<<some, 256, 0, st>>>(out + (size_t)t0 * h->N, ln.offs, idx_out, capacity, h->N);
                     count_launch(h);
                 }
             }
@@ -2518,7 +2522,7 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
     const bool want_sets = nz_count_out || nz_index_out || nz_total_out;
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     const int T = infer_tile_width(h);
-    const Route route = route_of(h, n_inputs, y_out != nullptr);
+    const Route route = route_of(h, n_inputs);
     const int width = route.width, lanes = n_inputs > T && !width ? infer_lanes(h, T) : 1;
     if ((rc = lanes_begin(h, lanes))) return rc;
     if (width && (rc = infer_resident(h, h->lane[0], width, x0, n_inputs, y_out, nz_count_out, nz_index_out, nz_index_capacity, want_sets, nz_index_out || nz_total_out))) return rc;
@@ -2562,7 +2566,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // the two halves share the stages of one tile
     const int first = halved ? resident_half(h->N, n_inputs, h->sms) : 0;  // inputs of the first half, where both go through whole networks
     Route route;                                                           // of both halves
-    if (first) route = route_of(h, n_inputs, y_out != nullptr);
+    if (first) route = route_of(h, n_inputs);
     const int64_t half = route.width ? first : T;
     if (!h->copy_stream) {
         CU(h, cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
@@ -2596,10 +2600,10 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         CU(h, cudaMemcpyAsync(stage[q], x0 + (size_t)t0 * h->N, bytes, cudaMemcpyHostToDevice, h->copy_stream));
         CU(h, cudaEventRecord(h->ev_copied[q], h->copy_stream));
         CU(h, cudaStreamWaitEvent(ln.stream, h->ev_copied[q], 0));
-        if (!halved) route = route_of(h, cnt, y_out != nullptr);
+        if (!halved) route = route_of(h, cnt);
         h->other_rows = route.other;
         if (route.width)
-            rc = infer_resident(h, ln, halved ? 1 : route.width, stage[q], cnt, ln.stage_out, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
+            rc = infer_resident(h, ln, halved ? 1 : route.width, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
                                 want_sets, want_sets, h->ev_consumed[q]);
         else rc = infer_tile(h, ln, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
                              nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity, want_sets, h->ev_consumed[q]);

@@ -441,6 +441,11 @@ def test_networks_held_in_shared_memory(torch_cuda, n, cnt, ragged):  # noqa: F8
     ids = ids.cpu().numpy()
     assert np.array_equal(ids[:total], np.nonzero(y)[1]) and (ids[total:] == -1).all()
 
+    ids2, c2 = torch.full((cnt * n,), -1, dtype=torch.int32, device="cuda"), torch.full((cnt,), -1, dtype=torch.int32, device="cuda")
+    h.infer_batch(x, cnt, None, c2)                                # without the outputs: the same counts and ids
+    assert np.array_equal(c2.cpu().numpy(), c)
+    assert h.infer_batch(x, cnt, None, None, ids2, cnt * n, want_total=True) == total and np.array_equal(ids2.cpu().numpy(), ids)
+
     yh = np.empty((cnt, n), dtype=np.float32)
     h.infer_batch(x0, cnt, yh, None, host=True)
     check_close(yh[pick], ora.infer(x0[pick]), "x^L through host buffers")
@@ -490,6 +495,10 @@ def test_dead_inputs_dropped_from_networks_held_in_shared_memory(torch_cuda, n, 
             total = h.infer_batch(x, cnt, y, c, ids, cnt * n, want_total=True)
             torch.cuda.synchronize()
             outs.append((y.cpu().numpy(), c.cpu().numpy(), ids.cpu().numpy(), total))
+            live = list(h.get_liveness()) if h is drop else None
+            c2, ids2 = torch.full_like(c, -1), torch.full_like(ids, -1)
+            assert h.infer_batch(x, cnt, None, c2, ids2, cnt * n, want_total=True) == total      # the same without the outputs
+            assert torch.equal(c, c2) and torch.equal(ids, ids2) and (live is None or list(h.get_liveness()) == live)
         assert all(np.array_equal(a, b) for a, b in zip(*outs))
         last = (cnt - 1) // drop.infer_tile_width() * drop.infer_tile_width()
         live, want = x0[last:], []
