@@ -70,7 +70,8 @@ typedef enum {
 #define SDNN_FLAG_SKIP_DEAD   0x08u /* allow data-dependent skipping; default is dense mode: every layer streams   */
                                     /* its weights and processes every input.  Inference: inputs whose activation  */
                                     /* vector has become all zero are dropped from the tile (whole chunks of 64    */
-                                    /* columns at a time); only done while no layer has a positive bias, because   */
+                                    /* columns at a time; one by one, after some layers, where whole networks run  */
+                                    /* in shared memory: larger batches, up to 8192 neurons); only done while no layer has a positive bias, because   */
                                     /* only then does an all-zero vector stay all zero.  Training: a unit of rows  */
                                     /* whose delta is zero for every input skips its entries (not for B <= 4,      */
                                     /* whose kernels have no such test).  Results are the same as in dense mode.   */
