@@ -18,8 +18,8 @@
 // Memory: a ring of slots.  A layer's outputs go behind its inputs; where both do not fit (4096 neurons, 8 inputs: 128 KB of
 // inputs and 97 KB free) the last units' outputs wait in registers until every warp has read the layer.
 // What bounds it is the shared-memory pipe (4096 neurons, 8 inputs a CTA: 0.27 wavefronts per entry and 8 inputs for operands, 0.05 for the
-// entry itself; the pipe 88 % busy under ncu before rows were grouped as they are now).  4096 x 120, 10000 inputs: 32.7 -> 25.7 ms,
-// with dead inputs dropped, 5000 inputs a third of which survive: 9.58 -> 5.74; 2048 x 24, 2368 inputs: 34.9 -> 22.3 us a layer.
+// entry itself; the pipe 86 % busy under ncu).  4096 x 120, 10000 inputs: 32.5 -> 25.6 ms,
+// with dead inputs dropped, 5000 inputs a third of which survive: 9.58 -> 5.71; 2048 x 24, 2368 inputs: 34.9 -> 22.3 us a layer.
 // 16 warps: with 20, 24 and 32 the same layer of 4096 takes 12, 10 and 6 % longer at 8 inputs a CTA (registers: fewer reads
 // together), 4 inputs gain 4 % with 32.
 #pragma once

@@ -581,6 +581,14 @@ bool entry_parallel(const sdnn* h, int ld) {
 bool moved(const LayerMem& lm, int ld);
 float* delta_tile(sdnn* h, int layer, size_t tile);
 
+// what the launch after one of these will read of its layer's entries (nothing where there is none)
+NextEntries next_entries(const sdnn* h, int layer, bool transposed) {
+    if (layer < (transposed ? 1 : 0) || layer >= h->L || h->lay[layer].windowed) return NextEntries{nullptr, nullptr, 0, 0};
+    const LayerMem& lm = h->lay[layer];
+    const int64_t elems = std::min<int64_t>(transposed ? lm.c_elems : lm.r_elems, 1 << 29);
+    return NextEntries{transposed ? lm.c_idx : lm.r_idx, transposed ? lm.c_val : lm.r_val, (unsigned)(elems * (h->idx16 ? 2 : 4)), (unsigned)(elems * 4)};
+}
+
 // Layers that do not fill the device.  ls = 0: of a training handle, at the width of its minibatches, by its list of units; else every row is split.
 template <int G, bool I16>
 void launch_forward_split(sdnn* h, int layer, const float* xin, float* xout, int ld, int ls, int last) {
@@ -588,7 +596,7 @@ void launch_forward_split(sdnn* h, int layer, const float* xin, float* xout, int
     const int rows = 32 / G >> ls, nunits = ls ? (h->N + rows - 1) / rows : lm.r_nunits;
     launch_k(h, forward_split_kernel<G, I16>, dim3((nunits + SPLIT_WARPS - 1) / SPLIT_WARPS), dim3(32 * SPLIT_WARPS), h->pdl, rows_of(h, layer),
              ls ? (const unsigned*)nullptr : (const unsigned*)lm.r_units, ls, nunits, (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp,
-             h->cfg.activation, h->pdl ? h->fwd_pdl : 0, last);
+             h->cfg.activation, h->pdl ? h->fwd_pdl : 0, last, next_entries(h, layer + 1, false));
     count_launch(h);
 }
 template <int G, bool I16>
@@ -598,7 +606,7 @@ void launch_backward_split(sdnn* h, int layer, int ld) {
     const float* acts = h->bwd_acts ? h->bwd_acts : h->d_acts;
     launch_on(h, backward_split_kernel<G, I16>, dim3(lm.c_nunits), dim3(32), 0, h->pdl, moved(lm, ld), cols_of(h, layer), (const unsigned*)lm.c_units, lm.c_nunits,
               acts + (size_t)layer * tile, (const float*)delta_tile(h, layer, tile), delta_tile(h, layer - 1, tile), h->N, h->cfg.clamp, h->cfg.activation,
-              (const StepParams*)h->d_sp, h->pdl ? PDL_EARLY : 0, acts + (size_t)(layer - 1) * tile, (unsigned)(tile * sizeof(float)));
+              (const StepParams*)h->d_sp, h->pdl ? PDL_EARLY : 0, acts + (size_t)(layer - 1) * tile, (unsigned)(tile * sizeof(float)), next_entries(h, layer - 1, true));
     count_launch(h);
 }
 #define SDNN_BY_WIDTH(WIDTH, FN, ...)                     \
@@ -610,9 +618,10 @@ void launch_backward_split(sdnn* h, int layer, int ld) {
         default: FN<16, I16>(__VA_ARGS__); break;         \
     }
 
-// Lists the units of one copy of a layer for them (off: its slice offsets).  beside_rows: the launch shares the device with row units,
-// which are done later when it takes all of it (us per backward layer, none split / 70 % / 100 % of the warps that fit: 6007 neurons, 28
-// inputs 5.62 / 5.12 / 5.79, ragged 6.13 / 5.46 / 6.48; 16384, 12, ragged 9.40 / 8.36 / 9.38); moves leave it all (6007, 37: 8.37 / 7.34 / 7.01).
+// Lists the units of one copy of a layer for them (off: its slice offsets).  beside_rows: the launch shares the device with row units: both
+// have to fit in one round, and the row units are done later when the columns take most of it (us per backward layer, as it was / 70 % / 100 %
+// of the warps that fit: 6007 neurons, 28 inputs 5.62 / 5.12 / 5.79, ragged 6.13 / 5.46 / 6.48; 6867 x 56, 28 inputs, where 70 % and the
+// row units do not fit 5.82 / 6.40, 53 %: 5.45); moves leave it all (6007, 37: 8.37 / 7.34 / 7.01).
 template <bool I16>
 int build_units(sdnn* h, const std::vector<int>& off, bool backward, bool beside_rows, unsigned** units, int* nunits) {
     if (!h->split || h->ld_max < 8 || h->ld_max > 128) return SDNN_OK;
@@ -628,7 +637,8 @@ int build_units(sdnn* h, const std::vector<int>& off, bool backward, bool beside
     }
 #undef SDNN_KERNEL
     const int64_t slots = (int64_t)h->sms * resident_ctas(h, kernel, block) * (block / 32);
-    const std::vector<unsigned> list = split_units(off, h->N, 32 / (h->ld_max / 8), h->ld_max * 4, h->sms, beside_rows ? slots * 7 / 10 : slots, backward);
+    const int rows = 32 / (h->ld_max / 8), whole = (h->N + rows - 1) / rows;      // row units beside
+    const std::vector<unsigned> list = split_units(off, h->N, rows, h->ld_max * 4, h->sms, beside_rows ? std::min<int64_t>(slots * 7 / 10, slots - whole) : slots, backward);
     if (list.empty()) return SDNN_OK;
     int rc;
     if ((rc = dev_alloc(h, units, list.size(), false))) return rc;
