@@ -23,8 +23,10 @@ inline int padded_width(int b) {
 // 32 inputs or of 16, 8 or 4: whole chunks are all the padding it needs.
 constexpr int64_t SHAPE_WORK = 32 << 20;      // stored elements x inputs per layer
 struct TileShape { int cw, cols; };
-inline TileShape tile_shape(int cnt, int64_t elems, bool windows) {
+// ls: see split_rows; a tile whose rows are shared is of whole lanes, which hold 8 inputs (the last tile of a call may have fewer).
+inline TileShape tile_shape(int cnt, int64_t elems, bool windows, int ls = 0) {
     TileShape best{std::min(padded_width(cnt), 256), padded_width(cnt)};
+    if (ls && best.cols < 8) best = {8, 8};
     if (windows) return cnt <= 32 ? best : TileShape{32, (cnt + 31) / 32 * 32};
     if (cnt <= 64 || elems * cnt < SHAPE_WORK) return best;
     double least = best.cols;
@@ -51,14 +53,14 @@ inline bool tile_as_graph(int layers, int64_t elems, int cols, bool track) { ret
 // the one not asked for longest makes room for one that serves any tile of this shape.  So batches that vary at will make a lane
 // fill its places, and after that one graph per shape (as long as there are no more shapes than places).
 // Returns the place; `make` is set where the graph has to be made first, with want.used columns (which may have been raised).
-struct GraphKey { int cw = 0, cols = 0, used = 0, pdl = 0; bool track = false, other = false; };      // other: of the reordered copies
+struct GraphKey { int cw = 0, cols = 0, used = 0, pdl = 0, ls = 0; bool track = false, other = false; };      // ls: see split_rows; other: of the reordered copies
 inline int pick_graph(const GraphKey* have, const int64_t* asked, int n, GraphKey& want, bool& make) {      // asked[q] = 0: empty
     int room = -1, serves = -1, oldest = 0;
     make = false;
     for (int q = 0; q < n; ++q) {
         if (!asked[q]) { if (room < 0) room = q; continue; }
         const GraphKey& g = have[q];
-        if (g.cw == want.cw && g.cols == want.cols && g.pdl == want.pdl && g.track == want.track && g.other == want.other && g.used >= want.used) {
+        if (g.cw == want.cw && g.cols == want.cols && g.pdl == want.pdl && g.ls == want.ls && g.track == want.track && g.other == want.other && g.used >= want.used) {
             if (g.used == want.used) return q;
             if (serves < 0 || g.used < have[serves].used) serves = q;
         }
@@ -82,8 +84,8 @@ inline double gathers_per_us(int row_bytes, int sms) { return (row_bytes <= 64 ?
 
 // Inference: log2 of the groups of lanes that share a row, the same for every row: as many as leave no more units than 2048 warps, the
 // device's fill, and no more than a row has steps of 8 entries in the mean; none where a layer's gathers take long beside the round
-// trips of a row (0.77 us a step).  A function of the net and the tile's chunk alone, so that
-// the kernels that drop dead inputs, in narrower chunks, add up in the same order.  us a layer, one group / this: 700 neurons of 32 entries,
+// trips of a row (0.77 us a step).  A function of the net and the chunk of a call's whole tiles (call_rows) alone, so that
+// the kernels that drop dead inputs, in narrower chunks, add up in the same order, and so does the call's last, narrower tile.  us a layer, one group / this: 700 neurons of 32 entries,
 // 6 inputs 3.63 / 2.26, 50 inputs 3.20 / 2.18, 100 inputs 3.22 / 2.62; 3000, 12 inputs 3.88 / 2.60, 50 inputs 3.80 / 3.46; 6000, 12 inputs 4.06 / 3.65;
 // left alone: 6000, 28 inputs, rows of 8 to 56 entries 5.34 / 5.46; 16384, 12 inputs 4.91 / 4.99; 30000, 6 inputs 6.79 / 7.04.
 inline int split_rows(int n, int64_t elems, int cw, int sms) {
@@ -92,6 +94,11 @@ inline int split_rows(int n, int64_t elems, int cw, int sms) {
     const int lanes = cw / 8;      // of a group
     while ((lanes << (ls + 1)) <= 32 && (((int64_t)n * lanes) << (ls + 1)) <= 2048 * 32 && (int64_t)n * 8 << (ls + 1) <= elems) ++ls;
     return ls;
+}
+// ... of all tiles of a call whose whole tiles have `tile` inputs; none where those are of several chunks
+inline int call_rows(int n, int64_t elems, int tile, int sms) {
+    const TileShape whole = tile_shape(tile, elems, false);
+    return whole.cw == whole.cols ? split_rows(n, elems, whole.cw, sms) : 0;
 }
 
 // Units of a layer that does not fill the device, one per warp (see forward_split_kernel): first row * 8 + log2 of the groups of

@@ -1221,7 +1221,7 @@ int alloc_lane(sdnn* h, InferLane& ln, bool own_stream) {
 
 // The launches of a tile's layers, as a graph where tile_as_graph says so; used: columns that the launches gather for.
 template <typename Layers>
-int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, bool track, const Layers& layers) {
+int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, int ls, bool track, const Layers& layers) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (h->infer_calls < 2 || !tile_as_graph(h->L, h->mean_elems, cols, track) || (h->cfg.flags & SDNN_FLAG_NO_GRAPH) || cudaStreamIsCapturing(ln.stream, &capturing) != cudaSuccess ||
         capturing != cudaStreamCaptureStatusNone) {
@@ -1229,7 +1229,7 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, bool trac
         return SDNN_OK;
     }
     GraphKey key;
-    key.cw = cw; key.cols = cols; key.used = used; key.pdl = h->fwd_pdl; key.track = track; key.other = h->other_rows;
+    key.cw = cw; key.cols = cols; key.used = used; key.pdl = h->fwd_pdl; key.ls = ls; key.track = track; key.other = h->other_rows;
     bool make = false;
     const int q = pick_graph(ln.graph_key, ln.graph_asked, TILE_GRAPHS, key, make);
     TileGraph& g = ln.graphs[q];
@@ -1255,8 +1255,8 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, bool trac
 }
 
 // One tile of inference on device buffers, on lane `ln`: x0 [cnt][N] -> outputs for these cnt inputs.
-// consumed (or NULL): recorded once x0 has been read.
-int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, int* cnt_out, int* idx_out, long long capacity,
+// ls: of the call, not of this tile (call_rows).  consumed (or NULL): recorded once x0 has been read.
+int infer_tile(sdnn* h, InferLane& ln, int ls, const float* x0, int cnt, float* y_out, int* cnt_out, int* idx_out, long long capacity,
                bool want_sets, cudaEvent_t consumed = nullptr) {
     NvtxRange call("sdnn inference tile");
     const int ld = h->ld_max;
@@ -1265,11 +1265,8 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     h->launch_stream = st;
     const bool track = drops_dead(h);
     // dropping dead inputs works on chunks of 64 whatever the padding
-    const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->mean_elems, h->windowed_layers == h->L);
+    const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->mean_elems, h->windowed_layers == h->L, ls);
     const int cw = shape.cw, cols = shape.cols;
-    // by the shape that the tile has without dropping; tiles of several chunks are not split, nor what stands in for whole networks
-    const TileShape dense = tile_shape(cnt, h->mean_elems, false);
-    const int ls = dense.cw == dense.cols && !h->other_rows ? split_rows(h->N, h->mean_elems, dense.cw, h->sms) : 0;
     launch_transpose_in(h, x0, ln.tile[0], cnt, cols, ld, h->d_in_label);
     if (consumed) CU(h, cudaEventRecord(consumed, st));
     auto layers = [&](int used) {      // used: columns to gather for, a multiple of a lane's
@@ -1311,7 +1308,7 @@ int infer_tile(sdnn* h, InferLane& ln, const float* x0, int cnt, float* y_out, i
     {
         // of the columns the tracked and the windowed kernels take whole chunks
         const int used = track || h->windowed_layers == h->L ? cols : std::min((cnt + 7) / 8 * 8, cols);
-        const int rc = enqueue_layers(h, ln, cw, cols, used, track, layers);
+        const int rc = enqueue_layers(h, ln, cw, cols, used, ls, track, layers);
         if (rc) return rc;
     }
     const int cur = (h->L + (track ? 1 : 0)) & 1;
@@ -1572,16 +1569,19 @@ int launch_resident(sdnn* h, ResidentArgs a, int p, cudaStream_t st) {
     return SDNN_OK;
 }
 
-// How a call's inputs go: the width of resident_infer_kernel's CTAs, or 0 for the layer launches, which then read the reordered copies
-// (other) where the kernel would have taken the inputs had none of them been expected to die: with dead inputs dropped or not, the
-// bits are the same.
-struct Route { int width = 0; bool other = false; };
-Route route_of(const sdnn* h, int64_t inputs) {
+// How all tiles of a call go, so that it adds every input's sums in one order: the width of resident_infer_kernel's CTAs, or 0 for the layer
+// launches.  These share rows between 2^ls groups of lanes, or read the reordered copies (other) where the kernel would have taken the inputs had
+// none of them been expected to die: with dead inputs dropped or not, the bits are the same.
+struct Route { int width = 0, ls = 0; bool other = false; };
+// inputs: that go one after the other (of a call on device buffers all, on host buffers those of a tile); tile: of a whole tile
+Route route_of(const sdnn* h, int64_t inputs, int tile) {
     Route r;
-    if (!h->resident.units) return r;
-    const int tile = infer_tile_width(h), dense = resident_width(h->N, h->resident_elems, inputs, h->sms, tile, false);
-    r.width = dense && drops_dead(h) ? resident_width(h->N, h->resident_elems, inputs, h->sms, tile, true) : dense;
-    r.other = dense && !r.width;
+    if (h->resident.units) {
+        const int T = infer_tile_width(h), dense = resident_width(h->N, h->resident_elems, inputs, h->sms, T, false);
+        r.width = dense && drops_dead(h) ? resident_width(h->N, h->resident_elems, inputs, h->sms, T, true) : dense;
+        r.other = dense && !r.width;
+    }
+    if (!r.width && !r.other) r.ls = call_rows(h->N, h->mean_elems, tile, h->sms);
     return r;
 }
 
@@ -2532,7 +2532,7 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
     const bool want_sets = nz_count_out || nz_index_out || nz_total_out;
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     const int T = infer_tile_width(h);
-    const Route route = route_of(h, n_inputs);
+    const Route route = route_of(h, n_inputs, (int)std::min<int64_t>(n_inputs, T));
     const int width = route.width, lanes = n_inputs > T && !width ? infer_lanes(h, T) : 1;
     if ((rc = lanes_begin(h, lanes))) return rc;
     if (width && (rc = infer_resident(h, h->lane[0], width, x0, n_inputs, y_out, nz_count_out, nz_index_out, nz_index_capacity, want_sets, nz_index_out || nz_total_out))) return rc;
@@ -2540,7 +2540,7 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
     int64_t tile_no = 0;
     for (int64_t t0 = 0; t0 < n_inputs && !width; t0 += T, ++tile_no) {
         const int cnt = (int)((n_inputs - t0 < T) ? (n_inputs - t0) : T);
-        rc = infer_tile(h, h->lane[tile_no % lanes], x0 + (size_t)t0 * h->N, cnt, y_out ? y_out + (size_t)t0 * h->N : nullptr,
+        rc = infer_tile(h, h->lane[tile_no % lanes], route.ls, x0 + (size_t)t0 * h->N, cnt, y_out ? y_out + (size_t)t0 * h->N : nullptr,
                         nz_count_out ? nz_count_out + t0 : nullptr, nz_index_out, nz_index_capacity, want_sets);
         if (rc) break;
     }
@@ -2575,8 +2575,8 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     const int T = host_tile_width(h, n_inputs);
     const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // the two halves share the stages of one tile
     const int first = halved ? resident_half(h->N, n_inputs, h->sms) : 0;  // inputs of the first half, where both go through whole networks
-    Route route;                                                           // of both halves
-    if (first) route = route_of(h, n_inputs);
+    const int tile = (int)std::min<int64_t>(n_inputs, T);
+    const Route route = !halved ? route_of(h, tile, tile) : first ? route_of(h, n_inputs, T) : Route{0, call_rows(h->N, h->mean_elems, T, h->sms), false};
     const int64_t half = route.width ? first : T;
     if (!h->copy_stream) {
         CU(h, cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
@@ -2610,12 +2610,11 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         CU(h, cudaMemcpyAsync(stage[q], x0 + (size_t)t0 * h->N, bytes, cudaMemcpyHostToDevice, h->copy_stream));
         CU(h, cudaEventRecord(h->ev_copied[q], h->copy_stream));
         CU(h, cudaStreamWaitEvent(ln.stream, h->ev_copied[q], 0));
-        if (!halved) route = route_of(h, cnt);
         h->other_rows = route.other;
         if (route.width)
             rc = infer_resident(h, ln, halved ? 1 : route.width, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
                                 want_sets, want_sets, h->ev_consumed[q]);
-        else rc = infer_tile(h, ln, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
+        else rc = infer_tile(h, ln, route.ls, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
                              nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity, want_sets, h->ev_consumed[q]);
         h->other_rows = false;
         if (rc) break;

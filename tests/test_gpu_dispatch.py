@@ -570,3 +570,45 @@ def test_inference_with_rows_shared_by_groups_of_lanes(torch_cuda, n, cnt, ragge
         h.destroy()
     check_close(outs[0].cpu().numpy(), want, "x^L")
     assert all(torch.equal(y, outs[0]) for y in outs)
+
+
+@pytest.mark.parametrize("n,tile,cnt,host", [
+    (1024, 1024, 1100, True), (2000, 600, 1250, True), (1500, 450, 455, True),      # whole networks in shared memory, a last tile too small for them
+    (700, 100, 103, False), (700, 100, 106, True), (3000, 12, 29, False), (1500, 28, 60, False), (700, 8, 9, False),      # rows shared by groups of lanes
+    (700, 300, 303, False), (4100, 400, 450, False), (4100, 257, 300, True), (700, 4, 11, False), (900, 256, 257, True)])
+@pytest.mark.parametrize("kind", ["uniform", "ragged", "dying", "windows"])
+def test_bits_do_not_depend_on_an_inputs_place_in_the_call(torch_cuda, n, tile, cnt, host, kind):  # noqa: F811
+    """A call adds every input's sums in one order: the inputs of its last, narrower tile (or second half) are also its first ones, and give
+    the same bits there; from the first call's launches and the later ones' graphs."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    layers, flags = 5, 0
+    arrays = ragged_net(rng, n=n, layers=layers, kmax=60, scale=0.3) if kind == "ragged" else uniform_net(rng, n, 32, layers)
+    if kind == "dying":
+        flags = pkg.FLAG_SKIP_DEAD
+        arrays = [*arrays[:2], [np.full(n * 32, 1.0 / 16.0, dtype=np.float32)] * layers, [np.full(n, -0.35, dtype=np.float32)] * layers]
+    elif kind == "windows":
+        flags = pkg.FLAG_REORDER | pkg.FLAG_SMEM_WINDOWS
+        first = np.minimum(np.arange(n) // 100, n // 100 - 1) * 100      # blocks of 100 neurons, what is left belongs to the last one
+        size = np.where(first == first[-1], n - first, 100)
+        cols = [np.concatenate([np.sort(f + rng.choice(m, size=16, replace=False)) for f, m in zip(first, size)]).astype(np.int32) for _ in range(layers)]
+        arrays = ([np.arange(n + 1, dtype=np.int32) * 16] * layers, cols, [rng.uniform(-1, 1, size=n * 16).astype(np.float32) for _ in range(layers)], arrays[3])
+    h = pkg.Sdnn.create(*arrays, max_batch=tile, flags=flags)
+    assert kind != "windows" or h.windowed_layers() == layers
+    whole = min(tile, h.infer_tile_width())
+    again = cnt % whole if cnt > tile else cnt // 3               # inputs that come twice
+    x0 = vectors(rng, cnt, n) if kind != "dying" else (rng.random((cnt, n)) < rng.uniform(0.05, 0.5, size=(cnt, 1))).astype(np.float32)
+    x0[cnt - again:] = x0[:again]
+    for _ in range(3):
+        if host:
+            y = np.full((cnt, n), -1.0, dtype=np.float32)
+            h.infer_batch(x0, cnt, y, host=True)
+        else:
+            yd = torch.full((cnt, n), -1.0, device="cuda")
+            h.infer_batch(torch.from_numpy(x0).cuda(), cnt, yd)
+            y = yd.cpu().numpy()
+        assert np.array_equal(y[cnt - again:], y[:again])
+    pick = np.unique(np.concatenate([[0, cnt - 1], rng.integers(0, cnt, size=10)]))
+    if kind != "dying":
+        check_close(y[pick], OracleNet(*arrays).infer(x0[pick]), "x^L")
+    h.destroy()

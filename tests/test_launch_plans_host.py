@@ -17,6 +17,16 @@ extern "C" int cols(int cnt, long long elems, int windows) { return tile_shape(c
 extern "C" int chunk(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cw; }
 extern "C" int graph(int layers, long long elems, int cols, int track) { return tile_as_graph(layers, elems, cols, track); }
 extern "C" int rows_log(int n, long long elems, int cw) { return split_rows(n, elems, cw, 148); }
+extern "C" int call_log(int n, long long elems, int tile) { return call_rows(n, elems, tile, 148); }
+extern "C" int shared_chunk(int cnt, long long elems, int ls) { const TileShape t = tile_shape(cnt, elems, false, ls); return t.cw == t.cols ? t.cw : 0; }
+extern "C" int graphs_of_two_orders() {
+    GraphKey have[4], want;
+    int64_t asked[4] = {1, 0, 0, 0};
+    bool make = false;
+    have[0].cw = have[0].cols = have[0].used = 16; want = have[0];
+    have[0].ls = 2;
+    return pick_graph(have, asked, 4, want, make) != 0 && make;
+}
 extern "C" int units(const int* off, int n, int rows, int bytes, long long slots, int backward, unsigned* out) {
     const std::vector<unsigned> list = split_units(std::vector<int>(off, off + (n + 15) / 16 + 1), n, rows, bytes, 148, slots, backward != 0);
     std::copy(list.begin(), list.end(), out);
@@ -91,6 +101,23 @@ def test_rows_shared_in_inference(plan):
                 parts = 1 << plan.rows_log(n, n * per_row, cw)
                 assert parts == 1 or (cw // 8 * parts <= 32 and n * (cw // 8) * parts <= 65536 and parts * 8 <= per_row)
     assert plan.rows_log(700, 700 * 32, 64) == 2 and plan.rows_log(16384, 16384 * 32, 64) == 0
+
+
+def test_the_last_tile_of_a_call_shares_its_rows_like_the_others(plan):
+    """Rows are shared by what a call's whole tiles hold.  A narrower last tile keeps to that: one chunk of whole lanes, whose groups fit a
+    warp, and a graph of its own where a tile of its width in another call shares rows otherwise."""
+    plan.call_log.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+    plan.shared_chunk.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+    for n in (17, 700, 1500, 4096, 9000, 30000):
+        for per_row in (8, 32, 300):
+            for tile in (1, 4, 5, 8, 12, 28, 60, 100, 128, 129, 300):
+                ls = plan.call_log(n, n * per_row, tile)
+                assert ls == 0 if tile <= 4 or tile > 128 else ls == plan.rows_log(n, n * per_row, plan.cols(tile, n * per_row, 0))
+                for last in range(1, tile + 1) if ls else ():
+                    cw = plan.shared_chunk(last, n * per_row, ls)
+                    assert 8 <= cw <= plan.cols(tile, n * per_row, 0) and cw // 8 << ls <= 32 and last <= cw
+    assert plan.call_log(700, 700 * 32, 100) == 1 and plan.call_log(700, 700 * 32, 12) == 2
+    assert plan.graphs_of_two_orders()
 
 
 def test_tile_shapes(plan):
