@@ -1234,8 +1234,8 @@ backward_kernel(const BackwardArgs a) {
 // us a layer, as it was / split: 6007 neurons, rows of 8 to 56 entries, 37 inputs: forward 7.17 / 5.12, backward 8.37 / 7.01; 3000 neurons,
 // 32 a row, 12 inputs: 3.92 / 2.56, 5.11 / 3.92; 700 neurons, 64 inputs: 3.58 / 2.21, 4.77 / 3.24.
 // A warp has one unit and so nothing to ask for ahead of time but what the next launch will read: the entries of its layer, in pieces
-// of 4 KB (of nets that outgrow L2 they come out of HBM: a step of 6007 x 56, 37 inputs 689 -> 655 us, 3000 x 56, 100 inputs 622 -> 597;
-// a chain of the narrowest layers pays 2 %).
+// of 4 KB, where a pass over the net walks so much that they are not at hand (sdnn_plan::asks_ahead; a step of 6007 x 56, 37 inputs 691 -> 654
+// us, 3000 x 56, 100 inputs 625 -> 596; 700 x 24, 16 inputs, which do not ask, 142 -> 134).
 struct NextEntries { const void* idx; const float* val; unsigned idx_bytes, val_bytes; };
 __device__ __forceinline__ void ask_for(const void* base, unsigned bytes, unsigned first, unsigned stride) {
     for (unsigned long long lo = (unsigned long long)first << 12; lo < bytes; lo += (unsigned long long)stride << 12)

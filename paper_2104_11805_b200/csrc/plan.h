@@ -140,4 +140,12 @@ inline std::vector<unsigned> split_units(const std::vector<int>& off, int n, int
     return list;
 }
 
+// Whether the launches of layers that do not fill the device ask for the next launch's entries while they work (see forward_split_kernel).
+// bytes: what a pass over the net walks: of an inference call the row-major copies, of a train step both copies, the activations and the
+// deltas; width: columns of a train step's tiles, 0: inference.  A pass whose entries are near at hand pays for asking; how near they have to
+// be was measured (us with / without, 24 to 480 layers of 640 to 6007 neurons, L2 126 MB): inference of 8 to 60 inputs 1.02 .. 1.07 up to 18 MB, 0.92 ..
+// 0.99 from 23 MB on; train steps of 37 and 100 inputs 1.00 .. 1.01 up to 34 MB, 0.95 .. 1.00 from 47 MB (700 neurons x 100, 100 inputs,
+// 99 MB: 0.88); of 8 to 28 inputs, whose launches wait for round trips and not for bytes, 1.00 .. 1.04 up to L2's size and 0.985 .. 1.02 beyond.
+inline bool asks_ahead(int64_t bytes, int width, int64_t l2) { return width == 0 ? 6 * bytes > l2 : width >= 64 ? 3 * bytes > l2 : bytes > l2; }
+
 }  // namespace sdnn_plan

@@ -173,6 +173,7 @@ struct sdnn {
     std::vector<std::vector<int>> labels;   // [L + 1] host: tile row of neuron i at boundary k (x^k, delta^k); empty = identity
     int windowed_layers = 0;
     int64_t mean_elems = 0;             // stored elements per layer, padding included
+    bool ask_infer = false, ask_train = false;      // asks_ahead for calls of inference, for train steps at the handle's width
     VectorLayer* d_vector = nullptr;    // [L] table of vector_infer_kernel (NULL: the net is not for it)
     int vector_kpad = 0;                // entries per row of every slice of every layer (the same everywhere, or no table)
     int* vector_status = nullptr;       // pinned: raised by a whole-network kernel whose wait for its neighbours ran out
@@ -581,9 +582,9 @@ bool entry_parallel(const sdnn* h, int ld) {
 bool moved(const LayerMem& lm, int ld);
 float* delta_tile(sdnn* h, int layer, size_t tile);
 
-// what the launch after one of these will read of its layer's entries (nothing where there is none)
-NextEntries next_entries(const sdnn* h, int layer, bool transposed) {
-    if (layer < (transposed ? 1 : 0) || layer >= h->L || h->lay[layer].windowed) return NextEntries{nullptr, nullptr, 0, 0};
+// what the launch after one of these will read of its layer's entries (nothing where there is none, or it is not to be asked for)
+NextEntries next_entries(const sdnn* h, bool ask, int layer, bool transposed) {
+    if (!ask || layer < (transposed ? 1 : 0) || layer >= h->L || h->lay[layer].windowed) return NextEntries{nullptr, nullptr, 0, 0};
     const LayerMem& lm = h->lay[layer];
     const int64_t elems = std::min<int64_t>(transposed ? lm.c_elems : lm.r_elems, 1 << 29);
     return NextEntries{transposed ? lm.c_idx : lm.r_idx, transposed ? lm.c_val : lm.r_val, (unsigned)(elems * (h->idx16 ? 2 : 4)), (unsigned)(elems * 4)};
@@ -596,7 +597,7 @@ void launch_forward_split(sdnn* h, int layer, const float* xin, float* xout, int
     const int rows = 32 / G >> ls, nunits = ls ? (h->N + rows - 1) / rows : lm.r_nunits;
     launch_k(h, forward_split_kernel<G, I16>, dim3((nunits + SPLIT_WARPS - 1) / SPLIT_WARPS), dim3(32 * SPLIT_WARPS), h->pdl, rows_of(h, layer),
              ls ? (const unsigned*)nullptr : (const unsigned*)lm.r_units, ls, nunits, (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp,
-             h->cfg.activation, h->pdl ? h->fwd_pdl : 0, last, next_entries(h, layer + 1, false));
+             h->cfg.activation, h->pdl ? h->fwd_pdl : 0, last, next_entries(h, ls ? h->ask_infer : h->ask_train, layer + 1, false));
     count_launch(h);
 }
 template <int G, bool I16>
@@ -606,7 +607,7 @@ void launch_backward_split(sdnn* h, int layer, int ld) {
     const float* acts = h->bwd_acts ? h->bwd_acts : h->d_acts;
     launch_on(h, backward_split_kernel<G, I16>, dim3(lm.c_nunits), dim3(32), 0, h->pdl, moved(lm, ld), cols_of(h, layer), (const unsigned*)lm.c_units, lm.c_nunits,
               acts + (size_t)layer * tile, (const float*)delta_tile(h, layer, tile), delta_tile(h, layer - 1, tile), h->N, h->cfg.clamp, h->cfg.activation,
-              (const StepParams*)h->d_sp, h->pdl ? PDL_EARLY : 0, acts + (size_t)(layer - 1) * tile, (unsigned)(tile * sizeof(float)), next_entries(h, layer - 1, true));
+              (const StepParams*)h->d_sp, h->pdl ? PDL_EARLY : 0, acts + (size_t)(layer - 1) * tile, (unsigned)(tile * sizeof(float)), next_entries(h, h->ask_train, layer - 1, true));
     count_launch(h);
 }
 #define SDNN_BY_WIDTH(WIDTH, FN, ...)                     \
@@ -2458,9 +2459,12 @@ int sdnn_finalize(sdnn_t* h) {
         int rc;
         if ((rc = build_moves(h)) || (rc = build_vector(h)) || (rc = build_resident(h))) return rc;
     }
-    int64_t elems = 0;
-    for (const LayerMem& lm : h->lay) elems += lm.windowed ? lm.w_elems : lm.r_elems;
+    int64_t elems = 0, transposed = 0;
+    for (const LayerMem& lm : h->lay) { elems += lm.windowed ? lm.w_elems : lm.r_elems; transposed += lm.c_elems; }
     h->mean_elems = elems / h->L;
+    const int64_t entry = h->idx16 ? 6 : 8;
+    h->ask_infer = asks_ahead(elems * entry, 0, h->l2_bytes);
+    h->ask_train = asks_ahead((elems + transposed) * entry + 2 * (int64_t)h->L * h->N * h->ld_max * (int64_t)sizeof(float), h->ld_max, h->l2_bytes);
     CU(h, cudaStreamSynchronize(h->stream));
     h->finalized = true;
     return SDNN_OK;

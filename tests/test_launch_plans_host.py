@@ -19,6 +19,7 @@ extern "C" int graph(int layers, long long elems, int cols, int track) { return 
 extern "C" int rows_log(int n, long long elems, int cw) { return split_rows(n, elems, cw, 148); }
 extern "C" int call_log(int n, long long elems, int tile) { return call_rows(n, elems, tile, 148); }
 extern "C" int shared_chunk(int cnt, long long elems, int ls) { const TileShape t = tile_shape(cnt, elems, false, ls); return t.cw == t.cols ? t.cw : 0; }
+extern "C" int asks(long long bytes, int width) { return asks_ahead(bytes, width, 132644864); }
 extern "C" int graphs_of_two_orders() {
     GraphKey have[4], want;
     int64_t asked[4] = {1, 0, 0, 0};
@@ -118,6 +119,18 @@ def test_the_last_tile_of_a_call_shares_its_rows_like_the_others(plan):
                     assert 8 <= cw <= plan.cols(tile, n * per_row, 0) and cw // 8 << ls <= 32 and last <= cw
     assert plan.call_log(700, 700 * 32, 100) == 1 and plan.call_log(700, 700 * 32, 12) == 2
     assert plan.graphs_of_two_orders()
+
+
+def test_entries_at_hand_are_not_asked_for(plan):
+    """Launches ask for the next one's entries where a pass over the net walks more than stays at hand: a third of L2 in wide train steps,
+    all of it in narrow ones, a sixth in inference."""
+    plan.asks.argtypes = [ctypes.c_longlong, ctypes.c_int]
+
+    def step(n, layers, width):
+        return plan.asks(n * 32 * 12 * layers + 8 * layers * n * width, width)
+    assert [step(700, 24, w) for w in (8, 16, 32, 64, 128)] == [0] * 5
+    assert step(6007, 56, 64) and step(6007, 24, 64) and step(700, 100, 128) and step(6007, 56, 32) and not step(700, 100, 32) and not step(1500, 100, 16)
+    assert not plan.asks(700 * 32 * 6 * 120, 0) and plan.asks(1500 * 32 * 6 * 120, 0)
 
 
 def test_tile_shapes(plan):
