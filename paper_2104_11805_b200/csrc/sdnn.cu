@@ -77,6 +77,7 @@ struct LayerMem {
     int r_nunits = 0, c_nunits = 0;
     Move move{};                           // how r_val is filled from c_val after an update (nb = 0: row units compute theirs)
     std::vector<int> r_slice_off;          // host copy of the row-major slice offsets
+    std::vector<int> c_slice_off;          // ... of the transposed copy's, until sdnn_finalize
     RowShape shape;
     // set-up reordering (SDNN_FLAG_REORDER): how the stored rows and entries map back to the caller's CSR arrays
     std::vector<int> row_src;              // [N] stored row -> caller's row (empty: identity)
@@ -642,7 +643,7 @@ int build_units(sdnn* h, const std::vector<int>& off, bool backward, bool beside
     const std::vector<unsigned> list = split_units(off, h->N, rows, h->ld_max * 4, h->sms, beside_rows ? std::min<int64_t>(slots * 7 / 10, slots - whole) : slots, backward);
     if (list.empty()) return SDNN_OK;
     int rc;
-    if ((rc = dev_alloc(h, units, list.size(), false))) return rc;
+    if ((rc = dev_alloc(h, units, list.size(), false))) return rc == SDNN_ERR_OOM ? SDNN_OK : rc;      // it saves time and is not needed
     CU(h, cudaMemcpyAsync(*units, list.data(), list.size() * sizeof(unsigned), cudaMemcpyHostToDevice, h->stream));
     CU(h, cudaStreamSynchronize(h->stream));
     *nunits = (int)list.size();
@@ -1902,6 +1903,20 @@ int build_moves(sdnn* h) {
     return rc;
 }
 
+// Column units of the layers that have a transposed copy (called by sdnn_finalize, when it is known which of them have maps: the row units
+// of a layer that does without run beside its column units and need room).
+int build_column_units(sdnn* h) {
+    for (LayerMem& lm : h->lay) {
+        if (lm.c_slice_off.empty()) continue;
+        const bool beside_rows = !moved(lm, h->ld_max);
+        const int rc = h->idx16 ? build_units<true>(h, lm.c_slice_off, true, beside_rows, &lm.c_units, &lm.c_nunits)
+                                : build_units<false>(h, lm.c_slice_off, true, beside_rows, &lm.c_units, &lm.c_nunits);
+        if (rc) return rc;
+        std::vector<int>().swap(lm.c_slice_off);
+    }
+    return SDNN_OK;
+}
+
 // Lays out one validated layer (caller's or reordered CSR, host arrays) in the kernels' sliced format and uploads it.
 // out_label (host, or NULL): tile row that each given row writes, for a layer whose rows are stored group by group.
 int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_idx, const float* values, const float* bias,
@@ -2017,7 +2032,6 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
                     c_idx[(size_t)sliced_pos(c_off.data(), place[j], q)] = out_label ? out_label[i] : i;      // the delta tile's row
                 }
         }
-        if ((rc = h->idx16 ? build_units<true>(h, c_off, true, !moves(lm, h->ld_max), &lm.c_units, &lm.c_nunits) : build_units<false>(h, c_off, true, !moves(lm, h->ld_max), &lm.c_units, &lm.c_nunits))) return rc;
         if ((rc = alloc_indices(h, &lm.c_idx, (size_t)lm.c_elems))) return rc;
         if ((rc = dev_alloc(h, &lm.c_val, (size_t)lm.c_elems, true))) return rc;
         CU(h, cudaMemcpyAsync(h->d_c_slice_off + (size_t)layer * (NS + 1), c_off.data(), (size_t)(NS + 1) * sizeof(int), cudaMemcpyHostToDevice, h->stream));
@@ -2025,6 +2039,7 @@ int upload_layer(sdnn* h, int layer, const int32_t* row_ptr, const int32_t* col_
         CU(h, cudaMemcpyAsync(h->d_c_order + (size_t)layer * N, order.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         if (lm.c_elems && (rc = upload_indices(h, lm.c_idx, c_idx))) return rc;
         if (!move_shape(h, layer).nb && (rc = refresh_mirror(h, layer, nullptr))) return rc;      // else with its maps, in sdnn_finalize
+        lm.c_slice_off = c_off;      // copied: its upload may still be on its way
     }
     CU(h, cudaStreamSynchronize(h->stream));   // the host vectors above go out of scope; the caller may reuse its arrays
     {
@@ -2457,7 +2472,7 @@ int sdnn_finalize(sdnn_t* h) {
     }
     {
         int rc;
-        if ((rc = build_moves(h)) || (rc = build_vector(h)) || (rc = build_resident(h))) return rc;
+        if ((rc = build_moves(h)) || (rc = build_column_units(h)) || (rc = build_vector(h)) || (rc = build_resident(h))) return rc;
     }
     int64_t elems = 0, transposed = 0;
     for (const LayerMem& lm : h->lay) { elems += lm.windowed ? lm.w_elems : lm.r_elems; transposed += lm.c_elems; }

@@ -612,3 +612,49 @@ def test_bits_do_not_depend_on_an_inputs_place_in_the_call(torch_cuda, n, tile, 
     if kind != "dying":
         check_close(y[pick], OracleNet(*arrays).infer(x0[pick]), "x^L")
     h.destroy()
+
+
+def launched(torch, call, name):
+    """Blocks of every launch that `call` makes of kernels of that name."""
+    import json
+    import os
+    import tempfile
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        call()
+        torch.cuda.synchronize()
+    with tempfile.TemporaryDirectory() as d:
+        trace = os.path.join(d, "trace.json")
+        p.export_chrome_trace(trace)
+        with open(trace) as f:
+            events = [e for e in json.load(f)["traceEvents"] if e.get("cat") == "kernel"]
+    if not events:
+        pytest.skip("no kernels in the trace")
+    return [e["args"]["grid"][0] for e in events if name in e["name"]]
+
+
+@pytest.mark.parametrize("n,k,B", [(3000, 64, 37), (6007, 32, 37), (2600, 112, 20)])
+def test_column_units_leave_room_for_row_units_where_no_maps_are_made(torch_cuda, all_but, n, k, B):  # noqa: F811
+    """A layer large enough for maps has none where the gradient is kept or memory does not allow it.  Its column units then run beside row
+    units, and both fit the device (16 warps an SM) in one round; with maps the column units have it to themselves."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n)
+    arrays = uniform_net(rng, n, k, 3)
+    x, y = (torch.from_numpy(vectors(rng, B, n)).cuda() for _ in range(2))
+    slots = 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    groups = 32 // (8 if B > 32 else 4)
+    rows, taken, weights = (n + groups - 1) // groups, [], []
+    for flags in (0, pkg.FLAG_KEEP_DEBUG, 0):
+        if len(taken) == 2:
+            all_but(taken[0] + (40 << 20))                        # room for the net, not for what the maps leave to later calls
+        h = pkg.Sdnn.create(*arrays, max_batch=B, train=True, activation=pkg.ACT_SIGMOID, flags=flags | pkg.FLAG_NO_GRAPH)
+        taken.append(h.device_bytes())
+        moves = launched(torch, lambda: h.train_step(x, y, B, 0.5), "split_values_kernel")
+        units = launched(torch, lambda: h.train_step(x, y, B, 0.5), "backward_split_kernel")
+        assert len(moves) == (2 if len(taken) == 1 else 0)
+        assert all(u <= (slots if moves else slots - rows) for u in units) and (units or not moves)
+        weights.append([h.get_weights(l, want_bias=False) for l in range(3)])
+        h.destroy()
+    for w in weights[1:]:
+        for a, b in zip(w, weights[0]):
+            check_close(a, b, "W after two steps")
