@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsdnn.so")
 SOURCES = [os.path.join(CSRC, "sdnn.cu")]
-DEPENDS = SOURCES + [os.path.join(CSRC, "kernels.cuh"), os.path.join(CSRC, "vector.cuh"), os.path.join(CSRC, "resident.cuh"), os.path.join(CSRC, "resident.h"), os.path.join(CSRC, "plan.h"), os.path.join(CSRC, "reorder.h"), os.path.join(HERE, "..", "include", "sdnn.h")]
+DEPENDS = SOURCES + [os.path.join(CSRC, "kernels.cuh"), os.path.join(CSRC, "vector.cuh"), os.path.join(CSRC, "resident.cuh"), os.path.join(CSRC, "resident.h"), os.path.join(CSRC, "plan.h"), os.path.join(CSRC, "capture.h"), os.path.join(CSRC, "reorder.h"), os.path.join(HERE, "..", "include", "sdnn.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

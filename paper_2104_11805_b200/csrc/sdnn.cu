@@ -4,6 +4,7 @@
 // arithmetic step runs in the kernels of kernels.cuh.
 #include "../../include/sdnn.h"
 #include "kernels.cuh"
+#include "capture.h"
 #include "plan.h"
 #include "vector.cuh"
 #include "resident.cuh"
@@ -1085,13 +1086,14 @@ int infer_vector(sdnn* h, const float* x0, int cnt, float* y, int* nz_count) {
 // timing events are recorded (as external event-record nodes while capturing a graph).
 // averaged: the forward chain runs on the whole batch, then the batch means of x^0..x^L and the averaged delta^L are
 // formed and the backward chain runs on those single vectors (tiles of padded width 4).
-void enqueue_step_body(sdnn* h, int ld, int v, unsigned flags, bool averaged) {
+int enqueue_step_body(sdnn* h, int ld, int v, unsigned flags, bool averaged) {
     const size_t tile = (size_t)h->N * ld;
     cudaEventRecordWithFlags(h->ev[0], h->stream, flags);
     {
         NvtxRange chain("sdnn forward chain");
-        if (v) forward_vector(h, v);
-        else for (int k = 0; k < h->L; ++k) {
+        if (v) {
+            if (const int rc = forward_vector(h, v)) return rc;
+        } else for (int k = 0; k < h->L; ++k) {
             NvtxRange pass("forward layer", k + 1);
             launch_forward(h, k, h->d_acts + (size_t)k * tile, h->d_acts + (size_t)(k + 1) * tile, ld, ld, ld, h->used);
         }
@@ -1117,6 +1119,26 @@ void enqueue_step_body(sdnn* h, int ld, int v, unsigned flags, bool averaged) {
         h->bwd_acts = nullptr;
     }
     cudaEventRecordWithFlags(h->ev[2], h->stream, flags);
+    return SDNN_OK;
+}
+
+// Captures what `body` enqueues on `stream` (0 or an SDNN_ERR from it) as a graph; launches: how many it holds.
+struct StreamCapture {
+    using Graph = cudaGraph_t;
+    cudaStream_t stream;
+    cudaError_t begin() const { return cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal); }
+    cudaError_t end(cudaGraph_t* g) const { return cudaStreamEndCapture(stream, g); }
+    cudaError_t last_error() const { return cudaGetLastError(); }
+    cudaError_t instantiate(cudaGraphExec_t* exec, cudaGraph_t g) const { return cudaGraphInstantiate(exec, g, 0); }
+    void destroy(cudaGraph_t g) const { cudaGraphDestroy(g); }
+};
+template <typename Body>
+int capture_on(sdnn* h, cudaStream_t stream, cudaGraphExec_t* exec, int64_t* launches, const Body& body) {
+    const int64_t before = h->launches;
+    const int rc = capture_graph(StreamCapture{stream}, exec, body, [&](cudaError_t e, const char* what) { return cuda_fail(h, e, what); });
+    *launches = h->launches - before;
+    h->launches = before;
+    return rc;
 }
 
 int train_step_device(sdnn* h, const float* x0, const float* target, int B, float eta, float* loss_out, bool averaged = false) {
@@ -1137,7 +1159,7 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
                                                          averaged ? h->d_sp_batch : (StepParams*)nullptr, eta, h->d_loss);
     count_launch(h);
     if (h->cfg.flags & SDNN_FLAG_NO_GRAPH) {
-        enqueue_step_body(h, ld, v, cudaEventRecordDefault, averaged);
+        if (const int rc = enqueue_step_body(h, ld, v, cudaEventRecordDefault, averaged)) return rc;
     } else {
         cudaGraphExec_t& graph = averaged ? h->graph_avg : h->graph;
         int& graph_ld = averaged ? h->graph_avg_ld : h->graph_ld;
@@ -1147,17 +1169,7 @@ int train_step_device(sdnn* h, const float* x0, const float* target, int B, floa
         // a graph made for more inputs of the same padded width serves fewer as well (the short batch at the end of an epoch)
         if (!graph || graph_ld != ld || graph_v != v || graph_used < h->used) {
             if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
-            cudaGraph_t g = nullptr;
-            const int64_t before = h->launches;
-            CU(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-            enqueue_step_body(h, ld, v, cudaEventRecordExternal, averaged);
-            cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-            graph_launches = h->launches - before;
-            h->launches = before;
-            if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
-            e = cudaGraphInstantiate(&graph, g, 0);
-            cudaGraphDestroy(g);
-            if (e != cudaSuccess) { graph = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
+            if (const int rc = capture_on(h, h->stream, &graph, &graph_launches, [&] { return enqueue_step_body(h, ld, v, cudaEventRecordExternal, averaged); })) return rc;
             graph_ld = ld; graph_v = v; graph_used = h->used;
         }
         CU(h, cudaGraphLaunch(graph, h->stream));
@@ -1237,17 +1249,7 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, int ls, b
     TileGraph& g = ln.graphs[q];
     if (make) {
         if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; ln.graph_asked[q] = 0; }
-        cudaGraph_t graph = nullptr;
-        const int64_t before = h->launches;
-        CU(h, cudaStreamBeginCapture(ln.stream, cudaStreamCaptureModeThreadLocal));
-        layers(key.used);
-        cudaError_t e = cudaStreamEndCapture(ln.stream, &graph);
-        g.launches = h->launches - before;
-        h->launches = before;
-        if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&g.exec, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) { g.exec = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
+        if (const int rc = capture_on(h, ln.stream, &g.exec, &g.launches, [&] { layers(key.used); return SDNN_OK; })) return rc;
         ln.graph_key[q] = key;
     }
     ln.graph_asked[q] = h->infer_calls;

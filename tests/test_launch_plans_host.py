@@ -405,3 +405,42 @@ def test_steps_of_eight_rows(resident, spread):
         assert seen == before
         if not spread and skew == 1:
             assert waves == steps + max(abs(c - steps) for c in total)
+
+
+CAPTURE_WRAPPER = """
+#include "capture.h"
+// calls that fail where `which` says so (1 begin, 2 end, 3 a launch, 4 instantiation; 5: the body itself) and note what happened
+static int which, open_captures, graphs, execs;
+struct Fake {
+    using Graph = int;
+    int begin() const { if (which == 1) return 100; ++open_captures; return 0; }
+    int end(int* g) const { --open_captures; if (which == 2) return 200; ++graphs; *g = 7; return 0; }
+    int last_error() const { return which == 3 ? 300 : 0; }
+    int instantiate(int* exec, int) const { if (which == 4) return 400; ++execs; *exec = 9; return 0; }
+    void destroy(int) const { --graphs; }
+};
+extern "C" int capture(int fails, int* state) {
+    which = fails; open_captures = graphs = execs = 0;
+    int exec = 0;
+    const int rc = sdnn_plan::capture_graph(Fake{}, &exec, [] { return which == 5 ? -5 : 0; }, [](int e, const char*) { return -e; });
+    state[0] = open_captures; state[1] = graphs; state[2] = execs; state[3] = exec;
+    return rc;
+}
+"""
+
+
+def test_no_graph_is_kept_of_a_capture_that_failed(tmp_path):
+    """A capture that was begun is ended, the captured graph is given back, and there is something to launch only if everything went well:
+    not where the body gave up, a launch failed, or a call did."""
+    src, lib = tmp_path / "capture.cpp", tmp_path / "libcapture.so"
+    src.write_text(CAPTURE_WRAPPER)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)])
+    lib = ctypes.CDLL(str(lib))
+    state = (ctypes.c_int * 4)()
+    for fails, rc in ((0, 0), (1, -100), (2, -200), (3, -300), (4, -400), (5, -5)):
+        assert lib.capture(fails, state) == rc
+        assert list(state) == ([0, 0, 1, 9] if fails == 0 else [0, 0, 0, 0]), fails
+    source = open(os.path.join(CSRC, "sdnn.cu")).read()
+    product, probes = source.split('extern "C" int sdnn_probe_gather_rate')[:2]
+    assert product.count("cudaStreamBeginCapture(") == product.count("cudaGraphInstantiate(") == 1      # both in what capture_graph is given
+    assert "if (const int rc = forward_vector(h, v)) return rc;" in product
