@@ -1258,6 +1258,16 @@ int enqueue_layers(sdnn* h, InferLane& ln, int cw, int cols, int used, int ls, b
     return SDNN_OK;
 }
 
+// The launch helpers work for a lane, until the tile's call returns: also where it returns early, so that what the handle launches next is
+// on its own stream again.
+struct LaneScope {
+    sdnn* h;
+    LaneScope(sdnn* handle, InferLane& ln) : h(handle) { h->cur = &ln; h->launch_stream = ln.stream; }
+    ~LaneScope() { h->launch_stream = nullptr; h->cur = &h->lane[0]; }
+    LaneScope(const LaneScope&) = delete;
+    LaneScope& operator=(const LaneScope&) = delete;
+};
+
 // One tile of inference on device buffers, on lane `ln`: x0 [cnt][N] -> outputs for these cnt inputs.
 // ls: of the call, not of this tile (call_rows).  consumed (or NULL): recorded once x0 has been read.
 int infer_tile(sdnn* h, InferLane& ln, int ls, const float* x0, int cnt, float* y_out, int* cnt_out, int* idx_out, long long capacity,
@@ -1265,8 +1275,7 @@ int infer_tile(sdnn* h, InferLane& ln, int ls, const float* x0, int cnt, float* 
     NvtxRange call("sdnn inference tile");
     const int ld = h->ld_max;
     cudaStream_t st = ln.stream;
-    h->cur = &ln;
-    h->launch_stream = st;
+    const LaneScope scope(h, ln);
     const bool track = drops_dead(h);
     // dropping dead inputs works on chunks of 64 whatever the padding
     const TileShape shape = track && cnt > 32 ? TileShape{TRACK_CHUNK, (cnt + TRACK_CHUNK - 1) / TRACK_CHUNK * TRACK_CHUNK} : tile_shape(cnt, h->mean_elems, h->windowed_layers == h->L, ls);
@@ -1316,8 +1325,6 @@ int infer_tile(sdnn* h, InferLane& ln, int ls, const float* x0, int cnt, float* 
         if (rc) return rc;
     }
     const int cur = (h->L + (track ? 1 : 0)) & 1;
-    h->launch_stream = nullptr;
-    h->cur = &h->lane[0];
     const float* xl = ln.tile[cur];
     if (y_out) {
         dim3 grid((h->N + TRANSPOSE_ROWS - 1) / TRANSPOSE_ROWS, (cnt + 31) / 32), block(256);

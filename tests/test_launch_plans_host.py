@@ -444,3 +444,12 @@ def test_no_graph_is_kept_of_a_capture_that_failed(tmp_path):
     product, probes = source.split('extern "C" int sdnn_probe_gather_rate')[:2]
     assert product.count("cudaStreamBeginCapture(") == product.count("cudaGraphInstantiate(") == 1      # both in what capture_graph is given
     assert "if (const int rc = forward_vector(h, v)) return rc;" in product
+
+
+def test_a_tile_gives_the_launch_stream_back_wherever_it_returns():
+    """The launch helpers' stream is a lane's only while an object lives whose end gives it back; the backward chain sets and clears it around
+    launches that do not return."""
+    source = open(os.path.join(CSRC, "sdnn.cu")).read()
+    tile = source[source.index("\nint infer_tile("):source.index("// Inputs per inference tile.")]
+    assert "const LaneScope scope(h, ln);" in tile and "h->launch_stream =" not in tile and "h->cur =" not in tile
+    assert source.count("h->launch_stream = ln.stream") == 1 and "~LaneScope() { h->launch_stream = nullptr; h->cur = &h->lane[0]; }" in source
