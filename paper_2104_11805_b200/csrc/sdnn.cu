@@ -1429,8 +1429,9 @@ void reorder_rows(sdnn* h, int layer, int layers) {
     resident_reorder_kernel<<<dim3((h->N + 7) / 8, layers), 256, 0, h->stream>>>(set, h->N, h->resident_idx2, h->resident_val2);
 }
 
-// Lays the net out for resident_infer_kernel where batches of max_batch inputs would go through it, or where the handle is for
-// large batches and larger ones would (called by sdnn_finalize).
+// Lays the net out for resident_infer_kernel where batches of max_batch inputs go through it (called by sdnn_finalize): 7 bytes for a
+// stored entry, 13 to 15 with SDNN_FLAG_SKIP_DEAD.  Not for what larger batches might: a handle for 640 inputs of 4096 neurons would hold its net
+// twice to answer batches of thousands, should they ever come, in three quarters of the time.
 int build_resident(sdnn* h) {
     if (h->cfg.train || h->reorder || h->N > 65536 - 2 * RES_UNIT || !resident_shape(h->N, 1).ok) return SDNN_OK;
     const int N = h->N, L = h->L, units = resident_shape(N, 1).units;
@@ -1466,8 +1467,7 @@ int build_resident(sdnn* h) {
     }
     unit_at[(size_t)L * units] = (int)run;
     const double elems = 128.0 * run / L;
-    auto takes = [&](int64_t inputs) { return resident_width(N, elems, inputs, h->sms, infer_tile_width(h), false) != 0; };
-    if (!takes(h->cfg.max_batch) && !(h->cfg.max_batch >= 512 && takes(10 * (int64_t)h->cfg.max_batch))) return SDNN_OK;
+    if (!resident_width(N, elems, h->cfg.max_batch, h->sms, infer_tile_width(h), false)) return SDNN_OK;
 
     auto room = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t rows = (size_t)L * units * RES_UNIT, entries = (size_t)run * 128;
@@ -1479,9 +1479,10 @@ int build_resident(sdnn* h) {
                             h->compaction ? (size_t)elems_stored * (h->idx16 ? 2 : 4) : 0, h->compaction ? (size_t)elems_stored * sizeof(float) : 0, L * sizeof(int*), L * sizeof(float*)};
     size_t bytes = 0, left = 0, whole = 0;
     for (size_t b : sizes) bytes += room(b);
-    // it saves time and is not needed: not where it would take what later calls allocate (a second lane, staging of host batches)
+    // it saves time and is not needed: not where it would take what later calls allocate (a second lane, staging of host batches), and the
+    // last quarter of the device is left to handles and tensors that come later
     CU(h, cudaMemGetInfo(&left, &whole));
-    if (bytes + 6 * (size_t)N * h->ld_max * sizeof(float) + ((size_t)64 << 20) > left) return SDNN_OK;
+    if (bytes + std::max(6 * (size_t)N * h->ld_max * sizeof(float) + ((size_t)64 << 20), whole / 4) > left) return SDNN_OK;
     char* at = nullptr;
     int rc = dev_alloc(h, &at, bytes, false);
     if (rc) return rc == SDNN_ERR_OOM ? SDNN_OK : rc;

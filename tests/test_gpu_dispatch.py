@@ -658,3 +658,25 @@ def test_column_units_leave_room_for_row_units_where_no_maps_are_made(torch_cuda
     for w in weights[1:]:
         for a, b in zip(w, weights[0]):
             check_close(a, b, "W after two steps")
+
+
+@pytest.mark.parametrize("n,tile,cnt,quarter", [(4096, 640, 5000, False), (2048, 600, 3000, False), (2048, 1024, 3000, True)])
+def test_nets_are_laid_out_twice_only_for_batches_of_the_handles_own_size(torch_cuda, all_but, n, tile, cnt, quarter):  # noqa: F811
+    """A handle whose batches of max_batch inputs go through the layer launches holds its net once, whatever larger ones would take; and so does
+    every handle made when less than a quarter of the device is free.  Larger batches give the same outputs."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n)
+    layers, k = 60, 32
+    arrays = uniform_net(rng, n, k, layers)
+    if quarter:
+        all_but(torch.cuda.get_device_properties(0).total_memory // 5)
+    h = pkg.Sdnn.create(*arrays, max_batch=tile, activation=pkg.ACT_SIGMOID)
+    once = 6 * n * k * layers + 2 * 4 * n * ((tile + 255) // 256 * 256) + (24 << 20)      # entries, two tiles, lists and the last block of small arrays
+    assert h.device_bytes() < once, (h.device_bytes(), once)
+    x0 = vectors(rng, cnt, n)
+    y = torch.full((cnt, n), -1.0, device="cuda")
+    before = h.kernel_launches()
+    h.infer_batch(torch.from_numpy(x0).cuda(), cnt, y)
+    assert h.kernel_launches() - before > layers
+    check_close(y[-8:].cpu().numpy(), OracleNet(*arrays, activation="sigmoid").infer(x0[-8:]), "x^L")
+    h.destroy()
