@@ -2602,11 +2602,11 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     // two input stages and a copy stream: the copy of tile t+1 runs under the layers of tile t
     const int T = host_tile_width(h, n_inputs);
-    const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // the two halves share the stages of one tile
+    const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // its pieces (two halves, or narrow tiles of a wide net) share the stages of one tile
     const int first = halved ? resident_half(h->N, n_inputs, h->sms) : 0;  // inputs of the first half, where both go through whole networks
     const int tile = (int)std::min<int64_t>(n_inputs, T);
     const Route route = !halved ? route_of(h, tile, tile) : first ? route_of(h, n_inputs, T) : Route{0, call_rows(h->N, h->mean_elems, T, h->sms), false};
-    const int64_t half = route.width ? first : T;
+    const int64_t piece = halved && route.width ? first : T;               // inputs of each but the last
     if (!h->copy_stream) {
         CU(h, cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
         for (int q = 0; q < 2; ++q) {
@@ -2615,7 +2615,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         }
     }
     if (!halved && !h->d_stage_a2 && (rc = dev_alloc(h, &h->d_stage_a2, (size_t)h->cfg.max_batch * h->N, false))) return rc;
-    float* stage[2] = {h->d_stage_a, halved ? h->d_stage_a + (size_t)half * h->N : h->d_stage_a2};
+    float* stage[2] = {h->d_stage_a, halved ? h->d_stage_a + (size_t)piece * h->N : h->d_stage_a2};
     CU(h, cudaEventRecord(h->ev_consumed[0], h->stream));       // the stages may still be read by earlier work on the stream
     CU(h, cudaEventRecord(h->ev_consumed[1], h->stream));
     const int lanes = n_inputs > T ? infer_lanes(h, T) : 1;
@@ -2626,11 +2626,11 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     }
     h->lane[0].stage_out = h->d_stage_b;
     h->lane[0].stage_cnt = h->d_stage_cnt;
-    h->lane[1].stage_out = halved ? h->d_stage_b + (size_t)half * h->N : h->d_stage_b2;
-    h->lane[1].stage_cnt = halved ? h->d_stage_cnt + half : h->d_stage_cnt2;
+    h->lane[1].stage_out = halved ? h->d_stage_b + (size_t)piece * h->N : h->d_stage_b2;
+    h->lane[1].stage_cnt = halved ? h->d_stage_cnt + piece : h->d_stage_cnt2;
     int64_t tile_no = 0;
     for (int64_t t0 = 0, t1; t0 < n_inputs; t0 = t1, ++tile_no) {
-        t1 = halved ? (tile_no ? n_inputs : half) : std::min<int64_t>(n_inputs, t0 + T);
+        t1 = std::min<int64_t>(n_inputs, t0 + piece);
         const int cnt = (int)(t1 - t0);
         const size_t bytes = (size_t)cnt * h->N * sizeof(float);
         const int q = (int)(tile_no & 1);

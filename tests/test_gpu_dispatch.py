@@ -680,3 +680,36 @@ def test_nets_are_laid_out_twice_only_for_batches_of_the_handles_own_size(torch_
     assert h.kernel_launches() - before > layers
     check_close(y[-8:].cpu().numpy(), OracleNet(*arrays, activation="sigmoid").infer(x0[-8:]), "x^L")
     h.destroy()
+
+
+@pytest.mark.parametrize("n,cnt,drop", [(20011, 700, False), (20011, 900, True), (40000, 500, False), (40000, 400, True)])
+def test_host_batches_of_wide_nets_keep_to_the_tile_width(torch_cuda, n, cnt, drop):  # noqa: F811
+    """A batch within max_batch whose tiles are narrower for L2's sake goes in as many tiles from host memory as from device memory: the same launches, outputs,
+    ids and live inputs of the last tile."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    layers, k = 3, 8
+    arrays = uniform_net(rng, n, k, layers)
+    if drop:
+        arrays = [*arrays[:2], [np.full(n * k, 1.0 / 4.0, dtype=np.float32)] * layers, [np.full(n, -0.6, dtype=np.float32)] * layers]
+    x0 = (rng.random((cnt, n)) < rng.uniform(0.0, 0.5, size=(cnt, 1)) ** 3).astype(np.float32) if drop else vectors(rng, cnt, n)
+    x0[-3:] = 0.0
+    h = pkg.Sdnn.create(*arrays, max_batch=cnt, flags=pkg.FLAG_SKIP_DEAD if drop else 0)
+    T = h.infer_tile_width()
+    assert T < cnt / 2
+    outs = []
+    for host in (False, True):
+        y, c, ids = np.full((cnt, n), -1.0, dtype=np.float32), np.full(cnt, -1, dtype=np.int32), np.full(cnt * n, -1, dtype=np.int32)
+        at = [torch.from_numpy(a) if host else torch.from_numpy(a).cuda() for a in (x0, y, c, ids)]
+        args = [a.numpy() for a in at] if host else at
+        before = h.kernel_launches()
+        total = h.infer_batch(args[0], cnt, args[1], args[2], args[3], cnt * n, want_total=True, host=host)
+        torch.cuda.synchronize()
+        outs.append([a.cpu().numpy() for a in at[1:]] + [total, h.kernel_launches() - before, list(h.get_liveness()) if drop else None])
+    assert all(np.array_equal(a, b) for a, b in zip(outs[0][:3], outs[1][:3])) and outs[0][3:] == outs[1][3:]
+    if drop:
+        last = (cnt - 1) // T * T
+        assert outs[0][5][-1] == np.count_nonzero(outs[0][1][last:]) and 0 < outs[0][5][0] <= cnt - last
+    pick = np.array([0, T, cnt - 1])
+    check_close(outs[1][0][pick], OracleNet(*arrays).infer(x0[pick]), "x^L")
+    h.destroy()
