@@ -578,17 +578,19 @@ __device__ __forceinline__ void prefetch_unit(const Sliced& m, int u, int rpw, i
 // multiplied by the zeros of delta's padding or never read), which adds no sector to a request: rows wider than 64 bytes cost by
 // their bytes (40000 neurons, 8 layers, 90 inputs: 319 -> 299 us).
 // TRACK (dropping dead inputs): one grid for all chunks, whose warps walk the units of the chunks that still hold live inputs
-// (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.  ls: 2^ls groups of
-// lanes share a row, as in forward_split_kernel, which runs the same layers when nothing is dropped.
-template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false, bool TRACK = false>
+// (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.  SHARE: 2^ls groups of
+// lanes share a row, as in forward_split_kernel, which runs the same layers when nothing is dropped; an instantiation of its own, as a
+// number of rows per unit that is known only at run time costs every unit divisions (us for 12 layers, with / without: 20000 neurons, 30 inputs
+// 175 / 160; 8000, 257 inputs of which a third survive 258 / 229; 3500, 257 inputs that all do 220 / 204).
+template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false, bool TRACK = false, bool SHARE = false>
 __global__ void __launch_bounds__(256, CPS > 2 ? 1 : 2)
 forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
                int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span, int last, int ls) {
-    const int RPW = 32 / G >> (TRACK ? ls : 0);
+    const int RPW = 32 / G >> (SHARE ? ls : 0);
     const int UPS = (RPW >= SLICE) ? 1 : SLICE / RPW;      // units per slice
     const int lane = threadIdx.x & 31;
-    const int sub = lane % G, grp = lane / G >> (TRACK ? ls : 0);
-    const int part = TRACK ? (lane / G) & ((1 << ls) - 1) : 0, hop = TRACK ? CPS << ls : CPS, skip = part * CPS;      // this group's steps of its row
+    const int sub = lane % G, grp = lane / G >> (SHARE ? ls : 0);
+    const int part = SHARE ? (lane / G) & ((1 << ls) - 1) : 0, hop = SHARE ? CPS << ls : CPS, skip = part * CPS;      // this group's steps of its row
     const int wpb = blockDim.x >> 5;
     const int all_units = (n + RPW - 1) / RPW;
     const int nunits = SPAN ? min(all_units, ((int)blockIdx.x + 1) * span) : all_units;
@@ -646,7 +648,7 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
             }
         }
         if (nch <= skip && nnch > skip) load_idx<CPS, I16>(c, m, nbase + skip * CHUNK_ROW);      // no step: nothing prefetched across the boundary yet
-        if (TRACK) {
+        if (SHARE) {
             __syncwarp();
             for (int o = G; o < G << ls; o <<= 1) lane_join(acc, o);
         }

@@ -553,25 +553,26 @@ void launch_forward_gv(sdnn* h, int layer, const float* xin, float* xout, int ld
 // input as 256 on dense tiles of 4096 neurons; of 1024 inputs a third of which survive, 6 of 16 such chunks are left, not 2 of 4
 // of 256), only the live ones, and each column that stays live marked.
 constexpr int TRACK_CHUNK = 64;
-template <bool I16, int G, int V>
+template <bool I16, int G, int V, bool SHARE>
 void launch_forward_tracked(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int ls) {
     const int rows = 32 / G >> ls, units = (h->N + rows - 1) / rows, chunks = cols / (V * G);
-    auto plan = plan_grid(h, (const void*)forward_kernel<G, V, 2, I16, false, false, true>, units * chunks, 1);
+    const auto kernel = forward_kernel<G, V, 2, I16, false, false, true, SHARE>;
+    auto plan = plan_grid(h, (const void*)kernel, units * chunks, 1);
     Sliced m = rows_of(h, layer);
     if (h->other_rows) { m.idx = h->lay[layer].r_idx2; m.val = h->lay[layer].r_val2; }
-    launch_k(h, forward_kernel<G, V, 2, I16, false, false, true>, dim3(plan.first), dim3(plan.second), h->pdl, m,
+    launch_k(h, kernel, dim3(plan.first), dim3(plan.second), h->pdl, m,
              (const float*)(h->d_bias + (size_t)layer * h->N), xin, xout, h->N, ld, h->cfg.clamp, h->cfg.activation, h->pdl ? h->fwd_pdl : 0,
              (const int*)h->cur->cs.ncols, h->cur->cs.flags + (size_t)layer * h->ld_max, 0, 0, ls);
     count_launch(h);
 }
-template <bool I16>
+template <bool I16, bool SHARE>
 void launch_forward_tracked_i(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int ls) {
     switch (std::min(cols, TRACK_CHUNK)) {
-        case 4: launch_forward_tracked<I16, 1, 4>(h, layer, xin, xout, ld, cols, ls); break;
-        case 8: launch_forward_tracked<I16, 1, 8>(h, layer, xin, xout, ld, cols, ls); break;
-        case 16: launch_forward_tracked<I16, 2, 8>(h, layer, xin, xout, ld, cols, ls); break;
-        case 32: launch_forward_tracked<I16, 4, 8>(h, layer, xin, xout, ld, cols, ls); break;
-        default: launch_forward_tracked<I16, 8, 8>(h, layer, xin, xout, ld, cols, ls); break;
+        case 4: launch_forward_tracked<I16, 1, 4, SHARE>(h, layer, xin, xout, ld, cols, ls); break;
+        case 8: launch_forward_tracked<I16, 1, 8, SHARE>(h, layer, xin, xout, ld, cols, ls); break;
+        case 16: launch_forward_tracked<I16, 2, 8, SHARE>(h, layer, xin, xout, ld, cols, ls); break;
+        case 32: launch_forward_tracked<I16, 4, 8, SHARE>(h, layer, xin, xout, ld, cols, ls); break;
+        default: launch_forward_tracked<I16, 8, 8, SHARE>(h, layer, xin, xout, ld, cols, ls); break;
     }
 }
 
@@ -682,8 +683,8 @@ void launch_forward_i(sdnn* h, int layer, const float* xin, float* xout, int ld,
 // the kernels are instantiated for both index widths of the sliced copies; used: columns that hold inputs; ls: see split_rows, -1 in a train step
 void launch_forward(sdnn* h, int layer, const float* xin, float* xout, int ld, int cols, int cw, int used, bool track = false, int ls = -1) {
     if (track) {
-        if (h->idx16) launch_forward_tracked_i<true>(h, layer, xin, xout, ld, cols, ls);
-        else launch_forward_tracked_i<false>(h, layer, xin, xout, ld, cols, ls);
+        if (h->idx16) ls > 0 ? launch_forward_tracked_i<true, true>(h, layer, xin, xout, ld, cols, ls) : launch_forward_tracked_i<true, false>(h, layer, xin, xout, ld, cols, 0);
+        else ls > 0 ? launch_forward_tracked_i<false, true>(h, layer, xin, xout, ld, cols, ls) : launch_forward_tracked_i<false, false>(h, layer, xin, xout, ld, cols, 0);
     } else if (h->idx16) launch_forward_i<true>(h, layer, xin, xout, ld, cols, cw, used, ls);
     else launch_forward_i<false>(h, layer, xin, xout, ld, cols, cw, used, ls);
 }
