@@ -580,24 +580,37 @@ __device__ __forceinline__ void prefetch_unit(const Sliced& m, int u, int rpw, i
 // TRACK (dropping dead inputs): one grid for all chunks, whose warps walk the units of the chunks that still hold live inputs
 // (*ncols_dev of them), so that the whole device works on what is left; the columns that stay live are marked in live_flags.  SHARE: 2^ls groups of
 // lanes share a row, as in forward_split_kernel, which runs the same layers when nothing is dropped; an instantiation of its own, as a
-// number of rows per unit that is known only at run time costs every unit divisions (us for 12 layers, with / without: 20000 neurons, 30 inputs
+// number of rows per unit that is known only at run time costs every unit (us for 12 layers, with / without: 20000 neurons, 30 inputs
 // 175 / 160; 8000, 257 inputs of which a third survive 258 / 229; 3500, 257 inputs that all do 220 / 204).
+// In launches of more than LIVE_WARPS warps the marks of a CTA's rows meet in shared memory and a CTA stores each once: every warp's storing the same few
+// words on its own is what such a launch ends with (us a layer, 60 inputs: 2048 neurons 8.7 -> 6.9, 1465 7.15 -> 6.15; 8000 neurons, 257 inputs
+// 35 -> 25), while the barrier costs a smaller one 0.3 us (700 neurons, 8 inputs, 88 warps: 4.6, with it 5.0; 2048, 16 inputs, 512: 4.7, 5.0; 1024, 60 inputs, 1024: 5.8,
+// 5.6).  Columns beyond LIVE_COLS are marked by their warps.
+constexpr int LIVE_WARPS = 768;
+constexpr int LIVE_COLS = 4096;
 template <int G, int V, int CPS, bool I16, bool CG = false, bool SPAN = false, bool TRACK = false, bool SHARE = false>
 __global__ void __launch_bounds__(256, CPS > 2 ? 1 : 2)
 forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict__ xin, float* __restrict__ xout,
                int n, int ld, float clamp, int act, int pdl, const int* __restrict__ ncols_dev, int* __restrict__ live_flags, int span, int last, int ls) {
-    const int RPW = 32 / G >> (SHARE ? ls : 0);
-    const int UPS = (RPW >= SLICE) ? 1 : SLICE / RPW;      // units per slice
+    constexpr int LOG_GROUPS = G == 1 ? 5 : G == 2 ? 4 : G == 4 ? 3 : G == 8 ? 2 : G == 16 ? 1 : 0;
+    const int log_rows = LOG_GROUPS - (SHARE ? ls : 0), RPW = 1 << log_rows;
+    const int UPS = (RPW >= SLICE) ? 1 : SLICE >> log_rows;      // units per slice
     const int lane = threadIdx.x & 31;
     const int sub = lane % G, grp = lane / G >> (SHARE ? ls : 0);
     const int part = SHARE ? (lane / G) & ((1 << ls) - 1) : 0, hop = SHARE ? CPS << ls : CPS, skip = part * CPS;      // this group's steps of its row
     const int wpb = blockDim.x >> 5;
-    const int all_units = (n + RPW - 1) / RPW;
+    const int all_units = (n + RPW - 1) >> log_rows;
     const int nunits = SPAN ? min(all_units, ((int)blockIdx.x + 1) * span) : all_units;
     const int stride = SPAN ? wpb : gridDim.x * wpb;
     int boff = (TRACK ? 0 : blockIdx.y * (V * G)) + sub * V;
     const unsigned pitch = (unsigned)ld * 4u;
     const float* __restrict__ val = m.val;
+    __shared__ unsigned s_live[TRACK ? LIVE_COLS / 32 : 1];      // a bit per column that a row of this CTA keeps alive
+    const bool meet = TRACK && stride > LIVE_WARPS;
+    if (meet) {
+        for (int c = threadIdx.x; c < LIVE_COLS / 32; c += blockDim.x) s_live[c] = 0u;
+        __syncthreads();
+    }
 
     int unit = (SPAN ? blockIdx.x * span : blockIdx.x * wpb) + (threadIdx.x >> 5);
     int chunks_left = 0x7fffffff;      // TRACK: chunks from the current one on
@@ -615,7 +628,12 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
     if (nch > skip) load_idx<CPS, I16>(c, m, base + skip * CHUNK_ROW);
     if (pdl) grid_dependency_wait();
     if (pdl == 2) grid_launch_dependents();
-    if (TRACK) chunks_left += (*ncols_dev + V * G - 1) / (V * G) - 0x7fffffff;
+    int live_cols = 0;
+    if (TRACK) {
+        live_cols = (*ncols_dev + V * G - 1) / (V * G);
+        chunks_left += live_cols - 0x7fffffff;
+        live_cols *= V * G;
+    }
     unsigned live = 0u;       // bit e: column boff + e of some row this lane produced is nonzero
 
     while (unit < nunits && (!TRACK || chunks_left > 0)) {
@@ -657,16 +675,28 @@ forward_kernel(Sliced m, const float* __restrict__ bias, const float* __restrict
             lane_store(tile_row(xout + boff, to, pitch), acc);
             if (TRACK) live |= lane_nonzero_bits(acc);
         }
-        if (TRACK && live && (nboff != boff || nleft <= 0)) {      // this warp's last unit of the chunk
+        if (TRACK && (nboff != boff || nleft <= 0)) {      // this warp's last unit of the chunk
+            if (meet && boff < LIVE_COLS) {
+                __syncwarp();
 #pragma unroll
-            for (int e = 0; e < V; ++e)
-                if ((live >> e) & 1u) live_flags[boff + e] = 1;      // many lanes may store the same 1
+                for (int o = G; o < 32; o <<= 1) live |= __shfl_xor_sync(0xffffffffu, live, o);
+                if (lane < G && live) atomicOr(&s_live[boff / 32], live << (boff % 32));
+            } else {
+#pragma unroll
+                for (int e = 0; e < V; ++e)
+                    if ((live >> e) & 1u) live_flags[boff + e] = 1;      // many lanes may store the same 1
+            }
             live = 0u;
         }
         unit = nunit; row = nrow; base = nbase; nch = nnch; b = nb; to = nto;
         if (TRACK) { boff = nboff; chunks_left = nleft; }
     }
 #undef SDNN_WRAP
+    if (meet) {
+        __syncthreads();
+        for (int c = threadIdx.x; c < min(live_cols, LIVE_COLS); c += blockDim.x)
+            if ((s_live[c / 32] >> (c % 32)) & 1u) live_flags[c] = 1;
+    }
     if (pdl == 1) grid_launch_dependents();
 }
 

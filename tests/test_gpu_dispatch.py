@@ -713,3 +713,28 @@ def test_host_batches_of_wide_nets_keep_to_the_tile_width(torch_cuda, n, cnt, dr
     pick = np.array([0, T, cnt - 1])
     check_close(outs[1][0][pick], OracleNet(*arrays).infer(x0[pick]), "x^L")
     h.destroy()
+
+
+@pytest.mark.parametrize("n,cnt", [(500, 4100), (300, 8300), (700, 4160), (2048, 60), (1465, 100), (3000, 30), (9000, 33)])
+def test_marks_of_live_inputs(torch_cuda, n, cnt):  # noqa: F811
+    """Which inputs are alive after each layer, from launches whose marks meet per CTA and from smaller ones, and in batches of more columns than
+    a CTA keeps marks for: the same bits as without dropping, and as many live inputs as have an output that is not zero."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    layers, k = 3, 256                                     # rows too long for whole networks in shared memory
+    rp, cols, _, _ = uniform_net(rng, n, k, layers)
+    vals, bias = [np.full(n * k, 1.0 / 128.0, dtype=np.float32)] * layers, [np.full(n, -0.35, dtype=np.float32)] * layers
+    x0 = (rng.random((cnt, n)) < rng.uniform(0.0, 0.5, size=(cnt, 1))).astype(np.float32)
+    x0[rng.random(cnt) < 0.3] = 0.0
+    x, outs = torch.from_numpy(x0).cuda(), []
+    for depth, flags in ((1, pkg.FLAG_SKIP_DEAD), (2, pkg.FLAG_SKIP_DEAD), (layers, pkg.FLAG_SKIP_DEAD), (layers, 0)):
+        h = pkg.Sdnn.create(rp[:depth], cols[:depth], vals[:depth], bias[:depth], max_batch=cnt, flags=flags)
+        assert h.infer_tile_width() == cnt
+        y = torch.full((cnt, n), -1.0, device="cuda")
+        h.infer_batch(x, cnt, y)
+        outs.append(y.cpu().numpy())
+        if flags:
+            live = list(h.get_liveness())
+            assert live == [np.count_nonzero(o.any(axis=1)) for o in outs] and 0 < live[0] < cnt
+        h.destroy()
+    assert np.array_equal(outs[2], outs[3])
