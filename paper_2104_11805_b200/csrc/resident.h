@@ -147,39 +147,67 @@ SDNN_HD void resident_share(int total, int sms, int p, int q, int* begin, int* e
     *begin = q == p ? 0 : main;
     *end = own ? total : q == p ? main : *begin;
 }
-// The width for `inputs` inputs, 0 where the layer launches, in tiles of `tile` inputs, are faster.  Clocks per layer, fitted to both
-// over 640 .. 8000 neurons and 32 .. 4000 inputs (24 layers; us per layer, layer launches / this kernel):
+// A layer: neurons, stored elements (padding included), entries of the longest row, whether rows differ in length.
+struct ResidentLayer { int n; double elems; int longest; bool several; };
+// What a layer takes, in clocks, one way and the other, fitted to measurements of both (24 layers of 600 .. 8000 neurons, 16, 32 and 56 entries a row, 8 to 56
+// and Poisson(32); us per layer, layer launches / this kernel, 32 entries):
 //   neurons   256 inputs      400             592             1184            2368            4000
 //     640     3.49 / 3.83     4.59 / 3.88     4.75 / 3.90     7.71 / 5.22     13.5 / 8.2      18.7 / 14.8
 //    1024     3.50 / 4.75     4.72 / 4.75     6.85 / 4.79     9.52 / 6.84     18.5 / 11.4     27.2 / 20.5
 //    2048     4.86 / 8.35     7.96 / 8.39     11.0 / 8.45     17.3 / 12.7     34.9 / 22.3     54.0 / 39.6
 //    4096     8.75 / 15.5     17.4 / 15.5     19.9 / 15.6     33.4 / 24.9     67.0 / 50.0     109 / 90.7
 //    8000     17.0 / 33.2     27.1 / 33.8     38.4 / 34.7     66.2 / 70.4     131 / 134
-// A CTA: wavefronts of operands (1.06 for eight of them), entries (6 bytes each) and outputs; a single piece of 4 inputs leaves the
-// pipe waiting for entries, units held in registers cost addresses; 2500 clocks for the ends of a layer.  The layer launches:
-// 66 bytes of operands per clock and SM, and the round trips at the ends of a launch, which a second tile in flight fills.
-inline double resident_clocks(int n, double elems, int p) {
-    const double pipe = elems * (p * 1.06 / 8 + 6.0 / 128) + n * p / 4.0;
-    const int held = resident_shape(n, p).held;
-    return pipe * (p == 1 ? 1.10 : 1.0) * (held == 4 ? 1.18 : held ? 1.04 : 1.0) + 2500;
+// A round of CTAs: wavefronts of operands (1.06 for eight of them), entries (6 bytes each) and outputs.  Units held in registers cost addresses, warps
+// without a unit in the last round idle; at 4 inputs a CTA a warp waits for its entries, more so where rows differ in length (their chunks
+// come in no fours; 7000 neurons, 8 to 56 entries, 592 inputs: 33.9 us, 32 each: 27.5) and where a layer of them is large.
+inline double resident_clocks(const ResidentLayer& l, int p) {
+    const ResidentShape s = resident_shape(l.n, p);
+    const double idle = (double)((s.units + RES_WARPS - 1) / RES_WARPS * RES_WARPS) / s.units - 1;
+    const double pipe = (l.elems * (p * 1.06 / 8 + 6.0 / 128) + l.n * p / 4.0) * (s.held == 4 ? 1.10 : s.held ? 1.04 : 1.0);
+    const double wait = p == 1 ? 1.20 + 0.45 * idle + (l.several ? 0.13 : 0.0) + 0.056e-5 * std::max(0.0, l.elems - 130000)
+                               : 1.03 + 0.035 * (p - 1) + (p == 2 ? 0.20 : 0.165) * idle + (l.several ? 0.02 : 0.0);
+    return pipe * wait + 2400;
 }
-// drop: dead inputs are dropped.  A third is taken to be left after a few layers, and the layer launches to take 1.8 times as long for what
-// is left (a tile of 1024 inputs is then a tile of 340, with what finding and moving them costs: 4096 x 120, 5000 inputs, us a layer:
-// 80 / 47; 1024 x 120, 3000: 15.9 / 8.1; 1465 x 120, 449: 6.9 / 7.1).
-inline int resident_width(int n, double elems, int64_t inputs, int sms, int tile, bool drop) {
+// ... for `inputs` inputs in rounds of width p; a rest behind whole rounds finds the CTAs out of step, which then read other parts of the network
+// (5000 neurons, 16 entries, 1500 and 1776 inputs: 38 and 34 us a layer)
+inline double resident_clocks(const ResidentLayer& l, int64_t inputs, int sms, int p) {
+    const int64_t round = (int64_t)4 * p * sms;
+    const int q = resident_rest_width((int)(inputs % round), sms);
+    const double whole = (double)(inputs / round) * resident_clocks(l, p);
+    return (whole + (q ? resident_clocks(l, q) : 0.0)) * (whole > 0 && q ? (p == 1 ? 1.08 : 1.03) : 1.0);
+}
+// The layer launches, in tiles of `tile` inputs: 66 bytes of operands per clock and SM (some of which L1 has: 80 for a row's entries, which its end takes a part of), and the round trips of
+// the longest row, which a second tile in flight fills in part.  A small batch pays for a part of the padding to whole chunks of 256.
+inline double launch_clocks(const ResidentLayer& l, int64_t inputs, int sms, int tile) {
+    const double trips = 4640 + 177.0 * l.longest;
+    const double padded = (double)inputs + (inputs <= tile && l.elems * (double)inputs < (32 << 20) ? 0.3 * (double)((256 - inputs % 256) % 256) : 0.0);
+    const double gathers = (0.82 * l.elems + 7.5 * l.n) * padded * 4.0 / (66.0 * sms);
+    const double tiles = (double)((inputs + tile - 1) / tile);
+    return inputs <= tile ? std::max(trips, gathers + 0.48 * trips) : std::max(0.66 * tiles * trips, gathers + 0.19 * tiles * trips);
+}
+// ... dropping dead inputs, where `inputs` of those in all tiles are left
+inline double dropping_clocks(const ResidentLayer& l, int64_t inputs, int sms, int tiles) {
+    const double trips = 4640 + 177.0 * l.longest, gathers = (0.82 * l.elems + 7.5 * l.n) * (double)inputs * 4.0 / (66.0 * sms);
+    return tiles == 1 ? 1.5 * gathers + 0.85 * trips + 1800 : 1.25 * gathers + 0.5 * tiles * trips + 1500;
+}
+// The width for `inputs` inputs, 0 where the layer launches, in tiles of `tile` inputs, are faster.  drop: dead inputs are dropped.  How many are left
+// after a few layers is not known: a third decides between the two ways, and the width is one that is right for a third and for all of them.
+inline int resident_width(const ResidentLayer& l, int64_t inputs, int sms, int tile, bool drop) {
     int best = 0;
     if (inputs <= 256) return best;      // a single chunk of inputs: the table's first column
-    if (drop) inputs = (inputs + 2) / 3;
-    const double gathers = elems * (double)inputs * 4.0 / (66.0 * sms);
-    double least = drop ? 1.8 * std::max(6300.0, gathers + 2800) : inputs > tile ? gathers : std::max(8700.0, gathers + 4500);
-    for (int p = 1; p <= 4; ++p) {
-        if (!resident_shape(n, p).ok) break;      // nor does a wider one
-        const int64_t round = (int64_t)4 * p * sms;
-        const int q = resident_rest_width((int)(inputs % round), sms);
-        const double all = (double)(inputs / round) * resident_clocks(n, elems, p) + (q ? resident_clocks(n, elems, q) : 0.0);
+    double least = launch_clocks(l, inputs, sms, tile);
+    for (int p = 1; p <= 4 && resident_shape(l.n, p).ok; ++p) {      // where a width does not fit, nor does a wider one
+        const double all = resident_clocks(l, inputs, sms, p);
         if (all < least) { least = all; best = p; }
     }
-    return best;
+    if (!drop || !best) return best;
+    const int64_t third = (inputs + 2) / 3;
+    auto either = [&](int p) { return resident_clocks(l, inputs, sms, p) + 3 * resident_clocks(l, third, sms, p); };
+    for (int p = 1; p <= 4 && resident_shape(l.n, p).ok; ++p) if (either(p) < either(best)) best = p;
+    return resident_clocks(l, third, sms, best) < dropping_clocks(l, third, sms, (int)((inputs + tile - 1) / tile)) ? best : 0;
+}
+inline int resident_width(int n, double elems, int64_t inputs, int sms, int tile, bool drop) {      // rows of one length
+    return resident_width(ResidentLayer{n, elems, (int)(elems / n), false}, inputs, sms, tile, drop);
 }
 
 // A batch from host memory that is one tile goes in two pieces, so that one's copies run under the other's layers.  Halves of 4 inputs a

@@ -181,7 +181,7 @@ struct sdnn {
     int* vector_status = nullptr;       // pinned: raised by a whole-network kernel whose wait for its neighbours ran out
     Resident resident{};                // the net as resident_infer_kernel reads it (units = 0: it does not)
     ResidentSetup resident_setup{};
-    double resident_elems = 0;          // stored elements per layer there, padding included
+    ResidentLayer resident_layer{};     // a layer of it
     int* const* resident_idx2 = nullptr; float* const* resident_val2 = nullptr;      // device: [L] r_idx2, r_val2 (NULL: none)
     bool other_rows = false;            // the launch helpers currently read those
     bool compaction = false;            // SDNN_FLAG_SKIP_DEAD asked for; effective while no bias is positive
@@ -1468,7 +1468,8 @@ int build_resident(sdnn* h) {
     }
     unit_at[(size_t)L * units] = (int)run;
     const double elems = 128.0 * run / L;
-    if (!resident_width(N, elems, h->cfg.max_batch, h->sms, infer_tile_width(h), false)) return SDNN_OK;
+    const ResidentLayer layer{N, elems, longest, !uniform};
+    if (!resident_width(layer, h->cfg.max_batch, h->sms, infer_tile_width(h), false)) return SDNN_OK;
 
     auto room = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t rows = (size_t)L * units * RES_UNIT, entries = (size_t)run * 128;
@@ -1525,7 +1526,7 @@ int build_resident(sdnn* h) {
     }
     CU(h, cudaGetLastError());
     CU(h, cudaStreamSynchronize(h->stream));
-    h->resident = net; h->resident_setup = set; h->resident_elems = elems;
+    h->resident = net; h->resident_setup = set; h->resident_layer = layer;
     if (h->compaction) {
         CU(h, cudaMemsetAsync(part[12], 0, sizes[12], h->stream));      // padding: index 0, value 0
         CU(h, cudaMemsetAsync(part[13], 0, sizes[13], h->stream));
@@ -1590,8 +1591,8 @@ struct Route { int width = 0, ls = 0; bool other = false; };
 Route route_of(const sdnn* h, int64_t inputs, int tile) {
     Route r;
     if (h->resident.units) {
-        const int T = infer_tile_width(h), dense = resident_width(h->N, h->resident_elems, inputs, h->sms, T, false);
-        r.width = dense && drops_dead(h) ? resident_width(h->N, h->resident_elems, inputs, h->sms, T, true) : dense;
+        const int T = infer_tile_width(h), dense = resident_width(h->resident_layer, inputs, h->sms, T, false);
+        r.width = dense && drops_dead(h) ? resident_width(h->resident_layer, inputs, h->sms, T, true) : dense;
         r.other = dense && !r.width;
     }
     if (!r.width && !r.other) r.ls = call_rows(h->N, h->mean_elems, tile, h->sms);

@@ -286,6 +286,12 @@ RESIDENT = """
 #include "resident.h"
 using namespace sdnn_plan;
 extern "C" int width(int n, double elems, long long inputs, int sms, int tile, int drop) { return resident_width(n, elems, inputs, sms, tile, drop != 0); }
+extern "C" int layer_width(int n, int chunks, int longest, int several, long long inputs, int tile, int drop) {
+    return resident_width(ResidentLayer{n, 4.0 * chunks * n, longest, several != 0}, inputs, 148, tile, drop != 0);
+}
+extern "C" double cost(int n, int chunks, int longest, int several, long long inputs, int p) {
+    return resident_shape(n, p).ok ? resident_clocks(ResidentLayer{n, 4.0 * chunks * n, longest, several != 0}, inputs, 148, p) : 1e30;
+}
 extern "C" void shape(int n, int p, int* out) {
     const ResidentShape s = resident_shape(n, p);
     out[0] = s.ok; out[1] = s.units; out[2] = s.slots; out[3] = s.cap; out[4] = s.held;
@@ -360,6 +366,26 @@ def test_shares_of_networks_held_in_shared_memory(resident):
                     if q < p:
                         assert out[1] - out[0] <= 4 * q * sms
                 assert taken == list(range(total))
+
+
+def test_widths_of_networks_held_in_shared_memory(resident):
+    """The way that was measured to be the faster one (us per layer, layer launches / whole networks), rows of 32 and of 8 to 56 entries; with dead
+    inputs dropped a width that is right for all inputs as well as for a third of them."""
+    measured = [(700, 32, 300, 300, 4.7, 4.1), (6000, 16, 1500, 1024, 38, 44), (1024, 32, 256, 256, 3.5, 4.8), (1024, 32, 1000, 1000, 8.2, 6.8),
+                (4096, 32, 10000, 1024, 269, 208), (8000, 32, 592, 592, 38.4, 34.3), (8000, 32, 1184, 1024, 66.2, 68.7), (5000, 56, 2368, 1024, 134, 147),
+                (1024, 0, 592, 592, 8.9, 5.4), (3000, 0, 592, 592, 18.6, 13.7), (7000, 0, 1776, 1024, 89.8, 109), (6000, 0, 2368, 1024, 108, 120), (8000, 0, 592, 592, 39.2, 42.7)]
+    resident.layer_width.argtypes = [ctypes.c_int] * 4 + [ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    resident.cost.argtypes, resident.cost.restype = [ctypes.c_int] * 4 + [ctypes.c_longlong, ctypes.c_int], ctypes.c_double
+    for n, k, inputs, tile, launches, whole in measured:
+        layer = (n, k // 4, k, 0) if k else (n, 9, 56, 1)
+        assert (resident.layer_width(*layer, inputs, tile, 0) > 0) == (whole < launches), (n, k, inputs)
+    for n in (640, 1024, 1465, 2048, 4096, 8000):
+        for layer in ((n, 4, 16, 0), (n, 8, 32, 0), (n, 9, 56, 1)):
+            for inputs in list(range(260, 2400, 37)) + [3000, 5000, 12057, 20000]:
+                p = resident.layer_width(*layer, inputs, 1024, 1)
+                assert p == 0 or resident.layer_width(*layer, inputs, 1024, 0)
+                for left in (inputs, (inputs + 2) // 3) if p else ():
+                    assert resident.cost(*layer, left, p) <= 1.06 * min(resident.cost(*layer, left, q) for q in range(1, 5)), (layer, inputs, left)
 
 
 def test_halves_of_a_batch_from_host_memory(resident):
