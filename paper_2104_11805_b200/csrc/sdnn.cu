@@ -2600,7 +2600,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         if ((rc = dev_alloc(h, &h->d_stage_idx, (size_t)nz_index_capacity, false))) return rc;   // grows; old block freed at destroy
         h->stage_idx_cap = nz_index_capacity;
     }
-    const bool want_sets = nz_count_out || nz_index_out || nz_total_out;
+    const bool want_sets = nz_count_out || nz_index_out || nz_total_out, want_total = nz_index_out || nz_total_out;
     if (want_sets) CU(h, cudaMemsetAsync(h->d_running, 0, sizeof(long long), h->stream));
     // two input stages and a copy stream: the copy of tile t+1 runs under the layers of tile t
     const int T = host_tile_width(h, n_inputs);
@@ -2644,7 +2644,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
         h->other_rows = route.other;
         if (route.width)
             rc = infer_resident(h, ln, halved ? 1 : route.width, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr, nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity,
-                                want_sets, want_sets, h->ev_consumed[q]);
+                                want_sets, want_total, h->ev_consumed[q]);
         else rc = infer_tile(h, ln, route.ls, stage[q], cnt, y_out ? ln.stage_out : nullptr, nz_count_out ? ln.stage_cnt : nullptr,
                              nz_index_out ? h->d_stage_idx : nullptr, nz_index_capacity, want_sets, h->ev_consumed[q]);
         h->other_rows = false;
@@ -2655,7 +2655,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     const int rc_end = lanes_end(h, lanes);
     if (rc || rc_end) return rc ? rc : rc_end;
     long long total = 0;
-    if (want_sets) CU(h, cudaMemcpyAsync(&total, h->d_running, sizeof total, cudaMemcpyDeviceToHost, h->stream));
+    if (want_total) CU(h, cudaMemcpyAsync(&total, h->d_running, sizeof total, cudaMemcpyDeviceToHost, h->stream));
     CU(h, cudaStreamSynchronize(h->stream));
     if ((rc = vector_check(h))) return rc;
     if (nz_total_out) *nz_total_out = total;

@@ -738,3 +738,22 @@ def test_marks_of_live_inputs(torch_cuda, n, cnt):  # noqa: F811
             assert live == [np.count_nonzero(o.any(axis=1)) for o in outs] and 0 < live[0] < cnt
         h.destroy()
     assert np.array_equal(outs[2], outs[3])
+
+
+@pytest.mark.parametrize("n,tile,cnt", [(1024, 1000, 3500), (2000, 592, 590), (1500, 450, 455)])
+def test_counts_alone_take_no_running_total(torch_cuda, n, tile, cnt):  # noqa: F811
+    """Host batches through whole networks in shared memory: the counts come with the outputs' launches; only a total or ids need more."""
+    rng, pkg = np.random.default_rng(n), sdnn()
+    arrays = uniform_net(rng, n, 32, 4)
+    h = pkg.Sdnn.create(*arrays, max_batch=tile)
+    x0 = vectors(rng, cnt, n)
+    y, c, launches = np.empty((cnt, n), dtype=np.float32), np.full((2, cnt), -1, dtype=np.int32), []
+    for args in ((y,), (y, c[0]), (None, c[1])):
+        before = h.kernel_launches()
+        h.infer_batch(x0, cnt, *args, host=True)
+        launches.append(h.kernel_launches() - before)
+    assert launches[0] == launches[1] == launches[2] < 4 * ((cnt + tile - 1) // tile), launches
+    assert np.array_equal(c[0], np.count_nonzero(y, axis=1)) and np.array_equal(c[1], c[0])
+    before = h.kernel_launches()
+    assert h.infer_batch(x0, cnt, None, c[1], want_total=True, host=True) == c[0].sum() and h.kernel_launches() - before > launches[0]
+    h.destroy()
