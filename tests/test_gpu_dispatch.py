@@ -757,3 +757,60 @@ def test_counts_alone_take_no_running_total(torch_cuda, n, tile, cnt):  # noqa: 
     before = h.kernel_launches()
     assert h.infer_batch(x0, cnt, None, c[1], want_total=True, host=True) == c[0].sum() and h.kernel_launches() - before > launches[0]
     h.destroy()
+
+
+@pytest.mark.parametrize("n,cnt,launches", [(4096, 592, True), (3001, 590, True), (1024, 1000, False), (1465, 449, False)])
+def test_dead_inputs_dropped_after_new_weights(torch_cuda, n, cnt, launches):  # noqa: F811
+    """Rows of several lengths with weights all different, so that an entry in another's place shows: the same bits with dead inputs dropped as without, through whole
+    networks and through layer launches that stand in for them, from the first weights, from new ones, and from biases that end the dropping and
+    begin it again."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    layers = 6
+    rps, cols = [], []
+    for _ in range(layers):
+        length = rng.integers(8, 57, size=n)
+        rps.append(np.concatenate([[0], np.cumsum(length)]).astype(np.int32))
+        cols.append(np.concatenate([np.sort(rng.choice(n, size=m, replace=False)) for m in length]).astype(np.int32))
+
+    def weights():
+        return ([(rng.standard_normal(len(c)) * 0.22).astype(np.float32) for c in cols], [-rng.uniform(0.1, 0.3, size=n).astype(np.float32) for _ in range(layers)])
+    vals, bias = weights()
+    dense, drop = (pkg.Sdnn.create(rps, cols, vals, bias, max_batch=cnt, flags=f) for f in (0, pkg.FLAG_SKIP_DEAD))
+    x0 = ((rng.random((cnt, n)) < 0.3) * np.exp(rng.uniform(np.log(0.02), np.log(20.0), size=(cnt, 1)))).astype(np.float32)
+    x = torch.from_numpy(x0).cuda()
+
+    def compare(dropping):
+        outs, made = [], []
+        for h in (dense, drop):
+            y, c = torch.full((cnt, n), -1.0, device="cuda"), torch.full((cnt,), -1, dtype=torch.int32, device="cuda")
+            before = h.kernel_launches()
+            h.infer_batch(x, cnt, y, c)
+            torch.cuda.synchronize()
+            made.append(h.kernel_launches() - before)
+            outs.append((y.cpu().numpy(), c.cpu().numpy()))
+        assert all(np.array_equal(a, b) for a, b in zip(*outs))
+        assert made[0] <= 2 and (made[1] > 2 * layers) == (launches and dropping), made
+        if dropping:
+            live = list(drop.get_liveness())
+            assert live[-1] == np.count_nonzero(outs[1][1]) and 0 < live[-1] < live[0] < cnt, live
+        pick = np.unique(np.concatenate([np.argsort(outs[0][1])[[0, cnt // 2, cnt - 1]], rng.integers(0, cnt, size=5)]))
+        check_close(outs[1][0][pick], OracleNet(rps, cols, vals, bias).infer(x0[pick]), "x^L")
+    compare(True)
+    vals, bias = weights()
+    for l in range(layers):
+        for h in (dense, drop):
+            h.set_weights(l, vals[l], bias[l])
+    compare(True)
+    kept, bias[2] = bias[2], bias[2].copy()
+    bias[2][n // 2] = 0.25
+    for h in (dense, drop):
+        h.set_weights(2, None, bias[2])
+    compare(False)
+    bias[2], vals[4] = kept, weights()[0][4]
+    for h in (dense, drop):
+        h.set_weights(2, None, bias[2])
+        h.set_weights(4, vals[4], None)
+    compare(True)
+    dense.destroy()
+    drop.destroy()
