@@ -684,6 +684,7 @@ def main():
                           "launch, not one launch's start-to-end duration" if in_flight > 1 else "")}
         if launches < args.steps * L:          # fewer launches than layers: whole networks, with the operands in shared memory
             dom = "resident_infer_kernel" if n_inputs > 4 else "vector_infer_kernel"
+            extra["tiles_in_flight"] = 0
             extra["note"] = ("a launch runs the whole network: launch_ms is the call's time per layer and tile of inputs, the bytes and gathers are "
                              "those of one layer and tile; the operands come out of shared memory, not as gathers out of L2")
     # what bounds these launches instead of HBM: random gathers of tile rows out of L2 (measured now, on this device)

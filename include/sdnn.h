@@ -71,8 +71,9 @@ typedef enum {
                                     /* its weights and processes every input.  Inference: inputs whose activation  */
                                     /* vector has become all zero are dropped from the tile (whole chunks of 64    */
                                     /* columns at a time; one by one, after some layers, where whole networks run  */
-                                    /* in shared memory: larger batches, up to 8192 neurons); only done while no layer has a positive bias, because   */
-                                    /* only then does an all-zero vector stay all zero.  Training: a unit of rows  */
+                                    /* in shared memory, see sdnn_infer_batch); only done while no layer has a     */
+                                    /* positive bias, because only then does an all-zero vector stay all zero.     */
+                                    /* Training: a unit of rows                                                    */
                                     /* whose delta is zero for every input skips its entries (not for B <= 4,      */
                                     /* whose kernels have no such test).  Results are the same as in dense mode.   */
 #define SDNN_FLAG_NO_GRAPH    0x10u /* launch the layer chain kernel by kernel instead of through a CUDA graph     */
@@ -169,7 +170,15 @@ int sdnn_finalize(sdnn_t* h);
  * the first such call), so that the start and tail of one tile's launches are filled by the other's;
  * SDNN_FLAG_ONE_TILE turns that off.  The call is ordered on the handle's stream either way:
  * work enqueued there before it is seen, and everything the call launched is complete once that stream has caught
- * up.  If nz_index_out is given and the
+ * up.
+ * Nets of up to 8192 neurons with rows of up to 248 entries take batches of more than 256 inputs without tiles where that is the faster way
+ * (decided by the net, the batch and cfg.max_batch): whole networks run in shared memory, a few inputs at a time, on the handle's stream alone.
+ * A handle holds its net in a second layout for this, 7 bytes per stored entry (13 to 15 with SDNN_FLAG_SKIP_DEAD), if batches of max_batch
+ * inputs go this way and a quarter of the device's memory stays free.
+ * The order in which a row's products are added depends on the number of inputs in the call (on the way they take, and up to 128 inputs on how
+ * many lanes share a row), and on whether the arrays are in device or host memory.  So the same input may give results that differ by
+ * rounding in calls of different sizes; within one call all inputs are added up in one order, and a repeated call gives the same bits.
+ * If nz_index_out is given and the
  * capacity is too small, only the ids at positions below the capacity are written, *nz_total_out
  * (if given) holds the needed capacity and the call returns SDNN_ERR_INVALID_ARG; y_out and
  * nz_count_out are still valid.  n_inputs == 0 is a valid no-op.
@@ -178,15 +187,16 @@ int sdnn_infer_batch(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
                      int32_t* nz_count_out, int32_t* nz_index_out, int64_t nz_index_capacity,
                      int64_t* nz_total_out);
 
-/* Inputs per tile that sdnn_infer_batch uses on this handle (see above); 0 before sdnn_finalize. */
+/* Inputs per tile that sdnn_infer_batch uses on this handle where a batch goes in tiles (see above); 0 before sdnn_finalize. */
 int32_t sdnn_infer_tile_width(const sdnn_t* h);
 
-/* Tiles that sdnn_infer_batch keeps in flight on this handle when a batch has more than one (1 or 2; see above);
- * 0 before sdnn_finalize. */
+/* Tiles that sdnn_infer_batch keeps in flight on this handle when a batch goes in more than one (1 or 2; see above; a batch
+ * that runs whole networks in shared memory has none); 0 before sdnn_finalize. */
 int32_t sdnn_infer_tiles_in_flight(const sdnn_t* h);
 
 /* Same call with every array in HOST memory (pinned or pageable); the library stages the
- * copies itself, tile by tile, and returns when the outputs are in place. */
+ * copies itself, tile by tile (a batch of one tile in two halves, if these are large enough), and returns when the outputs are in
+ * place.  The way of a whole tile, or of both halves, is that of every tile. */
 int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y_out,
                           int32_t* nz_count_out, int32_t* nz_index_out, int64_t nz_index_capacity,
                           int64_t* nz_total_out);
@@ -396,7 +406,8 @@ int sdnn_get_liveness(sdnn_t* h, int32_t* live_inputs_out);
  * a latency-critical loop that cannot afford the device-wide synchronisation an allocation may
  * imply, or a plug-in interface that forbids allocating after initialisation).
  *
- * Same arithmetic as sdnn_infer_batch with y_out only (L forward layers, one tile), but with no
+ * The same layers as sdnn_infer_batch with y_out only (one tile; 32-bit sums as there, a row's products added in an order of
+ * its own, which depends on the number of inputs and of neurons), but with no
  * handle: the network stays in the caller's device arrays and the two ping-pong activation tiles
  * live in a fixed array inside the library (SDNN_NOALLOC_SCRATCH_BYTES, held by every GPU that
  * loads the library until the process exits).  The call makes no cudaMalloc / cudaFree and uses

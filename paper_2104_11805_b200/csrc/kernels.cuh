@@ -570,7 +570,8 @@ __device__ __forceinline__ void prefetch_unit(const Sliced& m, int u, int rpw, i
 // Forward layer (feedforward equation): Xout[i,:] = clamp(bias[i] + sum_q val[i,q] * Xin[idx[i,q],:]).
 // Persistent grid: a warp takes units (32/G consecutive rows) in a grid-stride loop, or (span > 0) within its CTA's
 // run of `span` consecutive units.  One group of G lanes
-// per row; each lane accumulates V batch entries with fp32 FMAs in stored (ascending column) order.
+// per row (SHARE: 2^ls groups, whose sums meet at the row's end); each lane accumulates V batch entries with fp32 FMAs in stored order: ascending
+// columns, or, in the copies that stand in for whole networks (resident_reorder_kernel), the order in which those read a row's entries.
 // While it works on a unit a warp asks for the entries of its next unit to be brought into L2.
 // CG: the gathers go past L1 (64-byte rows of a layer without padding entries).
 // SPAN: a CTA takes a run of `span` consecutive units instead of walking the units in a grid-wide stride.

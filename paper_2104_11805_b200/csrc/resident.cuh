@@ -1,8 +1,8 @@
 // Whole networks for many inputs in one launch: a CTA takes 4, 8, 12 or 16 inputs through all layers with their activations in its
 // shared memory.
 //
-// Inference of nets whose layers fit (up to 8192 neurons).  The layer kernels gather every operand out of L2, 64 bytes per clock and
-// SM, and run at that; shared memory delivers 128.  Inputs are independent, so a CTA needs nothing from another one: no tile, no
+// Inference of nets whose layers fit (up to 8192 neurons).  The layer kernels gather every operand out of L2, which delivers 64 bytes
+// per clock and SM, and run at that (66 operand bytes with what L1 happens to hold); shared memory delivers 128.  Inputs are independent, so a CTA needs nothing from another one: no tile, no
 // launch and no barrier per layer on the device, and the network streams past out of L2, 6 bytes per entry and CTA.
 //
 // A slot holds one neuron's activations: P pieces of 4 inputs (16 bytes), each in a plane of its own.  A lane owns a row and reads P
