@@ -101,6 +101,31 @@ inline int call_rows(int n, int64_t elems, int tile, int sms) {
     return whole.cw == whole.cols ? split_rows(n, elems, whole.cw, sms) : 0;
 }
 
+// Allocation-free calls: groups of lanes that share a row of the caller's CSR arrays (at least so many), and whether a single group is of lanes of 4
+// inputs instead of 8 (`narrow`).  width: inputs of a chunk; per_row: entries of a row in the mean.  A launch of few rows is over when its longest row
+// is: the row goes to as many groups as 2048 warps (the device's fill) leave room for; with one lane a group four pay at any size, eight up to 5000
+// rows.  us per layer of 24, 4096 rows of 8 to 56 entries (of 32 in brackets), one group / this: 4 inputs 6.9 / 2.8 (4.5 / 2.8), 8 inputs 7.8 / 3.0
+// (5.1 / 3.1), 16 inputs 5.3 / 3.4 (3.7 / 3.4), 32 inputs 5.2 / 4.2 (3.9 / 3.4), 64 inputs 7.1 / 5.8 (5.4 / 4.4); 700 rows, 128 inputs 6.3 / 4.5
+// (4.9 / 3.4), 8 inputs 7.3 / 2.5.  More rows than that: 128 inputs, 4096 rows 8.5 with one group, 9.0 with two; two chunks, 2000 rows 4.8 and 5.0; 16 inputs,
+// 16000 rows lanes of four inputs 8.2, two groups 8.4; 32 inputs, 10000 rows 7.2 with lanes of four inputs, 8.0 of eight, from 12000 on the other way round.
+// A short row has nothing to share (one group / several: 3000 rows of 8, 16 inputs 3.3 / 3.9; 30000 of 8, 8 inputs 4.4 / 5.9; 2000 of 16, 32 inputs 3.5 / 3.9),
+// and less of it where a lane holds few inputs or many groups wait already (8 inputs or 64: rows of 12 gain 4 to 20 %) and several chunks fill the device
+// (1300 rows of 24, 384 inputs 4.0 / 4.8).
+struct CsrGroups { int groups; bool narrow; };
+inline CsrGroups csr_groups(int n, double per_row, int width, int chunks) {
+    const bool between = width == 16 || width == 32;
+    int groups = width <= 8 ? (n <= 5120 ? 8 : 4) : (int)std::min<int64_t>(8, 2048 * 32 / std::max<int64_t>(1, (int64_t)n * (width / 8)));
+    if (width > 4 && per_row < (between ? 20 : width == 8 && n > 16384 ? 28 : 10)) groups = 1;
+    if ((chunks == 2 && n > 1700) || (chunks > 1 && n > (chunks == 2 ? 1000 : 800) && per_row < 28)) groups = 1;
+    return CsrGroups{groups, n <= (per_row < 20 ? 9200 : 11000)};
+}
+// ... entries of a row of layer l, as far as the offsets of the layers tell (which may lie in any order, and do not tell where the last one ends)
+inline double csr_row(const int64_t* offset, int layers, int l, int n) {
+    const int k = l + 1 < layers ? l : l - 1;
+    const double entries = k < 0 ? 0.0 : (double)offset[k + 1] - (double)offset[k];
+    return entries > 0 ? entries / n : 32.0;
+}
+
 // Units of a layer that does not fill the device, one per warp (see forward_split_kernel): first row * 8 + log2 of the groups of
 // lanes that share a row.  off: offsets of the slices of 16 rows; a step is 8 entries of a row; `rows`: rows a warp works on at once with
 // a group each; `slots`: warps that fit the device.  A slice's rows are split into as many parts as bring its steps down to the fewest

@@ -3524,21 +3524,15 @@ extern "C" int sdnn_infer_noalloc(int32_t n_layers, int32_t n_neurons, const int
         const float* val = values + layer_offset[l];
         const float* b = bias + (size_t)l * n_neurons;
 #define SDNN_NOALLOC(...) noalloc_forward_g<__VA_ARGS__>(st, rp, col, val, b, tile[cur], tile[cur ^ 1], n_neurons, ld, chunks, n_inputs, clamp, bad)
-        // Lanes per group, inputs per lane, entries of a group in flight per step, groups per row.  A launch of few rows is over when its
-        // longest row is: the row goes to as many groups as 2048 warps (the device's fill) leave room for; with one lane a group four
-        // pay at any size, eight up to 5000 rows.  us per layer of 24, 4096 rows of 8 to 56 entries (of 32 in brackets), one group / this:
-        // 4 inputs 6.9 / 2.8 (4.5 / 2.8), 8 inputs 7.8 / 3.0 (5.1 / 3.1), 16 inputs 5.3 / 3.4 (3.7 / 3.4), 32 inputs 5.2 / 4.2
-        // (3.9 / 3.4), 64 inputs 7.1 / 5.8 (5.4 / 4.4); 700 rows, 128 inputs 6.3 / 4.5 (4.9 / 3.4), 8 inputs 7.3 / 2.5.  More rows than that:
-        // 128 inputs, 4096 rows 8.5 with one group, 9.0 with two; 16 inputs, 16000 rows lanes of four inputs 8.2, two groups 8.4.
-        const int fill = 2048 * 32;      // lanes
-        const int groups = (int)std::min<int64_t>(8, fill / std::max<int64_t>(1, (int64_t)n_neurons * std::max(1, ld / chunks / 8)));
+        // lanes per group, inputs per lane, entries of a group in flight per step, groups per row
+        const sdnn_plan::CsrGroups g = sdnn_plan::csr_groups(n_neurons, sdnn_plan::csr_row(layer_offset, n_layers, l, n_neurons), ld / chunks, chunks);
         switch (ld / chunks) {
-            case 4: if (n_neurons <= 5120) SDNN_NOALLOC(1, 4, 8, 8); else SDNN_NOALLOC(1, 4, 8, 4); break;
-            case 8: if (n_neurons <= 5120) SDNN_NOALLOC(1, 8, 8, 8); else SDNN_NOALLOC(1, 8, 8, 4); break;
-            case 16: if (groups >= 8) SDNN_NOALLOC(2, 8, 8, 8); else if (groups >= 4) SDNN_NOALLOC(2, 8, 8, 4); else SDNN_NOALLOC(4, 4, 16, 1); break;
-            case 32: if (groups >= 8) SDNN_NOALLOC(4, 8, 8, 8); else if (groups >= 4) SDNN_NOALLOC(4, 8, 8, 4); else if (groups >= 2) SDNN_NOALLOC(4, 8, 8, 2); else SDNN_NOALLOC(4, 8, 8, 1); break;
-            case 64: if (groups >= 4) SDNN_NOALLOC(8, 8, 8, 4); else if (groups >= 2) SDNN_NOALLOC(8, 8, 8, 2); else SDNN_NOALLOC(8, 8, 8, 1); break;
-            default: if (groups >= 2) SDNN_NOALLOC(16, 8, 8, 2); else SDNN_NOALLOC(16, 8, 8, 1); break;
+            case 4: if (g.groups >= 8) SDNN_NOALLOC(1, 4, 8, 8); else SDNN_NOALLOC(1, 4, 8, 4); break;
+            case 8: if (g.groups >= 8) SDNN_NOALLOC(1, 8, 8, 8); else if (g.groups >= 4) SDNN_NOALLOC(1, 8, 8, 4); else SDNN_NOALLOC(1, 8, 8, 1); break;
+            case 16: if (g.groups >= 8) SDNN_NOALLOC(2, 8, 8, 8); else if (g.groups >= 4) SDNN_NOALLOC(2, 8, 8, 4); else SDNN_NOALLOC(4, 4, 16, 1); break;
+            case 32: if (g.groups >= 8) SDNN_NOALLOC(4, 8, 8, 8); else if (g.groups >= 4) SDNN_NOALLOC(4, 8, 8, 4); else if (g.groups >= 2) SDNN_NOALLOC(4, 8, 8, 2); else if (g.narrow) SDNN_NOALLOC(8, 4, 16, 1); else SDNN_NOALLOC(4, 8, 8, 1); break;
+            case 64: if (g.groups >= 4) SDNN_NOALLOC(8, 8, 8, 4); else if (g.groups >= 2) SDNN_NOALLOC(8, 8, 8, 2); else SDNN_NOALLOC(8, 8, 8, 1); break;
+            default: if (g.groups >= 2) SDNN_NOALLOC(16, 8, 8, 2); else SDNN_NOALLOC(16, 8, 8, 1); break;
         }
 #undef SDNN_NOALLOC
         cur ^= 1;

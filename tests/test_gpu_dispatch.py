@@ -814,3 +814,27 @@ def test_dead_inputs_dropped_after_new_weights(torch_cuda, n, cnt, launches):  #
     compare(True)
     dense.destroy()
     drop.destroy()
+
+
+@pytest.mark.parametrize("n,cnt,kmax", [(3000, 7, 16), (17000, 8, 40), (2000, 14, 30), (1500, 30, 24), (9201, 32, 24), (10999, 32, 60), (11001, 29, 60), (900, 50, 16), (700, 120, 14),
+                                        (1701, 200, 60), (900, 300, 40), (1699, 256, 60), (5200, 4, 12)])
+def test_allocation_free_call_with_short_rows(torch_cuda, n, cnt, kmax):  # noqa: F811
+    """One group of lanes a row for short rows and on either side of the other lines, of lanes of 4 and of 8 inputs; layers with a gap behind them and
+    a last one whose end the offsets do not tell."""
+    torch, pkg = torch_cuda, sdnn()
+    rng = np.random.default_rng(n + cnt)
+    rp, cols, vals, bias = ragged_net(rng, n=n, layers=3, kmax=kmax, scale=0.3)
+    at = [64]
+    for c in cols[:-1]:
+        at.append((at[-1] + len(c) + 3) // 4 * 4)
+    at[2] += 128
+    col, val = np.zeros(at[2] + len(cols[2]), dtype=np.int32), np.zeros(at[2] + len(cols[2]), dtype=np.float32)
+    for l in range(3):
+        col[at[l]:at[l] + len(cols[l])] = cols[l]
+        val[at[l]:at[l] + len(vals[l])] = vals[l]
+    x0 = vectors(rng, cnt, n)
+    got = torch.full((cnt, n), -1.0, device="cuda")
+    pkg.infer_noalloc(3, n, *(torch.from_numpy(a).cuda() for a in (np.stack(rp), col, val)), np.asarray(at, dtype=np.int64),
+                      torch.from_numpy(np.stack(bias)).cuda(), torch.from_numpy(x0).cuda(), cnt, got)
+    torch.cuda.synchronize()
+    check_close(got.cpu().numpy(), OracleNet(rp, cols, vals, bias).infer(x0), f"{n} neurons, {cnt} inputs")

@@ -17,6 +17,8 @@ extern "C" int cols(int cnt, long long elems, int windows) { return tile_shape(c
 extern "C" int chunk(int cnt, long long elems, int windows) { return tile_shape(cnt, elems, windows).cw; }
 extern "C" int graph(int layers, long long elems, int cols, int track) { return tile_as_graph(layers, elems, cols, track); }
 extern "C" int rows_log(int n, long long elems, int cw) { return split_rows(n, elems, cw, 148); }
+extern "C" int csr(int n, double per_row, int width, int chunks) { const CsrGroups g = csr_groups(n, per_row, width, chunks); return g.groups * 2 + g.narrow; }
+extern "C" double row_of(const int64_t* offset, int layers, int l, int n) { return csr_row(offset, layers, l, n); }
 extern "C" int call_log(int n, long long elems, int tile) { return call_rows(n, elems, tile, 148); }
 extern "C" int shared_chunk(int cnt, long long elems, int ls) { const TileShape t = tile_shape(cnt, elems, false, ls); return t.cw == t.cols ? t.cw : 0; }
 extern "C" int asks(long long bytes, int width) { return asks_ahead(bytes, width, 132644864); }
@@ -102,6 +104,22 @@ def test_rows_shared_in_inference(plan):
                 parts = 1 << plan.rows_log(n, n * per_row, cw)
                 assert parts == 1 or (cw // 8 * parts <= 32 and n * (cw // 8) * parts <= 65536 and parts * 8 <= per_row)
     assert plan.rows_log(700, 700 * 32, 64) == 2 and plan.rows_log(16384, 16384 * 32, 64) == 0
+
+
+def test_rows_of_allocation_free_calls(plan):
+    """Groups for every size, none for rows of a few entries; what the offsets say of a row, in any order of the layers, and what they don't."""
+    plan.csr.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_int, ctypes.c_int]
+    plan.row_of.restype = ctypes.c_double
+    for n in (1, 17, 700, 1699, 4096, 5121, 9201, 16385, 30000, 262144, 2**31 - 1):
+        for width, chunks in [(4, 1), (8, 1), (16, 1), (32, 1), (64, 1), (128, 1), (128, 2), (128, 3), (128, 8192)]:
+            for per_row in (0.0, 8.0, 12.0, 24.0, 32.0, 300.0):
+                groups = plan.csr(n, per_row, width, chunks) // 2
+                assert 0 <= groups <= 8 and (groups >= 4 if width == 4 else groups <= 1 or per_row >= 10)
+    assert plan.csr(4096, 32.0, 128, 1) // 2 == 1 and plan.csr(700, 32.0, 128, 1) // 2 == 5 and plan.csr(700, 8.0, 128, 1) // 2 == 1
+    offsets = (ctypes.c_int64 * 4)(0, 3200, 6400, 800)
+    assert [plan.row_of(offsets, 4, l, 100) for l in range(4)] == [32.0, 32.0, 32.0, 32.0]      # the third layer's end is not known: nor is the fourth's
+    offsets = (ctypes.c_int64 * 3)(0, 800, 2**62)
+    assert plan.row_of(offsets, 3, 0, 100) == 8.0 and plan.row_of(offsets, 3, 2, 100) > 1e15 and plan.row_of(offsets, 1, 0, 100) == 32.0
 
 
 def test_the_last_tile_of_a_call_shares_its_rows_like_the_others(plan):
