@@ -219,5 +219,9 @@ constexpr int RES_HALVES = 3072;      // most neurons
 inline int resident_half(int n, int64_t inputs, int sms) {
     return n <= RES_HALVES && inputs >= 8 && (inputs + 3) / 4 <= sms ? (int)((inputs + 7) / 8) * 4 : 0;
 }
+// ... and only where it pays: halves of up to 256 inputs are a single chunk of the layer launches, which wider nets then go through faster (time of
+// halves / of layer launches, 40 layers, equal rows: 2048 neurons, 450 inputs 1.20 (381 us in layer launches), 1800, 500 1.21, 2048, 550 0.90, 1024, 450 1.01,
+// 700, 450 0.89).
+inline int resident_half_pays(int n, int64_t inputs, int sms) { return inputs > 512 || n <= 1024 ? resident_half(n, inputs, sms) : 0; }
 
 }  // namespace sdnn_plan

@@ -2605,7 +2605,7 @@ int sdnn_infer_batch_host(sdnn_t* h, const float* x0, int64_t n_inputs, float* y
     // two input stages and a copy stream: the copy of tile t+1 runs under the layers of tile t
     const int T = host_tile_width(h, n_inputs);
     const bool halved = n_inputs > T && n_inputs <= h->cfg.max_batch;      // its pieces (two halves, or narrow tiles of a wide net) share the stages of one tile
-    const int first = halved ? resident_half(h->N, n_inputs, h->sms) : 0;  // inputs of the first half, where both go through whole networks
+    const int first = halved ? resident_half_pays(h->N, n_inputs, h->sms) : 0;  // inputs of the first half, where both go through whole networks
     const int tile = (int)std::min<int64_t>(n_inputs, T);
     const Route route = !halved ? route_of(h, tile, tile) : first ? route_of(h, n_inputs, T) : Route{0, call_rows(h->N, h->mean_elems, T, h->sms), false};
     const int64_t piece = halved && route.width ? first : T;               // inputs of each but the last

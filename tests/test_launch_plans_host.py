@@ -316,6 +316,7 @@ extern "C" void shape(int n, int p, int* out) {
 }
 extern "C" void share(int total, int sms, int p, int q, int* out) { resident_share(total, sms, p, q, out, out + 1); }
 extern "C" int half(int n, long long inputs, int sms) { return resident_half(n, inputs, sms); }
+extern "C" int pays(int n, long long inputs, int sms) { return resident_half_pays(n, inputs, sms); }
 // steps of a group: left[row][class] entries; read[step][row] = class, 8 + class of the zeros for a row that waits
 extern "C" void steps(int* left, int steps, int* read) {
     int total[8] = {};
@@ -384,6 +385,15 @@ def test_shares_of_networks_held_in_shared_memory(resident):
                     if q < p:
                         assert out[1] - out[0] <= 4 * q * sms
                 assert taken == list(range(total))
+
+
+def test_halves_of_single_chunks_stay_with_the_layer_launches(resident):
+    """Wider nets' halves of up to 256 inputs go through the layer launches, larger ones and those of narrow nets as before."""
+    resident.pays.argtypes = resident.half.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+    for n in (700, 1024, 1025, 2048, 3000, 4000):
+        for inputs in (7, 260, 300, 512, 513, 592, 593):
+            want = 0 if n > 1024 and inputs <= 512 else resident.half(n, inputs, 148)
+            assert resident.pays(n, inputs, 148) == want
 
 
 def test_widths_of_networks_held_in_shared_memory(resident):
